@@ -65,7 +65,7 @@ __host__ __device__ constexpr int mode_level(int m) { return mode_splat(m) ? (in
 
 template <int TILE, int STG, int MODE>
 __host__ __device__ __forceinline__ size_t warp_smem_bytes(int K) {
-    return (size_t)(TILE * TILE * (mode_fills(MODE) ? 2 : 1) + 32) * 4 + stage_bytes(STG, K, mode_level(MODE)) +
+    return (size_t)(TILE * TILE * (mode_fills(MODE) ? 2 : 1) + 64) * 4 + stage_bytes(STG, K, mode_level(MODE)) +
            (mode_splat(MODE) ? (size_t)STG * sizeof(SplatSlot) : 0);
 }
 
@@ -99,7 +99,8 @@ __global__ void __launch_bounds__(kRastWarps * 32) raster_kernel(const __grid_co
     uint32_t *s_cnt = reinterpret_cast<uint32_t *>(mine);   // [TILE*TILE] fragments so far
     uint32_t *s_base = s_cnt + TILE * TILE;                   // [TILE*TILE] record offsets (fill)
     uint32_t *s_nf = s_cnt + TILE * TILE * (FILL ? 2 : 1);    // [32] fragments per lane of a batch
-    char *stage_base = mine + (size_t)(TILE * TILE * (FILL ? 2 : 1) + 32) * 4;
+    uint32_t *s_map = s_nf + 32;                               // [32] staged fans that have tests
+    char *stage_base = mine + (size_t)(TILE * TILE * (FILL ? 2 : 1) + 64) * 4;
     const Stage S = stage_ptrs(stage_base, STG, K, LEVEL);
     SplatSlot *s_spl = reinterpret_cast<SplatSlot *>(stage_base + stage_bytes(STG, K, LEVEL));
     const int tx0 = (tile % tiles_x) * TILE, ty0 = (tile / tiles_x) * TILE;
@@ -184,15 +185,18 @@ __global__ void __launch_bounds__(kRastWarps * 32) raster_kernel(const __grid_co
             mbase = __shfl_sync(0xffffffffu, mbase, 0);
         }
         if (MODE == kFill) my_moff = pinf.x;
+        const uint32_t live = __ballot_sync(0xffffffffu, my_n != 0);   // staged fans with tests, in order
+        if (my_n) s_map[__popc(live & ((1u << lane) - 1u))] = (uint32_t)lane;
+        __syncwarp();
         uint32_t fan_hit = 0;   // count pass: bit f set when staged fan f covers some pixel centre
         for (int base = 0; base < total; base += 32) {
             const int idx = base + lane;
-            int f = 0;   // first lane (fan) whose inclusive count exceeds idx
-#pragma unroll
-            for (int step = 16; step > 0; step >>= 1) {
-                const int v = __shfl_sync(0xffffffffu, incl, f + step - 1);
-                if (v <= idx) f += step;
-            }
+            // the fan of each index: the fans with tests start one after another, so an index's
+            // fan is the last one that starts at or before it
+            const int before = __popc(__ballot_sync(0xffffffffu, my_n != 0 && excl < base));
+            const uint32_t here = my_n != 0 && excl >= base && excl < base + 32 ? 1u << (excl - base) : 0u;
+            const uint32_t starts = __reduce_or_sync(0xffffffffu, here);
+            const int f = (int)s_map[before + __popc(starts & (0xffffffffu >> (31 - lane))) - 1];
             const int fexcl = __shfl_sync(0xffffffffu, excl, f);
             const uint32_t fmoff = __shfl_sync(0xffffffffu, my_moff, f);
             const uint32_t fgeo = __shfl_sync(0xffffffffu, my_geo, f);
@@ -204,7 +208,7 @@ __global__ void __launch_bounds__(kRastWarps * 32) raster_kernel(const __grid_co
                 const int rx0 = tx0 + (int)(fgeo & 63u), ry0 = ty0 + (int)((fgeo >> 6) & 63u);
                 const int w = (int)((fgeo >> 12) & 63u) + 1, local = idx - fexcl;
                 // (local + 0.5) / w is at least 1/(2w) away from an integer: exact row
-                const int yy = (int)(((float)local + 0.5f) * (1.0f / (float)w));
+                const int yy = (int)__fdividef((float)local + 0.5f, (float)w);
                 px = rx0 + (local - yy * w);
                 py = ry0 + yy;
                 if (SPLAT)
