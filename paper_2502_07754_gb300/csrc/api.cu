@@ -155,7 +155,7 @@ RenderLayout render_layout(int64_t n_fans, int K, const ms_camera *cams, int n_v
     L.off_masks = o;             o = align_up(o + 2 * (size_t)L.mask_cap, 256);
     L.off_counts = o;            o = align_up(o + 4 * (size_t)npx, 256);
     L.off_offsets = o;           o = align_up(o + 4 * (size_t)npx, 256);
-    L.off_perm = o;              o = align_up(o + 8 * (size_t)npx, 256);   // forward, backward pixel orders
+    L.off_perm = o;              o = align_up(o + 8 * (size_t)npx, 256);   // pixel order (pixel, record offset)
     L.off_frags = o;             o = align_up(o + 16 * kRecFwd * (size_t)fcap, 256);
     L.off_adj = o;               o = align_up(o + 32 * (size_t)fcap, 256);   // adjoint records
     L.off_corder = o;            o = align_up(o + 4 * (size_t)fcap, 256);

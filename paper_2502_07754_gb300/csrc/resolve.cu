@@ -1,46 +1,47 @@
 // Per-pixel resolve of the fragment buffer: exact depth order and front-to-back
 // compositing (forward), and its adjoint (backward).
 //
-// One thread per pixel.  A pixel's fragment records sit contiguously in tile-list
-// order, i.e. sorted by their fans' depth bounds.  The thread streams them through a
-// small sorted register buffer: the front fragment is composited ("committed") once
-// the next record's depth bound exceeds it -- every later fragment lies at least that
-// deep, so the order is exact.  If the buffer overflows, the thread remembers the
-// nearest dropped fragment and the earliest record it dropped, finishes the pass with
-// everything strictly nearer, and re-reads its own records from that point, skipping
-// fragments at or before the last committed one.  Order: (depth, triangle id), the depth
-// a double-float value (high part in the record's first word, low part in its fourth).
+// A pixel's fragment records sit contiguously.  Order: (depth, triangle id), the depth a
+// double-float value (high part in the record's first word, low part in its fourth).
 // Compositing stops once the transmittance falls below T_eps.
 //
-// Both passes visit the pixels in orders that pixel_order_kernel builds after the pixel
-// scan (by fragment count), so a warp's lanes run loops of about the same length instead
-// of all waiting for the deepest pixel among 32 neighbours.
+// Pixels are resolved by groups of 8, 16 or 32 lanes, by their fragment count, one record a
+// lane: the records are read coalesced, a record's place is the number of records before it,
+// counted against the group's keys in shared memory, and the composite's products and sums run
+// over the sorted values in front-to-back order, each rounded as a sequential composite rounds
+// it.  A warp takes a deeper pixel alone: up to 64 records are placed at once and composited in
+// two rounds of 32; beyond that, every pass over the records keeps the 32 nearest beyond the last
+// composited one (merging 32 records at a time), so the order is exact for any depth complexity.
+// A round after the first counts as an extra pass.
+//
+// pixel_order_kernel sorts the pixels by descending fragment count after the pixel scan, so
+// that each class is one range of the order and a warp's groups run loops of about the same
+// length; it writes the background of pixels without fragments itself.  Warps take units of the
+// order in turn and fetch the next units' entries and counts while they work.
 //
 // The forward also records, per pixel, the record index of each committed fragment in
-// commit order.  The backward walks that list (no pending buffer, no re-reads), and at
+// commit order.  The backward walks that list (no sorting), and at
 // each committed fragment f forms, from the recomputed transmittance T_f,
 // dC/dc_f = T_f a_f, dC/da_f = T_f c_f - (C_out - C_{<=f}) / (1 - a_f) and
 // dA/da_f = T_out / (1 - a_f).  It writes dL/dc_f and dL/da_f, with the fragment's
 // triangle and pixel, as an adjoint record (the pixel's c-th composited fragment in slot
 // c of its record range); the chain pass (chain.cu) takes them to the vertices record by
 // record, so this pass does no atomics.
+//
+// What bounds them: the forward issues on about half of its cycles and waits on scattered
+// record reads otherwise (1M fans at 1080p, 10.4M fragments: 0.27 ms; one thread a pixel with a
+// sorted register buffer, 114 registers and 11 of 32 lanes active: 0.54 ms).  The backward
+// waits on its record reads.
 #include "raster_common.cuh"
 
 namespace ms {
 
 namespace {
 
-// Pixels differ widely in their fragment counts: small blocks let an SM refill the slots
-// of warps that finished early instead of holding them until the block's slowest warp.
-constexpr int kResolveThreads = 64;
-
 struct ResolveArgs {
-    int K;
     int64_t npx;
-    const uint32_t *counts, *offsets;
-    float4 *frags;
+    const float4 *frags;
     int64_t frag_cap;
-    int depth_bits;
     float T_eps, bg0, bg1, bg2;
     Status *st;
     float *tfinal;
@@ -48,19 +49,15 @@ struct ResolveArgs {
     float4 *adj;               // backward: per composited fragment, in commit order within the
                                // pixel's record range: (dL/dc * T a, dL/da), (triangle, pixel, 0, 0)
     uint32_t *corder;          // per pixel: record indices in commit order (same offsets as records)
-    const uint32_t *perm;      // visiting order of the pixels
-    const uint32_t *zrange;    // per view depth range of the keys' quantisation (bin.cu)
+    const uint2 *order;        // pixels with fragments, by descending count: (pixel, record offset)
+    const uint32_t *counts;
+    const uint32_t *hist;      // [kCountBuckets] pixels of each count
     ViewTable vt;
 };
 
-// Resolve orders, built after the pixel scan.  Forward: all pixels in descending order of
-// their fragment counts (a counting sort over the histogram the tile prefix gathered), so
-// the 32 lanes of a warp walk lists of about the same length and the deepest pixels
-// start first instead of trailing at the end of the grid.  Backward: the same sort within
-// spans of kOrderSpan consecutive pixels only: that pass does little arithmetic per
-// record and is bound by memory latency, and the pixels of one span (part of a row) have
-// their records in the regions of the row's tiles (records are laid out tile by tile).
-// The order within one count varies from run to run; no pixel's result depends on it.
+// Pixel order, built after the pixel scan: the pixels with fragments in descending order of
+// their counts (a counting sort over the counts' histogram).  The order within one count
+// varies from run to run; no pixel's result depends on it.
 constexpr int kOrderThreads = 256, kOrderItems = 4, kOrderSpan = kOrderThreads * kOrderItems;
 
 // Exclusive prefix of v over the buckets in descending order (thread t holds bucket 255 - t).
@@ -80,238 +77,426 @@ __device__ __forceinline__ uint32_t desc_prefix(uint32_t v, uint32_t *s_warp) {
     return before + x - v;
 }
 
-__global__ void __launch_bounds__(kOrderThreads) pixel_order_kernel(const uint32_t *__restrict__ counts, int64_t npx,
-                                                                    const uint32_t *__restrict__ hist,
+__global__ void __launch_bounds__(kOrderThreads) pixel_order_kernel(const uint32_t *__restrict__ offsets,
                                                                     uint32_t *__restrict__ fill,
-                                                                    uint32_t *__restrict__ perm_fwd,
-                                                                    uint32_t *__restrict__ perm_bwd) {
-    __shared__ uint32_t s_cnt[kCountBuckets], s_span[kCountBuckets], s_glob[kCountBuckets], s_warp[kOrderThreads / 32];
+                                                                    uint2 *__restrict__ order,
+                                                                    const __grid_constant__ ResolveArgs a) {
+    __shared__ uint32_t s_cnt[kCountBuckets], s_glob[kCountBuckets], s_warp[kOrderThreads / 32];
     static_assert(kOrderThreads == kCountBuckets, "one thread per bucket");
     const int tid = threadIdx.x;
     const int64_t base = (int64_t)blockIdx.x * kOrderSpan;
     const int mb = kCountBuckets - 1 - tid;   // this thread's bucket in the scans
     s_cnt[tid] = 0;
-    const uint32_t g0 = desc_prefix(hist[mb], s_warp);   // (its barriers also order the clear)
+    const uint32_t g0 = desc_prefix(a.hist[mb], s_warp);   // (its barriers also order the clear)
     int bk[kOrderItems];
     uint32_t rk[kOrderItems];
 #pragma unroll
     for (int i = 0; i < kOrderItems; ++i) {
         const int64_t p = base + i * kOrderThreads + tid;
-        bk[i] = -1;
+        bk[i] = 0;
         rk[i] = 0;
-        if (p < npx) {
-            bk[i] = count_bucket(counts[p]);
+        if (p >= a.npx) continue;
+        bk[i] = count_bucket(a.counts[p]);
+        if (bk[i]) {
             rk[i] = atomicAdd(&s_cnt[bk[i]], 1u);
+        } else {   // no fragments: the background
+            const ViewDev &vw = a.vt.v[view_of_pixel(a.vt, (unsigned long long)p)];
+            reinterpret_cast<float4 *>(vw.out)[p - (int64_t)vw.pix_base] = make_float4(a.bg0, a.bg1, a.bg2, 0.0f);
+            a.tfinal[p] = 1.0f;
+            a.ncommit[p] = 0;
         }
     }
     __syncthreads();
-    const uint32_t h = s_cnt[mb];
-    s_span[mb] = desc_prefix(h, s_warp);
+    const uint32_t h = mb ? s_cnt[mb] : 0u;
     s_glob[mb] = h ? g0 + atomicAdd(&fill[mb], h) : 0u;
     __syncthreads();
 #pragma unroll
     for (int i = 0; i < kOrderItems; ++i)
-        if (bk[i] >= 0) {
-            const uint32_t p = (uint32_t)(base + i * kOrderThreads + tid);
-            // both positions are < npx: the span and the histogram count each pixel once
-            const int64_t ps = base + s_span[bk[i]] + rk[i];
+        if (bk[i]) {
+            const int64_t p = base + i * kOrderThreads + tid;
+            // the position is < npx: the histogram counts each pixel once
             const int64_t pg = (int64_t)s_glob[bk[i]] + rk[i];
-            if (ps < npx) perm_bwd[ps] = p;
-            if (pg < npx) perm_fwd[pg] = p;
+            if (pg < a.npx) order[pg] = make_uint2((uint32_t)p, offsets[p]);
         }
 }
 
-// (depth, triangle) order of two fragments; depths are normalised double-float values,
-// so comparing (high, low) lexicographically compares their values.
-__device__ __forceinline__ bool frag_less(float za, float la, uint32_t ta, float zb, float lb, uint32_t tb) {
-    return za < zb || (za == zb && (la < lb || (la == lb && ta < tb)));
-}
-
-template <int KB>
-__global__ void __launch_bounds__(kResolveThreads) resolve_kernel(const __grid_constant__ ResolveArgs a) {
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t pt = t < a.npx ? (int64_t)a.perm[t] : a.npx;
-    const bool valid = pt < a.npx;
-    const int64_t pix = valid ? pt : 0;
-    const int view = view_of_pixel(a.vt, (unsigned long long)pix);
-    const ViewDev &vw = a.vt.v[view];
-    const int64_t lpix = pix - (int64_t)vw.pix_base;   // index within the view's image
-    int n = valid ? (int)a.counts[pix] : 0;
-    const int64_t off = a.offsets[pix];
-    if (off + n > a.frag_cap) n = 0;   // the buffer overflowed: reported through the status block
-    const DepthQ dq = depth_quant(a.zrange, view, a.depth_bits);
-    constexpr int RS = kRecFwd;   // float4s per record
-    float4 *rec = a.frags + (size_t)RS * off;
-
-    float T = 1.0f, C0 = 0.0f, C1 = 0.0f, C2 = 0.0f;
-    float kz[KB], kl[KB];      // pending fragments sorted by (depth, triangle): depth high, low
-    uint32_t kt[KB], ki[KB];   // triangle id, record index
-    float4 kc[KB];             // colour and opacity, read with the depth (one sector per record)
-    int nb = 0;
-    float fz = 0.0f, fl = 0.0f;   // last committed (depth, triangle); depths are > 0
-    uint32_t ft = 0;
-    bool has_front = false;
-    float dz = 0.0f, dl = 0.0f;   // nearest dropped fragment of this pass
-    uint32_t dt = 0;
-    bool dropped = false;
-    int restart = 0x7fffffff;
-    bool done = !valid;
-    uint32_t ncom = 0;
-
-    auto commit_front = [&]() {
-        // colour and opacity travel in the pending buffer: a commit waits on no load
-        const float4 col = kc[0];
-        const float al = col.w;
-        const float c0 = col.x, c1 = col.y, c2 = col.z;
-        const float w = T * al;
-        C0 += w * c0;
-        C1 += w * c1;
-        C2 += w * c2;
-        T *= (1.0f - al);
-        a.corder[off + ncom] = ki[0];
-        ++ncom;
-        fz = kz[0];
-        fl = kl[0];
-        ft = kt[0];
-        has_front = true;
-#pragma unroll
-        for (int i = 0; i + 1 < KB; ++i) {
-            kz[i] = kz[i + 1]; kl[i] = kl[i + 1]; kt[i] = kt[i + 1]; ki[i] = ki[i + 1]; kc[i] = kc[i + 1];
-        }
-        --nb;
-        if (T < a.T_eps) {
-            done = true;
-            nb = 0;
-        }
-    };
-
-    int start = 0;
-    while (!done) {
-        for (int i = start; i < n && !done; ++i) {
-            const float4 r0 = rec[RS * i];
-            const float4 r1 = rec[RS * i + 1];
-            const float z = r0.x, zl = r0.w;
-            const uint32_t tri = __float_as_uint(r0.y), qk = __float_as_uint(r0.z);
-            while (nb > 0 && !done && depth_qv(dq, kz[0]) < qk) commit_front();
-            if (done) break;
-            if (has_front && !frag_less(fz, fl, ft, z, zl, tri)) continue;   // committed in an earlier pass
-            if (dropped && !frag_less(z, zl, tri, dz, dl, dt)) {
-                restart = min(restart, i);
-                continue;
-            }
-            if (nb == KB) {
-                if (frag_less(z, zl, tri, kz[KB - 1], kl[KB - 1], kt[KB - 1])) {
-                    dz = kz[KB - 1];   // evict the deepest pending fragment
-                    dl = kl[KB - 1];
-                    dt = kt[KB - 1];
-                    dropped = true;
-                    restart = min(restart, (int)ki[KB - 1]);
-                    --nb;
-                } else {
-                    if (!dropped || frag_less(z, zl, tri, dz, dl, dt)) {
-                        dz = z;
-                        dl = zl;
-                        dt = tri;
-                    }
-                    dropped = true;
-                    restart = min(restart, i);
-                    continue;
-                }
-            }
-            bool placed = false;
-#pragma unroll
-            for (int s = KB - 1; s >= 1; --s) {
-                if (s <= nb && !placed) {
-                    if (frag_less(z, zl, tri, kz[s - 1], kl[s - 1], kt[s - 1])) {
-                        kz[s] = kz[s - 1]; kl[s] = kl[s - 1]; kt[s] = kt[s - 1]; ki[s] = ki[s - 1];
-                        kc[s] = kc[s - 1];
-                    } else {
-                        kz[s] = z; kl[s] = zl; kt[s] = tri; ki[s] = (uint32_t)i; kc[s] = r1;
-                        placed = true;
-                    }
-                }
-            }
-            if (!placed) {
-                kz[0] = z; kl[0] = zl; kt[0] = tri; ki[0] = (uint32_t)i; kc[0] = r1;
-            }
-            ++nb;
-        }
-        // End of pass: everything pending is nearer than anything dropped.
-        while (nb > 0 && !done) commit_front();
-        if (!dropped || done) break;
-        atomicAdd(&a.st->extra_passes, 1ull);
-        start = restart;
-        dropped = false;
-        restart = 0x7fffffff;
+// The work of the resolve kernels: warps take units of the pixel order in turn, a unit being
+// one pixel of more than 16 records, two of 9 to 16 or four of 1 to 8.
+constexpr int kGroupThreads = 256, kResident = 4;   // threads a block, blocks a multiprocessor
+struct Units {
+    uint32_t f16, f8, end;        // order positions: [0, n32) more than 16 records (the first `deep` more
+                                  // than 32), [n32, f16) 9 to 16, [f16, end) 1 to 8
+    uint32_t deep, n32, n16, n8;  // unit bounds of the classes
+    // Called by a whole block of kGroupThreads threads.
+    __device__ __forceinline__ Units(const uint32_t *__restrict__ hist, int64_t npx) {
+        static_assert(kGroupThreads == kCountBuckets, "one thread per bucket");
+        __shared__ uint32_t s_n[4];
+        if (threadIdx.x < 4) s_n[threadIdx.x] = 0;
+        __syncthreads();
+        const int b = threadIdx.x;
+        const uint32_t h = b ? hist[b] : 0u;
+        if (h) atomicAdd(&s_n[b > 32 ? 0 : (b > 16 ? 1 : (b > 8 ? 2 : 3))], h);
+        __syncthreads();
+        const uint32_t most = (uint32_t)npx;
+        deep = min(s_n[0], most);
+        n32 = min(deep + s_n[1], most);
+        f16 = min(n32 + s_n[2], most);
+        end = min(f16 + s_n[3], most);
+        n16 = n32 + (f16 - n32 + 1) / 2;
+        n8 = n16 + (end - f16 + 3) / 4;
     }
-    {
-        if (valid) {
-            reinterpret_cast<float4 *>(vw.out)[lpix] =
-                make_float4(C0 + T * a.bg0, C1 + T * a.bg1, C2 + T * a.bg2, 1.0f - T);
-            a.tfinal[pix] = T;
-            a.ncommit[pix] = ncom;
+    // This lane's entry of unit u (no pixel: ~0).
+    __device__ __forceinline__ uint2 entry(const ResolveArgs &a, int64_t u, int lane) const {
+        int64_t q = u;
+        uint32_t e0 = n32;
+        if (u >= n16) {
+            q = f16 + 4 * (u - n16) + (lane >> 3);
+            e0 = end;
+        } else if (u >= n32) {
+            q = n32 + 2 * (u - n32) + (lane >> 4);
+            e0 = f16;
         }
-        const unsigned r = __reduce_add_sync(0xffffffffu, ncom);
-        if ((threadIdx.x & 31) == 0) atomicAdd(&a.st->commits, (unsigned long long)r);
+        uint2 e = make_uint2(~0u, 0u);
+        if (u < n8 && q < e0) e = __ldg(a.order + q);
+        return e;
     }
+};
+
+// A pixel with its records: count 0 where there is none, or where they did not fit the buffer
+// (reported through the status block).
+struct Pixel {
+    uint32_t pix, off, n;
+};
+__device__ __forceinline__ Pixel pixel_of(const ResolveArgs &a, const uint2 e) {
+    Pixel p = {e.x, e.y, 0u};
+    if (e.x < (uint64_t)a.npx) p.n = __ldg(a.counts + e.x);
+    return p;
+}
+__device__ __forceinline__ bool is_pixel(const ResolveArgs &a, const Pixel &p) { return p.pix < (uint64_t)a.npx; }
+__device__ __forceinline__ bool fits(const ResolveArgs &a, const Pixel &p) {
+    return (int64_t)p.off + p.n <= a.frag_cap;
 }
 
-// Backward: replay the forward's committed fragments in their recorded order.
-__global__ void __launch_bounds__(kResolveThreads) resolve_bwd_kernel(const __grid_constant__ ResolveArgs a) {
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= a.npx) return;
-    const int64_t pix = a.perm[t];
-    if (pix >= a.npx) return;
+// Shared words of one warp: sort keys and ids by record, then the values in sorted places.
+struct GroupMem {
+    unsigned long long key[64];
+    float oma[64], w[64], c[3][64];   // 1 - opacity, T a, colour
+    uint32_t tri[64], src[64];        // tie-break id, record of each place
+};
+
+// Depths are positive: their bits order like their values; the low part (either sign, zeros
+// alike) maps to an unsigned order.
+__device__ __forceinline__ unsigned long long sort_key(const float4 &r0) {
+    const uint32_t lb = __float_as_uint(r0.w + 0.0f);
+    return (unsigned long long)__float_as_uint(r0.x) << 32 | ((lb & 0x80000000u) ? ~lb : (lb | 0x80000000u));
+}
+
+__device__ __forceinline__ void put(GroupMem &m, int at, bool has, const float4 &r1, uint32_t src) {
+    m.oma[at] = has ? 1.0f - r1.w : 1.0f;
+    m.w[at] = has ? r1.w : 0.0f;
+    m.c[0][at] = r1.x;
+    m.c[1][at] = r1.y;
+    m.c[2][at] = r1.z;
+    m.src[at] = src;
+}
+
+// Transmittance in front of place `sub` (T0 in front of place 0), multiplied front to back.
+__device__ __forceinline__ float front_product(const float *oma, int sub, int nmax, float T0) {
+    float T = T0;
+    const float4 *op = reinterpret_cast<const float4 *>(oma);
+    for (int i = 0; i < nmax; i += 4) {
+        const float4 o = op[i >> 2];
+        if (i < sub) T *= o.x;
+        if (i + 1 < sub) T *= o.y;
+        if (i + 2 < sub) T *= o.z;
+        if (i + 3 < sub) T *= o.w;
+    }
+    return T;
+}
+
+// Composites the n <= G sorted places from g0 on (n <= nmax for every group of the warp) behind
+// transmittance T and the sums C (this lane's channel: sub % 4, the fourth idle); sets T to the
+// transmittance behind them and returns the number composited before T < T_eps (ended then set).
+template <int G>
+__device__ __forceinline__ int composite(GroupMem &m, int g0, int at0, int n, int nmax, float T_eps, float &T, float &C,
+                                         bool &ended) {
+    const int sub = (threadIdx.x & 31) - g0;
+    const int at = at0 + sub;
+    const float Tl = front_product(m.oma + at0, sub, nmax, T);
+    const float Tn = Tl * m.oma[at];
+    const uint32_t low = (__ballot_sync(0xffffffffu, sub < n && Tn < T_eps) >> g0) &
+                         (G == 32 ? 0xffffffffu : (1u << (G & 31)) - 1u);
+    ended = low != 0u;
+    const int ncom = ended ? __ffs(low) : n;
+    m.w[at] = sub < ncom ? Tl * m.w[at] : 0.0f;
+    if (sub >= ncom) m.c[0][at] = m.c[1][at] = m.c[2][at] = 0.0f;
+    __syncwarp();
+    const int ch = min(sub & 3, 2);
+    const float4 *wp = reinterpret_cast<const float4 *>(m.w + at0);
+    const float4 *cp = reinterpret_cast<const float4 *>(m.c[ch] + at0);
+    for (int i = 0; i < nmax; i += 4) {
+        const float4 x = wp[i >> 2], y = cp[i >> 2];
+        C += x.x * y.x;
+        C += x.y * y.y;
+        C += x.z * y.z;
+        C += x.w * y.w;
+    }
+    const float Tf = __shfl_sync(0xffffffffu, Tn, g0 + max(ncom - 1, 0));
+    if (n > 0) T = Tf;
+    return ncom;
+}
+
+__device__ __forceinline__ void write_pixel(const ResolveArgs &a, uint32_t pix, float T, float C0, float C1, float C2,
+                                            uint32_t ncom) {
     const ViewDev &vw = a.vt.v[view_of_pixel(a.vt, (unsigned long long)pix)];
-    const int64_t lpix = pix - (int64_t)vw.pix_base;
-    const uint32_t n = a.ncommit[pix];
-    const int64_t off = a.offsets[pix];
-    const uint32_t nrec = a.counts[pix];
-    if (n < nrec && off + nrec <= a.frag_cap) {
-        // slots past the composited fragments carry a zero gradient (the chain pass reads
-        // every slot of the pixel's range)
-        for (uint32_t i = n; i < nrec; ++i) {
-            a.adj[2 * (off + i)] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            a.adj[2 * (off + i) + 1] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    reinterpret_cast<float4 *>(vw.out)[(int64_t)pix - (int64_t)vw.pix_base] =
+        make_float4(C0 + T * a.bg0, C1 + T * a.bg1, C2 + T * a.bg2, 1.0f - T);
+    a.tfinal[pix] = T;
+    a.ncommit[pix] = ncom;
+}
+
+// One warp's 32 / G pixels (e per group); returns the fragments composited (first lanes).
+template <int G>
+__device__ __forceinline__ uint32_t resolve_group(const ResolveArgs &a, GroupMem &m, const Pixel e) {
+    const int lane = threadIdx.x & 31, sub = lane & (G - 1), g0 = lane & ~(G - 1);
+    const bool valid = is_pixel(a, e);
+    const int64_t off = e.off;
+    const int n = fits(a, e) && e.n <= (uint32_t)G ? (int)e.n : 0;
+    const int nmax = __reduce_max_sync(0xffffffffu, n);
+    const bool has = sub < n;
+    float4 r0 = make_float4(0.f, 0.f, 0.f, 0.f), r1 = r0;
+    if (has) {
+        const float4 *rec = a.frags + (size_t)kRecFwd * (size_t)(off + sub);
+        r0 = rec[0];
+        r1 = rec[1];
+    }
+    const unsigned long long key = has ? sort_key(r0) : ~0ull;
+    __syncwarp();   // the words are still read for the previous unit
+    m.key[lane] = key;
+    __syncwarp();
+    int rank = 0;
+    const ulonglong2 *kp = reinterpret_cast<const ulonglong2 *>(m.key + g0);
+    for (int i = 0; i < nmax; i += 2) {
+        const ulonglong2 k = kp[i >> 1];
+        rank += (int)(k.x < key) + (int)(k.y < key);
+    }
+    // equal depths leave two records on one place: then the triangle id decides
+    const uint32_t placed = __reduce_or_sync(0xffffffffu, has ? 1u << (g0 + rank) : 0u);
+    if (placed != __ballot_sync(0xffffffffu, has)) {
+        const uint32_t tri = __float_as_uint(r0.y);
+        m.tri[lane] = tri;
+        __syncwarp();
+        rank = 0;
+        for (int i = 0; i < nmax; ++i) {
+            const unsigned long long k = m.key[g0 + i];
+            rank += (int)(k < key || (k == key && i < n && m.tri[g0 + i] < tri));
         }
     }
+    put(m, g0 + (has ? rank : sub), has, r1, (uint32_t)sub);   // (the other lanes fill the places past n)
+    __syncwarp();
+    float T = 1.0f, C = 0.0f;
+    bool ended;
+    const int ncom = composite<G>(m, g0, g0, n, nmax, a.T_eps, T, C, ended);
+    const float C1 = __shfl_sync(0xffffffffu, C, g0 + 1), C2 = __shfl_sync(0xffffffffu, C, g0 + 2);
+    if (valid && sub < ncom) a.corder[off + sub] = m.src[lane];
+    if (valid && sub == 0) write_pixel(a, e.pix, T, C, C1, C2, (uint32_t)ncom);
+    return valid && sub == 0 ? (uint32_t)ncom : 0u;
+}
+
+// Places two records a lane (keys ka, kb; ~0: none) among the warp's 64 by (key, id).
+__device__ __forceinline__ void place64(GroupMem &m, unsigned long long ka, uint32_t ta, unsigned long long kb,
+                                        uint32_t tb, int &ra, int &rb) {
+    const int lane = threadIdx.x & 31;
+    __syncwarp();
+    m.key[lane] = ka;
+    m.key[lane + 32] = kb;
+    m.tri[lane] = ta;
+    m.tri[lane + 32] = tb;
+    __syncwarp();
+    ra = rb = 0;
+    const ulonglong2 *kp = reinterpret_cast<const ulonglong2 *>(m.key);
+    for (int i = 0; i < 32; ++i) {
+        const ulonglong2 k = kp[i];
+        ra += (int)(k.x < ka) + (int)(k.y < ka);
+        rb += (int)(k.x < kb) + (int)(k.y < kb);
+    }
+    const bool ha = ka != ~0ull, hb = kb != ~0ull;
+    const int n = __popc(__ballot_sync(0xffffffffu, ha)) + __popc(__ballot_sync(0xffffffffu, hb));
+    const uint32_t p0 = __reduce_or_sync(0xffffffffu, (ha && ra < 32 ? 1u << ra : 0u) | (hb && rb < 32 ? 1u << rb : 0u));
+    const uint32_t p1 = __reduce_or_sync(0xffffffffu, (ha && ra >= 32 ? 1u << (ra - 32) : 0u) |
+                                                          (hb && rb >= 32 ? 1u << (rb - 32) : 0u));
+    if (__popc(p0) + __popc(p1) != n) {   // equal depths: the id decides
+        ra = rb = 0;
+        for (int i = 0; i < 64; ++i) {
+            const unsigned long long k = m.key[i];
+            const uint32_t t = m.tri[i];
+            ra += (int)(k < ka || (k == ka && t < ta));
+            rb += (int)(k < kb || (k == kb && t < tb));
+        }
+    }
+    __syncwarp();
+}
+
+// One warp's pixel of any number of records.
+__device__ uint32_t resolve_deep(const ResolveArgs &a, GroupMem &m, const Pixel e) {
+    const int lane = threadIdx.x & 31;
+    if (!is_pixel(a, e)) return 0;
+    const int64_t off = e.off;
+    const int n = fits(a, e) ? (int)e.n : 0;
+    const float4 *rec = a.frags + (size_t)kRecFwd * (size_t)off;
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    float T = 1.0f, C = 0.0f;
+    uint32_t ncom = 0, extra = 0;
+    bool ended = false;
+    if (n <= 64) {
+        const bool ha = lane < n, hb = lane + 32 < n;
+        const float4 a0 = ha ? rec[kRecFwd * lane] : zero, a1 = ha ? rec[kRecFwd * lane + 1] : zero;
+        const float4 b0 = hb ? rec[kRecFwd * (lane + 32)] : zero, b1 = hb ? rec[kRecFwd * (lane + 32) + 1] : zero;
+        int ra, rb;
+        place64(m, ha ? sort_key(a0) : ~0ull, __float_as_uint(a0.y), hb ? sort_key(b0) : ~0ull, __float_as_uint(b0.y),
+                ra, rb);
+        put(m, ha ? ra : lane, ha, a1, (uint32_t)lane);
+        put(m, hb ? rb : lane + 32, hb, b1, (uint32_t)lane + 32u);   // (places past n lie in the upper half)
+        __syncwarp();
+        for (int at = 0; at < n && !ended; at += 32) {
+            const int k = min(n - at, 32);
+            const int c = composite<32>(m, 0, at, k, k, a.T_eps, T, C, ended);
+            if (lane < c) a.corder[off + ncom + lane] = m.src[at + lane];
+            ncom += c;
+            extra += at ? 1u : 0u;
+        }
+    } else {
+        unsigned long long last_k = 0;   // the last composited record; depths are > 0
+        uint32_t last_t = 0;
+        for (bool more = true; more && !ended; extra += more && !ended) {
+            // the 32 nearest records beyond the last composited one
+            unsigned long long bk = ~0ull;
+            uint32_t bt = 0xffffffffu, bs = 0;
+            more = false;
+            for (int i0 = 0; i0 < n; i0 += 32) {
+                const int i = i0 + lane;
+                unsigned long long k = ~0ull;
+                uint32_t t = 0xffffffffu;
+                if (i < n) {
+                    const float4 r0 = rec[kRecFwd * i];
+                    const unsigned long long kk = sort_key(r0);
+                    const uint32_t tt = __float_as_uint(r0.y);
+                    if (kk > last_k || (kk == last_k && tt > last_t)) {
+                        k = kk;
+                        t = tt;
+                    }
+                }
+                int ra, rb;
+                place64(m, bk, bt, k, t, ra, rb);
+                // (records that are not there tie behind all others: they go past them in any order)
+                if (bk != ~0ull) { m.key[ra] = bk; m.tri[ra] = bt; m.src[ra] = bs; }
+                if (k != ~0ull) { m.key[rb] = k; m.tri[rb] = t; m.src[rb] = (uint32_t)i; }
+                const int live = __popc(__ballot_sync(0xffffffffu, bk != ~0ull)) + __popc(__ballot_sync(0xffffffffu, k != ~0ull));
+                more |= live > 32;
+                __syncwarp();
+                bk = lane < live ? m.key[lane] : ~0ull;
+                bt = lane < live ? m.tri[lane] : 0xffffffffu;
+                bs = lane < live ? m.src[lane] : 0u;
+            }
+            const bool has = bk != ~0ull;
+            const int k = __popc(__ballot_sync(0xffffffffu, has));
+            if (k == 0) break;
+            __syncwarp();
+            put(m, lane, has, has ? rec[kRecFwd * bs + 1] : zero, bs);
+            __syncwarp();
+            const int c = composite<32>(m, 0, 0, k, k, a.T_eps, T, C, ended);
+            if (lane < c) a.corder[off + ncom + lane] = bs;
+            ncom += c;
+            last_k = __shfl_sync(0xffffffffu, bk, k - 1);
+            last_t = __shfl_sync(0xffffffffu, bt, k - 1);
+        }
+    }
+    const float C1 = __shfl_sync(0xffffffffu, C, 1), C2 = __shfl_sync(0xffffffffu, C, 2);
+    if (lane == 0) {
+        write_pixel(a, e.pix, T, C, C1, C2, ncom);
+        if (extra) atomicAdd(&a.st->extra_passes, (unsigned long long)extra);
+    }
+    return lane == 0 ? ncom : 0u;
+}
+
+__global__ void __launch_bounds__(kGroupThreads, kResident) resolve_kernel(const __grid_constant__ ResolveArgs a) {
+    __shared__ __align__(16) GroupMem s_mem[kGroupThreads / 32];
+    const Units U(a.hist, a.npx);
+    GroupMem &m = s_mem[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31;
+    const int64_t warps = (int64_t)gridDim.x * (kGroupThreads / 32);
+    uint32_t ncom = 0;
+    int64_t u = (int64_t)blockIdx.x * (kGroupThreads / 32) + (threadIdx.x >> 5);
+    // entries are fetched two units ahead, counts one unit ahead
+    Pixel e1 = pixel_of(a, U.entry(a, u, lane));
+    uint2 e2 = U.entry(a, u + warps, lane);
+    for (; u < U.n8; u += warps) {
+        const Pixel e = e1;
+        e1 = pixel_of(a, e2);
+        e2 = U.entry(a, u + 2 * warps, lane);
+        if (u < U.deep)
+            ncom += resolve_deep(a, m, e);
+        else if (u < U.n32)
+            ncom += resolve_group<32>(a, m, e);
+        else if (u < U.n16)
+            ncom += resolve_group<16>(a, m, e);
+        else
+            ncom += resolve_group<8>(a, m, e);
+    }
+    ncom = __reduce_add_sync(0xffffffffu, ncom);
+    if (lane == 0 && ncom) atomicAdd(&a.st->commits, (unsigned long long)ncom);
+}
+
+// Backward, one thread a pixel in the pixel order (a warp's lanes run loops of about the same
+// length): no sorting is left, so a lane's sequential walk takes far fewer instructions than the
+// groups' prefix sums (measured: 0.26 against 0.34 ms on 10.4M fragments).  The walk waits on
+// its records, so the record after the next one's index and the next record load while the
+// current one is worked on.
+constexpr int kBwdThreads = 64;
+__global__ void __launch_bounds__(kBwdThreads) resolve_bwd_kernel(const __grid_constant__ ResolveArgs a) {
+    const int64_t q = (int64_t)blockIdx.x * kBwdThreads + threadIdx.x;
+    if (q >= a.npx - (int64_t)__ldg(a.hist)) return;   // (the order holds the pixels with fragments)
+    const Pixel e = pixel_of(a, __ldg(a.order + q));
+    if (!is_pixel(a, e) || !fits(a, e)) return;
+    const int64_t off = e.off;
+    const uint32_t n = min(a.ncommit[e.pix], e.n);
+    const float4 zero = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    float4 *adj = a.adj + 2 * off;
+    // slots past the composited fragments carry a zero gradient (the chain pass reads
+    // every slot of the pixel's range)
+    for (uint32_t i = n; i < e.n; ++i) adj[2 * i] = adj[2 * i + 1] = zero;
     if (n == 0) return;
+    const ViewDev &vw = a.vt.v[view_of_pixel(a.vt, (unsigned long long)e.pix)];
+    const int64_t lpix = (int64_t)e.pix - (int64_t)vw.pix_base;
     const float4 *rec = a.frags + (size_t)kRecFwd * off;
     const uint32_t *ord = a.corder + off;
     const float4 g = reinterpret_cast<const float4 *>(vw.dL)[lpix];
     const float4 ov = reinterpret_cast<const float4 *>(vw.out_fwd)[lpix];
-    const float Tout = a.tfinal[pix];
+    const float Tout = a.tfinal[e.pix];
     float T = 1.0f, C0 = 0.0f, C1 = 0.0f, C2 = 0.0f;
-    uint32_t idx = ord[0];
+    const uint32_t i0 = ord[0];
+    uint32_t i2 = n > 1 ? ord[1] : 0u;
+    float tri1 = rec[(size_t)kRecFwd * i0].y;
+    float4 col1 = rec[(size_t)kRecFwd * i0 + 1];
     for (uint32_t c = 0; c < n; ++c) {
-        const uint32_t nidx = c + 1 < n ? ord[c + 1] : 0u;   // the next index loads early
-        const float4 *rc = rec + (size_t)kRecFwd * idx;
-        const float4 r0 = rc[0];
-        const float4 col = rc[1];
+        const float tri = tri1;
+        const float4 col = col1;
+        if (c + 1 < n) {
+            tri1 = rec[(size_t)kRecFwd * i2].y;
+            col1 = rec[(size_t)kRecFwd * i2 + 1];
+        }
+        if (c + 2 < n) i2 = ord[c + 2];
         const float al = col.w;
         const float w = T * al;
         const float nC0 = C0 + w * col.x, nC1 = C1 + w * col.y, nC2 = C2 + w * col.z;
         const float inv = 1.0f / fmaxf(1.0f - al, 1e-6f);
         const float ga = g.x * (T * col.x - (ov.x - nC0) * inv) + g.y * (T * col.y - (ov.y - nC1) * inv) +
                          g.z * (T * col.z - (ov.z - nC2) * inv) + g.w * Tout * inv;
-        a.adj[2 * (off + c)] = make_float4(g.x * w, g.y * w, g.z * w, ga);
-        a.adj[2 * (off + c) + 1] = make_float4(r0.y, __uint_as_float((uint32_t)pix), 0.0f, 0.0f);
+        adj[2 * c] = make_float4(g.x * w, g.y * w, g.z * w, ga);
+        adj[2 * c + 1] = make_float4(tri, __uint_as_float(e.pix), 0.0f, 0.0f);
         C0 = nC0; C1 = nC1; C2 = nC2;
         T *= (1.0f - al);
-        idx = nidx;
     }
-}
-
-cudaError_t launch_k(const ResolveArgs &ra, bool backward, int kbuf, int64_t npx, cudaStream_t st) {
-    const unsigned grid = (unsigned)((npx + kResolveThreads - 1) / kResolveThreads);
-    if (npx == 0) return cudaSuccess;
-    if (backward)
-        resolve_bwd_kernel<<<grid, kResolveThreads, 0, st>>>(ra);
-    else if (kbuf == 16)
-        resolve_kernel<16><<<grid, kResolveThreads, 0, st>>>(ra);
-    else
-        resolve_kernel<8><<<grid, kResolveThreads, 0, st>>>(ra);
-    return cudaGetLastError();
 }
 
 __global__ void grad_scatter_kernel(const float4 *__restrict__ g, int64_t V, float *__restrict__ dx,
@@ -330,17 +515,14 @@ __global__ void grad_scatter_kernel(const float4 *__restrict__ g, int64_t V, flo
 
 }  // namespace
 
-cudaError_t launch_resolve(const RenderArgs &ra, bool backward, cudaStream_t st) {
+namespace {
+
+ResolveArgs make_args(const RenderArgs &ra) {
     const RenderLayout &L = ra.L;
     ResolveArgs a;
-    a.K = ra.K;
     a.npx = L.npx;
-    a.counts = reinterpret_cast<const uint32_t *>(ra.ws + L.off_counts);
-    a.offsets = reinterpret_cast<const uint32_t *>(ra.ws + L.off_offsets);
-    a.frags = reinterpret_cast<float4 *>(ra.ws + L.off_frags);
+    a.frags = reinterpret_cast<const float4 *>(ra.ws + L.off_frags);
     a.frag_cap = L.frag_cap;
-    a.depth_bits = L.depth_bits;
-    a.zrange = reinterpret_cast<const uint32_t *>(ra.ws + L.off_zrange);
     a.T_eps = ra.prm.T_eps;
     a.bg0 = ra.prm.bg[0];
     a.bg1 = ra.prm.bg[1];
@@ -350,19 +532,36 @@ cudaError_t launch_resolve(const RenderArgs &ra, bool backward, cudaStream_t st)
     a.ncommit = reinterpret_cast<uint32_t *>(ra.ws + L.off_ncommit);
     a.adj = reinterpret_cast<float4 *>(ra.ws + L.off_adj);
     a.corder = reinterpret_cast<uint32_t *>(ra.ws + L.off_corder);
-    a.perm = reinterpret_cast<const uint32_t *>(ra.ws + L.off_perm) + (backward ? L.npx : 0);
+    a.order = reinterpret_cast<const uint2 *>(ra.ws + L.off_perm);
+    a.counts = reinterpret_cast<const uint32_t *>(ra.ws + L.off_counts);
+    a.hist = reinterpret_cast<const uint32_t *>(ra.ws + L.off_pbucket);
     a.vt = ra.vt;
-    return launch_k(a, backward, L.kbuf, L.npx, st);
+    return a;
+}
+
+}  // namespace
+
+cudaError_t launch_resolve(const RenderArgs &ra, bool backward, cudaStream_t st) {
+    const RenderLayout &L = ra.L;
+    if (L.npx == 0) return cudaSuccess;
+    // the classes' sizes are known on the device only: a persistent grid of the resident blocks,
+    // at most one warp a pixel
+    const unsigned grid = (unsigned)min64((L.npx + kGroupThreads / 32 - 1) / (kGroupThreads / 32), 152 * kResident);
+    if (backward)
+        resolve_bwd_kernel<<<(unsigned)((L.npx + kBwdThreads - 1) / kBwdThreads), kBwdThreads, 0, st>>>(
+            make_args(ra));
+    else
+        resolve_kernel<<<grid, kGroupThreads, 0, st>>>(make_args(ra));
+    return cudaGetLastError();
 }
 
 cudaError_t launch_pixel_order(const RenderArgs &ra, cudaStream_t st) {
     const RenderLayout &L = ra.L;
     if (L.npx == 0) return cudaSuccess;
-    const uint32_t *hist = reinterpret_cast<const uint32_t *>(ra.ws + L.off_pbucket);
     uint32_t *fill = reinterpret_cast<uint32_t *>(ra.ws + L.off_pbucket) + kCountBuckets;
-    uint32_t *perm = reinterpret_cast<uint32_t *>(ra.ws + L.off_perm);
     pixel_order_kernel<<<(unsigned)((L.npx + kOrderSpan - 1) / kOrderSpan), kOrderThreads, 0, st>>>(
-        reinterpret_cast<const uint32_t *>(ra.ws + L.off_counts), L.npx, hist, fill, perm, perm + L.npx);
+        reinterpret_cast<const uint32_t *>(ra.ws + L.off_offsets), fill,
+        reinterpret_cast<uint2 *>(ra.ws + L.off_perm), make_args(ra));
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) count_launches(1);
     return e;
