@@ -814,19 +814,19 @@ MS_API ms_status ms_mlp_forward(const float *log_scales, const float *quats, con
     return MS_OK;
 }
 
-MS_API size_t ms_mlp_train_workspace_size(int64_t n) { return n < 0 ? 0 : mlp_act_bytes(n); }
+MS_API size_t ms_mlp_train_workspace_size(int64_t n) { return n < 0 ? 0 : mlp_train_bytes(n); }
 
 MS_API ms_status ms_mlp_grads(const float *X, const float *T, int64_t n, int32_t n_out, const void *packed,
                               float *grads, float *loss, void *workspace, size_t ws_bytes, void *stream) {
     if (n < 0 || n_out < 1 || n_out > 32) return fail(MS_ERR_INVALID, "bad n or n_out");
     if (!packed || !grads || !loss || (n > 0 && (!X || !T || !workspace))) return fail(MS_ERR_INVALID, "NULL pointer");
-    if (ws_bytes < mlp_act_bytes(n)) return fail(MS_ERR_INVALID, "workspace %zu < %zu", ws_bytes, mlp_act_bytes(n));
+    if (ws_bytes < mlp_train_bytes(n)) return fail(MS_ERR_INVALID, "workspace %zu < %zu", ws_bytes, mlp_train_bytes(n));
     if ((reinterpret_cast<uintptr_t>(packed) | reinterpret_cast<uintptr_t>(workspace)) & 255)
         return fail(MS_ERR_INVALID, "packed weights / workspace not 256-byte aligned");
-    cudaError_t e = launch_mlp_grads(X, T, n, n_out, static_cast<const char *>(packed), static_cast<char *>(workspace),
-                                     grads, loss, (cudaStream_t)stream);
+    cudaError_t e = launch_mlp_grads(X, T, n, n_out, static_cast<const char *>(packed), grads, loss,
+                                     (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(e, "mlp gradient launch");
-    if (n > 0) count_launches(2);
+    if (n > 0) count_launches(1);
     return MS_OK;
 }
 

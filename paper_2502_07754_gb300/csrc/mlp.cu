@@ -8,11 +8,11 @@
 //              (smem) -> Z2 -> H2 -> Z3 -> corrections (global FP32), or, fused, the
 //              conversion of each row's Gaussian with its corrections still in registers
 //              (the corrections never reach HBM).
-//   training   mlp_act_kernel: the same forward plus the activation adjoint of the mean
-//              squared error (dY, dZ2 = (dY W3^T) gelu'(Z2), dZ1 = (dZ2 W2^T) gelu'(Z1)),
-//              writing the per-tile operands of the weight gradients transposed;
-//              mlp_wgrad_kernel: dW1^T, dW2^T, dW3 summed over tiles in tensor memory
-//              (operands brought in by one bulk copy per tile), added atomically.
+//   training   mlp_train_kernel: persistent CTAs of 512 threads, one 128-row tile at a time:
+//              the same forward, the activation adjoint of the mean squared error (dY,
+//              dZ2 = (dY W3^T) gelu'(Z2), dZ1 = (dZ2 W2^T) gelu'(Z1)), and the weight
+//              gradients dW1^T, dW2^T, dW3 summed over the CTA's tiles in tensor memory, from
+//              the tile's operands where they lie (added atomically at the end).
 // Every product is BF16 x BF16 with FP32 accumulation; the bf16 rounding points are the
 // operands (inputs, weights, h1, h2, dy, dz2, dz1).  Weights are kept as FP32 masters and
 // packed to bf16 tiles in the canonical K-major layout of tc05.cuh.
@@ -41,15 +41,6 @@ constexpr uint32_t kW2b = kW3b + kHid * kOutPad * 2;    // [128 h1][128 h2]
 constexpr uint32_t kPackedBytes = kW2b + kHid * kHid * 2;
 constexpr uint32_t kStatusOff = kPackedBytes;           // uint32 timeouts, then pad
 constexpr uint32_t kPackedTotal = kPackedBytes + 256;
-
-// Per-tile operands of the weight gradients, [feature][row] K-major (K = the 128 rows).
-constexpr uint32_t kTXt = 0;                            // X^T   [16][128]
-constexpr uint32_t kTH1t = kTXt + kIn * kRows * 2;      // H1^T  [128][128]
-constexpr uint32_t kTH2t = kTH1t + kHid * kRows * 2;    // H2^T
-constexpr uint32_t kTdYt = kTH2t + kHid * kRows * 2;    // dY^T  [32][128]
-constexpr uint32_t kTdZ2t = kTdYt + kOutPad * kRows * 2;   // dZ2^T [128][128]
-constexpr uint32_t kTdZ1t = kTdZ2t + kHid * kRows * 2;     // dZ1^T [128][128]
-constexpr uint32_t kTileBytes = kTdZ1t + kHid * kRows * 2;
 
 // GELU x Phi(x) in binary32.  With z = |x| / sqrt 2 and E = erfc(z) / 2, Phi(x) is 1 - E
 // for x >= 0 and E for x < 0, written Phi = fma(1 - 2 step, E, step) with step = [x >= 0];
@@ -91,18 +82,7 @@ constexpr float kGeluT = 0.35355339059327376f;        // (1 / 2) / sqrt 2: t = 1
 constexpr float kGeluX2 = -0.72134752044448170f;      // -log2(e) / 2
 __device__ __forceinline__ float gelu_step(float x) { return x >= 0.0f ? 1.0f : 0.0f; }
 
-// Phi(x), one value (the derivative's first term).
-__device__ __forceinline__ float gelu_phi(float x) {
-    constexpr float c[] = {MS_GELU_POLY};
-    const float t = rcp_approx(fmaf(fabsf(x), kGeluT, 1.0f));
-    float q = c[kGeluDeg];
-#pragma unroll
-    for (int i = kGeluDeg - 1; i >= 0; --i) q = fmaf(q, t, c[i]);
-    const float E = t * ex2_approx(fmaf(x * x, kGeluX2, q));
-    const float st = gelu_step(x);
-    return fmaf(fmaf(st, -2.0f, 1.0f), E, st);
-}
-// GELU of a pair, in place; the same roundings as x * gelu_phi(x) for each value.
+// GELU of a pair, in place.
 __device__ __forceinline__ void gelu2(float &a, float &b) {
     constexpr float c[] = {MS_GELU_POLY};
     const uint64_t t = f2(rcp_approx(fmaf(fabsf(a), kGeluT, 1.0f)), rcp_approx(fmaf(fabsf(b), kGeluT, 1.0f)));
@@ -117,8 +97,24 @@ __device__ __forceinline__ void gelu2(float &a, float &b) {
     const uint64_t phi = fma2(fma2(st, f2(-2.0f, -2.0f), f2(1.0f, 1.0f)), E, st);
     unf2(mul2(x, phi), a, b);
 }
-__device__ __forceinline__ float gelu_grad(float x) {
-    return gelu_phi(x) + x * 0.39894228040143268f * __expf(-0.5f * x * x);
+// The same, with the derivative Phi(x) + x phi(x) of each value in da, db.
+__device__ __forceinline__ void gelu2_grad(float &a, float &b, float &da, float &db) {
+    constexpr float c[] = {MS_GELU_POLY};
+    const uint64_t t = f2(rcp_approx(fmaf(fabsf(a), kGeluT, 1.0f)), rcp_approx(fmaf(fabsf(b), kGeluT, 1.0f)));
+    const uint64_t x = f2(a, b);
+    uint64_t q = f2(c[kGeluDeg], c[kGeluDeg]);
+#pragma unroll
+    for (int i = kGeluDeg - 1; i >= 0; --i) q = fma2(q, t, f2(c[i], c[i]));
+    const uint64_t xx = mul2(x, x);
+    float ga, gb, ha, hb;
+    unf2(fma2(xx, f2(kGeluX2, kGeluX2), q), ga, gb);
+    unf2(mul2(xx, f2(kGeluX2, kGeluX2)), ha, hb);
+    const uint64_t E = mul2(t, f2(ex2_approx(ga), ex2_approx(gb)));
+    const uint64_t st = f2(gelu_step(a), gelu_step(b));
+    const uint64_t phi = fma2(fma2(st, f2(-2.0f, -2.0f), f2(1.0f, 1.0f)), E, st);
+    constexpr float k = 0.39894228040143268f;   // 1 / sqrt(2 pi)
+    unf2(fma2(mul2(x, f2(k, k)), f2(ex2_approx(ha), ex2_approx(hb)), phi), da, db);
+    unf2(mul2(x, phi), a, b);
 }
 __device__ __forceinline__ void gelu16(float v[16]) {
 #pragma unroll
@@ -222,11 +218,6 @@ __device__ __forceinline__ void raw_features(const MlpSrc &s, const char *row, f
     features_from(r[0], r[1], r[2], *reinterpret_cast<const float4 *>(row + 16), r[3], dc, f);
 }
 
-struct TcState {
-    uint64_t mbar;
-    uint32_t tmem;
-};
-
 // Issue the K-slices of one product D (+)= A B^T by thread 0 and commit it.
 __device__ __forceinline__ void issue(uint32_t d, const char *A, const char *B, int Kc, int N, bool acc_first,
                                       uint64_t *mbar) {
@@ -237,55 +228,13 @@ __device__ __forceinline__ void issue(uint32_t d, const char *A, const char *B, 
     if (mbar) tc::commit(mbar);
 }
 
-// Shared-memory operands were written: make them visible to the tensor cores, order
-// against earlier tensor-memory reads, and (thread 0) issue the product.
-__device__ __forceinline__ void sync_then(bool issuer) {
-    tc::fence_proxy_async();
-    tc::fence_before_sync();
-    __syncthreads();
-    if (issuer) tc::fence_after_sync();
-}
-
-// Every thread tracks the barrier's phase parity in its own register.
-__device__ __forceinline__ bool wait_mma(TcState *S, uint32_t &phase, uint32_t *timeouts) {
-    const bool ok = tc::mbar_wait(&S->mbar, phase, kTcWaitLimit);
-    phase ^= 1u;
-    if (!ok && threadIdx.x == 0) atomicAdd(timeouts, 1u);
-    tc::fence_after_sync();
-    return ok;
-}
-
-// Slot version: every thread of the slot waits on the slot's mbarrier.
-__device__ __forceinline__ bool wait_mma_slot(uint64_t *mbar, uint32_t &phase, uint32_t *timeouts, bool counter) {
+// Every thread that reads a product waits on its mbarrier and tracks the phase parity itself.
+__device__ __forceinline__ bool wait_mma(uint64_t *mbar, uint32_t &phase, uint32_t *timeouts, bool counter) {
     const bool ok = tc::mbar_wait(mbar, phase, kTcWaitLimit);
     phase ^= 1u;
     if (!ok && counter) atomicAdd(timeouts, 1u);
     tc::fence_after_sync();
     return ok;
-}
-
-// Shared prologue: weights into shared memory, barrier, tensor memory.
-__device__ __forceinline__ void setup(char *smem, const char *packed, uint32_t wbytes_lo, uint32_t wbytes_hi,
-                                      char *wdst, TcState *S, uint32_t ncols) {
-    const uint4 *src = reinterpret_cast<const uint4 *>(packed + wbytes_lo);
-    uint4 *dst = reinterpret_cast<uint4 *>(wdst);
-    for (uint32_t i = threadIdx.x; i < (wbytes_hi - wbytes_lo) / 16; i += blockDim.x) dst[i] = src[i];
-    if (threadIdx.x == 0) {
-        tc::mbar_init(&S->mbar, 1);
-        tc::mbar_init_fence();
-    }
-    if (threadIdx.x < 32) tc::tmem_alloc(&S->tmem, ncols);
-    tc::fence_before_sync();
-    __syncthreads();
-    tc::fence_after_sync();
-    (void)smem;
-}
-
-__device__ __forceinline__ void teardown(TcState *S, uint32_t ncols) {
-    tc::fence_before_sync();
-    __syncthreads();
-    tc::fence_after_sync();
-    if (threadIdx.x < 32) tc::tmem_dealloc(S->tmem, ncols);
 }
 
 // ------------------------------------------------------------------ inference
@@ -443,15 +392,15 @@ __global__ void __launch_bounds__(kFwdThreads, 1) mlp_fwd_kernel(const MlpSrc s,
             tc::fence_after_sync();
             issue(tz0, X, W1, kIn, kHid, false, mbar);
         }
-        ok = wait_mma_slot(mbar, phase, timeouts, issuer);
+        ok = wait_mma(mbar, phase, timeouts, issuer);
         gelu_cols64(tz, H, r, c0);
         slot_sync_then(slot, issuer);
         if (issuer) issue(tz0, H, W2, kHid, kHid, false, mbar);
-        ok = wait_mma_slot(mbar, phase, timeouts, issuer) && ok;
+        ok = wait_mma(mbar, phase, timeouts, issuer) && ok;
         gelu_cols64(tz, H, r, c0);   // the product has read H1: H2 replaces it
         slot_sync_then(slot, issuer);
         if (issuer) issue(tz0, H, W3, kHid, kOutPad, false, mbar);
-        ok = wait_mma_slot(mbar, phase, timeouts, issuer) && ok;
+        ok = wait_mma(mbar, phase, timeouts, issuer) && ok;
         float y[32];
         if (row_owner) {
             tc::tmem_ld16(tz, *reinterpret_cast<float(*)[16]>(y));
@@ -495,215 +444,219 @@ __global__ void __launch_bounds__(kFwdThreads, 1) mlp_fwd_kernel(const MlpSrc s,
     if (threadIdx.x < 32) tc::tmem_dealloc(*tmem_base, 128 * kSlots);
 }
 
-// ------------------------------------------------------------------ training: activations
+// ------------------------------------------------------------------ training
 
-constexpr uint32_t kAW = kW1f, kAWEnd = kPackedBytes;    // all five weight tiles
-constexpr uint32_t kAX = kAWEnd - kAW;                   // X  [128][16]
-constexpr uint32_t kAH1 = kAX + kRows * kIn * 2;         // H1, later dZ2 [128][128]
-constexpr uint32_t kAH2 = kAH1 + kRows * kHid * 2;       // H2
-constexpr uint32_t kAdY = kAH2 + kRows * kHid * 2;       // dY [128][32]
-constexpr uint32_t kAT = kAdY + kRows * kOutPad * 2;     // transpose staging [128][128]
-constexpr uint32_t kAState = kAT + kHid * kRows * 2;
-constexpr uint32_t kActSmem = kAState + 64;
+// One CTA of 16 warps per SM and one 128-row tile at a time.  Warp w reads tensor-memory lanes
+// 32 (w % 4) .. + 31 (rows) and a quarter (w / 4) of a product's columns; a thread keeps
+// gelu'(Z1) and gelu'(Z2) of its row and columns in registers between the forward and the
+// adjoint.  Every operand of the weight gradients is in shared memory as [row][feature] already,
+// which the tensor cores also take with the rows contracted (rowslice_desc), so nothing is
+// transposed, staged or written to HBM, and those products run under the next epilogue.
+// Tensor memory: 128 columns for the product in hand, 32 for Y, 176 for the three sums.
+// What bounds it: the chain of five products and their epilogues per tile (3907 tiles of 500k pairs
+// on 152 SMs); a tile's operands fill the shared memory, so one tile is in flight.  Measured on 500k
+// pairs, K = 8: 0.214 ms, against 0.515 ms for 128-thread CTAs that also wrote the weight gradients'
+// operands transposed (140 KB a tile) plus 0.098 ms for the kernel that read them back.
+constexpr int kTrainThreads = 512;
+constexpr uint32_t kTrX = 0;                               // X [128][16], two buffers
+constexpr uint32_t kTrH1 = kTrX + 2 * kRows * kIn * 2;     // H1 [128][128]
+constexpr uint32_t kTrH2 = kTrH1 + kRows * kHid * 2;       // H2, later dZ1
+constexpr uint32_t kTrdZ2 = kTrH2 + kRows * kHid * 2;      // dZ2
+constexpr uint32_t kTrdY = kTrdZ2 + kRows * kHid * 2;      // dY [128][32]
+constexpr uint32_t kTrW = kTrdY + kRows * kOutPad * 2;     // the five weight tiles
+constexpr uint32_t kTrState = kTrW + kPackedBytes;         // mbarrier, TMEM base
+constexpr uint32_t kTrainSmem = kTrState + 16;
+static_assert(kTrainSmem <= 227 * 1024, "shared memory");
+constexpr uint32_t kTmZ = 0, kTmY = 128, kTmD2 = 160, kTmD3 = 288, kTmD1 = 320, kTmCols = 512;
 
-// Writes column values v[0..n) of this thread's row r into the staging tile laid out as
-// [feature][row] (K = rows), at features f0..f0+n.
-__device__ __forceinline__ void stage_t(char *T, int r, int f0, const float *v, int n) {
-    for (int i = 0; i < n; ++i)
-        *reinterpret_cast<uint16_t *>(T + tc::cm_offset(f0 + i, r, kRows)) = bf16_bits(v[i]);
+// D (128 x N, sums) += A^T B over the tile's 128 rows: A has Ka features, B has N.
+__device__ __forceinline__ void issue_rows(uint32_t d, const char *A, int Ka, const char *B, int N, bool acc_first) {
+    const uint32_t id = tc::idesc_bf16_f32_mn(128, N);
+    const uint32_t a = tc::smem_u32(A), b = tc::smem_u32(B);
+    for (int s = 0; s < kRows / 16; ++s)
+        tc::mma_bf16(d, tc::rowslice_desc(a, Ka, s), tc::rowslice_desc(b, N, s), id, acc_first || s > 0);
 }
-// Copies `bytes` of the staging tile to global (all threads, after a barrier).
-__device__ __forceinline__ void flush_t(const char *T, char *dst, uint32_t bytes) {
-    __syncthreads();
-    const uint4 *s = reinterpret_cast<const uint4 *>(T);
-    uint4 *d = reinterpret_cast<uint4 *>(dst);
-    for (uint32_t i = threadIdx.x; i < bytes / 16; i += blockDim.x) d[i] = s[i];
-    __syncthreads();
-}
 
-__global__ void __launch_bounds__(128, 1) mlp_act_kernel(const float *__restrict__ Xin, const float *__restrict__ Tgt,
-                                                         int64_t n, int n_out, const char *__restrict__ packed,
-                                                         char *__restrict__ act, float *__restrict__ loss) {
+__global__ void __launch_bounds__(kTrainThreads, 1) mlp_train_kernel(const float *__restrict__ Xin,
+                                                                     const float *__restrict__ Tgt, int64_t n,
+                                                                     int n_out, const char *__restrict__ packed,
+                                                                     float *__restrict__ dW1, float *__restrict__ dW2,
+                                                                     float *__restrict__ dW3, float *__restrict__ loss) {
     extern __shared__ __align__(1024) char smem[];
-    TcState *S = reinterpret_cast<TcState *>(smem + kAState);
+    uint64_t *mbar = reinterpret_cast<uint64_t *>(smem + kTrState);
+    uint32_t *tmem_base = reinterpret_cast<uint32_t *>(smem + kTrState + 8);
     uint32_t *timeouts = reinterpret_cast<uint32_t *>(const_cast<char *>(packed) + kStatusOff);
-    setup(smem, packed, kAW, kAWEnd, smem, S, 512);
-    const char *W1 = smem + kW1f, *W2 = smem + kW2f, *W3 = smem + kW3f, *W3b = smem + kW3b, *W2b = smem + kW2b;
-    char *X = smem + kAX, *H1 = smem + kAH1, *H2 = smem + kAH2, *dY = smem + kAdY, *T = smem + kAT;
-    const int r = threadIdx.x, warp = r >> 5;
-    const uint32_t lo = (uint32_t)(warp * 32) << 16;
-    const uint32_t tZ1 = S->tmem, tZ2 = S->tmem + 128, tZ3 = S->tmem + 256, tdH2 = S->tmem + 384,
-                   tdH1 = S->tmem + 128;
+    {   // weights, barrier, tensor memory
+        const uint4 *src = reinterpret_cast<const uint4 *>(packed);
+        uint4 *dst = reinterpret_cast<uint4 *>(smem + kTrW);
+        for (uint32_t i = threadIdx.x; i < kPackedBytes / 16; i += blockDim.x) dst[i] = src[i];
+        if (threadIdx.x == 0) {
+            tc::mbar_init(mbar, 1);
+            tc::mbar_init_fence();
+        }
+        if (threadIdx.x < 32) tc::tmem_alloc(tmem_base, kTmCols);
+        tc::fence_before_sync();
+        __syncthreads();
+        tc::fence_after_sync();
+    }
+    const char *W1 = smem + kTrW + kW1f, *W2 = smem + kTrW + kW2f, *W3 = smem + kTrW + kW3f;
+    const char *W3b = smem + kTrW + kW3b, *W2b = smem + kTrW + kW2b;
+    char *H1 = smem + kTrH1, *H2 = smem + kTrH2, *dZ2 = smem + kTrdZ2, *dY = smem + kTrdY;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, cg = w >> 2;
+    const int r = 32 * (w & 3) + lane;   // row of the tile (tensor-memory lane)
+    const int c0 = 32 * cg;              // this thread's columns
+    const bool issuer = threadIdx.x == 0;
+    const uint32_t tm = *tmem_base, tl = tm + ((uint32_t)(32 * (w & 3)) << 16);
     const int64_t tiles = (n + kRows - 1) / kRows;
     const float dscale = 2.0f / ((float)n * (float)n_out);
-    float my_loss = 0.0f;
+    const bool xvec = (reinterpret_cast<uintptr_t>(Xin) & 15) == 0;
+    auto load_x = [&](int64_t t, float x[4]) {   // this thread's four inputs of a tile's row
+        const int64_t g = t * kRows + r;
+        if (t >= tiles || g >= n) {
+            x[0] = x[1] = x[2] = x[3] = 0.0f;
+        } else if (xvec) {
+            const float4 v = __ldg(reinterpret_cast<const float4 *>(Xin + g * kIn) + cg);
+            x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
+        } else {
+            for (int i = 0; i < 4; ++i) x[i] = __ldg(Xin + g * kIn + 4 * cg + i);
+        }
+    };
+    // operands were written: visible to the tensor cores, ordered after earlier tensor-memory reads
+    auto sync = [&]() {
+        tc::fence_proxy_async();
+        tc::fence_before_sync();
+        __syncthreads();
+        if (issuer) tc::fence_after_sync();
+    };
+    float my_loss = 0.0f, x[4];
     uint32_t phase = 0;
-    bool ok = true;
-    for (int64_t t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
+    bool ok = true, first = true;
+    int buf = 0;
+    load_x(blockIdx.x, x);
+    for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x, buf ^= 1) {
         const int64_t g = t * kRows + r;
         const bool live = g < n;
-        char *out = act + (size_t)t * kTileBytes;
-        float f[kIn];
-#pragma unroll
-        for (int i = 0; i < kIn; ++i) f[i] = live ? Xin[g * kIn + i] : 0.0f;
-        put8(X, kIn, r, 0, f);
-        put8(X, kIn, r, 8, f + 8);
-        stage_t(T, r, 0, f, kIn);
-        flush_t(T, out + kTXt, kIn * kRows * 2);
-        // forward
-        sync_then(r == 0);
-        if (r == 0) issue(tZ1, X, W1, kIn, kHid, false, &S->mbar);
-        ok = wait_mma(S, phase, timeouts) && ok;
-        for (int c0 = 0; c0 < kHid; c0 += 16) {
-            float v[16];
-            tc::tmem_ld16(tZ1 + lo + c0, v);
-            gelu16(v);
-            put8(H1, kHid, r, c0, v);
-            put8(H1, kHid, r, c0 + 8, v + 8);
-            stage_t(T, r, c0, v, 16);
-        }
-        flush_t(T, out + kTH1t, kHid * kRows * 2);
-        sync_then(r == 0);
-        if (r == 0) issue(tZ2, H1, W2, kHid, kHid, false, &S->mbar);
-        ok = wait_mma(S, phase, timeouts) && ok;
-        for (int c0 = 0; c0 < kHid; c0 += 16) {
-            float v[16];
-            tc::tmem_ld16(tZ2 + lo + c0, v);
-            gelu16(v);
-            put8(H2, kHid, r, c0, v);
-            put8(H2, kHid, r, c0 + 8, v + 8);
-            stage_t(T, r, c0, v, 16);
-        }
-        flush_t(T, out + kTH2t, kHid * kRows * 2);
-        sync_then(r == 0);
-        if (r == 0) issue(tZ3, H2, W3, kHid, kOutPad, false, &S->mbar);
-        ok = wait_mma(S, phase, timeouts) && ok;
-        {
-            float y[32];
-            tc::tmem_ld16(tZ3 + lo, *reinterpret_cast<float(*)[16]>(y));
-            tc::tmem_ld16(tZ3 + lo + 16, *reinterpret_cast<float(*)[16]>(y + 16));
-            for (int o = 0; o < kOutPad; ++o) {
-                float d = 0.0f;
-                if (live && o < n_out) {
-                    const float e = y[o] - Tgt[g * n_out + o];
-                    my_loss += e * e;
-                    d = dscale * e;
-                }
-                y[o] = d;
-            }
-            for (int c0 = 0; c0 < kOutPad; c0 += 8) put8(dY, kOutPad, r, c0, y + c0);
-            stage_t(T, r, 0, y, kOutPad);
-            flush_t(T, out + kTdYt, kOutPad * kRows * 2);
-        }
-        // adjoint: dH2 = dY W3^T, dZ2 = dH2 gelu'(Z2)
-        sync_then(r == 0);
-        if (r == 0) issue(tdH2, dY, W3b, kOutPad, kHid, false, &S->mbar);
-        ok = wait_mma(S, phase, timeouts) && ok;
-        for (int c0 = 0; c0 < kHid; c0 += 16) {
-            float z[16], d[16];
-            tc::tmem_ld16(tZ2 + lo + c0, z);
-            tc::tmem_ld16(tdH2 + lo + c0, d);
-            for (int i = 0; i < 16; ++i) d[i] *= gelu_grad(z[i]);
-            put8(H1, kHid, r, c0, d);          // H1's product finished: the buffer now holds dZ2
-            put8(H1, kHid, r, c0 + 8, d + 8);
-            stage_t(T, r, c0, d, 16);
-        }
-        flush_t(T, out + kTdZ2t, kHid * kRows * 2);
-        // dH1 = dZ2 W2^T, dZ1 = dH1 gelu'(Z1)
-        sync_then(r == 0);
-        if (r == 0) issue(tdH1, H1, W2b, kHid, kHid, false, &S->mbar);
-        ok = wait_mma(S, phase, timeouts) && ok;
-        for (int c0 = 0; c0 < kHid; c0 += 16) {
-            float z[16], d[16];
-            tc::tmem_ld16(tZ1 + lo + c0, z);
-            tc::tmem_ld16(tdH1 + lo + c0, d);
-            for (int i = 0; i < 16; ++i) d[i] *= gelu_grad(z[i]);
-            stage_t(T, r, c0, d, 16);
-        }
-        flush_t(T, out + kTdZ1t, kHid * kRows * 2);
+        char *X = smem + kTrX + buf * (kRows * kIn * 2);
+        // (the sums over the tile before last have read this buffer: a later product was waited for)
+        *reinterpret_cast<uint2 *>(X + tc::cm_offset(r, 4 * cg, kIn)) = make_uint2(pack2(x[0], x[1]), pack2(x[2], x[3]));
+        tc::fence_proxy_async();
         tc::fence_before_sync();
-        ok = __syncthreads_and(ok);
+        if (!__syncthreads_and(ok)) {
+            ok = false;
+            break;
+        }
+        if (issuer) {
+            tc::fence_after_sync();
+            issue(tm + kTmZ, X, W1, kIn, kHid, false, mbar);
+        }
+        load_x(t + gridDim.x, x);
+        float tv[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int o = 8 * cg + i;
+            tv[i] = live && o < n_out ? __ldg(Tgt + g * n_out + o) : 0.0f;
+        }
+        float g1[32], g2[32];
+        ok = wait_mma(mbar, phase, timeouts, issuer) && ok;   // (also: the last tile's sums are complete)
+#pragma unroll
+        for (int h = 0; h < 32; h += 16) {
+            float v[16];
+            tc::tmem_ld16(tl + kTmZ + c0 + h, v);
+#pragma unroll
+            for (int i = 0; i < 16; i += 2) gelu2_grad(v[i], v[i + 1], g1[h + i], g1[h + i + 1]);
+            put8(H1, kHid, r, c0 + h, v);
+            put8(H1, kHid, r, c0 + h + 8, v + 8);
+        }
+        sync();
+        if (issuer) issue(tm + kTmZ, H1, W2, kHid, kHid, false, mbar);
+        ok = wait_mma(mbar, phase, timeouts, issuer) && ok;
+#pragma unroll
+        for (int h = 0; h < 32; h += 16) {
+            float v[16];
+            tc::tmem_ld16(tl + kTmZ + c0 + h, v);
+#pragma unroll
+            for (int i = 0; i < 16; i += 2) gelu2_grad(v[i], v[i + 1], g2[h + i], g2[h + i + 1]);
+            put8(H2, kHid, r, c0 + h, v);
+            put8(H2, kHid, r, c0 + h + 8, v + 8);
+        }
+        sync();
+        if (issuer) issue(tm + kTmY, H2, W3, kHid, kOutPad, false, mbar);
+        ok = wait_mma(mbar, phase, timeouts, issuer) && ok;
+        {
+            float y[8];
+            tc::tmem_ld8(tl + kTmY + 8 * cg, y);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const float e = live && 8 * cg + i < n_out ? y[i] - tv[i] : 0.0f;
+                my_loss += e * e;
+                y[i] = dscale * e;
+            }
+            put8(dY, kOutPad, r, 8 * cg, y);
+        }
+        sync();
+        if (issuer) {
+            issue(tm + kTmZ, dY, W3b, kOutPad, kHid, false, mbar);           // dH2 = dY W3^T
+            issue_rows(tm + kTmD3, H2, kHid, dY, kOutPad, !first);           // dW3
+        }
+        ok = wait_mma(mbar, phase, timeouts, issuer) && ok;
+#pragma unroll
+        for (int h = 0; h < 32; h += 16) {
+            float v[16];
+            tc::tmem_ld16(tl + kTmZ + c0 + h, v);
+#pragma unroll
+            for (int i = 0; i < 16; ++i) v[i] *= g2[h + i];
+            put8(dZ2, kHid, r, c0 + h, v);
+            put8(dZ2, kHid, r, c0 + h + 8, v + 8);
+        }
+        sync();
+        if (issuer) {
+            issue(tm + kTmZ, dZ2, W2b, kHid, kHid, false, mbar);             // dH1 = dZ2 W2^T
+            issue_rows(tm + kTmD2, dZ2, kHid, H1, kHid, !first);             // dW2^T
+        }
+        ok = wait_mma(mbar, phase, timeouts, issuer) && ok;   // (dW3's product, issued before, has read H2)
+#pragma unroll
+        for (int h = 0; h < 32; h += 16) {
+            float v[16];
+            tc::tmem_ld16(tl + kTmZ + c0 + h, v);
+#pragma unroll
+            for (int i = 0; i < 16; ++i) v[i] *= g1[h + i];
+            put8(H2, kHid, r, c0 + h, v);
+            put8(H2, kHid, r, c0 + h + 8, v + 8);
+        }
+        sync();
+        if (issuer) issue_rows(tm + kTmD1, H2, kHid, X, kIn, !first);        // dW1^T
+        first = false;
     }
     for (int o = 16; o > 0; o >>= 1) my_loss += __shfl_xor_sync(0xffffffffu, my_loss, o);
-    if ((r & 31) == 0) atomicAdd(loss, my_loss / ((float)n * (float)n_out));
-    if (!ok) tc::mbar_wait(&S->mbar, phase, kTcWaitLimit);
-    teardown(S, 512);
-}
-
-// ------------------------------------------------------------------ training: weight gradients
-
-constexpr uint32_t kGState = kTileBytes;
-constexpr uint32_t kGradSmem = kGState + 64;
-
-__global__ void __launch_bounds__(128, 1) mlp_wgrad_kernel(const char *__restrict__ act, int64_t tiles, int n_out,
-                                                           uint32_t *timeouts, float *__restrict__ dW1,
-                                                           float *__restrict__ dW2, float *__restrict__ dW3) {
-    extern __shared__ __align__(1024) char smem[];
-    TcState *S = reinterpret_cast<TcState *>(smem + kGState);
-    __shared__ uint64_t load_bar;
-    if (threadIdx.x == 0) {
-        tc::mbar_init(&S->mbar, 1);
-        tc::mbar_init(&load_bar, 1);
-        tc::mbar_init_fence();
+    if (lane == 0) atomicAdd(loss, my_loss / ((float)n * (float)n_out));
+    if (ok) {
+        if (issuer) tc::commit(mbar);
+        ok = wait_mma(mbar, phase, timeouts, issuer);
+        if (ok && !first) {
+            float v[16], u[8];
+#pragma unroll
+            for (int h = 0; h < 32; h += 16) {   // row = h2 unit, columns = h1 units
+                tc::tmem_ld16(tl + kTmD2 + c0 + h, v);
+#pragma unroll
+                for (int i = 0; i < 16; ++i) atomicAdd(&dW2[(c0 + h + i) * kHid + r], v[i]);
+            }
+            tc::tmem_ld8(tl + kTmD3 + 8 * cg, u);   // row = h2 unit, columns = outputs
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                if (8 * cg + i < n_out) atomicAdd(&dW3[r * n_out + 8 * cg + i], u[i]);
+            if (cg == 0) {                           // row = h1 unit, columns = inputs
+                tc::tmem_ld16(tl + kTmD1, v);
+#pragma unroll
+                for (int i = 0; i < kIn; ++i) atomicAdd(&dW1[i * kHid + r], v[i]);
+            }
+        }
+    } else {
+        tc::mbar_wait(mbar, phase, kTcWaitLimit);   // let an unfinished product drain
     }
-    if (threadIdx.x < 32) tc::tmem_alloc(&S->tmem, 256);
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
-    const uint32_t tD1 = S->tmem, tD2 = S->tmem + 32, tD3 = S->tmem + 160;
-    uint32_t load_phase = 0, phase = 0;
-    bool ok = true, first = true;
-    for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
-        // one bulk copy brings the tile's six operands (all laid out K-major, K = rows)
-        if (threadIdx.x == 0) {
-            tc::mbar_expect_tx(&load_bar, kTileBytes);
-            const char *src = act + (size_t)t * kTileBytes;
-            const uint32_t parts[7] = {kTXt, kTH1t, kTH2t, kTdYt, kTdZ2t, kTdZ1t, kTileBytes};
-            for (int i = 0; i < 6; ++i) tc::bulk_g2s(smem + parts[i], src + parts[i], parts[i + 1] - parts[i], &load_bar);
-        }
-        const bool loaded = tc::mbar_wait(&load_bar, load_phase, kTcWaitLimit);
-        load_phase ^= 1u;
-        if (!__syncthreads_and(loaded)) {
-            if (threadIdx.x == 0) atomicAdd(timeouts, 1u);
-            // the copy may still land: wait for it once more before the smem is released
-            tc::mbar_wait(&load_bar, load_phase ^ 1u, kTcWaitLimit);
-            ok = false;
-            break;
-        }
-        if (threadIdx.x == 0) {
-            tc::fence_after_sync();
-            issue(tD1, smem + kTdZ1t, smem + kTXt, kRows, kIn, !first, nullptr);       // dW1^T
-            issue(tD2, smem + kTdZ2t, smem + kTH1t, kRows, kHid, !first, nullptr);     // dW2^T
-            issue(tD3, smem + kTH2t, smem + kTdYt, kRows, kOutPad, !first, &S->mbar);  // dW3
-        }
-        const bool done = wait_mma(S, phase, timeouts);
-        first = false;
-        if (!__syncthreads_and(done)) {
-            ok = false;
-            break;
-        }
-    }
-    if (ok && !first) {
-        const int r = threadIdx.x, warp = r >> 5;
-        const uint32_t lo = (uint32_t)(warp * 32) << 16;
-        float v[16];
-        tc::tmem_ld16(tD1 + lo, v);                    // row r = h1 unit, columns = inputs
-        for (int i = 0; i < kIn; ++i) atomicAdd(&dW1[i * kHid + r], v[i]);
-        for (int c0 = 0; c0 < kHid; c0 += 16) {         // row r = h2 unit, columns = h1 units
-            tc::tmem_ld16(tD2 + lo + c0, v);
-            for (int i = 0; i < 16; ++i) atomicAdd(&dW2[(c0 + i) * kHid + r], v[i]);
-        }
-        for (int c0 = 0; c0 < kOutPad; c0 += 16) {      // row r = h2 unit, columns = outputs
-            tc::tmem_ld16(tD3 + lo + c0, v);
-            for (int i = 0; i < 16; ++i)
-                if (c0 + i < n_out) atomicAdd(&dW3[r * n_out + c0 + i], v[i]);
-        }
-    }
-    if (!ok) tc::mbar_wait(&S->mbar, phase, kTcWaitLimit);   // let an unfinished product drain
-    tc::fence_before_sync();
-    __syncthreads();
-    tc::fence_after_sync();
-    if (threadIdx.x < 32) tc::tmem_dealloc(S->tmem, 256);
+    if (threadIdx.x < 32) tc::tmem_dealloc(tm, kTmCols);
 }
 
 // ------------------------------------------------------------------ packing and Adam
@@ -766,7 +719,7 @@ int sm_count() {
 }  // namespace
 
 size_t mlp_packed_bytes() { return kPackedTotal; }
-size_t mlp_act_bytes(int64_t n) { return (size_t)((n + kRows - 1) / kRows) * kTileBytes; }
+size_t mlp_train_bytes(int64_t n) { return n > 0 ? 256 : 0; }   // (the training kernel keeps its operands on chip)
 size_t mlp_param_count(int n_out) { return (size_t)kIn * kHid + (size_t)kHid * kHid + (size_t)kHid * n_out; }
 uint32_t mlp_status_offset() { return kStatusOff; }
 
@@ -831,20 +784,18 @@ cudaError_t launch_mesh_build_mlp(const float *means, const MlpSrc &s, int64_t N
     }
 }
 
-cudaError_t launch_mlp_grads(const float *X, const float *T, int64_t n, int n_out, const char *packed, char *act,
-                             float *grads, float *loss, cudaStream_t st) {
+cudaError_t launch_mlp_grads(const float *X, const float *T, int64_t n, int n_out, const char *packed, float *grads,
+                             float *loss, cudaStream_t st) {
     const size_t np = mlp_param_count(n_out);
     cudaError_t e = cudaMemsetAsync(grads, 0, np * sizeof(float), st);
     if (e == cudaSuccess) e = cudaMemsetAsync(loss, 0, sizeof(float), st);
     if (e != cudaSuccess || n == 0) return e;
     const int64_t tiles = (n + kRows - 1) / kRows;
     const int grid = (int)min64(tiles, sm_count());
-    cudaFuncSetAttribute(mlp_act_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kActSmem);
-    mlp_act_kernel<<<grid, 128, kActSmem, st>>>(X, T, n, n_out, packed, act, loss);
-    cudaFuncSetAttribute(mlp_wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGradSmem);
-    uint32_t *timeouts = reinterpret_cast<uint32_t *>(const_cast<char *>(packed) + kStatusOff);
-    mlp_wgrad_kernel<<<grid, 128, kGradSmem, st>>>(act, tiles, n_out, timeouts, grads, grads + kIn * kHid,
-                                                   grads + kIn * kHid + kHid * kHid);
+    e = cudaFuncSetAttribute(mlp_train_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTrainSmem);
+    if (e != cudaSuccess) return e;
+    mlp_train_kernel<<<grid, kTrainThreads, kTrainSmem, st>>>(X, T, n, n_out, packed, grads, grads + kIn * kHid,
+                                                              grads + kIn * kHid + kHid * kHid, loss);
     return cudaGetLastError();
 }
 

@@ -70,7 +70,7 @@ struct MlpSrc {
     int sh_dtype, sh_degree;
 };
 size_t mlp_packed_bytes();
-size_t mlp_act_bytes(int64_t n);
+size_t mlp_train_bytes(int64_t n);
 size_t mlp_param_count(int n_out);
 uint32_t mlp_status_offset();
 cudaError_t launch_mlp_pack(const float *W1, const float *W2, const float *W3, int n_out, char *packed,
@@ -81,8 +81,8 @@ cudaError_t launch_mlp_forward(const MlpSrc &s, int64_t N, const char *packed, i
 // The conversion fused behind the initializer's inference (flat fans, n_out = 2(K+1)).
 cudaError_t launch_mesh_build_mlp(const float *means, const MlpSrc &s, int64_t N, const char *packed,
                                   const MeshBuildConst &kc, float *xyz, float *rgb, float *alpha, cudaStream_t st);
-cudaError_t launch_mlp_grads(const float *X, const float *T, int64_t n, int n_out, const char *packed, char *act,
-                             float *grads, float *loss, cudaStream_t st);
+cudaError_t launch_mlp_grads(const float *X, const float *T, int64_t n, int n_out, const char *packed, float *grads,
+                             float *loss, cudaStream_t st);
 cudaError_t launch_mlp_adam(float *W, const float *grads, float *m, float *v, int n_out, int32_t *d_step, float lr,
                             float b1, float b2, float eps, char *packed, cudaStream_t st);
 

@@ -38,9 +38,23 @@ __device__ __forceinline__ uint64_t kslice_desc(uint32_t tile_saddr, int Kc, int
     return smem_desc(tile_saddr + (uint32_t)s * 256u, 128u, (uint32_t)(Kc >> 3) * 128u);
 }
 
+// The same tile, [row][feature] as above, as the operand of a product that contracts over the
+// rows (features are the M or N dimension, contiguous: "MN-major"): the slice of rows
+// [16 s, 16 s + 16).  Core matrices follow each other at 128 bytes along the features and at
+// (Kc / 8) * 128 along the rows.
+__device__ __forceinline__ uint64_t rowslice_desc(uint32_t tile_saddr, int Kc, int s) {
+    const uint32_t row_group = (uint32_t)(Kc >> 3) * 128u;
+    return smem_desc(tile_saddr + (uint32_t)s * 2u * row_group, row_group, 128u);
+}
+
 // Instruction descriptor of kind::f16 with BF16 A and B, FP32 D, both K-major.
 __host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+}
+
+// The same with both operands MN-major (rowslice_desc).
+__host__ __device__ constexpr uint32_t idesc_bf16_f32_mn(int M, int N) {
+    return idesc_bf16_f32(M, N) | (1u << 15) | (1u << 16);
 }
 
 __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
@@ -92,6 +106,17 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+// 8 consecutive FP32 columns.
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
+    uint32_t r[8];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
 }
 
 // ------------------------------------------------------------------ mbarrier
