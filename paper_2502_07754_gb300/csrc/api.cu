@@ -257,7 +257,7 @@ static ms_status render_views(const float *xyz, const float *rgb, const float *a
     {
         StageScope sc(MS_STAGE_RASTER, st);
         if ((e = launch_raster_count(a, st)) != cudaSuccess) return cuda_fail(e, "raster count launch");
-        if ((e = launch_raster(a, true, st)) != cudaSuccess) return cuda_fail(e, "raster fill launch");
+        if ((e = launch_fill(a, st)) != cudaSuccess) return cuda_fail(e, "raster fill launch");
         if ((e = launch_resolve(a, false, st)) != cudaSuccess) return cuda_fail(e, "resolve launch");
     }
     if (n_fans > 0) count_launches(1 + 3 + L.passes);
@@ -346,7 +346,7 @@ static ms_status splat_views(const float *means, const float *log_scales, const 
     if ((e = launch_bin(a, st)) != cudaSuccess) return cuda_fail(e, "bin launch");
     if ((e = launch_sort(a, st)) != cudaSuccess) return cuda_fail(e, "sort launch");
     if ((e = launch_raster_count(a, st)) != cudaSuccess) return cuda_fail(e, "splat count launch");
-    if ((e = launch_raster(a, true, st)) != cudaSuccess) return cuda_fail(e, "splat fill launch");
+    if ((e = launch_splat_fill(a, st)) != cudaSuccess) return cuda_fail(e, "splat fill launch");
     if ((e = launch_resolve(a, false, st)) != cudaSuccess) return cuda_fail(e, "resolve launch");
     if (N > 0) count_launches(2 + 3 + L.passes);
     count_launches(1);

@@ -102,7 +102,8 @@ cudaError_t sort_u64(unsigned long long *a, unsigned long long *b, int64_t n, in
                      cudaStream_t st, unsigned long long **result);
 constexpr int kItemFans = 64;   // fans per raster work item
 
-cudaError_t launch_raster(const RenderArgs &a, bool fill, cudaStream_t st);
+cudaError_t launch_fill(const RenderArgs &a, cudaStream_t st);         // fragment records of the fans
+cudaError_t launch_splat_fill(const RenderArgs &a, cudaStream_t st);   // fragment records of the source Gaussians
 cudaError_t launch_raster_count(const RenderArgs &a, cudaStream_t st);   // items, count, prefix, pixel scan
 cudaError_t launch_record_chain(const RenderArgs &a, cudaStream_t st);   // adjoint: records -> fan vertices
 constexpr int kRecFwd = 2;   // float4s per fragment record

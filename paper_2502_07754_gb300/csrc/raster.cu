@@ -13,10 +13,10 @@
 // when the pair covers no pixel centre, so the fill skips it).  A
 // per-tile prefix over the tile's items turns the counts into each item's starting slot
 // within the pixel and gives the pixel totals; an exclusive scan over pixels gives record
-// offsets.  Fill pass: the same walk, reading the stored masks and rectangles instead of
-// staging the decisions and testing again, writes one 32-byte record per fragment at offset + item slot + running
-// index -- depth (high), triangle id, the fan's depth bound, depth (low), colour, opacity -- so a
-// pixel's records come out in tile-list order, which the resolve relies on.
+// offsets.  The fill pass (fill.cu) walks the same items with the stored masks and rectangles
+// and writes the records.
+#include <algorithm>
+
 #include "raster_common.cuh"
 
 namespace ms {
@@ -43,7 +43,8 @@ struct RastArgs {
                                // pixel rectangle clipped to the tile (pair_geo; 0 if empty)
     uint16_t *masks;           // coverage masks (bit j: triangle j) of the count pass's tests
     int64_t mask_cap;
-    uint32_t *mask_cursor;     // [kMaskRegions] fill levels of the mask regions (zeroed per render)
+    uint32_t mask_regions;
+    uint32_t *mask_cursor;     // [mask_regions] fill levels of the mask regions (zeroed per render)
 };
 
 constexpr int kRastWarps = 2;   // warps (work items) per block: items differ widely in cost
@@ -54,18 +55,17 @@ __device__ __forceinline__ uint32_t pair_geo(int rx0, int ry0, int w, int h) {
     return 0x80000000u | (uint32_t)rx0 | (uint32_t)ry0 << 6 | (uint32_t)(w - 1) << 12 | (uint32_t)(h - 1) << 18;
 }
 
-// Pass kinds: count fragments; fill their 32-byte forward records.  The splat passes draw
+// Pass kinds: count the fans' fragments (fill.cu writes their records).  The splat passes draw
 // the source Gaussians themselves (count, then 32-byte records) over the tile lists of
 // their circumscribing polygons.
-enum RasterMode { kCount = 0, kFill = 1, kSplatCount = 3, kSplatFill = 4 };
+enum RasterMode { kCount = 0, kSplatCount = 3, kSplatFill = 4 };
 
-__host__ __device__ constexpr bool mode_fills(int m) { return m == kFill || m == kSplatFill; }
+__host__ __device__ constexpr bool mode_fills(int m) { return m == kSplatFill; }
 __host__ __device__ constexpr bool mode_splat(int m) { return m >= kSplatCount; }
-__host__ __device__ constexpr int mode_level(int m) { return mode_splat(m) ? (int)kStageDecide : m; }
 
 template <int TILE, int STG, int MODE>
 __host__ __device__ __forceinline__ size_t warp_smem_bytes(int K) {
-    return (size_t)(TILE * TILE * (mode_fills(MODE) ? 2 : 1) + 64) * 4 + stage_bytes(STG, K, mode_level(MODE)) +
+    return (size_t)(TILE * TILE * (mode_fills(MODE) ? 2 : 1) + 64) * 4 + stage_bytes(STG, K) +
            (mode_splat(MODE) ? (size_t)STG * sizeof(SplatSlot) : 0);
 }
 
@@ -73,7 +73,6 @@ template <int TILE, int STG, int KT, int MODE>
 __global__ void __launch_bounds__(kRastWarps * 32) raster_kernel(const __grid_constant__ RastArgs a) {
     constexpr bool FILL = mode_fills(MODE);   // passes that address records
     constexpr bool SPLAT = mode_splat(MODE);
-    constexpr int LEVEL = mode_level(MODE);
     extern __shared__ __align__(16) char smem[];
     const int K = KT > 0 ? KT : a.K;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -101,8 +100,8 @@ __global__ void __launch_bounds__(kRastWarps * 32) raster_kernel(const __grid_co
     uint32_t *s_nf = s_cnt + TILE * TILE * (FILL ? 2 : 1);    // [32] fragments per lane of a batch
     uint32_t *s_map = s_nf + 32;                               // [32] staged fans that have tests
     char *stage_base = mine + (size_t)(TILE * TILE * (FILL ? 2 : 1) + 64) * 4;
-    const Stage S = stage_ptrs(stage_base, STG, K, LEVEL);
-    SplatSlot *s_spl = reinterpret_cast<SplatSlot *>(stage_base + stage_bytes(STG, K, LEVEL));
+    const Stage S = stage_ptrs(stage_base, STG, K);
+    SplatSlot *s_spl = reinterpret_cast<SplatSlot *>(stage_base + stage_bytes(STG, K));
     const int tx0 = (tile % tiles_x) * TILE, ty0 = (tile / tiles_x) * TILE;
     const int tx1 = min(tx0 + TILE, sc.W) - 1, ty1 = min(ty0 + TILE, sc.H) - 1;
     uint32_t *icnt = a.icnt + (size_t)item * TILE * TILE;
@@ -124,11 +123,6 @@ __global__ void __launch_bounds__(kRastWarps * 32) raster_kernel(const __grid_co
     __syncwarp();
     for (uint32_t cb = it.y; cb < it.z; cb += STG) {
         const int cnt = (int)min((uint32_t)STG, it.z - cb);
-        // The fill pass takes a chunk whose pairs all have their masks stored without the
-        // decision stage: the count pass left each pair's rectangle beside its mask index.
-        uint2 pinf = make_uint2(~0u, 0u);
-        if (MODE == kFill && lane < cnt) pinf = __ldg(a.pinfo + cb + lane);
-        const bool stored = MODE == kFill && __all_sync(0xffffffffu, lane >= cnt || pinf.x != ~0u);
         {
             constexpr int LPF = 32 / STG;   // lanes staging one fan
             const int slot = lane / LPF;
@@ -139,10 +133,7 @@ __global__ void __launch_bounds__(kRastWarps * 32) raster_kernel(const __grid_co
                 q = (uint32_t)((e >> a.fan_bits) & ((1ull << a.depth_bits) - 1ull));
                 fan = (uint32_t)(e & ((1ull << a.fan_bits) - 1ull));
             }
-            // a stored chunk skips the values of pairs that the count pass found without any
-            // covered pixel centre (their rectangle word is 0)
-            const uint32_t sgeo = __shfl_sync(0xffffffffu, pinf.y, slot);
-            stage_fans<LPF>(sc, S, K, lane, slot < cnt && (!stored || sgeo != 0u), fan, q, LEVEL, !stored);
+            stage_fans<LPF>(sc, S, K, lane, slot < cnt, fan, q);
             if (SPLAT && lane < cnt)
                 s_spl[lane] = splat_setup(a.spl, *sc.cam,
                                           (uint32_t)(__ldg(a.keys + cb + lane) & ((1ull << a.fan_bits) - 1ull)));
@@ -152,9 +143,7 @@ __global__ void __launch_bounds__(kRastWarps * 32) raster_kernel(const __grid_co
         // index space, fan-major, so every lane tests a pixel even when fans are tiny.
         int my_n = 0;
         uint32_t my_geo = 0;
-        if (stored) {
-            my_geo = pinf.y;
-        } else if (lane < cnt) {
+        if (lane < cnt) {
             const int4 r = S.rect[lane];
             const int rx0 = max(r.x, tx0), rx1 = min(r.y, tx1), ry0 = max(r.z, ty0), ry1 = min(r.w, ty1);
             if (S.flags[lane] != 0 && rx0 <= rx1 && ry0 <= ry1)
@@ -172,19 +161,18 @@ __global__ void __launch_bounds__(kRastWarps * 32) raster_kernel(const __grid_co
         // The count pass stores the coverage mask of every test of the chunk (one range per
         // chunk, reserved with one atomic) and each pair's first index; the fill pass reads
         // them instead of testing again.  Both walk a fan's rectangle in the same order.
-        uint32_t mbase = ~0u, my_moff = ~0u;
+        uint32_t mbase = ~0u;
         if (MODE == kCount) {
-            // kMaskRegions cursors, the item picking one by its index, so that the reservations
-            // of millions of chunks do not queue on one address
+            // up to kMaskRegions cursors, the item picking one by its index, so that the
+            // reservations of millions of chunks do not queue on one address
             if (lane == 0 && total > 0) {
-                const uint32_t reg = item % kMaskRegions;
-                const uint32_t rsz = (uint32_t)(a.mask_cap / kMaskRegions);
+                const uint32_t reg = item % a.mask_regions;
+                const uint32_t rsz = (uint32_t)(a.mask_cap / a.mask_regions);
                 const uint32_t b = atomicAdd(a.mask_cursor + reg, (uint32_t)total);
                 if ((uint64_t)b + (uint64_t)total <= (uint64_t)rsz) mbase = reg * rsz + b;
             }
             mbase = __shfl_sync(0xffffffffu, mbase, 0);
         }
-        if (MODE == kFill) my_moff = pinf.x;
         const uint32_t live = __ballot_sync(0xffffffffu, my_n != 0);   // staged fans with tests, in order
         if (my_n) s_map[__popc(live & ((1u << lane) - 1u))] = (uint32_t)lane;
         __syncwarp();
@@ -198,7 +186,6 @@ __global__ void __launch_bounds__(kRastWarps * 32) raster_kernel(const __grid_co
             const uint32_t starts = __reduce_or_sync(0xffffffffu, here);
             const int f = (int)s_map[before + __popc(starts & (0xffffffffu >> (31 - lane))) - 1];
             const int fexcl = __shfl_sync(0xffffffffu, excl, f);
-            const uint32_t fmoff = __shfl_sync(0xffffffffu, my_moff, f);
             const uint32_t fgeo = __shfl_sync(0xffffffffu, my_geo, f);
             uint32_t hits = 0, flags = 0;
             int lp = -1, px = 0, py = 0;
@@ -214,8 +201,6 @@ __global__ void __launch_bounds__(kRastWarps * 32) raster_kernel(const __grid_co
                 if (SPLAT)
                     hits = splat_hit(s_spl[f], *sc.cam, a.spl.trunc, (double)px + 0.5, (double)py + 0.5, sp_t, sp_a)
                                ? 1u : 0u;
-                else if (MODE == kFill && fmoff != ~0u)
-                    hits = __ldg(a.masks + fmoff + (uint32_t)local);
                 else {   // decisions in the fan's relative frame (the origin is an integer)
                     flags = S.flags[f];
                     hits = cover_mask<KT>(S, STG, K, f, flags, (float)(px - (int)S.ox[f]) + 0.5f,
@@ -252,39 +237,6 @@ __global__ void __launch_bounds__(kRastWarps * 32) raster_kernel(const __grid_co
                     float4 *rec = a.frags + (size_t)kRecFwd * ((size_t)b + slot);
                     rec[0] = make_float4(sp_t, __uint_as_float(S.fan[f]), __uint_as_float(S.q[f]), 0.0f);
                     rec[1] = make_float4(sl.col[0], sl.col[1], sl.col[2], sp_a);
-                }
-            }
-            if (MODE == kFill && nf) {
-                const uint32_t b = s_base[lp];
-                if (b != 0xffffffffu) {
-                    const float pxc = (float)px + 0.5f, pyc = (float)py + 0.5f;
-                    for (uint32_t hm = hits; hm; hm &= hm - 1, ++slot) {
-                        const int j = __ffs(hm) - 1;
-                        const int jn = (j + 1 == K) ? 0 : j + 1;
-                        const float izc = S.viz[f];
-                        const float izj = S.viz[(1 + j) * STG + f], izn = S.viz[(1 + jn) * STG + f];
-                        const dfl zf = frag_depth_df(S, STG, K, f, j, pxc, pyc, *sc.cam);
-                        // perspective-correct barycentrics from the accurate centre offsets
-                        const float ox = __fsub_rn(S.cxh[f], pxc) + S.cxl[f];
-                        const float oy = __fsub_rn(S.cyh[f], pyc) + S.cyl[f];
-                        const float ujx = ox + S.du[j * STG + f], ujy = oy + S.dv[j * STG + f];
-                        const float unx = ox + S.du[jn * STG + f], uny = oy + S.dv[jn * STG + f];
-                        const float w0 = (ujx * uny - ujy * unx) * izc;
-                        const float w1 = (unx * oy - uny * ox) * izj;
-                        const float w2 = (ox * ujy - oy * ujx) * izn;
-                        const float Wsum = w0 + w1 + w2;
-                        const float iW = 1.0f / Wsum;
-                        const float m0 = w0 * iW, m1 = w1 * iW, m2 = w2 * iW;
-                        const int vc = f, vj = (1 + j) * STG + f, vn = (1 + jn) * STG + f;
-                        const float al = m0 * S.ca[vc] + m1 * S.ca[vj] + m2 * S.ca[vn];
-                        const float c0 = m0 * S.cr[vc] + m1 * S.cr[vj] + m2 * S.cr[vn];
-                        const float c1 = m0 * S.cg[vc] + m1 * S.cg[vj] + m2 * S.cg[vn];
-                        const float c2 = m0 * S.cb[vc] + m1 * S.cb[vj] + m2 * S.cb[vn];
-                        const uint32_t tri = S.fan[f] * (uint32_t)K + (uint32_t)j;
-                        float4 *rec = a.frags + (size_t)kRecFwd * ((size_t)b + slot);
-                        rec[0] = make_float4(zf.h, __uint_as_float(tri), __uint_as_float(S.q[f]), zf.l);
-                        rec[1] = make_float4(c0, c1, c2, al);
-                    }
                 }
             }
             __syncwarp();   // the next batch may append to the same pixels
@@ -484,7 +436,7 @@ cudaError_t launch_t(const RastArgs &ra, int64_t max_items, int K, cudaStream_t 
     // fans staged per chunk: small enough that the shared-memory stage of a warp lets
     // many warps share an SM (the passes are latency-bound), large enough to keep the
     // packed (fan, pixel) batches full
-    constexpr int STG = (MODE == kCount || MODE == kSplatCount) ? 16 : 8;
+    constexpr int STG = mode_fills(MODE) ? 8 : 16;
     const size_t smem = kRastWarps * warp_smem_bytes<TILE, STG, MODE>(K);
     auto fn = raster_kernel<TILE, STG, KT, MODE>;
     cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -539,6 +491,9 @@ RastArgs make_args(const RenderArgs &ra) {
     a.pinfo = reinterpret_cast<uint2 *>(ra.ws + L.off_maskoff);
     a.masks = reinterpret_cast<uint16_t *>(ra.ws + L.off_masks);
     a.mask_cap = L.mask_cap;
+    // regions of at least 2^16 masks, so that a small image's chunks (up to 16 fans of a whole
+    // tile) fit one
+    a.mask_regions = (uint32_t)std::min<int64_t>(kMaskRegions, std::max<int64_t>(1, L.mask_cap >> 16));
     a.mask_cursor = reinterpret_cast<uint32_t *>(ra.ws + L.off_mask_cursor);
     return a;
 }
@@ -584,15 +539,9 @@ cudaError_t launch_raster_count(const RenderArgs &ra, cudaStream_t st) {
     return e;
 }
 
-cudaError_t launch_raster(const RenderArgs &ra, bool fill, cudaStream_t st) {
-    const RenderLayout &L = ra.L;
-    if (L.n_tiles == 0) return cudaSuccess;
-    const RastArgs a = make_args(ra);
-    cudaError_t e;
-    if (ra.splat)
-        e = fill ? launch_dispatch<kSplatFill>(a, L, ra.K, st) : launch_dispatch<kSplatCount>(a, L, ra.K, st);
-    else
-        e = fill ? launch_dispatch<kFill>(a, L, ra.K, st) : launch_dispatch<kCount>(a, L, ra.K, st);
+cudaError_t launch_splat_fill(const RenderArgs &ra, cudaStream_t st) {
+    if (ra.L.n_tiles == 0) return cudaSuccess;
+    const cudaError_t e = launch_dispatch<kSplatFill>(make_args(ra), ra.L, ra.K, st);
     if (e == cudaSuccess) count_launches(1);
     return e;
 }

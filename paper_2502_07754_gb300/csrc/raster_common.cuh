@@ -1,7 +1,7 @@
 // Shared pieces of the rasterisation kernels: double-float projection of a fan
-// centre (value path), the shared-memory stage of a chunk of fans, the per-pixel
+// centre (value path), the shared-memory stage of a chunk of fans' decisions, and the per-pixel
 // coverage walk over a staged fan's K triangles with the binary32 decision formulas on
-// fan-relative vertex positions, and the double-float fragment depth that orders them.
+// fan-relative vertex positions.
 #pragma once
 
 #include "fan_geom.cuh"
@@ -119,25 +119,13 @@ struct Stage {
     float2 *sd;                   // [K][CH] spoke directions b_i - c
     float *rdx, *rdy;             // [K][CH] rim directions, lower index to higher
     float *area;                  // [K][CH] |area2|
-    float *cxh, *cxl, *cyh, *cyl; // [CH] double-float screen position of the centre (values)
-    float *du, *dv;               // [K][CH] screen offsets of the boundary vertices (values)
-    float *cr, *cg, *cb, *ca;     // [KV][CH] vertex colour and opacity (values)
-    float *viz;                   // [KV][CH] 1 / depth (values: barycentric weights)
-    // exact-order depth (frag_depth_df), double-float (high, low):
-    float *pc;                    // [6][CH] fx X_c, fy Y_c, Z_c of the centre
-    float *exh, *exl, *eyh, *eyl, *ezh, *ezl;   // [K][CH] view offsets R (b_i - c) of the boundary vertices
 };
 
-// What a stage holds: decisions only (count), or decisions and values (fill).
-enum StageLevel { kStageDecide = 0, kStageValues = 1 };
-
-__host__ __device__ __forceinline__ size_t stage_bytes(int CH, int K, int level) {
-    const int dec = 2 * (K + 1) + 5 * K;
-    const int val = level >= kStageValues ? 4 + 2 * K + 4 * (K + 1) + (K + 1) + 6 + 6 * K : 0;
-    return (size_t)CH * (16 + 20 + 8 + 4 * (dec + val));
+__host__ __device__ __forceinline__ size_t stage_bytes(int CH, int K) {
+    return (size_t)CH * (16 + 20 + 8 + 4 * (2 * (K + 1) + 5 * K));
 }
 
-__device__ __forceinline__ Stage stage_ptrs(char *base, int CH, int K, int level) {
+__device__ __forceinline__ Stage stage_ptrs(char *base, int CH, int K) {
     const int KV = K + 1;
     Stage s;
     s.rect = reinterpret_cast<int4 *>(base);
@@ -154,27 +142,7 @@ __device__ __forceinline__ Stage stage_ptrs(char *base, int CH, int K, int level
     s.sd = reinterpret_cast<float2 *>(f); f += 2 * K * CH;   // (CH is even: 8-byte aligned)
     s.rdx = f; f += K * CH;
     s.rdy = f; f += K * CH;
-    s.area = f; f += K * CH;
-    if (level >= kStageValues) {
-        s.cxh = f; f += CH;
-        s.cxl = f; f += CH;
-        s.cyh = f; f += CH;
-        s.cyl = f; f += CH;
-        s.du = f; f += K * CH;
-        s.dv = f; f += K * CH;
-        s.cr = f; f += KV * CH;
-        s.cg = f; f += KV * CH;
-        s.cb = f; f += KV * CH;
-        s.ca = f; f += KV * CH;
-        s.viz = f; f += KV * CH;
-        s.pc = f; f += 6 * CH;
-        s.exh = f; f += K * CH;
-        s.exl = f; f += K * CH;
-        s.eyh = f; f += K * CH;
-        s.eyl = f; f += K * CH;
-        s.ezh = f; f += K * CH;
-        s.ezl = f;
-    }
+    s.area = f;
     return s;
 }
 
@@ -275,78 +243,14 @@ __device__ __forceinline__ void stage_decisions(const SceneDev &a, const Stage &
         s.rect[slot] = make_int4(r.i0, r.i1, r.j0, r.j1);
     }
 }
-// The value part of stage_fans (fill passes): the double-float centre projection, the
-// boundary vertices' screen offsets and view offsets, 1 / depth, colours and opacities.
-template <int LPF>
-__device__ __forceinline__ void stage_values(const SceneDev &a, const Stage &s, int K, int slot, int sub, uint32_t fan,
-                                             const float *p) {
-    constexpr int CH = 32 / LPF;
-    const int KV = K + 1;
-    const float m[3] = {__ldg(p), __ldg(p + 1), __ldg(p + 2)};
-    const CentreProj cp = project_centre(*a.cam, m);
-    const dfl zc = df_fast_two_sum(cp.Zh, cp.Zl);
-    if (sub == 0) {
-        s.cxh[slot] = cp.xh;
-        s.cxl[slot] = cp.xl;
-        s.cyh[slot] = cp.yh;
-        s.cyl[slot] = cp.yl;
-        s.viz[slot] = 1.0f / zc.h;
-        const dfl xf = df_mul_f(df_fast_two_sum(cp.Xh, cp.Xl), a.cam->fx);
-        const dfl yf = df_mul_f(df_fast_two_sum(cp.Yh, cp.Yl), a.cam->fy);
-        s.pc[slot] = xf.h;
-        s.pc[CH + slot] = xf.l;
-        s.pc[2 * CH + slot] = yf.h;
-        s.pc[3 * CH + slot] = yf.l;
-        s.pc[4 * CH + slot] = zc.h;
-        s.pc[5 * CH + slot] = zc.l;
-    }
-    for (int i = sub; i < K; i += LPF) {
-        const float *pi = p + 3 * (1 + i);
-        const float d[3] = {__ldg(pi) - m[0], __ldg(pi + 1) - m[1], __ldg(pi + 2) - m[2]};
-        float du, dv, X, Y, Z;
-        vertex_offset(*a.cam, cp, d, du, dv, X, Y, Z);
-        s.du[i * CH + slot] = du;
-        s.dv[i * CH + slot] = dv;
-        // the exact view offset e = R (b_i - c) in double-float, for the fragment depths
-        const DfVec e = df_view_offset(*a.cam, m, pi);
-        s.viz[(1 + i) * CH + slot] = 1.0f / df_add(zc, e.z).h;
-        const int u = i * CH + slot;
-        s.exh[u] = e.x.h;
-        s.exl[u] = e.x.l;
-        s.eyh[u] = e.y.h;
-        s.eyl[u] = e.y.l;
-        s.ezh[u] = e.z.h;
-        s.ezl[u] = e.z.l;
-    }
-    const float *col = a.rgb + (size_t)fan * KV * 3;
-    const float *al = a.alpha + (size_t)fan * KV;
-    for (int k = sub; k < KV; k += LPF) {
-        s.cr[k * CH + slot] = __ldg(col + 3 * k);
-        s.cg[k * CH + slot] = __ldg(col + 3 * k + 1);
-        s.cb[k * CH + slot] = __ldg(col + 3 * k + 2);
-        s.ca[k * CH + slot] = __ldg(al + k);
-    }
-}
-
 // Stages CH = 32 / LPF fans into slots 0..CH-1 with the whole warp: the LPF lanes of slot
-// lane / LPF share the fan's vertices, triangles and colours (every lane of the warp
+// lane / LPF share the fan's vertices and triangles (every lane of the warp
 // calls this; a lane whose slot is not active does no loads or stores but takes part in
-// the shuffles).  The staged words are the same as one lane per fan would write.  With
-// `decide` false (warp-uniform) only the fan id, depth bound and the values are staged:
-// the caller already holds the fans' coverage masks and pixel rectangles.
+// the shuffles).  The staged words are the same as one lane per fan would write.
 template <int LPF>
 __device__ __forceinline__ void stage_fans(const SceneDev &a, const Stage &s, int K, int lane, bool active,
-                                           uint32_t fan, uint32_t q, int level, bool decide = true) {
-    const int slot = lane / LPF, sub = lane % LPF;
-    const float *p = a.xyz + (size_t)fan * (K + 1) * 3;
-    if (decide)
-        stage_decisions<LPF>(a, s, K, slot, sub, active, fan, q);
-    else if (active && sub == 0) {
-        s.q[slot] = q;
-        s.fan[slot] = fan;
-    }
-    if (level < kStageValues || !active) return;
-    stage_values<LPF>(a, s, K, slot, sub, fan, p);
+                                           uint32_t fan, uint32_t q) {
+    stage_decisions<LPF>(a, s, K, lane / LPF, lane % LPF, active, fan, q);
 }
 // Coverage of the pixel centre (pxc, pyc) by staged fan f: bit j is set when triangle j
 // covers it.  Each spoke value is computed once and turned into two pass bits (as the
@@ -406,44 +310,6 @@ __device__ __forceinline__ uint32_t cover_mask(const Stage &S, int CH, int K, in
         if (E0 > 0.0f || (E0 == 0.0f && ((rtie >> (flip ? 16 + j : j)) & 1u))) hits |= 1u << j;
     }
     return hits;
-}
-
-// Depth of triangle j = (c, b_j, b_j+1) of staged fan f at the pixel centre (pxc, pyc)
-// (absolute screen coordinates), in double-float: the view depth where the pixel's ray
-// r = ((x - cx) / fx, (y - cy) / fy, 1) meets the triangle's plane, Z = n . P_c / n . r with
-// n = e_j x e_j+1 the normal from the vertices' exact view offsets and P_c the centre's
-// view position (numerator and denominator both scaled by fx fy), which equals
-// 1 / sum_k (lambda_k / Z_k) of the perspective-correct barycentrics.  Clamped to the
-// triangle's vertex depths, where a covered centre lies (the clamp acts only where the
-// decided coverage and the exact plane differ by rounding; a ray parallel to the plane
-// takes the least vertex depth).
-__device__ __forceinline__ dfl frag_depth_df(const Stage &S, int CH, int K, int f, int j, float pxc, float pyc,
-                                             const CamDev &c) {
-    const int jn = (j + 1 == K) ? 0 : j + 1;
-    const int u = j * CH + f, w = jn * CH + f;
-    const dfl e1x = {S.exh[u], S.exl[u]}, e1y = {S.eyh[u], S.eyl[u]}, e1z = {S.ezh[u], S.ezl[u]};
-    const dfl e2x = {S.exh[w], S.exl[w]}, e2y = {S.eyh[w], S.eyl[w]}, e2z = {S.ezh[w], S.ezl[w]};
-    const dfl xf = {S.pc[f], S.pc[CH + f]}, yf = {S.pc[2 * CH + f], S.pc[3 * CH + f]};
-    const dfl zc = {S.pc[4 * CH + f], S.pc[5 * CH + f]};
-    const dfl nx = df_add_fast(df_mul(e1y, e2z), df_neg(df_mul(e1z, e2y)));
-    const dfl ny = df_add_fast(df_mul(e1z, e2x), df_neg(df_mul(e1x, e2z)));
-    const dfl nz = df_add_fast(df_mul(e1x, e2y), df_neg(df_mul(e1y, e2x)));
-    const dfl pa = df_mul_f(nx, c.fy), pb = df_mul_f(ny, c.fx), pn = df_mul_f(df_mul_f(nz, c.fx), c.fy);
-    const dfl num = df_add_fast(df_add_fast(df_mul(pa, xf), df_mul(pb, yf)), df_mul(pn, zc));
-    const dfl den = df_add_fast(df_add_fast(df_mul(pa, df_two_sum(pxc, -c.cx)), df_mul(pb, df_two_sum(pyc, -c.cy))),
-                                pn);
-    const dfl z1 = df_add_fast(zc, e1z), z2 = df_add_fast(zc, e2z);
-    dfl lo = zc, hi = zc;
-    if (df_lt(z1, lo)) lo = z1;
-    if (df_lt(z2, lo)) lo = z2;
-    if (df_lt(hi, z1)) hi = z1;
-    if (df_lt(hi, z2)) hi = z2;
-    if (den.h == 0.0f) return lo;
-    dfl z = df_div_rcp(num, den);
-    if (!(z.h == z.h)) return lo;   // NaN
-    if (df_lt(z, lo)) z = lo;
-    if (df_lt(hi, z)) z = hi;
-    return z;
 }
 
 // ------------------------------------------------------------------------------------
