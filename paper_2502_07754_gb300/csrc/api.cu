@@ -311,6 +311,10 @@ constexpr double kSplatTrunc = 2.7;           // truncation radius in scales (th
 constexpr float kSplatKeyScale = 0.9990234375f;   // 1 - 2^-10: depth keys stay below every hit
 
 static size_t splat_poly_bytes(int64_t N) { return align_up((size_t)N * (kSplatK + 1) * 12, 256); }
+// what a splat workspace holds beyond the render layout: polygons, then coefficients
+static size_t splat_extra_bytes(int64_t N, int n_views) {
+    return splat_poly_bytes(N) + align_up(splat_coef_bytes(N, n_views), 256);
+}
 
 static ms_status splat_views(const float *means, const float *log_scales, const float *quats, const float *opacity,
                              const float *rgb, int64_t N, int axis_rule, const ms_camera *cams, int n_views,
@@ -324,8 +328,9 @@ static ms_status splat_views(const float *means, const float *log_scales, const 
     if (N >= (1ll << 31)) return fail(MS_ERR_INVALID, "too many Gaussians");
     RenderLayout L;
     // the layout check sees a placeholder soup pointer: the polygons are made below
+    const size_t extra = N > 0 && n_views > 0 ? splat_extra_bytes(N, n_views) : 0;
     ms_status s = check_render_args(N > 0 ? means : nullptr, means, means, N, kSplatK, cams, n_views, p, workspace,
-                                    ws_bytes > splat_poly_bytes(N) ? ws_bytes - splat_poly_bytes(N) : 0, L);
+                                    ws_bytes > extra ? ws_bytes - extra : 0, L);
     if (s != MS_OK) return s;
     if (!out) return fail(MS_ERR_INVALID, "output image list is NULL");
     for (int v = 0; v < n_views; ++v)
@@ -338,11 +343,13 @@ static ms_status splat_views(const float *means, const float *log_scales, const 
     memset(&a, 0, sizeof(a));
     a.xyz = poly; a.n_fans = N; a.K = kSplatK; a.prm = p; a.L = L; a.ws = ws;
     a.splat = true;
+    a.splat_coef = reinterpret_cast<float4 *>(ws + L.total + splat_poly_bytes(N));
     a.key_scale = kSplatKeyScale;
     a.spl.means = means; a.spl.log_scales = log_scales; a.spl.quats = quats; a.spl.opacity = opacity;
     a.spl.rgb = rgb; a.spl.axis_rule = axis_rule; a.spl.trunc = kSplatTrunc;
     a.vt = make_views(cams, n_views, L, out, nullptr, nullptr);
     if ((e = launch_splat_polygons(a.spl, N, poly, st)) != cudaSuccess) return cuda_fail(e, "polygon launch");
+    if ((e = launch_splat_setup(a, st)) != cudaSuccess) return cuda_fail(e, "splat setup launch");
     if ((e = launch_bin(a, st)) != cudaSuccess) return cuda_fail(e, "bin launch");
     if ((e = launch_sort(a, st)) != cudaSuccess) return cuda_fail(e, "sort launch");
     if ((e = launch_raster_count(a, st)) != cudaSuccess) return cuda_fail(e, "splat count launch");
@@ -554,7 +561,7 @@ MS_API ms_status ms_batch_render_backward(const float *xyz, const float *rgb, co
 MS_API size_t ms_splat_workspace_size(int64_t N, const ms_camera *cams, int32_t n_views,
                                       const ms_render_params *params) {
     const size_t base = ms_batch_workspace_size(N, kSplatK, cams, n_views, params);
-    return base ? base + splat_poly_bytes(N) : 0;
+    return base ? base + splat_extra_bytes(N, n_views) : 0;
 }
 
 MS_API ms_status ms_splat_render(const float *means, const float *log_scales, const float *quats,

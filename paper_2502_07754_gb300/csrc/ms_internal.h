@@ -60,6 +60,7 @@ struct RenderArgs {
     float *d_xyz, *d_rgb, *d_alpha;   // backward outputs
     bool splat;                // draw the source Gaussians of `spl` over the polygons in xyz
     float key_scale;           // binning: depth keys from key_scale * min Z (1 for fans)
+    float4 *splat_coef;        // splat passes: coefficients of every (view, Gaussian)
     SplatSrc spl;
 };
 
@@ -103,7 +104,11 @@ cudaError_t sort_u64(unsigned long long *a, unsigned long long *b, int64_t n, in
 constexpr int kItemFans = 64;   // fans per raster work item
 
 cudaError_t launch_fill(const RenderArgs &a, cudaStream_t st);         // fragment records of the fans
-cudaError_t launch_splat_fill(const RenderArgs &a, cudaStream_t st);   // fragment records of the source Gaussians
+// the source Gaussians: per-view coefficients, fragment counts, fragment records
+size_t splat_coef_bytes(int64_t N, int n_views);
+cudaError_t launch_splat_setup(const RenderArgs &a, cudaStream_t st);
+cudaError_t launch_splat_count(const RenderArgs &a, cudaStream_t st);
+cudaError_t launch_splat_fill(const RenderArgs &a, cudaStream_t st);
 cudaError_t launch_raster_count(const RenderArgs &a, cudaStream_t st);   // items, count, prefix, pixel scan
 cudaError_t launch_record_chain(const RenderArgs &a, cudaStream_t st);   // adjoint: records -> fan vertices
 constexpr int kRecFwd = 2;   // float4s per fragment record

@@ -24,24 +24,18 @@ namespace ms {
 namespace {
 
 struct RastArgs {
-    const float *xyz, *rgb, *alpha;
-    int K, depth_bits, fan_bits;
+    int K, fan_bits;
     ViewTable vt;
     const unsigned long long *keys;   // sorted elements tile | depth bound | fan id
     const uint4 *items;        // (tile, start, end, index within tile)
     uint32_t *icnt;            // [item][tile pixels]: counts, then in-pixel starting slots
-    const uint32_t *offsets;
-    const uint32_t *counts;
-    float4 *frags;
-    int64_t frag_cap;
     Status *st;
-    SplatSrc spl;              // source Gaussians (splat passes only)
     const float4 *dec;         // [view][vertex] decided vertices from binning
     int64_t V;
     const uint32_t *face_mask; // per fan, bit j = face j drawn; NULL = all
     uint2 *pinfo;              // per pair: index of its first coverage mask (~0 if none stored), and its
                                // pixel rectangle clipped to the tile (pair_geo; 0 if empty)
-    uint16_t *masks;           // coverage masks (bit j: triangle j) of the count pass's tests
+    uint16_t *masks;           // coverage masks (bit j: triangle j) of the tests
     int64_t mask_cap;
     uint32_t mask_regions;
     uint32_t *mask_cursor;     // [mask_regions] fill levels of the mask regions (zeroed per render)
@@ -49,30 +43,13 @@ struct RastArgs {
 
 constexpr int kRastWarps = 2;   // warps (work items) per block: items differ widely in cost
 
-// A pair's pixel rectangle clipped to its tile, relative to the tile's corner: x0 | y0 << 6 |
-// (w - 1) << 12 | (h - 1) << 18, bit 31 set; 0 for a pair with no pixel to test.
-__device__ __forceinline__ uint32_t pair_geo(int rx0, int ry0, int w, int h) {
-    return 0x80000000u | (uint32_t)rx0 | (uint32_t)ry0 << 6 | (uint32_t)(w - 1) << 12 | (uint32_t)(h - 1) << 18;
-}
-
-// Pass kinds: count the fans' fragments (fill.cu writes their records).  The splat passes draw
-// the source Gaussians themselves (count, then 32-byte records) over the tile lists of
-// their circumscribing polygons.
-enum RasterMode { kCount = 0, kSplatCount = 3, kSplatFill = 4 };
-
-__host__ __device__ constexpr bool mode_fills(int m) { return m == kSplatFill; }
-__host__ __device__ constexpr bool mode_splat(int m) { return m >= kSplatCount; }
-
-template <int TILE, int STG, int MODE>
+template <int TILE, int STG>
 __host__ __device__ __forceinline__ size_t warp_smem_bytes(int K) {
-    return (size_t)(TILE * TILE * (mode_fills(MODE) ? 2 : 1) + 64) * 4 + stage_bytes(STG, K) +
-           (mode_splat(MODE) ? (size_t)STG * sizeof(SplatSlot) : 0);
+    return (size_t)(TILE * TILE + 32) * 4 + stage_bytes(STG, K);
 }
 
-template <int TILE, int STG, int KT, int MODE>
-__global__ void __launch_bounds__(kRastWarps * 32) raster_kernel(const __grid_constant__ RastArgs a) {
-    constexpr bool FILL = mode_fills(MODE);   // passes that address records
-    constexpr bool SPLAT = mode_splat(MODE);
+template <int TILE, int STG, int KT>
+__global__ void __launch_bounds__(kRastWarps * 32) count_kernel(const __grid_constant__ RastArgs a) {
     extern __shared__ __align__(16) char smem[];
     const int K = KT > 0 ? KT : a.K;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -82,43 +59,20 @@ __global__ void __launch_bounds__(kRastWarps * 32) raster_kernel(const __grid_co
     const int view = view_of_tile(a.vt, it.x);
     const ViewDev &vw = a.vt.v[view];
     SceneDev sc;
-    sc.xyz = a.xyz;
-    sc.rgb = a.rgb;
-    sc.alpha = a.alpha;
-    sc.K = K;
-    sc.cam = &vw.cam;
     sc.W = vw.cam.width;
     sc.H = vw.cam.height;
     sc.dec = a.dec + (size_t)view * (size_t)a.V;
-    sc.face_mask = SPLAT ? nullptr : a.face_mask;
+    sc.face_mask = a.face_mask;
     const int tile = (int)(it.x - vw.tile_base);
     const int tiles_x = (int)vw.tiles_x;
-    const unsigned long long pix_base = vw.pix_base;
-    char *mine = smem + (size_t)warp * warp_smem_bytes<TILE, STG, MODE>(K);
+    char *mine = smem + (size_t)warp * warp_smem_bytes<TILE, STG>(K);
     uint32_t *s_cnt = reinterpret_cast<uint32_t *>(mine);   // [TILE*TILE] fragments so far
-    uint32_t *s_base = s_cnt + TILE * TILE;                   // [TILE*TILE] record offsets (fill)
-    uint32_t *s_nf = s_cnt + TILE * TILE * (FILL ? 2 : 1);    // [32] fragments per lane of a batch
-    uint32_t *s_map = s_nf + 32;                               // [32] staged fans that have tests
-    char *stage_base = mine + (size_t)(TILE * TILE * (FILL ? 2 : 1) + 64) * 4;
-    const Stage S = stage_ptrs(stage_base, STG, K);
-    SplatSlot *s_spl = reinterpret_cast<SplatSlot *>(stage_base + stage_bytes(STG, K));
+    uint32_t *s_map = s_cnt + TILE * TILE;                    // [32] staged fans that have tests
+    const Stage S = stage_ptrs(mine + (size_t)(TILE * TILE + 32) * 4, STG, K);
     const int tx0 = (tile % tiles_x) * TILE, ty0 = (tile / tiles_x) * TILE;
     const int tx1 = min(tx0 + TILE, sc.W) - 1, ty1 = min(ty0 + TILE, sc.H) - 1;
     uint32_t *icnt = a.icnt + (size_t)item * TILE * TILE;
-    for (int i = lane; i < TILE * TILE; i += 32) {
-        s_cnt[i] = 0;
-        if (FILL) {
-            const int x = tx0 + (i % TILE), y = ty0 + (i / TILE);
-            uint32_t b = 0xffffffffu;
-            if (x <= tx1 && y <= ty1) {
-                const size_t pix = pix_base + (size_t)y * sc.W + x;
-                const int64_t o = a.offsets[pix];
-                // a pixel whose records would not fit gets none (the overflow is reported)
-                if (o + a.counts[pix] <= a.frag_cap) b = (uint32_t)o + icnt[i];
-            }
-            s_base[i] = b;
-        }
-    }
+    for (int i = lane; i < TILE * TILE; i += 32) s_cnt[i] = 0;
     uint32_t c_rect = 0, c_frag = 0;
     __syncwarp();
     for (uint32_t cb = it.y; cb < it.z; cb += STG) {
@@ -126,17 +80,9 @@ __global__ void __launch_bounds__(kRastWarps * 32) raster_kernel(const __grid_co
         {
             constexpr int LPF = 32 / STG;   // lanes staging one fan
             const int slot = lane / LPF;
-            uint32_t q = 0, fan = 0;
-            if (slot < cnt) {
-                const uint32_t li = cb + slot;
-                const unsigned long long e = __ldg(a.keys + li);
-                q = (uint32_t)((e >> a.fan_bits) & ((1ull << a.depth_bits) - 1ull));
-                fan = (uint32_t)(e & ((1ull << a.fan_bits) - 1ull));
-            }
-            stage_fans<LPF>(sc, S, K, lane, slot < cnt, fan, q);
-            if (SPLAT && lane < cnt)
-                s_spl[lane] = splat_setup(a.spl, *sc.cam,
-                                          (uint32_t)(__ldg(a.keys + cb + lane) & ((1ull << a.fan_bits) - 1ull)));
+            uint32_t fan = 0;
+            if (slot < cnt) fan = (uint32_t)(__ldg(a.keys + cb + slot) & ((1ull << a.fan_bits) - 1ull));
+            stage_fans<LPF>(sc, S, K, lane, slot < cnt, fan);
         }
         __syncwarp();
         // The staged fans' rectangles (clipped to the tile) form one packed (fan, pixel)
@@ -158,11 +104,11 @@ __global__ void __launch_bounds__(kRastWarps * 32) raster_kernel(const __grid_co
         }
         const int excl = incl - my_n;
         const int total = __shfl_sync(0xffffffffu, incl, 31);
-        // The count pass stores the coverage mask of every test of the chunk (one range per
-        // chunk, reserved with one atomic) and each pair's first index; the fill pass reads
-        // them instead of testing again.  Both walk a fan's rectangle in the same order.
+        // The coverage mask of every test of the chunk is stored (one range per chunk, reserved
+        // with one atomic) with each pair's first index; the fill pass reads them instead of
+        // testing again.  Both walk a fan's rectangle in the same order.
         uint32_t mbase = ~0u;
-        if (MODE == kCount) {
+        {
             // up to kMaskRegions cursors, the item picking one by its index, so that the
             // reservations of millions of chunks do not queue on one address
             if (lane == 0 && total > 0) {
@@ -176,7 +122,7 @@ __global__ void __launch_bounds__(kRastWarps * 32) raster_kernel(const __grid_co
         const uint32_t live = __ballot_sync(0xffffffffu, my_n != 0);   // staged fans with tests, in order
         if (my_n) s_map[__popc(live & ((1u << lane) - 1u))] = (uint32_t)lane;
         __syncwarp();
-        uint32_t fan_hit = 0;   // count pass: bit f set when staged fan f covers some pixel centre
+        uint32_t fan_hit = 0;   // bit f set when staged fan f covers some pixel centre
         for (int base = 0; base < total; base += 32) {
             const int idx = base + lane;
             // the fan of each index: the fans with tests start one after another, so an index's
@@ -187,74 +133,35 @@ __global__ void __launch_bounds__(kRastWarps * 32) raster_kernel(const __grid_co
             const int f = (int)s_map[before + __popc(starts & (0xffffffffu >> (31 - lane))) - 1];
             const int fexcl = __shfl_sync(0xffffffffu, excl, f);
             const uint32_t fgeo = __shfl_sync(0xffffffffu, my_geo, f);
-            uint32_t hits = 0, flags = 0;
-            int lp = -1, px = 0, py = 0;
-            float sp_t = 0.0f, sp_a = 0.0f;
+            uint32_t hits = 0;
             if (idx < total) {
                 ++c_rect;
-                const int rx0 = tx0 + (int)(fgeo & 63u), ry0 = ty0 + (int)((fgeo >> 6) & 63u);
-                const int w = (int)((fgeo >> 12) & 63u) + 1, local = idx - fexcl;
+                const int local = idx - fexcl, w = (int)((fgeo >> 12) & 63u) + 1;
                 // (local + 0.5) / w is at least 1/(2w) away from an integer: exact row
                 const int yy = (int)__fdividef((float)local + 0.5f, (float)w);
-                px = rx0 + (local - yy * w);
-                py = ry0 + yy;
-                if (SPLAT)
-                    hits = splat_hit(s_spl[f], *sc.cam, a.spl.trunc, (double)px + 0.5, (double)py + 0.5, sp_t, sp_a)
-                               ? 1u : 0u;
-                else {   // decisions in the fan's relative frame (the origin is an integer)
-                    flags = S.flags[f];
-                    hits = cover_mask<KT>(S, STG, K, f, flags, (float)(px - (int)S.ox[f]) + 0.5f,
-                                          (float)(py - (int)S.oy[f]) + 0.5f);
-                }
-                if (MODE == kCount && mbase != ~0u) a.masks[mbase + (uint32_t)idx] = (uint16_t)hits;
-                if (hits) lp = (py - ty0) * TILE + (px - tx0);
+                const int x = (int)(fgeo & 63u) + (local - yy * w), y = (int)((fgeo >> 6) & 63u) + yy;
+                // decisions in the fan's relative frame (the origin is an integer)
+                hits = cover_mask<KT>(S, STG, K, f, S.flags[f], (float)(tx0 + x - (int)S.ox[f]) + 0.5f,
+                                      (float)(ty0 + y - (int)S.oy[f]) + 0.5f);
+                if (mbase != ~0u) a.masks[mbase + (uint32_t)idx] = (uint16_t)hits;
+                // the order of a pixel's slots does not matter yet
+                if (hits) atomicAdd(&s_cnt[y * TILE + x], (uint32_t)__popc(hits));
             }
-            if (MODE == kCount) fan_hit |= __reduce_or_sync(0xffffffffu, hits ? 1u << f : 0u);
-            const int nf = __popc(hits);
-            c_frag += nf;
-            if (!FILL) {   // counting: the order of a pixel's slots does not matter yet
-                if (nf) atomicAdd(&s_cnt[lp], (uint32_t)nf);
-                continue;
-            }
-            // Lanes that hit the same pixel take consecutive slots in lane order, which is
-            // fan order, so a pixel's records keep the depth-key order of the tile list.
-            const unsigned grp = __match_any_sync(0xffffffffu, lp);
-            if (nf) s_nf[lane] = (uint32_t)nf;
-            __syncwarp();
-            uint32_t slot = 0;
-            if (nf) {
-                uint32_t pre = 0;
-                for (unsigned lower = grp & ((1u << lane) - 1u); lower; lower &= lower - 1)
-                    pre += s_nf[__ffs(lower) - 1];
-                slot = s_cnt[lp] + pre;
-            }
-            __syncwarp();
-            if (nf && (grp >> lane) == 1u) s_cnt[lp] = slot + (uint32_t)nf;   // last lane of its group
-            if (SPLAT && FILL && nf) {
-                const uint32_t b = s_base[lp];
-                if (b != 0xffffffffu) {
-                    const SplatSlot &sl = s_spl[f];
-                    float4 *rec = a.frags + (size_t)kRecFwd * ((size_t)b + slot);
-                    rec[0] = make_float4(sp_t, __uint_as_float(S.fan[f]), __uint_as_float(S.q[f]), 0.0f);
-                    rec[1] = make_float4(sl.col[0], sl.col[1], sl.col[2], sp_a);
-                }
-            }
-            __syncwarp();   // the next batch may append to the same pixels
+            fan_hit |= __reduce_or_sync(0xffffffffu, hits ? 1u << f : 0u);
+            c_frag += __popc(hits);
         }
         // each pair's first mask index, and its rectangle if it covers any pixel centre
-        if (MODE == kCount && lane < cnt)
+        if (lane < cnt)
             a.pinfo[cb + lane] = make_uint2(mbase == ~0u ? ~0u : mbase + (uint32_t)excl,
                                             ((fan_hit >> lane) & 1u) ? my_geo : 0u);
         __syncwarp();
     }
-    if (!FILL) {
-        for (int i = lane; i < TILE * TILE; i += 32) icnt[i] = s_cnt[i];
-        const unsigned r0 = __reduce_add_sync(0xffffffffu, c_rect);
-        const unsigned r1 = __reduce_add_sync(0xffffffffu, c_frag);
-        if (lane == 0) {
-            atomicAdd(&a.st->rect_tests, (unsigned long long)r0);
-            atomicAdd(&a.st->fragments, (unsigned long long)r1);
-        }
+    for (int i = lane; i < TILE * TILE; i += 32) icnt[i] = s_cnt[i];
+    const unsigned r0 = __reduce_add_sync(0xffffffffu, c_rect);
+    const unsigned r1 = __reduce_add_sync(0xffffffffu, c_frag);
+    if (lane == 0) {
+        atomicAdd(&a.st->rect_tests, (unsigned long long)r0);
+        atomicAdd(&a.st->fragments, (unsigned long long)r1);
     }
 }
 
@@ -431,60 +338,41 @@ __global__ void __launch_bounds__(TILE *TILE) item_prefix_kernel(const uint32_t 
         if (s_hist[b]) atomicAdd(&hist[b], s_hist[b]);
 }
 
-template <int TILE, int KT, int MODE>
+template <int TILE, int KT>
 cudaError_t launch_t(const RastArgs &ra, int64_t max_items, int K, cudaStream_t st) {
     // fans staged per chunk: small enough that the shared-memory stage of a warp lets
-    // many warps share an SM (the passes are latency-bound), large enough to keep the
-    // packed (fan, pixel) batches full
-    constexpr int STG = mode_fills(MODE) ? 8 : 16;
-    const size_t smem = kRastWarps * warp_smem_bytes<TILE, STG, MODE>(K);
-    auto fn = raster_kernel<TILE, STG, KT, MODE>;
+    // many warps share an SM, large enough to keep the packed (fan, pixel) batches full
+    constexpr int STG = 16;
+    const size_t smem = kRastWarps * warp_smem_bytes<TILE, STG>(K);
+    auto fn = count_kernel<TILE, STG, KT>;
     cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     fn<<<(unsigned)((max_items + kRastWarps - 1) / kRastWarps), kRastWarps * 32, smem, st>>>(ra);
     return cudaGetLastError();
 }
 
-template <int MODE>
-cudaError_t launch_dispatch(const RastArgs &ra, const RenderLayout &L, int K, cudaStream_t st) {
-    if (mode_splat(MODE)) {   // the circumscribing polygons are K = 8 fans
-        if (L.tile == 8) return launch_t<8, kSplatK, MODE>(ra, L.max_items, K, st);
-        if (L.tile == 32) return launch_t<32, kSplatK, MODE>(ra, L.max_items, K, st);
-        return launch_t<16, kSplatK, MODE>(ra, L.max_items, K, st);
-    }
-    if (L.tile == 8) {
-        if (K == 8) return launch_t<8, 8, MODE>(ra, L.max_items, K, st);
-        if (K == 6) return launch_t<8, 6, MODE>(ra, L.max_items, K, st);
-        return launch_t<8, 0, MODE>(ra, L.max_items, K, st);
-    }
-    if (L.tile == 32) {
-        if (K == 8) return launch_t<32, 8, MODE>(ra, L.max_items, K, st);
-        if (K == 6) return launch_t<32, 6, MODE>(ra, L.max_items, K, st);
-        return launch_t<32, 0, MODE>(ra, L.max_items, K, st);
-    }
-    if (K == 8) return launch_t<16, 8, MODE>(ra, L.max_items, K, st);
-    if (K == 6) return launch_t<16, 6, MODE>(ra, L.max_items, K, st);
-    return launch_t<16, 0, MODE>(ra, L.max_items, K, st);
+template <int TILE>
+cudaError_t launch_k(const RastArgs &ra, int64_t max_items, int K, cudaStream_t st) {
+    if (K == 8) return launch_t<TILE, 8>(ra, max_items, K, st);
+    if (K == 6) return launch_t<TILE, 6>(ra, max_items, K, st);
+    return launch_t<TILE, 0>(ra, max_items, K, st);
+}
+
+cudaError_t launch_count(const RastArgs &ra, const RenderLayout &L, int K, cudaStream_t st) {
+    if (L.tile == 8) return launch_k<8>(ra, L.max_items, K, st);
+    if (L.tile == 32) return launch_k<32>(ra, L.max_items, K, st);
+    return launch_k<16>(ra, L.max_items, K, st);
 }
 
 RastArgs make_args(const RenderArgs &ra) {
     const RenderLayout &L = ra.L;
     RastArgs a;
-    a.xyz = ra.xyz;
-    a.rgb = ra.rgb;
-    a.alpha = ra.alpha;
     a.K = ra.K;
     a.vt = ra.vt;
-    a.depth_bits = L.depth_bits;
     a.fan_bits = L.fan_bits;
     a.keys = reinterpret_cast<const unsigned long long *>(ra.ws + (L.passes & 1 ? L.off_keys1 : L.off_keys0));
     a.items = reinterpret_cast<const uint4 *>(ra.ws + L.off_items);
     a.icnt = reinterpret_cast<uint32_t *>(ra.ws + L.off_icnt);
-    a.offsets = reinterpret_cast<const uint32_t *>(ra.ws + L.off_offsets);
-    a.counts = reinterpret_cast<const uint32_t *>(ra.ws + L.off_counts);
-    a.frags = reinterpret_cast<float4 *>(ra.ws + L.off_frags);
-    a.frag_cap = L.frag_cap;
     a.st = reinterpret_cast<Status *>(ra.ws + L.off_status);
-    a.spl = ra.spl;
     a.dec = reinterpret_cast<const float4 *>(ra.ws + L.off_dec);
     a.V = L.V;
     a.face_mask = ra.prm.face_mask;
@@ -516,7 +404,7 @@ cudaError_t launch_raster_count(const RenderArgs &ra, cudaStream_t st) {
     tile_item_emit_kernel<<<tg, 256, 0, st>>>(ranges, L.n_tiles, nitems, ibase,
                                               reinterpret_cast<uint4 *>(ws + L.off_items), L.max_items, status,
                                               (unsigned long long)L.frag_cap);
-    cudaError_t e = ra.splat ? launch_dispatch<kSplatCount>(a, L, ra.K, st) : launch_dispatch<kCount>(a, L, ra.K, st);
+    cudaError_t e = ra.splat ? launch_splat_count(ra, st) : launch_count(a, L, ra.K, st);
     if (e != cudaSuccess) return e;
     uint32_t *cnts = reinterpret_cast<uint32_t *>(ws + L.off_counts);
     uint32_t *hist = reinterpret_cast<uint32_t *>(ws + L.off_pbucket);
@@ -538,13 +426,5 @@ cudaError_t launch_raster_count(const RenderArgs &ra, cudaStream_t st) {
     if (e == cudaSuccess) e = launch_pixel_order(ra, st);
     return e;
 }
-
-cudaError_t launch_splat_fill(const RenderArgs &ra, cudaStream_t st) {
-    if (ra.L.n_tiles == 0) return cudaSuccess;
-    const cudaError_t e = launch_dispatch<kSplatFill>(make_args(ra), ra.L, ra.K, st);
-    if (e == cudaSuccess) count_launches(1);
-    return e;
-}
-
 
 }  // namespace ms

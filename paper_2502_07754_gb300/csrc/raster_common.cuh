@@ -15,10 +15,13 @@ __device__ __forceinline__ int count_bucket(uint32_t n) {
     return n < (uint32_t)kCountBuckets ? (int)n : kCountBuckets - 1;
 }
 
+// A pair's pixel rectangle clipped to its tile, relative to the tile's corner: x0 | y0 << 6 |
+// (w - 1) << 12 | (h - 1) << 18, bit 31 set; 0 for a pair with no pixel to test.
+__device__ __forceinline__ uint32_t pair_geo(int rx0, int ry0, int w, int h) {
+    return 0x80000000u | (uint32_t)rx0 | (uint32_t)ry0 << 6 | (uint32_t)(w - 1) << 12 | (uint32_t)(h - 1) << 18;
+}
+
 struct SceneDev {
-    const float *xyz, *rgb, *alpha;
-    int K;
-    const CamDev *cam;   // points into the kernel's __grid_constant__ view table
     int W, H;
     const float4 *dec;   // this view's decided vertices (xr, yr, Z or -1, origin), written by binning
     const uint32_t *face_mask;   // per fan, bit j = face j drawn; NULL = all
@@ -111,8 +114,6 @@ __device__ __forceinline__ DfVec df_view_offset(const CamDev &c, const float m[3
 struct Stage {
     int4 *rect;                   // [CH] i0, i1, j0, j1
     uint32_t *flags;              // [CH] bits 0..15 valid triangle, 16..31 negative orientation
-    uint32_t *q;                  // [CH] quantised depth bound
-    uint32_t *fan;                // [CH] fan id
     uint32_t *stie, *rtie;        // [CH] top-left tie bits of the spoke / rim directions
     float *ox, *oy;               // [CH] integer origin of the fan's relative positions
     float *vx, *vy;               // [KV][CH] decided vertices relative to the origin
@@ -122,7 +123,7 @@ struct Stage {
 };
 
 __host__ __device__ __forceinline__ size_t stage_bytes(int CH, int K) {
-    return (size_t)CH * (16 + 20 + 8 + 4 * (2 * (K + 1) + 5 * K));
+    return (size_t)CH * (16 + 12 + 8 + 4 * (2 * (K + 1) + 5 * K));
 }
 
 __device__ __forceinline__ Stage stage_ptrs(char *base, int CH, int K) {
@@ -130,9 +131,7 @@ __device__ __forceinline__ Stage stage_ptrs(char *base, int CH, int K) {
     Stage s;
     s.rect = reinterpret_cast<int4 *>(base);
     s.flags = reinterpret_cast<uint32_t *>(s.rect + CH);
-    s.q = s.flags + CH;
-    s.fan = s.q + CH;
-    s.stie = s.fan + CH;
+    s.stie = s.flags + CH;
     s.rtie = s.stie + CH;
     float *f = reinterpret_cast<float *>(s.rtie + CH);
     s.ox = f; f += CH;
@@ -170,7 +169,7 @@ __device__ __forceinline__ float group_max(float x) {
 // tie bits, valid-triangle flags and the pixel rectangle of every slot.
 template <int LPF>
 __device__ __forceinline__ void stage_decisions(const SceneDev &a, const Stage &s, int K, int slot, int sub,
-                                                bool active, uint32_t fan, uint32_t q) {
+                                                bool active, uint32_t fan) {
     constexpr int CH = 32 / LPF;
     const int KV = K + 1;
     const float4 *dv = a.dec + (size_t)fan * KV;
@@ -238,8 +237,6 @@ __device__ __forceinline__ void stage_decisions(const SceneDev &a, const Stage &
         s.stie[slot] = stie;
         s.rtie[slot] = rtie;
         s.flags[slot] = (tmask == 0 || r.empty) ? 0u : flags;
-        s.q[slot] = q;
-        s.fan[slot] = fan;
         s.rect[slot] = make_int4(r.i0, r.i1, r.j0, r.j1);
     }
 }
@@ -249,8 +246,8 @@ __device__ __forceinline__ void stage_decisions(const SceneDev &a, const Stage &
 // the shuffles).  The staged words are the same as one lane per fan would write.
 template <int LPF>
 __device__ __forceinline__ void stage_fans(const SceneDev &a, const Stage &s, int K, int lane, bool active,
-                                           uint32_t fan, uint32_t q) {
-    stage_decisions<LPF>(a, s, K, lane / LPF, lane % LPF, active, fan, q);
+                                           uint32_t fan) {
+    stage_decisions<LPF>(a, s, K, lane / LPF, lane % LPF, active, fan);
 }
 // Coverage of the pixel centre (pxc, pyc) by staged fan f: bit j is set when triangle j
 // covers it.  Each spoke value is computed once and turned into two pass bits (as the
@@ -313,20 +310,18 @@ __device__ __forceinline__ uint32_t cover_mask(const Stage &S, int CH, int K, in
 }
 
 // ------------------------------------------------------------------------------------
-// Source-Gaussian splats (FP64: the splat image is the reference the fans approximate,
-// drawn once per view, so precision is worth more than speed here)
+// Source-Gaussian splats in FP64 (the splat image is the reference that the fans approximate;
+// splat_raster.cu takes these formulas where its faster forms leave a case open)
 // ------------------------------------------------------------------------------------
 
-struct SplatSlot {
-    double mc[3], ua[3], ub[3], n[3];   // camera-space centre, kept unit axes, plane normal
-    double mcn, sa, sb;                 // mc . n, the two kept scales
-    float sigma, col[3];
+// The flat Gaussian g: rotation from the normalised quaternion (w, x, y, z), the two kept
+// axes by the same rule as the fan conversion.
+struct SplatAxes {
+    double m[3], ra[3], rb[3], sa, sb;   // centre, kept unit axes (world), their scales
+    float sigma;
 };
-
-// The flat Gaussian g in the camera frame: rotation from the normalised quaternion
-// (w, x, y, z), the two kept axes by the same rule as the fan conversion.
-__device__ __forceinline__ SplatSlot splat_setup(const SplatSrc &src, const CamDev &c, uint32_t g) {
-    SplatSlot o;
+__device__ __forceinline__ SplatAxes splat_axes(const SplatSrc &src, int64_t g) {
+    SplatAxes o;
     const float4 qf = *reinterpret_cast<const float4 *>(src.quats + 4 * (size_t)g);
     const double qn = sqrt((double)qf.x * qf.x + (double)qf.y * qf.y + (double)qf.z * qf.z + (double)qf.w * qf.w);
     const double w = qf.x / qn, x = qf.y / qn, y = qf.z / qn, z = qf.w / qn;
@@ -342,25 +337,41 @@ __device__ __forceinline__ SplatSlot splat_setup(const SplatSrc &src, const CamD
         if (s2 < sm) drop = 2;
     }
     const int ia = drop == 0 ? 1 : 0, ib = drop == 2 ? 1 : 2;
-    const float *m = src.means + 3 * (size_t)g;
-    const double dm[3] = {(double)m[0] - (double)c.C[0], (double)m[1] - (double)c.C[1], (double)m[2] - (double)c.C[2]};
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+        o.m[r] = (double)src.means[3 * (size_t)g + r];
+        o.ra[r] = ia == 0 ? R[3 * r] : R[3 * r + 1];
+        o.rb[r] = ib == 2 ? R[3 * r + 2] : R[3 * r + 1];
+    }
+    o.sa = exp((double)(ia == 0 ? s0 : s1));
+    o.sb = exp((double)(ib == 2 ? s2 : s1));
+    o.sigma = src.opacity[g];
+    return o;
+}
+
+struct SplatSlot {
+    double mc[3], ua[3], ub[3], n[3];   // camera-space centre, kept unit axes, plane normal
+    double mcn, sa, sb;                 // mc . n, the two kept scales
+    float sigma;
+};
+// The Gaussian in the camera frame of c.
+__device__ __forceinline__ SplatSlot splat_in_view(const SplatAxes &ax, const CamDev &c) {
+    SplatSlot o;
+    const double dm[3] = {ax.m[0] - (double)c.C[0], ax.m[1] - (double)c.C[1], ax.m[2] - (double)c.C[2]};
 #pragma unroll
     for (int r = 0; r < 3; ++r) {
         const double R0 = c.R[3 * r], R1 = c.R[3 * r + 1], R2 = c.R[3 * r + 2];
         o.mc[r] = R0 * dm[0] + R1 * dm[1] + R2 * dm[2];
-        o.ua[r] = R0 * R[ia] + R1 * R[3 + ia] + R2 * R[6 + ia];
-        o.ub[r] = R0 * R[ib] + R1 * R[3 + ib] + R2 * R[6 + ib];
+        o.ua[r] = R0 * ax.ra[0] + R1 * ax.ra[1] + R2 * ax.ra[2];
+        o.ub[r] = R0 * ax.rb[0] + R1 * ax.rb[1] + R2 * ax.rb[2];
     }
     o.n[0] = o.ua[1] * o.ub[2] - o.ua[2] * o.ub[1];
     o.n[1] = o.ua[2] * o.ub[0] - o.ua[0] * o.ub[2];
     o.n[2] = o.ua[0] * o.ub[1] - o.ua[1] * o.ub[0];
     o.mcn = o.mc[0] * o.n[0] + o.mc[1] * o.n[1] + o.mc[2] * o.n[2];
-    o.sa = exp((double)(ia == 0 ? s0 : s1));
-    o.sb = exp((double)(ib == 2 ? s2 : s1));
-    o.sigma = src.opacity[g];
-    o.col[0] = src.rgb[3 * (size_t)g];
-    o.col[1] = src.rgb[3 * (size_t)g + 1];
-    o.col[2] = src.rgb[3 * (size_t)g + 2];
+    o.sa = ax.sa;
+    o.sb = ax.sb;
+    o.sigma = ax.sigma;
     return o;
 }
 
