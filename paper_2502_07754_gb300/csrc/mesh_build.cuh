@@ -1,8 +1,7 @@
 // Per-Gaussian body of the Gaussian -> triangle-fan conversion (Sec. 3, "MeshSplats
 // Transformation for Flat Gaussians", Eq. 2 and the vertex equation after it; and
 // "Transformation for 3D Gaussians"), shared by the plain conversion kernel and the
-// conversion fused behind the learned initializer's inference.  One thread converts one
-// Gaussian into shared-memory staging; the caller stores the block's staging coalesced.
+// conversion fused behind the learned initializer's inference.
 #pragma once
 
 #include <math.h>
@@ -109,41 +108,52 @@ __device__ __forceinline__ void block_store(float *dst, const float *src, int n)
     }
 }
 
-// Converts Gaussian g into staging vertices lv .. lv + GV - 1 (s_xyz, s_rgb: 3 floats per
-// vertex; s_a: one).  cr: NULL, or the 2(K+1) corrections of g (radial dr_0..dr_K, then
-// log-opacity do_0..do_K; flat fans only): boundary vertex i moves to
-// m + (1 + dr_i)(cos th_i a + sin th_i b) and alpha_i <- clamp(alpha_i exp(do_i), 0, 1).
-template <int DEG, bool BF16>
-__device__ __forceinline__ void convert_gaussian(const Gaussians &G, const MeshBuildConst &kc, int64_t g,
-                                                 const float *cr, float *s_xyz, float *s_rgb, float *s_a,
-                                                 int lv) {
-    const int KV = kc.K + 1;
-    float m[3] = {__ldg(G.means + 3 * g), __ldg(G.means + 3 * g + 1), __ldg(G.means + 3 * g + 2)};
+// What a Gaussian's vertices are made of: centre, the scaled axes (a, b of the flat fan; all
+// three, in order, for three fans), colour, opacity.
+struct Frame {
+    float m[3], ax[3][3], col[3], sig;
+};
+template <int DEG, bool BF16, bool THREE>
+__device__ __forceinline__ Frame gaussian_frame(const Gaussians &G, const MeshBuildConst &kc, int64_t g) {
+    Frame F;
+    F.m[0] = __ldg(G.means + 3 * g);
+    F.m[1] = __ldg(G.means + 3 * g + 1);
+    F.m[2] = __ldg(G.means + 3 * g + 2);
     float s[3] = {__ldg(G.log_scales + 3 * g), __ldg(G.log_scales + 3 * g + 1), __ldg(G.log_scales + 3 * g + 2)};
     float4 q = __ldg(reinterpret_cast<const float4 *>(G.quats) + g);
+    F.sig = __ldg(G.opacity + g);
     float qn = rsqrtf(q.x * q.x + q.y * q.y + q.z * q.z + q.w * q.w);
     float w = q.x * qn, x = q.y * qn, y = q.z * qn, z = q.w * qn;
     // Rotation matrix, row-major; column c of R is the principal axis r_{c+1}.
     float R[9] = {1.f - 2.f * (y * y + z * z), 2.f * (x * y - w * z), 2.f * (x * z + w * y),
                   2.f * (x * y + w * z), 1.f - 2.f * (x * x + z * z), 2.f * (y * z - w * x),
                   2.f * (x * z - w * y), 2.f * (y * z + w * x), 1.f - 2.f * (x * x + y * y)};
-    int drop = 0;
-    if (kc.axis_rule == 1) {
-        if (s[1] < s[drop]) drop = 1;
-        if (s[2] < s[drop]) drop = 2;
-    }
-    const int ia = drop == 0 ? 1 : 0, ib = drop == 2 ? 1 : 2;
-    const float sa = kc.scale_mul * expf(s[ia]), sb = kc.scale_mul * expf(s[ib]);
-    float a[3], b[3];
+    if (THREE) {
 #pragma unroll
-    for (int r = 0; r < 3; ++r) {
-        a[r] = sa * R[3 * r + ia];
-        b[r] = sb * R[3 * r + ib];
+        for (int c = 0; c < 3; ++c) {
+            const float sc = kc.scale_mul * expf(s[c]);
+#pragma unroll
+            for (int r = 0; r < 3; ++r) F.ax[c][r] = sc * R[3 * r + c];
+        }
+    } else {
+        int drop = 0;
+        float sd = s[0];
+        if (kc.axis_rule == 1) {
+            if (s[1] < sd) { drop = 1; sd = s[1]; }
+            if (s[2] < sd) drop = 2;
+        }
+        const float sa = kc.scale_mul * expf(drop == 0 ? s[1] : s[0]), sb = kc.scale_mul * expf(drop == 2 ? s[1] : s[2]);
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+            F.ax[0][r] = sa * (drop == 0 ? R[3 * r + 1] : R[3 * r]);
+            F.ax[1][r] = sb * (drop == 2 ? R[3 * r + 1] : R[3 * r + 2]);
+            F.ax[2][r] = 0.0f;
+        }
     }
     constexpr int NB = (DEG + 1) * (DEG + 1);
     float Y[NB];
     int nuse = 1;
-    float dx = m[0] - kc.cc[0], dy = m[1] - kc.cc[1], dz = m[2] - kc.cc[2];
+    float dx = F.m[0] - kc.cc[0], dy = F.m[1] - kc.cc[1], dz = F.m[2] - kc.cc[2];
     float dn = dx * dx + dy * dy + dz * dz;
     if (DEG > 0 && kc.has_cam && dn > 0.0f) {
         float inv = rsqrtf(dn);
@@ -152,44 +162,34 @@ __device__ __forceinline__ void convert_gaussian(const Gaussians &G, const MeshB
     } else {
         Y[0] = kc.shc[0];
     }
-    float col[3];   // one per Gaussian, inherited by all its vertices
-    sh_colour<DEG, BF16>(G.sh, g, kc.sh_vec_ok, Y, nuse, col);
-    const float sig = __ldg(G.opacity + g);
-    if (kc.three) {
-        float sr[3][3];   // sr[c] = scale_mul exp(s_c) r_c
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const float sc = kc.scale_mul * expf(s[c]);
-#pragma unroll
-            for (int r = 0; r < 3; ++r) sr[c][r] = sc * R[3 * r + c];
-        }
-        for (int fan = 0; fan < 3; ++fan) {
-            const int fa = fan == 2 ? 1 : 0, fb = fan == 0 ? 1 : 2;
-            for (int k = 0; k < KV; ++k) {
-                const int v = lv + fan * KV + k;
-#pragma unroll
-                for (int r = 0; r < 3; ++r) {
-                    s_xyz[3 * v + r] = k == 0 ? m[r]
-                                              : m[r] + (kc.cs[k - 1] * sr[fa][r] + kc.sn[k - 1] * sr[fb][r]);
-                    s_rgb[3 * v + r] = col[r];
-                }
-                s_a[v] = k == 0 ? sig : kc.opac_mul * sig;
-            }
-        }
-        return;
-    }
+    sh_colour<DEG, BF16>(G.sh, g, kc.sh_vec_ok, Y, nuse, F.col);   // one per Gaussian, inherited by its vertices
+    return F;
+}
+
+// Converts Gaussian g into staging vertices lv .. lv + K (s_xyz, s_rgb: 3 floats per
+// vertex; s_a: one) of a flat fan.  cr: the 2(K+1) corrections of g (radial dr_0..dr_K, then
+// log-opacity do_0..do_K): boundary vertex i goes to
+// m + (1 + dr_i)(cos th_i a + sin th_i b) and alpha_i to clamp(alpha_i exp(do_i), 0, 1).
+template <int DEG, bool BF16>
+__device__ __forceinline__ void convert_gaussian(const Gaussians &G, const MeshBuildConst &kc, int64_t g,
+                                                 const float *cr, float *s_xyz, float *s_rgb, float *s_a,
+                                                 int lv) {
+    const int KV = kc.K + 1;
+    const Frame F = gaussian_frame<DEG, BF16, false>(G, kc, g);
+    const float *m = F.m, *a = F.ax[0], *b = F.ax[1], *col = F.col;
+    const float sig = F.sig;
     for (int k = 0; k < KV; ++k) {
         float p[3];
         if (k == 0) {
             p[0] = m[0]; p[1] = m[1]; p[2] = m[2];
         } else {
             const float c = kc.cs[k - 1], sn = kc.sn[k - 1];
-            const float rs = cr ? 1.0f + cr[k] : 1.0f;
+            const float rs = 1.0f + cr[k];
 #pragma unroll
             for (int r = 0; r < 3; ++r) p[r] = m[r] + rs * (c * a[r] + sn * b[r]);
         }
         float op = k == 0 ? sig : kc.opac_mul * sig;
-        if (cr) op = fminf(fmaxf(op * expf(cr[KV + k]), 0.0f), 1.0f);
+        op = fminf(fmaxf(op * expf(cr[KV + k]), 0.0f), 1.0f);
 #pragma unroll
         for (int r = 0; r < 3; ++r) {
             s_xyz[3 * (lv + k) + r] = p[r];
