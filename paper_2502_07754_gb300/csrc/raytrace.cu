@@ -11,7 +11,7 @@
 //     (1 - a_g) over every other triangle g the segment p -> L crosses (parameter strictly
 //     inside (1e-9, 1 - 1e-9)), and its colour becomes c (k + (1 - k) S), k the ambient
 //     share; a shadow ray stops once S < T_eps, the primary composite's own bound.
-// Intersections are decided in FP64 (Moller-Trumbore, edges closed), values in FP64.
+// Intersections are decided as in FP64 (Moller-Trumbore, edges closed).
 //
 // Acceleration: a linear BVH (Karras 2012, "Maximizing parallelism in the construction of
 // BVHs, octrees, and k-d trees"): 30-bit Morton codes of the triangle centroids in the
@@ -26,8 +26,10 @@
 // nearest crossings beyond the last composited one (by (t, triangle)), composites them in
 // order, and repeats while some crossing was left out and the transmittance is above
 // T_eps.  A pass skips boxes that end before the last composited crossing and, once its
-// buffer is full, boxes that start beyond the farthest kept one; a binary32 filter
-// (mt_may_hit) keeps the FP64 test for triangles the ray may cross.
+// buffer is full, boxes that start beyond the farthest kept one.  FP64 runs at a small fraction
+// of the binary32 rate here, so a triangle meets a binary32 filter (mt_may_hit), then a
+// double-float test (mt_df), and FP64 only where neither is certain (the ray within 2^-40 of an
+// edge): the decisions are those of FP64, the values within 2^-42 of it.
 #include "ms_common.cuh"
 #include "ms_internal.h"
 
@@ -41,7 +43,7 @@ constexpr int kTraceKB = 8;
 constexpr int kStack = 64;
 constexpr double kSegEps = 1e-9;
 
-struct BvhNode {
+struct alignas(16) BvhNode {
     float lo[3], hi[3];
     int left, right;   // children: < n - 1 internal, >= n - 1 leaf (n - 1 + sorted position)
 };
@@ -259,14 +261,15 @@ struct TraceArgs {
     unsigned *overflow;   // traversal stack overflows (status)
 };
 
+// A crossing: parameter and barycentrics as double-float values.
 struct Hit {
-    double t, u, v;
+    dfl t, u, v;
     int tri;
 };
 
 // Moller-Trumbore in FP64, edges closed: the crossing of o + t d with triangle (P0, P1, P2).
-__device__ __forceinline__ bool mt(const double o[3], const double d[3], const double P0[3], const double P1[3],
-                                   const double P2[3], double &t, double &u, double &v) {
+__device__ __noinline__ bool mt(const double o[3], const double d[3], const double P0[3], const double P1[3],
+                                const double P2[3], double &t, double &u, double &v) {
     const double e1[3] = {P1[0] - P0[0], P1[1] - P0[1], P1[2] - P0[2]};
     const double e2[3] = {P2[0] - P0[0], P2[1] - P0[1], P2[2] - P0[2]};
     const double pv[3] = {d[1] * e2[2] - d[2] * e2[1], d[2] * e2[0] - d[0] * e2[2], d[0] * e2[1] - d[1] * e2[0]};
@@ -291,39 +294,47 @@ __device__ __forceinline__ bool mt(const double o[3], const double d[3], const d
 // FP64 arithmetic runs at a small fraction of the binary32 rate on this GPU, and most
 // boxes the traversal reaches hold triangles the ray misses.
 struct RayF {
-    float o[3], d[3], ao[3], ad[3];
+    dfl o[3], d[3];   // double-float origin and direction; the filter takes the high parts
 };
+__device__ __forceinline__ dfl df_of(double x) {
+    const float h = (float)x;
+    return dfl{h, (float)(x - (double)h)};
+}
+__device__ __forceinline__ double to_double(dfl a) { return (double)a.h + (double)a.l; }
 __device__ __forceinline__ RayF ray_f(const double o[3], const double d[3]) {
     RayF r;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        r.o[k] = (float)o[k];
-        r.d[k] = (float)d[k];
-        r.ao[k] = fabsf(r.o[k]);
-        r.ad[k] = fabsf(r.d[k]);
+        r.o[k] = df_of(o[k]);
+        r.d[k] = df_of(d[k]);
     }
     return r;
 }
+// Error bounds of the filter's determinant and numerators.
+struct MtBounds {
+    float det, U, V, T;
+};
 __device__ __forceinline__ bool mt_may_hit(const RayF &r, const float P0[3], const float P1[3], const float P2[3],
-                                           float tmin, float tmax) {
+                                           float tmin, float tmax, MtBounds &e) {
     constexpr float kU = 64.0f * 0x1p-24f;
     float e1[3], e2[3], tv[3], E1[3], E2[3], TV[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         e1[k] = P1[k] - P0[k];
         e2[k] = P2[k] - P0[k];
-        tv[k] = r.o[k] - P0[k];
+        tv[k] = r.o[k].h - P0[k];
         const float a0 = fabsf(P0[k]);
         E1[k] = fabsf(P1[k]) + a0;
         E2[k] = fabsf(P2[k]) + a0;
-        TV[k] = r.ao[k] + a0;
+        TV[k] = fabsf(r.o[k].h) + a0;
     }
-    const float pv[3] = {r.d[1] * e2[2] - r.d[2] * e2[1], r.d[2] * e2[0] - r.d[0] * e2[2],
-                         r.d[0] * e2[1] - r.d[1] * e2[0]};
-    const float PV[3] = {r.ad[1] * E2[2] + r.ad[2] * E2[1], r.ad[2] * E2[0] + r.ad[0] * E2[2],
-                         r.ad[0] * E2[1] + r.ad[1] * E2[0]};
+    const float d0 = r.d[0].h, d1 = r.d[1].h, d2 = r.d[2].h;
+    const float a0 = fabsf(d0), a1 = fabsf(d1), a2 = fabsf(d2);
+    const float pv[3] = {d1 * e2[2] - d2 * e2[1], d2 * e2[0] - d0 * e2[2], d0 * e2[1] - d1 * e2[0]};
+    const float PV[3] = {a1 * E2[2] + a2 * E2[1], a2 * E2[0] + a0 * E2[2], a0 * E2[1] + a1 * E2[0]};
     const float det = e1[0] * pv[0] + e1[1] * pv[1] + e1[2] * pv[2];
     const float eDet = kU * (E1[0] * PV[0] + E1[1] * PV[1] + E1[2] * PV[2]);
+    e = MtBounds{eDet, 3.0e38f, 3.0e38f, 3.0e38f};   // (undetermined: all of it is left to FP64)
     if (!(fabsf(det) > eDet)) return true;
     const float sg = det > 0.0f ? 1.0f : -1.0f;
     const float U = tv[0] * pv[0] + tv[1] * pv[1] + tv[2] * pv[2];
@@ -331,15 +342,58 @@ __device__ __forceinline__ bool mt_may_hit(const RayF &r, const float P0[3], con
     if (sg * U < -eU) return false;
     const float qv[3] = {tv[1] * e1[2] - tv[2] * e1[1], tv[2] * e1[0] - tv[0] * e1[2], tv[0] * e1[1] - tv[1] * e1[0]};
     const float QV[3] = {TV[1] * E1[2] + TV[2] * E1[1], TV[2] * E1[0] + TV[0] * E1[2], TV[0] * E1[1] + TV[1] * E1[0]};
-    const float V = qv[0] * r.d[0] + qv[1] * r.d[1] + qv[2] * r.d[2];
-    const float eV = kU * (QV[0] * r.ad[0] + QV[1] * r.ad[1] + QV[2] * r.ad[2]);
+    const float V = qv[0] * d0 + qv[1] * d1 + qv[2] * d2;
+    const float eV = kU * (QV[0] * a0 + QV[1] * a1 + QV[2] * a2);
     if (sg * V < -eV) return false;
     if (sg * (U + V - det) > eU + eV + eDet) return false;
     const float Tn = e2[0] * qv[0] + e2[1] * qv[1] + e2[2] * qv[2];
     const float eT = kU * (E2[0] * QV[0] + E2[1] * QV[1] + E2[2] * QV[2]);
     const float t = Tn / det;
     const float dt = (eT + fabsf(t) * eDet) / (fabsf(det) - eDet) + kU * fabsf(t);
+    e = MtBounds{eDet, eU, eV, eT};
     return t + dt >= tmin && t - dt <= tmax;
+}
+
+// The same crossing in double-float, whose operations carry errors of at most 2^-42 of the same
+// sums: 1 crossing within (tmin, tmax), 0 none, -1 a quantity closer to its limit than 2^-40 of
+// the sums (64 units of 2^-24 scaled by 2^-22), which leaves the triangle to the FP64 test.
+// FP64's own rounding is far inside the margin, so the decisions are those of the FP64 test.
+__device__ __forceinline__ dfl df_det2(dfl a, dfl b, dfl c, dfl d) { return df_add_fast(df_mul(a, b), df_neg(df_mul(c, d))); }
+__device__ __forceinline__ dfl df_dot(const dfl a[3], const dfl b[3]) {
+    return df_add_fast(df_add_fast(df_mul(a[0], b[0]), df_mul(a[1], b[1])), df_mul(a[2], b[2]));
+}
+__device__ __forceinline__ int mt_df(const RayF &r, const float P0[3], const float P1[3], const float P2[3],
+                                     const MtBounds &e, dfl tmin, dfl tmax, Hit &h) {
+    constexpr float kS = 0x1p-22f;
+    const float eD = kS * e.det, eU = kS * e.U, eV = kS * e.V;
+    dfl e1[3], e2[3], tv[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        e1[k] = df_two_sum(P1[k], -P0[k]);
+        e2[k] = df_two_sum(P2[k], -P0[k]);
+        tv[k] = df_add_f(r.o[k], -P0[k]);
+    }
+    const dfl pv[3] = {df_det2(r.d[1], e2[2], r.d[2], e2[1]), df_det2(r.d[2], e2[0], r.d[0], e2[2]),
+                       df_det2(r.d[0], e2[1], r.d[1], e2[0])};
+    const dfl det = df_dot(e1, pv), U = df_dot(tv, pv);
+    // (below 2^-80 the products' low parts could leave binary32's range)
+    if (!(fabsf(det.h) > eD && fabsf(U.h) > eU && e.det > 0x1p-80f && e.U < 1.0e38f)) return -1;
+    const float sg = det.h > 0.0f ? 1.0f : -1.0f;
+    if (sg * U.h < 0.0f) return 0;
+    const dfl qv[3] = {df_det2(tv[1], e1[2], tv[2], e1[1]), df_det2(tv[2], e1[0], tv[0], e1[2]),
+                       df_det2(tv[0], e1[1], tv[1], e1[0])};
+    const dfl V = df_dot(qv, r.d);
+    const dfl W = df_add_fast(df_add_fast(U, V), df_neg(det));
+    if (!(fabsf(V.h) > eV && fabsf(W.h) > eU + eV + eD)) return -1;
+    if (sg * V.h < 0.0f || sg * W.h > 0.0f) return 0;
+    h.t = df_div_rcp(df_dot(e2, qv), det);
+    const float dt = kS * ((e.T + fabsf(h.t.h) * e.det) / fabsf(det.h)) + 0x1p-40f * fabsf(h.t.h);
+    const float below = df_add_fast(h.t, df_neg(tmin)).h, above = df_add_fast(h.t, df_neg(tmax)).h;
+    if (!(fabsf(below) > dt && fabsf(above) > dt)) return -1;
+    if (below < 0.0f || above > 0.0f) return 0;
+    h.u = df_div_rcp(U, det);
+    h.v = df_div_rcp(V, det);
+    return 1;
 }
 
 __device__ __forceinline__ void tri_f(const TraceArgs &a, int tri, float P[3][3]) {
@@ -351,100 +405,110 @@ __device__ __forceinline__ void tri_f(const TraceArgs &a, int tri, float P[3][3]
         for (int r = 0; r < 3; ++r) P[k][r] = __ldg(a.xyz + 3 * v[k] + r);
 }
 
-__device__ __forceinline__ void load_tri(const TraceArgs &a, int tri, int64_t v[3], double P[3][3]) {
-    tri_verts(a.tris, a.K, tri, v);
+// Whether the ray (o, d; rf its double-float form) crosses triangle P within (tmin, tmax): the
+// binary32 filter, then double-float, then FP64 where neither is certain.
+__device__ __forceinline__ bool crosses(const double o[3], const double d[3], const RayF &rf, const float P[3][3],
+                                        float f_min, float f_max, double tmin, double tmax, Hit &h) {
+    MtBounds e;
+    if (!mt_may_hit(rf, P[0], P[1], P[2], f_min, f_max, e)) return false;
+    const int c = mt_df(rf, P[0], P[1], P[2], e, df_of(tmin), df_of(tmax), h);
+    if (c >= 0) return c != 0;
+    double Q[3][3], t, u, v;
 #pragma unroll
     for (int k = 0; k < 3; ++k)
 #pragma unroll
-        for (int r = 0; r < 3; ++r) P[k][r] = (double)__ldg(a.xyz + 3 * v[k] + r);
+        for (int r = 0; r < 3; ++r) Q[k][r] = (double)P[k][r];
+    if (!(mt(o, d, Q[0], Q[1], Q[2], t, u, v) && t > tmin && t < tmax)) return false;
+    h.t = df_of(t);
+    h.u = df_of(u);
+    h.v = df_of(v);
+    return true;
 }
 
-// Slab test of the ray o + t d, t in [t0, t1], against a node box (binary32, widened).
-__device__ __forceinline__ bool box_hit(const BvhNode &nd, const float o[3], const float id[3], float t0, float t1) {
+// Slab test of the ray o + t d against a node box (binary32, widened): whether it meets [t0, t1],
+// and where (tn, tf).
+__device__ __forceinline__ bool box_span(const BvhNode *node, const float o[3], const float id[3], float t0, float t1,
+                                         float &tn, float &tf, int &left, int &right) {
+    const float4 a = __ldg(reinterpret_cast<const float4 *>(node)), b = __ldg(reinterpret_cast<const float4 *>(node) + 1);
+    const float lo[3] = {a.x, a.y, a.z}, hi[3] = {a.w, b.x, b.y};
+    left = __float_as_int(b.z);
+    right = __float_as_int(b.w);
 #pragma unroll
     for (int r = 0; r < 3; ++r) {
-        float a = (nd.lo[r] - o[r]) * id[r], b = (nd.hi[r] - o[r]) * id[r];
-        if (a > b) { const float tmp = a; a = b; b = tmp; }
-        if (!(a == a)) a = -3.0e38f;   // 0 * inf
-        if (!(b == b)) b = 3.0e38f;
-        t0 = fmaxf(t0, a);
-        t1 = fminf(t1, b);
-    }
-    return t0 <= t1;
-}
-
-// The same slab test returning the parameter interval [tn, tf] of the box (within t0, t1).
-__device__ __forceinline__ bool box_span(const BvhNode &nd, const float o[3], const float id[3], float t0, float t1,
-                                         float &tn, float &tf) {
-#pragma unroll
-    for (int r = 0; r < 3; ++r) {
-        float a = (nd.lo[r] - o[r]) * id[r], b = (nd.hi[r] - o[r]) * id[r];
-        if (a > b) { const float tmp = a; a = b; b = tmp; }
-        if (!(a == a)) a = -3.0e38f;   // 0 * inf
-        if (!(b == b)) b = 3.0e38f;
-        t0 = fmaxf(t0, a);
-        t1 = fminf(t1, b);
+        const float x = (lo[r] - o[r]) * id[r], y = (hi[r] - o[r]) * id[r];
+        // (0 * inf, a ray in the plane of a side, does not bound the interval)
+        t0 = fmaxf(t0, x == x && y == y ? fminf(x, y) : -3.0e38f);
+        t1 = fminf(t1, x == x && y == y ? fmaxf(x, y) : 3.0e38f);
     }
     tn = t0;
     tf = t1;
     return t0 <= t1;
 }
 
-__device__ __forceinline__ bool hit_less(double ta, int ia, double tb, int ib) { return ta < tb || (ta == tb && ia < ib); }
+__device__ __forceinline__ bool hit_less(dfl ta, int ia, dfl tb, int ib) {
+    return df_lt(ta, tb) || (ta.h == tb.h && ta.l == tb.l && ia < ib);
+}
+// a0 (1 - u - v) + a1 u + a2 v in double-float.
+__device__ __forceinline__ dfl bary_mix(dfl u, dfl v, float a0, float a1, float a2) {
+    const dfl w = df_add_f(df_neg(df_add_fast(u, v)), 1.0f);
+    return df_add_fast(df_add_fast(df_mul_f(w, a0), df_mul_f(u, a1)), df_mul_f(v, a2));
+}
 
 // Transmittance of the segment p -> L through every triangle but `own`.
 __device__ double shadow(const TraceArgs &a, const double p[3], int own) {
     const double d[3] = {a.L[0] - p[0], a.L[1] - p[1], a.L[2] - p[2]};
-    const float of[3] = {(float)p[0], (float)p[1], (float)p[2]};
     const RayF rf = ray_f(p, d);
-    float id[3];
+    float of[3], id[3];
 #pragma unroll
-    for (int r = 0; r < 3; ++r) id[r] = 1.0f / (float)d[r];
-    int stack[kStack];
-    int sp = 0;
-    stack[sp++] = 0;
-    double S = 1.0;
-    const int64_t n = a.T;
-    while (sp > 0) {
-        const int node = stack[--sp];
-        const BvhNode &nd = a.nodes[node];
-        if (!box_hit(nd, of, id, -1e-3f, 1.001f)) continue;
-        if (node >= n - 1) {
-            const int tri = a.leaf_tri[node - (n - 1)];
-            if (tri == own) continue;
-            {
-                float Pf[3][3];
-                tri_f(a, tri, Pf);
-                if (!mt_may_hit(rf, Pf[0], Pf[1], Pf[2], (float)kSegEps, (float)(1.0 - kSegEps))) continue;
-            }
-            int64_t v[3];
-            double P[3][3], t, u, w;
-            load_tri(a, tri, v, P);
-            if (mt(p, d, P[0], P[1], P[2], t, u, w) && t > kSegEps && t < 1.0 - kSegEps) {
-                const double al = (1.0 - u - w) * __ldg(a.alpha + v[0]) + u * __ldg(a.alpha + v[1]) +
-                                  w * __ldg(a.alpha + v[2]);
-                S *= 1.0 - al;
-                // the light is blocked to within T_eps: the colour's shadow factor moves by at
-                // most (1 - ambient) T_eps, the primary composite's own termination bound
-                if (S < a.T_eps) return S;
-            }
-            continue;
-        }
-        if (sp + 2 > kStack) {
-            atomicAdd(a.overflow, 1u);
-            continue;
-        }
-        stack[sp++] = nd.left;
-        stack[sp++] = nd.right;
+    for (int r = 0; r < 3; ++r) {
+        of[r] = rf.o[r].h;
+        id[r] = 1.0f / rf.d[r].h;
     }
-    return S;
+    const int n1 = (int)(a.T - 1);   // nodes from n1 on are leaves
+    int stack[kStack];
+    int sp = 0, node = 0;
+    dfl S = df_make(1.0f);
+    const float t0 = -1e-3f, t1 = 1.001f;
+    for (;;) {
+        // down to a leaf whose parent's test admitted it
+        while (node >= 0 && node < n1) {
+            const int left = __ldg(&a.nodes[node].left), right = __ldg(&a.nodes[node].right);
+            float tn, tf;
+            int x, y;
+            const bool hl = box_span(a.nodes + left, of, id, t0, t1, tn, tf, x, y);
+            const bool hr = box_span(a.nodes + right, of, id, t0, t1, tn, tf, x, y);
+            if (hl && hr) {
+                if (sp < kStack) stack[sp++] = right;
+                else atomicAdd(a.overflow, 1u);
+            }
+            node = hl ? left : (hr ? right : (sp > 0 ? stack[--sp] : -1));
+        }
+        if (node < 0) break;
+        const int tri = __ldg(a.leaf_tri + (node - n1));
+        node = sp > 0 ? stack[--sp] : -1;
+        if (tri == own) continue;
+        float P[3][3];
+        tri_f(a, tri, P);
+        Hit h;
+        if (!crosses(p, d, rf, P, (float)kSegEps, (float)(1.0 - kSegEps), kSegEps, 1.0 - kSegEps, h)) continue;
+        int64_t v[3];
+        tri_verts(a.tris, a.K, tri, v);
+        const dfl al = bary_mix(h.u, h.v, __ldg(a.alpha + v[0]), __ldg(a.alpha + v[1]), __ldg(a.alpha + v[2]));
+        S = df_mul(S, df_add_f(df_neg(al), 1.0f));
+        // the light is blocked to within T_eps: the colour's shadow factor moves by at
+        // most (1 - ambient) T_eps, the primary composite's own termination bound
+        if (to_double(S) < a.T_eps) break;
+    }
+    return to_double(S);
 }
 
+// One thread a pixel, a block an 8 x 8 tile of pixels (a warp 8 x 4), so that a warp's rays stay
+// together down the tree.
 __global__ void __launch_bounds__(kTraceThreads) trace_kernel(const __grid_constant__ TraceArgs a) {
-    const int64_t pix = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int W = a.cam.width, H = a.cam.height;
-    if (pix >= (int64_t)W * H) return;
-    const int px = (int)(pix % W), py = (int)(pix / W);
+    const int px = blockIdx.x * 8 + (threadIdx.x & 7), py = blockIdx.y * 8 + (threadIdx.x >> 3);
+    if (px >= W || py >= H) return;
+    const int64_t pix = (int64_t)py * W + px;
     const CamDev &c = a.cam;
     // ray with unit view depth: d = R^T ((x - cx) / fx, (y - cy) / fy, 1)
     const double dc[3] = {((double)px + 0.5 - (double)c.cx) / (double)c.fx,
@@ -455,84 +519,92 @@ __global__ void __launch_bounds__(kTraceThreads) trace_kernel(const __grid_const
         d[r] = ((double)c.R[r] * dc[0] + (double)c.R[3 + r] * dc[1]) + (double)c.R[6 + r] * dc[2];
         o[r] = (double)c.C[r];
     }
-    const float of[3] = {(float)o[0], (float)o[1], (float)o[2]};
-    float id[3];
-#pragma unroll
-    for (int r = 0; r < 3; ++r) id[r] = 1.0f / (float)d[r];
     const RayF rf = ray_f(o, d);
-    const int64_t n = a.T;
+    float of[3], id[3];
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+        of[r] = rf.o[r].h;
+        id[r] = 1.0f / rf.d[r].h;
+    }
+    const int n1 = (int)(a.T - 1);   // nodes from n1 on are leaves
     double T = 1.0, C0 = 0.0, C1 = 0.0, C2 = 0.0;
-    double after_t = -1.0e300;
+    dfl after_t = df_make(-3.0e38f);
     int after_i = -1;
-    for (int pass = 0; n > 0; ++pass) {
+    for (int pass = 0; a.T > 0; ++pass) {
         Hit buf[kTraceKB];
         int nb = 0;
         bool more = false;
         int stack[kStack];
-        int sp = 0;
-        stack[sp++] = 0;
+        int sp = 0, node = 0;
         // Boxes wholly before the last composited crossing hold nothing for this pass, and
         // boxes wholly beyond the farthest kept crossing of a full buffer only mean another
         // pass; both bounds are widened by 1e-5 relative, far above the slab test's rounding.
-        const float t_after = after_t > 0.0 ? (float)after_t * (1.0f - 1e-5f) : 0.0f;
-        while (sp > 0) {
-            const int node = stack[--sp];
-            const BvhNode &nd = a.nodes[node];
-            float tn, tf;
-            if (!box_span(nd, of, id, (float)c.znear * 0.999f, 3.0e38f, tn, tf)) continue;
-            if (tf < t_after) continue;
-            if (nb == kTraceKB && tn > (float)buf[kTraceKB - 1].t * (1.0f + 1e-5f)) {
-                more = true;
-                continue;
-            }
-            if (node >= n - 1) {
-                const int tri = a.leaf_tri[node - (n - 1)];
-                {
-                    // crossings before the last composited one were taken in an earlier pass
-                    float Pf[3][3];
-                    tri_f(a, tri, Pf);
-                    if (!mt_may_hit(rf, Pf[0], Pf[1], Pf[2], fmaxf(c.znear, (float)after_t), 3.0e38f)) continue;
-                }
-                int64_t v[3];
-                double P[3][3], t, u, w;
-                load_tri(a, tri, v, P);
-                if (!(mt(o, d, P[0], P[1], P[2], t, u, w) && t > (double)c.znear)) continue;
-                if (!hit_less(after_t, after_i, t, tri)) continue;   // composited in an earlier pass
+        const float t_after = after_t.h > 0.0f ? after_t.h * (1.0f - 1e-5f) : 0.0f;
+        const float t_near = c.znear * 0.999f;
+        for (;;) {
+            while (node >= 0 && node < n1) {
+                const int left = __ldg(&a.nodes[node].left), right = __ldg(&a.nodes[node].right);
+                float nl, fl, nr, fr;
+                int x, y;
+                bool hl = box_span(a.nodes + left, of, id, t_near, 3.0e38f, nl, fl, x, y) && fl >= t_after;
+                bool hr = box_span(a.nodes + right, of, id, t_near, 3.0e38f, nr, fr, x, y) && fr >= t_after;
                 if (nb == kTraceKB) {
-                    more = true;
-                    if (!hit_less(t, tri, buf[kTraceKB - 1].t, buf[kTraceKB - 1].tri)) continue;
-                    --nb;   // the farthest kept crossing waits for a later pass
+                    const float t_far = buf[kTraceKB - 1].t.h * (1.0f + 1e-5f);
+                    if (hl && nl > t_far) {
+                        hl = false;
+                        more = true;
+                    }
+                    if (hr && nr > t_far) {
+                        hr = false;
+                        more = true;
+                    }
                 }
-                int s = nb;
-                while (s > 0 && hit_less(t, tri, buf[s - 1].t, buf[s - 1].tri)) {
-                    buf[s] = buf[s - 1];
-                    --s;
+                // the nearer child first: the buffer fills with near crossings early
+                const bool swap = hl && hr && nr < nl;
+                const int first = swap || !hl ? right : left, second = swap ? left : right;
+                if (hl && hr) {
+                    if (sp < kStack) stack[sp++] = second;
+                    else atomicAdd(a.overflow, 1u);
                 }
-                buf[s] = Hit{t, u, w, tri};
-                ++nb;
-                continue;
+                node = hl || hr ? first : (sp > 0 ? stack[--sp] : -1);
             }
-            if (sp + 2 > kStack) {
-                atomicAdd(a.overflow, 1u);
-                continue;
+            if (node < 0) break;
+            const int tri = __ldg(a.leaf_tri + (node - n1));
+            node = sp > 0 ? stack[--sp] : -1;
+            float P[3][3];
+            tri_f(a, tri, P);
+            Hit h;
+            // crossings before the last composited one were taken in an earlier pass
+            if (!crosses(o, d, rf, P, fmaxf(c.znear, after_t.h), 3.0e38f, (double)c.znear, 1.0e300, h)) continue;
+            h.tri = tri;
+            if (!hit_less(after_t, after_i, h.t, tri)) continue;   // composited in an earlier pass
+            if (nb == kTraceKB) {
+                more = true;
+                if (!hit_less(h.t, tri, buf[kTraceKB - 1].t, buf[kTraceKB - 1].tri)) continue;
+                --nb;   // the farthest kept crossing waits for a later pass
             }
-            stack[sp++] = nd.left;
-            stack[sp++] = nd.right;
+            int s = nb;
+            while (s > 0 && hit_less(h.t, tri, buf[s - 1].t, buf[s - 1].tri)) {
+                buf[s] = buf[s - 1];
+                --s;
+            }
+            buf[s] = h;
+            ++nb;
         }
         bool stop = false;
         for (int k = 0; k < nb; ++k) {
             const Hit &h = buf[k];
             int64_t v[3];
             tri_verts(a.tris, a.K, h.tri, v);
-            const double w0 = 1.0 - h.u - h.v;
-            const double al = w0 * __ldg(a.alpha + v[0]) + h.u * __ldg(a.alpha + v[1]) + h.v * __ldg(a.alpha + v[2]);
+            const double al = to_double(bary_mix(h.u, h.v, __ldg(a.alpha + v[0]), __ldg(a.alpha + v[1]), __ldg(a.alpha + v[2])));
             double col[3];
 #pragma unroll
             for (int r = 0; r < 3; ++r)
-                col[r] = w0 * __ldg(a.rgb + 3 * v[0] + r) + h.u * __ldg(a.rgb + 3 * v[1] + r) +
-                         h.v * __ldg(a.rgb + 3 * v[2] + r);
+                col[r] = to_double(bary_mix(h.u, h.v, __ldg(a.rgb + 3 * v[0] + r), __ldg(a.rgb + 3 * v[1] + r),
+                                            __ldg(a.rgb + 3 * v[2] + r)));
             if (a.shadows) {
-                const double p[3] = {o[0] + h.t * d[0], o[1] + h.t * d[1], o[2] + h.t * d[2]};
+                const double t = to_double(h.t);
+                const double p[3] = {o[0] + t * d[0], o[1] + t * d[1], o[2] + t * d[2]};
                 const double f = a.ambient + (1.0 - a.ambient) * shadow(a, p, h.tri);
 #pragma unroll
                 for (int r = 0; r < 3; ++r) col[r] *= f;
@@ -637,8 +709,8 @@ extern "C" MS_API ms_status ms_raytrace(const float *xyz, const float *rgb, cons
     a.ambient = ambient;
     a.T_eps = T_eps;
     a.out = out_rgba;
-    const int64_t npx = (int64_t)cam->width * cam->height;
-    trace_kernel<<<(unsigned)((npx + kTraceThreads - 1) / kTraceThreads), kTraceThreads, 0, (cudaStream_t)stream>>>(a);
+    const dim3 grid((cam->width + 7) / 8, (cam->height + 7) / 8);
+    trace_kernel<<<grid, kTraceThreads, 0, (cudaStream_t)stream>>>(a);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return set_error(MS_ERR_CUDA, "trace_kernel: %s", cudaGetErrorString(e));
     count_launches(1);
