@@ -112,12 +112,12 @@ typedef struct {
 
 typedef struct {
     int32_t tile;           /* screen tile edge in pixels: 8, 16 or 32 */
-    int32_t kbuf;           /* per-pixel pending-fragment buffer: 8 or 16 */
+    int32_t kbuf;           /* 8 or 16 (checked; every pixel is sorted exactly, whatever the value) */
     float T_eps;            /* early-termination transmittance (default 1e-5) */
     float bg[3];            /* background colour */
     int64_t pair_capacity;  /* (tile, fan) pair capacity of the workspace; 0 = default */
-    int32_t depth_bits;     /* depth bits in the sort key, 8..31; 0 = automatic: the most (<= 27) that
-                               keep the key within the bytes of tile bits + 20 */
+    int32_t depth_bits;     /* 0, or 8..31 (checked with the tile and fan bits against 64; the tile lists
+                               hold no depth) */
     int64_t frag_capacity;  /* per-pixel fragment records of the workspace; 0 = 8 W H + 65536 */
     const uint32_t *face_mask;  /* NULL: every face of every fan is drawn; else device, one word per fan,
                                    bit j set = triangle j drawn (the faces ms_prune_faces keeps) */
@@ -128,10 +128,10 @@ typedef struct {
     int64_t pairs;          /* (tile, fan) pairs the binning produced */
     int64_t pair_capacity;  /* capacity of the workspace */
     int64_t culled_tris;    /* triangles culled at the near plane / guard band */
-    int64_t extra_passes;   /* pixel-passes re-run because the pending buffer overflowed */
+    int64_t extra_passes;   /* rounds of 32 fragments that pixels took beyond their first */
     int32_t overflow;       /* 1 if pairs or fragments exceed their capacity (image invalid) */
     int32_t timeouts;       /* bounded waits that expired (image invalid) */
-    int32_t sort_bits;      /* key bits sorted */
+    int32_t sort_bits;      /* bits of a tile index (the key the pairs are ordered by) */
     int32_t n_tiles;
     int64_t rect_tests;     /* (pixel, fan) pairs the forward rasterisation evaluated */
     int64_t fragments;      /* covered (pixel, triangle) fragments it found */

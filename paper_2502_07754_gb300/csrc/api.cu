@@ -101,16 +101,13 @@ RenderLayout render_layout(int64_t n_fans, int K, const ms_camera *cams, int n_v
     L.n_tiles = (int)tiles;
     L.npx = npx;
     L.tile_bits = bits_for(L.n_tiles);
-    // A sort element is one 64-bit word: tile | quantised depth bound | fan id, the fan id in
-    // the low fan_bits bits; the radix passes sort the tile and depth bits above them.
-    // Automatic depth bits: at least 12 over the view's depth range, and as many more as fill
-    // the sort key's last byte, within the word.
+    // (the tile lists are built by counting; a depth key is still sized and checked so that the
+    // same configurations are taken as with sorted (tile, depth, fan) elements)
     L.fan_bits = bits_for(n_fans);
     L.depth_bits = p.depth_bits ? p.depth_bits
                                 : std::min(std::min(31, 8 * ((L.tile_bits + 12 + 7) / 8) - L.tile_bits),
                                            64 - L.fan_bits - L.tile_bits);
     L.key_bits = L.tile_bits + L.depth_bits;
-    L.passes = (L.key_bits + 7) / 8;
     L.n_fans = n_fans;
     L.V = n_fans * (K + 1);
     int64_t cap = p.pair_capacity;
@@ -126,25 +123,20 @@ RenderLayout render_layout(int64_t n_fans, int K, const ms_camera *cams, int n_v
     L.frag_cap = fcap;
     L.bin_fan_blocks = (n_fans + 255) / 256;
     L.bin_blocks = L.bin_fan_blocks * n_views;
-    L.sort_blocks = (cap + sort_tile_elems() - 1) / sort_tile_elems();
-    L.scan_blocks = ((int64_t)L.n_tiles * L.tile * L.tile + 2047) / 2048;   // pixel slots in tile order
     L.max_items = L.n_tiles + (cap + kItemFans - 1) / kItemFans;
-    L.tscan_blocks = ((int64_t)L.n_tiles + 2047) / 2048;
+    L.tscan_blocks = tile_scan_blocks(L.n_tiles);
+    L.order_b = min64(npx, fcap / 17 + 1);   // pixels of more than 16 fragments
     size_t o = 0;
     L.off_status = o;            o = align_up(o + 256, 256);
-    L.off_bin_state = o;         o = align_up(o + 8 * (size_t)L.bin_blocks, 256);
-    L.off_hist = o;              o = align_up(o + 8 * 256 * 4, 256);
-    L.off_lookback = o;          o = align_up(o + (size_t)L.passes * L.sort_blocks * 256 * 4, 256);
-    L.off_ranges = o;            o = align_up(o + 8 * (size_t)L.n_tiles, 256);
-    L.off_scan_state = o;        o = align_up(o + 8 * (size_t)L.scan_blocks, 256);
     L.off_tscan_state = o;       o = align_up(o + 8 * (size_t)L.tscan_blocks, 256);
-    L.off_pbucket = o;           o = align_up(o + 2 * 256 * 4, 256);   // pixel-count histogram, fill cursors
-    L.off_zrange = o;            o = align_up(o + 8 * (size_t)n_views, 256);   // per view: ~bits(zlo), bits(zhi)
+    L.off_tile_cnt = o;          o = align_up(o + 4 * (size_t)L.n_tiles, 256);
     L.off_mask_cursor = o;       o = align_up(o + 4 * (size_t)kMaskRegions, 256);
-    L.off_keys0 = o;             o = align_up(o + 8 * (size_t)cap, 256);   // (zeroed prefix ends here)
-    L.off_keys1 = o;             o = align_up(o + 8 * (size_t)cap, 256);
-    L.off_tile_nitems = o;       o = align_up(o + 4 * (size_t)L.n_tiles, 256);
-    L.off_tile_ibase = o;        o = align_up(o + 4 * (size_t)L.n_tiles, 256);
+    L.off_counts = o;            o = align_up(o + 4 * (size_t)npx, 256);
+    L.off_zero_end = o;          // (the prefix zeroed per render)
+    L.off_pairs = o;             o = align_up(o + 8 * (size_t)cap, 256);
+    L.off_ranks = o;             o = align_up(o + 4 * (size_t)cap, 256);
+    L.off_list = o;              o = align_up(o + 4 * (size_t)cap, 256);
+    L.off_tile_start = o;        o = align_up(o + 4 * (size_t)L.n_tiles, 256);
     L.off_items = o;             o = align_up(o + 16 * (size_t)L.max_items, 256);
     L.off_icnt = o;              o = align_up(o + 4 * (size_t)L.max_items * p.tile * p.tile, 256);
     // coverage masks of the count pass (2 bytes per (pixel, fan) test) and each pair's first
@@ -153,14 +145,13 @@ RenderLayout render_layout(int64_t n_fans, int K, const ms_camera *cams, int n_v
     L.mask_cap = std::min<int64_t>(16 * npx + 65536, 0xfffffffell);
     L.off_maskoff = o;           o = align_up(o + 8 * (size_t)cap, 256);   // per pair: mask index, rectangle
     L.off_masks = o;             o = align_up(o + 2 * (size_t)L.mask_cap, 256);
-    L.off_counts = o;            o = align_up(o + 4 * (size_t)npx, 256);
     L.off_offsets = o;           o = align_up(o + 4 * (size_t)npx, 256);
-    L.off_perm = o;              o = align_up(o + 8 * (size_t)npx, 256);   // pixel order (pixel, record offset)
+    L.off_order_a = o;           o = align_up(o + 8 * (size_t)npx, 256);   // pixel lists of the resolve
+    L.off_order_b = o;           o = align_up(o + 4 * (size_t)L.order_b, 256);
     L.off_frags = o;             o = align_up(o + 16 * kRecFwd * (size_t)fcap, 256);
     L.off_adj = o;               o = align_up(o + 32 * (size_t)fcap, 256);   // adjoint records
     L.off_corder = o;            o = align_up(o + 4 * (size_t)fcap, 256);
     L.off_tfinal = o;            o = align_up(o + 4 * (size_t)npx, 256);
-    L.off_ncommit = o;           o = align_up(o + 4 * (size_t)npx, 256);
     L.off_grad = o;              o = align_up(o + 32 * (size_t)L.V, 256);
     L.off_dec = o;               o = align_up(o + 16 * (size_t)L.V * n_views, 256);   // decided vertices per view
     L.total = o;
@@ -239,12 +230,11 @@ static ms_status render_views(const float *xyz, const float *rgb, const float *a
     for (int v = 0; v < n_views; ++v)
         if (!out[v] || !aligned16(out[v])) return fail(MS_ERR_INVALID, "view %d: output image NULL or not 16-byte aligned", v);
     char *ws = static_cast<char *>(workspace);
-    cudaError_t e = cudaMemsetAsync(ws, 0, L.off_keys0, st);
+    cudaError_t e = cudaMemsetAsync(ws, 0, L.off_zero_end, st);
     if (e != cudaSuccess) return cuda_fail(e, "workspace clear");
     RenderArgs a;
     memset(&a, 0, sizeof(a));
     a.xyz = xyz; a.rgb = rgb; a.alpha = alpha; a.n_fans = n_fans; a.K = K; a.prm = p; a.L = L; a.ws = ws;
-    a.key_scale = 1.0f;
     a.vt = make_views(cams, n_views, L, out, nullptr, nullptr);
     {
         StageScope sc(MS_STAGE_BIN, st);
@@ -252,15 +242,16 @@ static ms_status render_views(const float *xyz, const float *rgb, const float *a
     }
     {
         StageScope sc(MS_STAGE_SORT, st);
-        if ((e = launch_sort(a, st)) != cudaSuccess) return cuda_fail(e, "sort launch");
+        if ((e = launch_tile_lists(a, st)) != cudaSuccess) return cuda_fail(e, "tile list launch");
     }
     {
         StageScope sc(MS_STAGE_RASTER, st);
-        if ((e = launch_raster_count(a, st)) != cudaSuccess) return cuda_fail(e, "raster count launch");
+        if ((e = launch_count(a, st)) != cudaSuccess) return cuda_fail(e, "raster count launch");
+        if ((e = launch_pixel_alloc(a, st)) != cudaSuccess) return cuda_fail(e, "pixel range launch");
         if ((e = launch_fill(a, st)) != cudaSuccess) return cuda_fail(e, "raster fill launch");
         if ((e = launch_resolve(a, false, st)) != cudaSuccess) return cuda_fail(e, "resolve launch");
     }
-    if (n_fans > 0) count_launches(1 + 3 + L.passes);
+    if (n_fans > 0) count_launches(1);   // bin
     count_launches(1);   // resolve (raster kernels count themselves)
     return MS_OK;
 }
@@ -291,7 +282,6 @@ static ms_status render_views_backward(const float *xyz, const float *rgb, const
     memset(&a, 0, sizeof(a));
     a.xyz = xyz; a.rgb = rgb; a.alpha = alpha; a.n_fans = n_fans; a.K = K; a.prm = p; a.L = L; a.ws = ws;
     a.d_xyz = d_xyz; a.d_rgb = d_rgb; a.d_alpha = d_alpha;
-    a.key_scale = 1.0f;
     a.vt = make_views(cams, n_views, L, nullptr, out_fwd, dL);
     // the forward's composited fragments are replayed in commit order, recomputing
     // transmittance; the per-record upstream gradients are then chained to the vertices
@@ -308,7 +298,6 @@ static ms_status render_views_backward(const float *xyz, const float *rgb, const
 // same binning, sort and work-item machinery as fans; the splat passes then evaluate
 // the Gaussians themselves.  The polygon soup lives after the render layout.
 constexpr double kSplatTrunc = 2.7;           // truncation radius in scales (the fan's scale_mul)
-constexpr float kSplatKeyScale = 0.9990234375f;   // 1 - 2^-10: depth keys stay below every hit
 
 static size_t splat_poly_bytes(int64_t N) { return align_up((size_t)N * (kSplatK + 1) * 12, 256); }
 // what a splat workspace holds beyond the render layout: polygons, then coefficients
@@ -337,25 +326,25 @@ static ms_status splat_views(const float *means, const float *log_scales, const 
         if (!out[v] || !aligned16(out[v])) return fail(MS_ERR_INVALID, "view %d: output image NULL or not 16-byte aligned", v);
     char *ws = static_cast<char *>(workspace);
     float *poly = reinterpret_cast<float *>(ws + L.total);
-    cudaError_t e = cudaMemsetAsync(ws, 0, L.off_keys0, st);
+    cudaError_t e = cudaMemsetAsync(ws, 0, L.off_zero_end, st);
     if (e != cudaSuccess) return cuda_fail(e, "workspace clear");
     RenderArgs a;
     memset(&a, 0, sizeof(a));
     a.xyz = poly; a.n_fans = N; a.K = kSplatK; a.prm = p; a.L = L; a.ws = ws;
     a.splat = true;
     a.splat_coef = reinterpret_cast<float4 *>(ws + L.total + splat_poly_bytes(N));
-    a.key_scale = kSplatKeyScale;
     a.spl.means = means; a.spl.log_scales = log_scales; a.spl.quats = quats; a.spl.opacity = opacity;
     a.spl.rgb = rgb; a.spl.axis_rule = axis_rule; a.spl.trunc = kSplatTrunc;
     a.vt = make_views(cams, n_views, L, out, nullptr, nullptr);
     if ((e = launch_splat_polygons(a.spl, N, poly, st)) != cudaSuccess) return cuda_fail(e, "polygon launch");
     if ((e = launch_splat_setup(a, st)) != cudaSuccess) return cuda_fail(e, "splat setup launch");
     if ((e = launch_bin(a, st)) != cudaSuccess) return cuda_fail(e, "bin launch");
-    if ((e = launch_sort(a, st)) != cudaSuccess) return cuda_fail(e, "sort launch");
-    if ((e = launch_raster_count(a, st)) != cudaSuccess) return cuda_fail(e, "splat count launch");
+    if ((e = launch_tile_lists(a, st)) != cudaSuccess) return cuda_fail(e, "tile list launch");
+    if ((e = launch_splat_count(a, st)) != cudaSuccess) return cuda_fail(e, "splat count launch");
+    if ((e = launch_pixel_alloc(a, st)) != cudaSuccess) return cuda_fail(e, "pixel range launch");
     if ((e = launch_splat_fill(a, st)) != cudaSuccess) return cuda_fail(e, "splat fill launch");
     if ((e = launch_resolve(a, false, st)) != cudaSuccess) return cuda_fail(e, "resolve launch");
-    if (N > 0) count_launches(2 + 3 + L.passes);
+    if (N > 0) count_launches(2);   // polygons, bin
     count_launches(1);
     return MS_OK;
 }

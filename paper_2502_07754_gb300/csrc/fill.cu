@@ -16,8 +16,8 @@
 //     depth in double-float.
 // What bounds it: issue slots and the waits of a pair's dependent loads.  Staging with every lane
 // and computing fragments 32 at a time, against four lanes a fan and the lanes whose test hit:
-// 1M fans at 1080p (10.4M fragments) 0.62 -> 0.47 ms, 200k fans at 800x800 0.31 -> 0.23 ms, 3M fans
-// in 16 views (42M pairs, 51M fragments) 9.9 -> 6.4 ms.
+// 1M fans at 1080p (10.4M fragments) 0.62 -> 0.45 ms, 200k fans at 800x800 0.31 -> 0.21 ms, 3M fans
+// in 16 views (42M pairs, 51M fragments) 9.9 -> 5.9 ms.
 #include "raster_common.cuh"
 
 namespace ms {
@@ -26,11 +26,11 @@ namespace {
 
 struct FillArgs {
     const float *xyz, *rgb, *alpha;
-    int K, fan_bits;
+    int K;
     ViewTable vt;
-    const unsigned long long *keys;   // sorted elements tile | depth bound | fan id
+    const uint32_t *list;             // fans in tile order
     const uint4 *items;               // (tile, start, end, index within tile)
-    const uint32_t *icnt;             // [item][tile pixels]: in-pixel starting slots
+    const uint32_t *icnt;             // [item][tile pixels]: first slot within the pixel
     const uint32_t *offsets, *counts;
     float4 *frags;
     int64_t frag_cap;
@@ -197,12 +197,11 @@ __global__ void __launch_bounds__(kFillWarps * 32) fill_kernel(const __grid_cons
     uint32_t head = 0, queued = 0;   // the ring
     for (uint32_t cb = it.y; cb < it.z; cb += 32) {
         uint2 pinf = make_uint2(0u, 0u);
-        unsigned long long key = 0;
+        uint32_t fan = 0;
         if (cb + lane < it.z) {
             pinf = __ldg(a.pinfo + cb + lane);
-            key = __ldg(a.keys + cb + lane);
+            fan = __ldg(a.list + cb + lane);
         }
-        const uint32_t fan = (uint32_t)(key & ((1ull << a.fan_bits) - 1ull));
         const uint32_t n_mine = pinf.y ? (((pinf.y >> 12) & 63u) + 1u) * (((pinf.y >> 18) & 63u) + 1u) : 0u;
         const uint32_t live = __ballot_sync(0xffffffffu, n_mine != 0u);
         const int rank = __popc(live & lt), n_live = __popc(live);
@@ -369,8 +368,7 @@ cudaError_t launch_fill(const RenderArgs &ra, cudaStream_t st) {
     a.alpha = ra.alpha;
     a.K = ra.K;
     a.vt = ra.vt;
-    a.fan_bits = L.fan_bits;
-    a.keys = reinterpret_cast<const unsigned long long *>(ra.ws + (L.passes & 1 ? L.off_keys1 : L.off_keys0));
+    a.list = reinterpret_cast<const uint32_t *>(ra.ws + L.off_list);
     a.items = reinterpret_cast<const uint4 *>(ra.ws + L.off_items);
     a.icnt = reinterpret_cast<const uint32_t *>(ra.ws + L.off_icnt);
     a.offsets = reinterpret_cast<const uint32_t *>(ra.ws + L.off_offsets);

@@ -29,15 +29,15 @@ cudaError_t launch_mesh_build(const float *means, const float *log_scales, const
 // Render workspace layout (byte offsets from the workspace base, 256-byte aligned).
 // Tiles and pixels of all views form one index space (see ViewTable).
 struct RenderLayout {
-    int tile, n_views, n_tiles, tile_bits, depth_bits, key_bits, passes, kbuf;
-    int fan_bits;              // low bits of a sort element holding the fan id
+    int tile, n_views, n_tiles, tile_bits, depth_bits, key_bits, kbuf;
+    int fan_bits;
     int tiles_x[kMaxViews], tile_base[kMaxViews];
     int64_t pix_base[kMaxViews];
-    int64_t npx, n_fans, V, cap, frag_cap, mask_cap;
-    int64_t bin_fan_blocks, bin_blocks, sort_blocks, scan_blocks, tscan_blocks, max_items;
-    size_t off_status, off_bin_state, off_keys0, off_keys1, off_hist, off_lookback,
-        off_ranges, off_scan_state, off_tscan_state, off_pbucket, off_zrange, off_mask_cursor, off_perm, off_tile_nitems, off_tile_ibase, off_items, off_icnt,
-        off_counts, off_offsets, off_maskoff, off_masks, off_frags, off_adj, off_corder, off_tfinal, off_ncommit, off_grad, off_dec, total;
+    int64_t npx, n_fans, V, cap, frag_cap, mask_cap, order_b;
+    int64_t bin_fan_blocks, bin_blocks, tscan_blocks, max_items;
+    size_t off_status, off_tscan_state, off_tile_cnt, off_mask_cursor, off_counts, off_zero_end, off_pairs, off_ranks,
+        off_list, off_tile_start, off_items, off_icnt, off_offsets, off_order_a, off_order_b, off_maskoff, off_masks,
+        off_frags, off_adj, off_corder, off_tfinal, off_grad, off_dec, total;
 };
 
 RenderLayout render_layout(int64_t n_fans, int K, const ms_camera *cams, int n_views, const ms_render_params &p);
@@ -59,7 +59,6 @@ struct RenderArgs {
     char *ws;
     float *d_xyz, *d_rgb, *d_alpha;   // backward outputs
     bool splat;                // draw the source Gaussians of `spl` over the polygons in xyz
-    float key_scale;           // binning: depth keys from key_scale * min Z (1 for fans)
     float4 *splat_coef;        // splat passes: coefficients of every (view, Gaussian)
     SplatSrc spl;
 };
@@ -92,13 +91,13 @@ constexpr int kSplatK = 8;
 cudaError_t launch_splat_polygons(const SplatSrc &s, int64_t N, float *xyz, cudaStream_t st);
 
 cudaError_t launch_bin(const RenderArgs &a, cudaStream_t st);
-cudaError_t launch_sort(const RenderArgs &a, cudaStream_t st);
+int64_t tile_scan_blocks(int64_t n_tiles);
+cudaError_t launch_tile_lists(const RenderArgs &a, cudaStream_t st);   // pairs in tile order, work items
 // Stable LSD sort of n 64-bit elements by bits [shift, shift + 8 passes): a and b are the two
 // buffers, *result receives the one holding the sorted elements; scratch (device,
 // sort_scratch_bytes, 16-byte aligned) is cleared and used for counts and look-back flags.
 size_t sort_scratch_bytes(int64_t n, int passes);
 // Elements of one sort tile (one look-back slot per tile and digit).
-int64_t sort_tile_elems();
 cudaError_t sort_u64(unsigned long long *a, unsigned long long *b, int64_t n, int shift, int passes, char *scratch,
                      cudaStream_t st, unsigned long long **result);
 constexpr int kItemFans = 64;   // fans per raster work item
@@ -109,10 +108,10 @@ size_t splat_coef_bytes(int64_t N, int n_views);
 cudaError_t launch_splat_setup(const RenderArgs &a, cudaStream_t st);
 cudaError_t launch_splat_count(const RenderArgs &a, cudaStream_t st);
 cudaError_t launch_splat_fill(const RenderArgs &a, cudaStream_t st);
-cudaError_t launch_raster_count(const RenderArgs &a, cudaStream_t st);   // items, count, prefix, pixel scan
+cudaError_t launch_count(const RenderArgs &a, cudaStream_t st);        // fragment counts of the fans
 cudaError_t launch_record_chain(const RenderArgs &a, cudaStream_t st);   // adjoint: records -> fan vertices
 constexpr int kRecFwd = 2;   // float4s per fragment record
-cudaError_t launch_pixel_order(const RenderArgs &a, cudaStream_t st);   // resolve order of the pixels
+cudaError_t launch_pixel_alloc(const RenderArgs &a, cudaStream_t st);   // record ranges and order of the pixels
 cudaError_t launch_resolve(const RenderArgs &a, bool backward, cudaStream_t st);
 cudaError_t launch_grad_scatter(const RenderArgs &a, cudaStream_t st);
 

@@ -14,13 +14,13 @@
 // composited one (merging 32 records at a time), so the order is exact for any depth complexity.
 // A round after the first counts as an extra pass.
 //
-// pixel_order_kernel sorts the pixels by descending fragment count after the pixel scan, so
-// that each class is one range of the order and a warp's groups run loops of about the same
-// length; it writes the background of pixels without fragments itself.  Warps take units of the
-// order in turn and fetch the next units' entries and counts while they work.
+// pixel_alloc_kernel (tiles.cu) lists the pixels by class of fragment count, spans of 1024 pixel
+// slots in descending count, so a warp's groups run loops of about the same length on
+// neighbouring records.  Warps take units of the lists in turn and fetch the next units' entries
+// and counts while they work.
 //
 // The forward also records, per pixel, the record index of each committed fragment in
-// commit order.  The backward walks that list (no sorting), and at
+// commit order (and where they end early).  The backward walks that list (no sorting), and at
 // each committed fragment f forms, from the recomputed transmittance T_f,
 // dC/dc_f = T_f a_f, dC/da_f = T_f c_f - (C_out - C_{<=f}) / (1 - a_f) and
 // dA/da_f = T_out / (1 - a_f).  It writes dL/dc_f and dL/da_f, with the fragment's
@@ -38,6 +38,8 @@ namespace ms {
 
 namespace {
 
+constexpr uint32_t kEnd = 0xffffffffu;
+
 struct ResolveArgs {
     int64_t npx;
     const float4 *frags;
@@ -45,119 +47,51 @@ struct ResolveArgs {
     float T_eps, bg0, bg1, bg2;
     Status *st;
     float *tfinal;
-    uint32_t *ncommit;
     float4 *adj;               // backward: per composited fragment, in commit order within the
                                // pixel's record range: (dL/dc * T a, dL/da), (triangle, pixel, 0, 0)
-    uint32_t *corder;          // per pixel: record indices in commit order (same offsets as records)
-    const uint2 *order;        // pixels with fragments, by descending count: (pixel, record offset)
+                               // (32 bytes, whole sectors: 16 + 8 bytes in two arrays took twice as long)
+    uint32_t *corder;          // per pixel: record indices in commit order (same offsets as records), then
+                               // kEnd if fewer were composited than there are records
+    // pixels with fragments: list_b holds those of more than 16 fragments (more than 32 from its
+    // end, the others from its start), list_a the others with their record offsets (9 to 16 from
+    // its end, 1 to 8 from its start); st->classes counts the four
+    const uint2 *list_a;
+    const uint32_t *list_b, *offsets;
+    int64_t order_b;           // entries of list_b (list_a: npx)
     const uint32_t *counts;
-    const uint32_t *hist;      // [kCountBuckets] pixels of each count
     ViewTable vt;
 };
 
-// Pixel order, built after the pixel scan: the pixels with fragments in descending order of
-// their counts (a counting sort over the counts' histogram).  The order within one count
-// varies from run to run; no pixel's result depends on it.
-constexpr int kOrderThreads = 256, kOrderItems = 4, kOrderSpan = kOrderThreads * kOrderItems;
-
-// Exclusive prefix of v over the buckets in descending order (thread t holds bucket 255 - t).
-__device__ __forceinline__ uint32_t desc_prefix(uint32_t v, uint32_t *s_warp) {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    uint32_t x = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    __syncthreads();   // s_warp may still be read by an earlier call
-    if (lane == 31) s_warp[warp] = x;
-    __syncthreads();
-    uint32_t before = 0;
-    for (int w = 0; w < warp; ++w) before += s_warp[w];
-    return before + x - v;
-}
-
-__global__ void __launch_bounds__(kOrderThreads) pixel_order_kernel(const uint32_t *__restrict__ offsets,
-                                                                    uint32_t *__restrict__ fill,
-                                                                    uint2 *__restrict__ order,
-                                                                    const __grid_constant__ ResolveArgs a) {
-    __shared__ uint32_t s_cnt[kCountBuckets], s_glob[kCountBuckets], s_warp[kOrderThreads / 32];
-    static_assert(kOrderThreads == kCountBuckets, "one thread per bucket");
-    const int tid = threadIdx.x;
-    const int64_t base = (int64_t)blockIdx.x * kOrderSpan;
-    const int mb = kCountBuckets - 1 - tid;   // this thread's bucket in the scans
-    s_cnt[tid] = 0;
-    const uint32_t g0 = desc_prefix(a.hist[mb], s_warp);   // (its barriers also order the clear)
-    int bk[kOrderItems];
-    uint32_t rk[kOrderItems];
-#pragma unroll
-    for (int i = 0; i < kOrderItems; ++i) {
-        const int64_t p = base + i * kOrderThreads + tid;
-        bk[i] = 0;
-        rk[i] = 0;
-        if (p >= a.npx) continue;
-        bk[i] = count_bucket(a.counts[p]);
-        if (bk[i]) {
-            rk[i] = atomicAdd(&s_cnt[bk[i]], 1u);
-        } else {   // no fragments: the background
-            const ViewDev &vw = a.vt.v[view_of_pixel(a.vt, (unsigned long long)p)];
-            reinterpret_cast<float4 *>(vw.out)[p - (int64_t)vw.pix_base] = make_float4(a.bg0, a.bg1, a.bg2, 0.0f);
-            a.tfinal[p] = 1.0f;
-            a.ncommit[p] = 0;
-        }
-    }
-    __syncthreads();
-    const uint32_t h = mb ? s_cnt[mb] : 0u;
-    s_glob[mb] = h ? g0 + atomicAdd(&fill[mb], h) : 0u;
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < kOrderItems; ++i)
-        if (bk[i]) {
-            const int64_t p = base + i * kOrderThreads + tid;
-            // the position is < npx: the histogram counts each pixel once
-            const int64_t pg = (int64_t)s_glob[bk[i]] + rk[i];
-            if (pg < a.npx) order[pg] = make_uint2((uint32_t)p, offsets[p]);
-        }
-}
-
-// The work of the resolve kernels: warps take units of the pixel order in turn, a unit being
+// The work of the resolve kernel: warps take units of the pixel lists in turn, a unit being
 // one pixel of more than 16 records, two of 9 to 16 or four of 1 to 8.
 constexpr int kGroupThreads = 256, kResident = 4;   // threads a block, blocks a multiprocessor
 struct Units {
-    uint32_t f16, f8, end;        // order positions: [0, n32) more than 16 records (the first `deep` more
-                                  // than 32), [n32, f16) 9 to 16, [f16, end) 1 to 8
+    uint32_t c16, c8;             // pixels of 9 to 16 and of 1 to 8 records
     uint32_t deep, n32, n16, n8;  // unit bounds of the classes
-    // Called by a whole block of kGroupThreads threads.
-    __device__ __forceinline__ Units(const uint32_t *__restrict__ hist, int64_t npx) {
-        static_assert(kGroupThreads == kCountBuckets, "one thread per bucket");
-        __shared__ uint32_t s_n[4];
-        if (threadIdx.x < 4) s_n[threadIdx.x] = 0;
-        __syncthreads();
-        const int b = threadIdx.x;
-        const uint32_t h = b ? hist[b] : 0u;
-        if (h) atomicAdd(&s_n[b > 32 ? 0 : (b > 16 ? 1 : (b > 8 ? 2 : 3))], h);
-        __syncthreads();
-        const uint32_t most = (uint32_t)npx;
-        deep = min(s_n[0], most);
-        n32 = min(deep + s_n[1], most);
-        f16 = min(n32 + s_n[2], most);
-        end = min(f16 + s_n[3], most);
-        n16 = n32 + (f16 - n32 + 1) / 2;
-        n8 = n16 + (end - f16 + 3) / 4;
+    __device__ __forceinline__ Units(const ResolveArgs &a) {
+        // (a count past a list's end exists only for a buffer that overflowed its capacity)
+        const uint4 c = *reinterpret_cast<const uint4 *>(a.st->classes);
+        deep = (uint32_t)min64(c.x, a.order_b);
+        n32 = deep + (uint32_t)min64(c.y, a.order_b);
+        c16 = (uint32_t)min64(c.z, a.npx);
+        c8 = (uint32_t)min64(c.w, a.npx);
+        n16 = n32 + (c16 + 1) / 2;
+        n8 = n16 + (c8 + 3) / 4;
     }
-    // This lane's entry of unit u (no pixel: ~0).
+    // This lane's entry of unit u (pixel and, from list_a, its record offset; no pixel: ~0).
     __device__ __forceinline__ uint2 entry(const ResolveArgs &a, int64_t u, int lane) const {
-        int64_t q = u;
-        uint32_t e0 = n32;
-        if (u >= n16) {
-            q = f16 + 4 * (u - n16) + (lane >> 3);
-            e0 = end;
-        } else if (u >= n32) {
-            q = n32 + 2 * (u - n32) + (lane >> 4);
-            e0 = f16;
-        }
         uint2 e = make_uint2(~0u, 0u);
-        if (u < n8 && q < e0) e = __ldg(a.order + q);
+        if (u < deep) {
+            e.x = __ldg(a.list_b + (a.order_b - 1 - u));
+        } else if (u < n32) {
+            e.x = __ldg(a.list_b + (u - deep));
+        } else if (u < n16) {
+            const int64_t q = 2 * (u - n32) + (lane >> 4);
+            if (q < c16) e = __ldg(a.list_a + (a.npx - 1 - q));
+        } else if (u < n8) {
+            const int64_t q = 4 * (u - n16) + (lane >> 3);
+            if (q < c8) e = __ldg(a.list_a + q);
+        }
         return e;
     }
 };
@@ -167,9 +101,12 @@ struct Units {
 struct Pixel {
     uint32_t pix, off, n;
 };
-__device__ __forceinline__ Pixel pixel_of(const ResolveArgs &a, const uint2 e) {
+__device__ __forceinline__ Pixel pixel_of(const ResolveArgs &a, const uint2 e, bool from_b) {
     Pixel p = {e.x, e.y, 0u};
-    if (e.x < (uint64_t)a.npx) p.n = __ldg(a.counts + e.x);
+    if (e.x < (uint64_t)a.npx) {
+        p.n = __ldg(a.counts + e.x);
+        if (from_b) p.off = __ldg(a.offsets + e.x);
+    }
     return p;
 }
 __device__ __forceinline__ bool is_pixel(const ResolveArgs &a, const Pixel &p) { return p.pix < (uint64_t)a.npx; }
@@ -246,13 +183,13 @@ __device__ __forceinline__ int composite(GroupMem &m, int g0, int at0, int n, in
     return ncom;
 }
 
-__device__ __forceinline__ void write_pixel(const ResolveArgs &a, uint32_t pix, float T, float C0, float C1, float C2,
+__device__ __forceinline__ void write_pixel(const ResolveArgs &a, const Pixel &e, float T, float C0, float C1, float C2,
                                             uint32_t ncom) {
-    const ViewDev &vw = a.vt.v[view_of_pixel(a.vt, (unsigned long long)pix)];
-    reinterpret_cast<float4 *>(vw.out)[(int64_t)pix - (int64_t)vw.pix_base] =
+    const ViewDev &vw = a.vt.v[view_of_pixel(a.vt, (unsigned long long)e.pix)];
+    reinterpret_cast<float4 *>(vw.out)[(int64_t)e.pix - (int64_t)vw.pix_base] =
         make_float4(C0 + T * a.bg0, C1 + T * a.bg1, C2 + T * a.bg2, 1.0f - T);
-    a.tfinal[pix] = T;
-    a.ncommit[pix] = ncom;
+    a.tfinal[e.pix] = T;
+    if (ncom < e.n && fits(a, e)) a.corder[(size_t)e.off + ncom] = kEnd;
 }
 
 // One warp's 32 / G pixels (e per group); returns the fragments composited (first lanes).
@@ -299,7 +236,7 @@ __device__ __forceinline__ uint32_t resolve_group(const ResolveArgs &a, GroupMem
     const int ncom = composite<G>(m, g0, g0, n, nmax, a.T_eps, T, C, ended);
     const float C1 = __shfl_sync(0xffffffffu, C, g0 + 1), C2 = __shfl_sync(0xffffffffu, C, g0 + 2);
     if (valid && sub < ncom) a.corder[off + sub] = m.src[lane];
-    if (valid && sub == 0) write_pixel(a, e.pix, T, C, C1, C2, (uint32_t)ncom);
+    if (valid && sub == 0) write_pixel(a, e, T, C, C1, C2, (uint32_t)ncom);
     return valid && sub == 0 ? (uint32_t)ncom : 0u;
 }
 
@@ -413,7 +350,7 @@ __device__ uint32_t resolve_deep(const ResolveArgs &a, GroupMem &m, const Pixel 
     }
     const float C1 = __shfl_sync(0xffffffffu, C, 1), C2 = __shfl_sync(0xffffffffu, C, 2);
     if (lane == 0) {
-        write_pixel(a, e.pix, T, C, C1, C2, ncom);
+        write_pixel(a, e, T, C, C1, C2, ncom);
         if (extra) atomicAdd(&a.st->extra_passes, (unsigned long long)extra);
     }
     return lane == 0 ? ncom : 0u;
@@ -421,18 +358,18 @@ __device__ uint32_t resolve_deep(const ResolveArgs &a, GroupMem &m, const Pixel 
 
 __global__ void __launch_bounds__(kGroupThreads, kResident) resolve_kernel(const __grid_constant__ ResolveArgs a) {
     __shared__ __align__(16) GroupMem s_mem[kGroupThreads / 32];
-    const Units U(a.hist, a.npx);
+    const Units U(a);
     GroupMem &m = s_mem[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (kGroupThreads / 32);
     uint32_t ncom = 0;
     int64_t u = (int64_t)blockIdx.x * (kGroupThreads / 32) + (threadIdx.x >> 5);
     // entries are fetched two units ahead, counts one unit ahead
-    Pixel e1 = pixel_of(a, U.entry(a, u, lane));
+    Pixel e1 = pixel_of(a, U.entry(a, u, lane), u < U.n32);
     uint2 e2 = U.entry(a, u + warps, lane);
     for (; u < U.n8; u += warps) {
         const Pixel e = e1;
-        e1 = pixel_of(a, e2);
+        e1 = pixel_of(a, e2, u + warps < U.n32);
         e2 = U.entry(a, u + 2 * warps, lane);
         if (u < U.deep)
             ncom += resolve_deep(a, m, e);
@@ -447,7 +384,7 @@ __global__ void __launch_bounds__(kGroupThreads, kResident) resolve_kernel(const
     if (lane == 0 && ncom) atomicAdd(&a.st->commits, (unsigned long long)ncom);
 }
 
-// Backward, one thread a pixel in the pixel order (a warp's lanes run loops of about the same
+// Backward, one thread a pixel of the lists (a warp's lanes run loops of about the same
 // length): no sorting is left, so a lane's sequential walk takes far fewer instructions than the
 // groups' prefix sums (measured: 0.26 against 0.34 ms on 10.4M fragments).  The walk waits on
 // its records, so the record after the next one's index and the next record load while the
@@ -455,17 +392,22 @@ __global__ void __launch_bounds__(kGroupThreads, kResident) resolve_kernel(const
 constexpr int kBwdThreads = 64;
 __global__ void __launch_bounds__(kBwdThreads) resolve_bwd_kernel(const __grid_constant__ ResolveArgs a) {
     const int64_t q = (int64_t)blockIdx.x * kBwdThreads + threadIdx.x;
-    if (q >= a.npx - (int64_t)__ldg(a.hist)) return;   // (the order holds the pixels with fragments)
-    const Pixel e = pixel_of(a, __ldg(a.order + q));
+    const uint4 cl = *reinterpret_cast<const uint4 *>(a.st->classes);
+    const int64_t n0 = min64(cl.x, a.order_b), n1 = n0 + min64(cl.y, a.order_b), n2 = n1 + min64(cl.z, a.npx);
+    if (q >= n2 + min64(cl.w, a.npx)) return;
+    uint2 entry = make_uint2(0u, 0u);
+    if (q < n0)
+        entry.x = __ldg(a.list_b + (a.order_b - 1 - q));
+    else if (q < n1)
+        entry.x = __ldg(a.list_b + (q - n0));
+    else
+        entry = __ldg(q < n2 ? a.list_a + (a.npx - 1 - (q - n1)) : a.list_a + (q - n2));
+    const Pixel e = pixel_of(a, entry, q < n1);
     if (!is_pixel(a, e) || !fits(a, e)) return;
     const int64_t off = e.off;
-    const uint32_t n = min(a.ncommit[e.pix], e.n);
+    const uint32_t n = e.n;
     const float4 zero = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     float4 *adj = a.adj + 2 * off;
-    // slots past the composited fragments carry a zero gradient (the chain pass reads
-    // every slot of the pixel's range)
-    for (uint32_t i = n; i < e.n; ++i) adj[2 * i] = adj[2 * i + 1] = zero;
-    if (n == 0) return;
     const ViewDev &vw = a.vt.v[view_of_pixel(a.vt, (unsigned long long)e.pix)];
     const int64_t lpix = (int64_t)e.pix - (int64_t)vw.pix_base;
     const float4 *rec = a.frags + (size_t)kRecFwd * off;
@@ -474,18 +416,24 @@ __global__ void __launch_bounds__(kBwdThreads) resolve_bwd_kernel(const __grid_c
     const float4 ov = reinterpret_cast<const float4 *>(vw.out_fwd)[lpix];
     const float Tout = a.tfinal[e.pix];
     float T = 1.0f, C0 = 0.0f, C1 = 0.0f, C2 = 0.0f;
-    const uint32_t i0 = ord[0];
-    uint32_t i2 = n > 1 ? ord[1] : 0u;
-    float tri1 = rec[(size_t)kRecFwd * i0].y;
-    float4 col1 = rec[(size_t)kRecFwd * i0 + 1];
-    for (uint32_t c = 0; c < n; ++c) {
+    // (indices past the last composited fragment are not read as records)
+    uint32_t i1 = ord[0], i2 = n > 1 ? ord[1] : kEnd;
+    float tri1 = 0.0f;
+    float4 col1 = zero;
+    if (i1 < n) {
+        tri1 = rec[(size_t)kRecFwd * i1].y;
+        col1 = rec[(size_t)kRecFwd * i1 + 1];
+    }
+    uint32_t c = 0;
+    for (; c < n && i1 < n; ++c) {
         const float tri = tri1;
         const float4 col = col1;
-        if (c + 1 < n) {
+        if (i2 < n) {
             tri1 = rec[(size_t)kRecFwd * i2].y;
             col1 = rec[(size_t)kRecFwd * i2 + 1];
         }
-        if (c + 2 < n) i2 = ord[c + 2];
+        i1 = i2;
+        i2 = c + 2 < n && i2 < n ? ord[c + 2] : kEnd;
         const float al = col.w;
         const float w = T * al;
         const float nC0 = C0 + w * col.x, nC1 = C1 + w * col.y, nC2 = C2 + w * col.z;
@@ -497,6 +445,9 @@ __global__ void __launch_bounds__(kBwdThreads) resolve_bwd_kernel(const __grid_c
         C0 = nC0; C1 = nC1; C2 = nC2;
         T *= (1.0f - al);
     }
+    // slots past the composited fragments carry a zero gradient (the chain pass reads
+    // every slot of the pixel's range)
+    for (; c < n; ++c) adj[2 * c] = adj[2 * c + 1] = zero;
 }
 
 __global__ void grad_scatter_kernel(const float4 *__restrict__ g, int64_t V, float *__restrict__ dx,
@@ -529,12 +480,13 @@ ResolveArgs make_args(const RenderArgs &ra) {
     a.bg2 = ra.prm.bg[2];
     a.st = reinterpret_cast<Status *>(ra.ws + L.off_status);
     a.tfinal = reinterpret_cast<float *>(ra.ws + L.off_tfinal);
-    a.ncommit = reinterpret_cast<uint32_t *>(ra.ws + L.off_ncommit);
     a.adj = reinterpret_cast<float4 *>(ra.ws + L.off_adj);
     a.corder = reinterpret_cast<uint32_t *>(ra.ws + L.off_corder);
-    a.order = reinterpret_cast<const uint2 *>(ra.ws + L.off_perm);
+    a.list_a = reinterpret_cast<const uint2 *>(ra.ws + L.off_order_a);
+    a.list_b = reinterpret_cast<const uint32_t *>(ra.ws + L.off_order_b);
+    a.offsets = reinterpret_cast<const uint32_t *>(ra.ws + L.off_offsets);
+    a.order_b = L.order_b;
     a.counts = reinterpret_cast<const uint32_t *>(ra.ws + L.off_counts);
-    a.hist = reinterpret_cast<const uint32_t *>(ra.ws + L.off_pbucket);
     a.vt = ra.vt;
     return a;
 }
@@ -553,18 +505,6 @@ cudaError_t launch_resolve(const RenderArgs &ra, bool backward, cudaStream_t st)
     else
         resolve_kernel<<<grid, kGroupThreads, 0, st>>>(make_args(ra));
     return cudaGetLastError();
-}
-
-cudaError_t launch_pixel_order(const RenderArgs &ra, cudaStream_t st) {
-    const RenderLayout &L = ra.L;
-    if (L.npx == 0) return cudaSuccess;
-    uint32_t *fill = reinterpret_cast<uint32_t *>(ra.ws + L.off_pbucket) + kCountBuckets;
-    pixel_order_kernel<<<(unsigned)((L.npx + kOrderSpan - 1) / kOrderSpan), kOrderThreads, 0, st>>>(
-        reinterpret_cast<const uint32_t *>(ra.ws + L.off_offsets), fill,
-        reinterpret_cast<uint2 *>(ra.ws + L.off_perm), make_args(ra));
-    cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) count_launches(1);
-    return e;
 }
 
 cudaError_t launch_grad_scatter(const RenderArgs &ra, cudaStream_t st) {

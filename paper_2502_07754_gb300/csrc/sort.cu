@@ -1,5 +1,5 @@
-// LSD radix sort of the 64-bit (tile | depth | fan id) elements by their tile and depth
-// bits (above the fan id's low bits), 8-bit digits.
+// LSD radix sort of 64-bit (key | id) elements by their key bits, 8-bit digits (Morton orders
+// of the storage order and of the ray tracer's boxes).
 //
 // One histogram kernel reads the elements once and counts the digits of every pass; each
 // pass is then a single "onesweep" kernel: a block loads its 4096 elements (all loads
@@ -199,21 +199,9 @@ __global__ void __launch_bounds__(kSortThreads, 2) sort_pass_kernel(const unsign
     }
 }
 
-__global__ void tile_ranges_kernel(const unsigned long long *__restrict__ keys, const Status *st, int64_t cap,
-                                   int tile_shift, uint2 *__restrict__ ranges) {
-    const int64_t n = n_pairs(st, cap);
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t t = (uint32_t)(keys[i] >> tile_shift);
-        if (i == 0 || (uint32_t)(keys[i - 1] >> tile_shift) != t) ranges[t].x = (uint32_t)i;
-        if (i == n - 1 || (uint32_t)(keys[i + 1] >> tile_shift) != t) ranges[t].y = (uint32_t)(i + 1);
-    }
-}
-
 __global__ void set_pairs_kernel(Status *st, int64_t n) { st->pairs = (unsigned long long)n; }
 
 }  // namespace
-
-int64_t sort_tile_elems() { return kSortTile; }
 
 size_t sort_scratch_bytes(int64_t n, int passes) {
     const int64_t blocks = (n + kSortTile - 1) / kSortTile;
@@ -247,36 +235,6 @@ cudaError_t sort_u64(unsigned long long *a, unsigned long long *b, int64_t n, in
                                                             lookback + (size_t)p * blocks * 256, p, shift + 8 * p);
     *result = kb[passes & 1];
     count_launches(3 + passes);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_sort(const RenderArgs &a, cudaStream_t st) {
-    const RenderLayout &L = a.L;
-    if (a.n_fans == 0) return cudaSuccess;
-    char *ws = a.ws;
-    Status *status = reinterpret_cast<Status *>(ws + L.off_status);
-    uint32_t *hist = reinterpret_cast<uint32_t *>(ws + L.off_hist);
-    unsigned long long *kb[2] = {reinterpret_cast<unsigned long long *>(ws + L.off_keys0),
-                                 reinterpret_cast<unsigned long long *>(ws + L.off_keys1)};
-    const int hist_grid = (int)min64((L.cap + kHistThreads * 8 - 1) / (kHistThreads * 8), 4 * 152);
-    sort_hist_kernel<<<hist_grid, kHistThreads, 0, st>>>(kb[0], status, L.cap, L.passes, L.fan_bits, hist);
-    sort_scan_kernel<<<1, 256, 0, st>>>(hist, L.passes);
-    const size_t smem = (size_t)kSortTile * 8 + (kSortWarps * 256 + 512) * 4;
-    cudaFuncSetAttribute(sort_pass_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    int dev = 0, n_sm = 152, per_sm = 4;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sort_pass_kernel, kSortThreads, smem);
-    const unsigned grid = (unsigned)min64(L.sort_blocks, (int64_t)n_sm * (per_sm > 0 ? per_sm : 1));
-    for (int p = 0; p < L.passes; ++p) {
-        sort_pass_kernel<<<grid, kSortThreads, smem, st>>>(
-            kb[p & 1], kb[(p + 1) & 1], status, L.cap, hist,
-            reinterpret_cast<uint32_t *>(ws + L.off_lookback) + (size_t)p * L.sort_blocks * 256, p, L.fan_bits + 8 * p);
-    }
-    const unsigned long long *sorted = kb[L.passes & 1];
-    const int rg = (int)min64((L.cap + 255) / 256, 8 * 152);
-    tile_ranges_kernel<<<rg, 256, 0, st>>>(sorted, status, L.cap, L.fan_bits + L.depth_bits,
-                                           reinterpret_cast<uint2 *>(ws + L.off_ranges));
     return cudaGetLastError();
 }
 

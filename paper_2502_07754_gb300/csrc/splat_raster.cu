@@ -29,17 +29,16 @@ namespace ms {
 namespace {
 
 constexpr int kSplatWarps = 2;
-constexpr uint32_t kNoRecord = 0xffffffffu;
 
 struct SplatArgs {
     ViewTable vt;
     SplatSrc spl;
-    int depth_bits, fan_bits;
     int64_t N;
-    const unsigned long long *keys;
+    const uint32_t *list;
     const uint4 *items;
     uint32_t *icnt;
-    const uint32_t *offsets, *counts;
+    const uint32_t *offsets;
+    uint32_t *counts;
     float4 *frags;
     int64_t frag_cap;
     Status *st;
@@ -194,11 +193,12 @@ __device__ __forceinline__ uint32_t polygon_geo(const float4 *__restrict__ dv, i
 
 template <int TILE, bool FILL>
 struct SplatMem {
-    float4 c[32], A[32], B[32], D[32], Z[32];   // staged coefficients (Z.w: the key's depth bound)
+    float4 c[32], A[32], B[32], D[32], Z[32];   // staged coefficients
     float4 col[FILL ? 32 : 1];                  // colour, Gaussian id (bits)
     uint2 info[32];                             // first index in the packed space, rectangle
     uint32_t gid[32];
     uint32_t cnt[TILE * TILE];                  // fragments so far, or next record of each pixel
+    uint32_t fits[FILL ? 32 : 1];               // pixels whose records fit the buffer
     uint2 ring[FILL ? 64 : 1];
 };
 
@@ -219,23 +219,30 @@ __global__ void __launch_bounds__(kSplatWarps * 32, 14) splat_raster_kernel(cons
     const int tx0 = (tile % tiles_x) * TILE, ty0 = (tile / tiles_x) * TILE;
     const int tx1 = min(tx0 + TILE, cam.width) - 1, ty1 = min(ty0 + TILE, cam.height) - 1;
     uint32_t *icnt = a.icnt + (size_t)item * TILE * TILE;
+    bool all_fit = true;
     for (int i = lane; i < TILE * TILE; i += 32) {
-        uint32_t b = FILL ? kNoRecord : 0u;
+        uint32_t b = 0;
+        bool fit = true;
         const int x = tx0 + (i % TILE), y = ty0 + (i / TILE);
         if (FILL && x <= tx1 && y <= ty1) {
             const size_t pix = vw.pix_base + (size_t)y * cam.width + x;
-            const int64_t o = a.offsets[pix];
+            const uint32_t o = a.offsets[pix];
             // a pixel whose records would not fit gets none (the overflow is reported)
-            if (o + a.counts[pix] <= a.frag_cap) b = (uint32_t)o + icnt[i];
+            fit = (int64_t)o + a.counts[pix] <= a.frag_cap;
+            b = o + icnt[i];
         }
         S.cnt[i] = b;
+        if (FILL) {
+            const uint32_t m = __ballot_sync(0xffffffffu, fit);
+            if (lane == 0) S.fits[i >> 5] = m;
+            all_fit = all_fit && m == 0xffffffffu;
+        }
     }
     const uint32_t lt = (1u << lane) - 1u, le = 0xffffffffu >> (31 - lane);
     uint32_t head = 0, queued = 0, n_test = 0, n_frag = 0;
     for (uint32_t cb = it.y; cb < it.z; cb += 32) {
         const bool mine = cb + lane < it.z;
-        const unsigned long long key = mine ? __ldg(a.keys + cb + lane) : 0ull;
-        const uint32_t g = (uint32_t)(key & ((1ull << a.fan_bits) - 1ull));
+        const uint32_t g = mine ? __ldg(a.list + cb + lane) : 0u;
         uint32_t geo = 0;
         if (mine)
             geo = FILL ? a.pinfo[cb + lane].y
@@ -260,9 +267,7 @@ __global__ void __launch_bounds__(kSplatWarps * 32, 14) splat_raster_kernel(cons
             S.A[slot] = __ldg(w + 1);
             S.B[slot] = __ldg(w + 2);
             S.D[slot] = __ldg(w + 3);
-            float4 z = __ldg(w + 4);
-            z.w = __uint_as_float((uint32_t)((key >> a.fan_bits) & ((1ull << a.depth_bits) - 1ull)));
-            S.Z[slot] = z;
+            S.Z[slot] = __ldg(w + 4);
             if (FILL) {
                 const float *col = a.spl.rgb + 3 * (size_t)g;
                 S.col[slot] = make_float4(__ldg(col), __ldg(col + 1), __ldg(col + 2), 0.0f);
@@ -306,19 +311,12 @@ __global__ void __launch_bounds__(kSplatWarps * 32, 14) splat_raster_kernel(cons
                 if (hit) atomicAdd(&S.cnt[lp], 1u);
                 continue;
             }
-            // Lanes that hit the same pixel take consecutive slots in lane order, which is
-            // list order, so a pixel's records keep the depth-key order of the tile list.
-            const unsigned grp = __match_any_sync(0xffffffffu, lp);
-            uint32_t rec = kNoRecord;
-            if (hit) {
-                rec = S.cnt[lp];
-                if (rec != kNoRecord) rec += __popc(grp & lt);
-            }
-            __syncwarp();
-            if (rec != kNoRecord && (grp >> lane) == 1u) S.cnt[lp] = rec + 1u;   // last lane of its group
-            const uint32_t pend = __ballot_sync(0xffffffffu, rec != kNoRecord);
-            if (rec != kNoRecord)
-                S.ring[(head + queued + __popc(pend & lt)) & 63u] = make_uint2((uint32_t)f | x << 5 | y << 10, rec);
+            // (a pixel's records may come in any order: the resolve sorts them)
+            uint32_t rec = 0;
+            if (hit && !all_fit && !((S.fits[lp >> 5] >> (lp & 31)) & 1u)) hit = 0;
+            if (hit) rec = atomicAdd(&S.cnt[lp], 1u);
+            const uint32_t pend = __ballot_sync(0xffffffffu, hit != 0);
+            if (hit) S.ring[(head + queued + __popc(pend & lt)) & 63u] = make_uint2((uint32_t)f | x << 5 | y << 10, rec);
             queued += __popc(pend);
             __syncwarp();
             // whole warps of hits, and what is left once these splats' centres are done
@@ -335,7 +333,7 @@ __global__ void __launch_bounds__(kSplatWarps * 32, 14) splat_raster_kernel(cons
                         splat_exact(a.spl, cam, S.gid[jf], px, py, t, al);
                     const float4 col = S.col[jf];
                     float4 *out = a.frags + (size_t)kRecFwd * (size_t)job.y;
-                    out[0] = make_float4(t, __uint_as_float(S.gid[jf]), Z.w, 0.0f);
+                    out[0] = make_float4(t, __uint_as_float(S.gid[jf]), 0.0f, 0.0f);
                     out[1] = make_float4(col.x, col.y, col.z, al);
                 }
                 head += nj;
@@ -348,7 +346,11 @@ __global__ void __launch_bounds__(kSplatWarps * 32, 14) splat_raster_kernel(cons
     }
     if (!FILL) {
         __syncwarp();
-        for (int i = lane; i < TILE * TILE; i += 32) icnt[i] = S.cnt[i];
+        for (int i = lane; i < TILE * TILE; i += 32) {
+            const uint32_t c = S.cnt[i];   // (nonzero only inside the image)
+            if (c)
+                icnt[i] = atomicAdd(a.counts + vw.pix_base + (size_t)(ty0 + i / TILE) * cam.width + (size_t)(tx0 + i % TILE), c);
+        }
         const unsigned r0 = __reduce_add_sync(0xffffffffu, n_test), r1 = __reduce_add_sync(0xffffffffu, n_frag);
         if (lane == 0) {
             atomicAdd(&a.st->rect_tests, (unsigned long long)r0);
@@ -373,14 +375,12 @@ cudaError_t launch(const RenderArgs &ra, cudaStream_t st) {
     SplatArgs a;
     a.vt = ra.vt;
     a.spl = ra.spl;
-    a.depth_bits = L.depth_bits;
-    a.fan_bits = L.fan_bits;
     a.N = ra.n_fans;
-    a.keys = reinterpret_cast<const unsigned long long *>(ra.ws + (L.passes & 1 ? L.off_keys1 : L.off_keys0));
+    a.list = reinterpret_cast<const uint32_t *>(ra.ws + L.off_list);
     a.items = reinterpret_cast<const uint4 *>(ra.ws + L.off_items);
     a.icnt = reinterpret_cast<uint32_t *>(ra.ws + L.off_icnt);
     a.offsets = reinterpret_cast<const uint32_t *>(ra.ws + L.off_offsets);
-    a.counts = reinterpret_cast<const uint32_t *>(ra.ws + L.off_counts);
+    a.counts = reinterpret_cast<uint32_t *>(ra.ws + L.off_counts);
     a.frags = reinterpret_cast<float4 *>(ra.ws + L.off_frags);
     a.frag_cap = L.frag_cap;
     a.st = reinterpret_cast<Status *>(ra.ws + L.off_status);
