@@ -637,7 +637,8 @@ MS_API ms_status ms_fine_tune_loss(const float *img_rgba, const float *target_rg
         return fail(MS_ERR_INVALID, "workspace %zu bytes < %zu needed", ws_bytes,
                     ms_fine_tune_loss_workspace_size(height, width));
     char *ws = static_cast<char *>(workspace);
-    float *scratch = reinterpret_cast<float *>(ws + ((256 - (reinterpret_cast<uintptr_t>(ws) & 255)) & 255));
+    // 16-byte alignment leaves at least 241 of the 256 spare bytes for the sum of the loss
+    char *scratch = ws + ((16 - (reinterpret_cast<uintptr_t>(ws) & 15)) & 15);
     cudaError_t e;
     {
         StageScope sc(MS_STAGE_LOSS, (cudaStream_t)stream);

@@ -88,9 +88,17 @@ struct FwdMem {
     float red[kThreads / 32];
 };
 
+// The loss over the blocks, summed in FP64: thousands of binary32 additions to one word would
+// carry an error of about 1e-6 of it, different from run to run.  The last block rounds it.
+struct LossSum {
+    double sum;
+    unsigned done, pad;
+};
+
 __global__ void __launch_bounds__(kThreads, 3) ssim_fwd_kernel(const float4 *__restrict__ img, const float4 *__restrict__ tgt,
                                                             int H, int W, float lam, float inv_n, Window win,
-                                                            float *__restrict__ G, float *__restrict__ loss) {
+                                                            float *__restrict__ G, LossSum *total,
+                                                            float *__restrict__ loss) {
     extern __shared__ __align__(16) char smem[];
     FwdMem &S = *reinterpret_cast<FwdMem *>(smem);
     const int tid = threadIdx.x;
@@ -192,7 +200,14 @@ __global__ void __launch_bounds__(kThreads, 3) ssim_fwd_kernel(const float4 *__r
         __syncthreads();   // the next channel's row pass overwrites the row sums
     }
     const float t = block_sum(acc, S.red);
-    if (tid == 0) atomicAdd(loss, t * inv_n);
+    if (tid == 0) {
+        atomicAdd(&total->sum, (double)t * (double)inv_n);
+        __threadfence();
+        if (atomicAdd(&total->done, 1u) == gridDim.x * gridDim.y - 1) {
+            __threadfence();
+            *loss = (float)atomicAdd(&total->sum, 0.0);
+        }
+    }
 }
 
 struct BwdMem {
@@ -305,21 +320,24 @@ Window make_window() {
 
 }  // namespace
 
-size_t ssim_scratch_bytes(int H, int W) { return (size_t)9 * sizeof(float) * (size_t)H * (size_t)W; }
+size_t ssim_scratch_bytes(int H, int W) { return (size_t)9 * sizeof(float) * (size_t)H * (size_t)W; }   // the planes
 
 cudaError_t launch_ssim_loss(const float *img, const float *tgt, int H, int W, float lam, float *dL, float *loss,
-                             float *scratch, cudaStream_t st) {
-    cudaError_t e = cudaMemsetAsync(loss, 0, sizeof(float), st);
-    if (e != cudaSuccess || H == 0 || W == 0) return e;
+                             char *scratch, cudaStream_t st) {
+    if (H == 0 || W == 0) return cudaMemsetAsync(loss, 0, sizeof(float), st);
+    LossSum *total = reinterpret_cast<LossSum *>(scratch);
+    float *G = reinterpret_cast<float *>(total + 1);
+    cudaError_t e = cudaMemsetAsync(total, 0, sizeof(LossSum), st);
+    if (e != cudaSuccess) return e;
     const dim3 grid((W + kT - 1) / kT, (H + kT - 1) / kT), block(kThreads);
     const float inv_n = (float)(1.0 / (3.0 * (double)H * (double)W));
     const Window win = make_window();
     e = cudaFuncSetAttribute(ssim_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(FwdMem));
     if (e != cudaSuccess) return e;
     ssim_fwd_kernel<<<grid, block, sizeof(FwdMem), st>>>(reinterpret_cast<const float4 *>(img), reinterpret_cast<const float4 *>(tgt),
-                                            H, W, lam, inv_n, win, scratch, loss);
+                                            H, W, lam, inv_n, win, G, total, loss);
     ssim_bwd_kernel<<<grid, block, 0, st>>>(reinterpret_cast<const float4 *>(img), reinterpret_cast<const float4 *>(tgt),
-                                            H, W, lam, inv_n, win, scratch, reinterpret_cast<float4 *>(dL));
+                                            H, W, lam, inv_n, win, G, reinterpret_cast<float4 *>(dL));
     return cudaGetLastError();
 }
 
