@@ -585,7 +585,7 @@ MS_API ms_status ms_render_get_info(const void *workspace, ms_render_info *info,
     info->sort_bits = (int32_t)st.sort_bits;
     info->overflow = st.pairs > st.cap ? 1 : 0;
     info->rect_tests = (int64_t)st.rect_tests;
-    info->fragments = (int64_t)st.fragments;
+    info->fragments = (int64_t)st.frags;   // (every covered fragment is given a record)
     info->commits = (int64_t)st.commits;
     info->frags = (int64_t)st.frags;
     info->frag_capacity = (int64_t)st.frag_cap;

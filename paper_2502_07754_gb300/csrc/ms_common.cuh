@@ -32,7 +32,6 @@ struct Status {
     unsigned int n_tiles;
     unsigned int sort_bits;
     unsigned long long rect_tests;   // forward rasterisation / resolve work counters
-    unsigned long long fragments;
     unsigned long long commits;
     unsigned long long frags;        // fragment records the pixels were given
     unsigned long long frag_cap;     // fragment record capacity of the workspace

@@ -1,7 +1,5 @@
-// Shared pieces of the rasterisation kernels: double-float projection of a fan
-// centre (value path), the shared-memory stage of a chunk of fans' decisions, and the per-pixel
-// coverage walk over a staged fan's K triangles with the binary32 decision formulas on
-// fan-relative vertex positions.
+// Shared pieces of the rasterisation kernels: a pair's rectangle word, the double-float projection
+// of a fan centre (value path), and the FP64 formulas of the source Gaussians.
 #pragma once
 
 #include "fan_geom.cuh"
@@ -20,12 +18,6 @@ __device__ __forceinline__ int count_bucket(uint32_t n) {
 __device__ __forceinline__ uint32_t pair_geo(int rx0, int ry0, int w, int h) {
     return 0x80000000u | (uint32_t)rx0 | (uint32_t)ry0 << 6 | (uint32_t)(w - 1) << 12 | (uint32_t)(h - 1) << 18;
 }
-
-struct SceneDev {
-    int W, H;
-    const float4 *dec;   // this view's decided vertices (xr, yr, Z or -1, origin), written by binning
-    const uint32_t *face_mask;   // per fan, bit j = face j drawn; NULL = all
-};
 
 // ------------------------------------------------------------------------------------
 // Double-float helpers of the value path (Knuth two-sum, FMA two-product)
@@ -105,208 +97,6 @@ __device__ __forceinline__ DfVec df_view_offset(const CamDev &c, const float m[3
     const dfl d0 = df_two_sum(__ldg(p), -m[0]), d1 = df_two_sum(__ldg(p + 1), -m[1]);
     const dfl d2 = df_two_sum(__ldg(p + 2), -m[2]);
     return DfVec{df_row_dot(c.R, d0, d1, d2), df_row_dot(c.R + 3, d0, d1, d2), df_row_dot(c.R + 6, d0, d1, d2)};
-}
-
-// ------------------------------------------------------------------------------------
-// Shared-memory stage (structure of arrays over CH slots)
-// ------------------------------------------------------------------------------------
-
-struct Stage {
-    int4 *rect;                   // [CH] i0, i1, j0, j1
-    uint32_t *flags;              // [CH] bits 0..15 valid triangle, 16..31 negative orientation
-    uint32_t *stie, *rtie;        // [CH] top-left tie bits of the spoke / rim directions
-    float *ox, *oy;               // [CH] integer origin of the fan's relative positions
-    float *vx, *vy;               // [KV][CH] decided vertices relative to the origin
-    float2 *sd;                   // [K][CH] spoke directions b_i - c
-    float *rdx, *rdy;             // [K][CH] rim directions, lower index to higher
-    float *area;                  // [K][CH] |area2|
-};
-
-__host__ __device__ __forceinline__ size_t stage_bytes(int CH, int K) {
-    return (size_t)CH * (16 + 12 + 8 + 4 * (2 * (K + 1) + 5 * K));
-}
-
-__device__ __forceinline__ Stage stage_ptrs(char *base, int CH, int K) {
-    const int KV = K + 1;
-    Stage s;
-    s.rect = reinterpret_cast<int4 *>(base);
-    s.flags = reinterpret_cast<uint32_t *>(s.rect + CH);
-    s.stie = s.flags + CH;
-    s.rtie = s.stie + CH;
-    float *f = reinterpret_cast<float *>(s.rtie + CH);
-    s.ox = f; f += CH;
-    s.oy = f; f += CH;
-    s.vx = f; f += KV * CH;
-    s.vy = f; f += KV * CH;
-    s.sd = reinterpret_cast<float2 *>(f); f += 2 * K * CH;   // (CH is even: 8-byte aligned)
-    s.rdx = f; f += K * CH;
-    s.rdy = f; f += K * CH;
-    s.area = f;
-    return s;
-}
-
-// OR / min / max over the LPF lanes of a fan's group (lanes lane & ~(LPF-1) .. + LPF-1).
-template <int LPF>
-__device__ __forceinline__ uint32_t group_or(uint32_t x) {
-#pragma unroll
-    for (int o = LPF / 2; o > 0; o >>= 1) x |= __shfl_xor_sync(0xffffffffu, x, o);
-    return x;
-}
-template <int LPF>
-__device__ __forceinline__ float group_min(float x) {
-#pragma unroll
-    for (int o = LPF / 2; o > 0; o >>= 1) x = fminf(x, __shfl_xor_sync(0xffffffffu, x, o));
-    return x;
-}
-template <int LPF>
-__device__ __forceinline__ float group_max(float x) {
-#pragma unroll
-    for (int o = LPF / 2; o > 0; o >>= 1) x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, o));
-    return x;
-}
-
-// The decision part of stage_fans: decided vertices, spoke and rim directions, areas,
-// tie bits, valid-triangle flags and the pixel rectangle of every slot.
-template <int LPF>
-__device__ __forceinline__ void stage_decisions(const SceneDev &a, const Stage &s, int K, int slot, int sub,
-                                                bool active, uint32_t fan) {
-    constexpr int CH = 32 / LPF;
-    const int KV = K + 1;
-    const float4 *dv = a.dec + (size_t)fan * KV;
-
-    uint32_t vmask = 0;
-    if (active)
-        for (int k = sub; k < KV; k += LPF) {
-            const float4 d = __ldg(dv + k);   // the binning pass's decide_vertex, bit for bit
-            s.vx[k * CH + slot] = d.x;
-            s.vy[k * CH + slot] = d.y;
-            if (d.z > 0.0f) vmask |= 1u << k;   // binning marks invalid vertices with Z = -1
-            if (k == 0) s.ox[slot] = d.w;
-            if (k == 1) s.oy[slot] = d.w;
-        }
-    vmask = group_or<LPF>(vmask);
-    __syncwarp();   // the group's vertex rows are complete
-    uint32_t tmask = tri_valid_mask(vmask, K);
-    if (a.face_mask && active) tmask &= __ldg(a.face_mask + fan);   // the same word in every lane of the fan
-    float mnx = 3.0e38f, mxx = -3.0e38f, mny = 3.0e38f, mxy = -3.0e38f;
-    uint32_t flags = 0, stie = 0, rtie = 0;
-    if (active) {
-        for (int k = sub; k < KV; k += LPF) {
-            if (!vertex_used(tmask, k, K)) continue;
-            const float x = s.vx[k * CH + slot], y = s.vy[k * CH + slot];
-            mnx = fminf(mnx, x); mxx = fmaxf(mxx, x);
-            mny = fminf(mny, y); mxy = fmaxf(mxy, y);
-        }
-        const float xc = s.vx[slot], yc = s.vy[slot];
-        for (int j = sub; j < K; j += LPF) {
-            const int b = 1 + j, c = 1 + (j + 1 == K ? 0 : j + 1);
-            const float xb = s.vx[b * CH + slot], yb = s.vy[b * CH + slot];
-            const float xn = s.vx[c * CH + slot], yn = s.vy[c * CH + slot];
-            const float sx = __fsub_rn(xb, xc), sy = __fsub_rn(yb, yc);
-            float rx, ry;
-            if (j + 1 == K) {   // rim (b_{K-1}, b_0): the lower index is b_0
-                rx = __fsub_rn(xb, xn);
-                ry = __fsub_rn(yb, yn);
-            } else {
-                rx = __fsub_rn(xn, xb);
-                ry = __fsub_rn(yn, yb);
-            }
-            s.sd[j * CH + slot] = make_float2(sx, sy);
-            s.rdx[j * CH + slot] = rx;
-            s.rdy[j * CH + slot] = ry;
-            const float ar = dec_area2(xc, yc, xb, yb, xn, yn);
-            s.area[j * CH + slot] = fabsf(ar);
-            if (((tmask >> j) & 1u) && ar != 0.0f) flags |= 1u << j;
-            if (ar < 0.0f) flags |= 1u << (16 + j);
-            // tie acceptance (E == 0) of each direction and of its reverse
-            if (sy < 0.0f || (sy == 0.0f && sx > 0.0f)) stie |= 1u << j;
-            if (sy > 0.0f || (sy == 0.0f && sx < 0.0f)) stie |= 1u << (16 + j);
-            if (ry < 0.0f || (ry == 0.0f && rx > 0.0f)) rtie |= 1u << j;
-            if (ry > 0.0f || (ry == 0.0f && rx < 0.0f)) rtie |= 1u << (16 + j);
-        }
-    }
-    mnx = group_min<LPF>(mnx);
-    mxx = group_max<LPF>(mxx);
-    mny = group_min<LPF>(mny);
-    mxy = group_max<LPF>(mxy);
-    flags = group_or<LPF>(flags);
-    stie = group_or<LPF>(stie);
-    rtie = group_or<LPF>(rtie);
-    if (active && sub == 0) {
-        const FanRect r = rect_from_bounds_rel(mnx, mxx, mny, mxy, (int)s.ox[slot], (int)s.oy[slot], a.W, a.H);
-        s.stie[slot] = stie;
-        s.rtie[slot] = rtie;
-        s.flags[slot] = (tmask == 0 || r.empty) ? 0u : flags;
-        s.rect[slot] = make_int4(r.i0, r.i1, r.j0, r.j1);
-    }
-}
-// Stages CH = 32 / LPF fans into slots 0..CH-1 with the whole warp: the LPF lanes of slot
-// lane / LPF share the fan's vertices and triangles (every lane of the warp
-// calls this; a lane whose slot is not active does no loads or stores but takes part in
-// the shuffles).  The staged words are the same as one lane per fan would write.
-template <int LPF>
-__device__ __forceinline__ void stage_fans(const SceneDev &a, const Stage &s, int K, int lane, bool active,
-                                           uint32_t fan) {
-    stage_decisions<LPF>(a, s, K, lane / LPF, lane % LPF, active, fan);
-}
-// Coverage of the pixel centre (pxc, pyc) by staged fan f: bit j is set when triangle j
-// covers it.  Each spoke value is computed once and turned into two pass bits (as the
-// edge c -> b_i and as its reverse), so a triangle's two spoke tests are a bit test; only
-// triangles passing both get the rim edge.  The result is the conjunction of the three edge
-// tests, as stated.  A spoke's bits are its value's sign bit, shifted into the mask by one
-// funnel shift; a value of zero (where the top-left tie bits decide) is noticed as a zero
-// minimum of the magnitudes and takes the general form below.  The count pass that runs it is
-// bound by issue slots (65-72% of them busy): setting two compared and tie-checked bits per
-// spoke took about 400 instructions a test; with the sign bits, one 8-byte load per spoke and
-// the fan of a test found from start flags instead of a five-step search, 200k fans at 800x800
-// went from 1.284 to 1.220 ms (forward and adjoint), 1k fans at 128x128 from 0.54 to 0.48 ms.
-template <int KT>
-__device__ __forceinline__ uint32_t cover_mask(const Stage &S, int CH, int K, int f, uint32_t flags, float pxc,
-                                               float pyc) {
-    const float qx = __fsub_rn(pxc, S.vx[f]), qy = __fsub_rn(pyc, S.vy[f]);
-    const uint32_t full = (1u << K) - 1u;
-    uint32_t N = 0;
-    float least = 3.0e38f;
-#pragma unroll(KT > 0 ? KT : 1)
-    for (int i = K - 1; i >= 0; --i) {   // (descending, so that spoke i lands in bit i)
-        const float2 d = S.sd[i * CH + f];
-        const float Si = __fsub_rn(__fmul_rn(d.x, qy), __fmul_rn(d.y, qx));
-        N = __funnelshift_l(__float_as_uint(Si), N, 1);
-        least = fminf(least, fabsf(Si));
-    }
-    uint32_t P = ~N & full;
-    if (least == 0.0f) {   // a centre on a spoke's line
-        const uint32_t stie = S.stie[f];
-        P = N = 0;
-#pragma unroll 1
-        for (int i = 0; i < K; ++i) {
-            const float2 d = S.sd[i * CH + f];
-            const float Si = __fsub_rn(__fmul_rn(d.x, qy), __fmul_rn(d.y, qx));
-            const bool z = Si == 0.0f;
-            P |= (uint32_t)(Si > 0.0f || (z && ((stie >> i) & 1u))) << i;
-            N |= (uint32_t)(Si < 0.0f || (z && ((stie >> (16 + i)) & 1u))) << i;
-        }
-    }
-    const uint32_t Pn = ((P >> 1) | (P << (K - 1))) & full;   // bit j: spoke j+1
-    const uint32_t Nn = ((N >> 1) | (N << (K - 1))) & full;
-    const uint32_t negm = flags >> 16;
-    uint32_t cand = ((P & Nn & ~negm) | (N & Pn & negm)) & flags & full;
-    uint32_t hits = 0;
-    const uint32_t rtie = S.rtie[f];
-    while (cand) {
-        const int j = __ffs(cand) - 1;
-        cand &= cand - 1;
-        const bool neg = (negm >> j) & 1u;
-        const bool wrap = (j + 1 == K);
-        const int lo = wrap ? 0 : j;
-        const float Rc = dec_edge(S.rdx[j * CH + f], S.rdy[j * CH + f], S.vx[(1 + lo) * CH + f],
-                                  S.vy[(1 + lo) * CH + f], pxc, pyc);
-        // oriented rim: b_j -> b_{j+1} for positive orientation, reversed otherwise
-        const bool flip = wrap != neg;
-        const float E0 = flip ? -Rc : Rc;
-        if (E0 > 0.0f || (E0 == 0.0f && ((rtie >> (flip ? 16 + j : j)) & 1u))) hits |= 1u << j;
-    }
-    return hits;
 }
 
 // ------------------------------------------------------------------------------------

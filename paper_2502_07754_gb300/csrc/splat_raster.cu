@@ -44,6 +44,7 @@ struct SplatArgs {
     Status *st;
     const float4 *dec;      // [view][vertex] decided polygon vertices
     int64_t V;
+    uint32_t *tests;        // [kMaskRegions] tests, in parts
     uint2 *pinfo;           // per pair: (0, rectangle within the tile; 0 if no centre is hit)
     const float4 *coef;     // [view][Gaussian][5]
     float r2;               // squared truncation radius in scales
@@ -239,7 +240,7 @@ __global__ void __launch_bounds__(kSplatWarps * 32, 14) splat_raster_kernel(cons
         }
     }
     const uint32_t lt = (1u << lane) - 1u, le = 0xffffffffu >> (31 - lane);
-    uint32_t head = 0, queued = 0, n_test = 0, n_frag = 0;
+    uint32_t head = 0, queued = 0, n_test = 0;
     for (uint32_t cb = it.y; cb < it.z; cb += 32) {
         const bool mine = cb + lane < it.z;
         const uint32_t g = mine ? __ldg(a.list + cb + lane) : 0u;
@@ -307,7 +308,6 @@ __global__ void __launch_bounds__(kSplatWarps * 32, 14) splat_raster_kernel(cons
             }
             if (!FILL) {   // counting: the order of a pixel's slots does not matter yet
                 hit_slots |= __reduce_or_sync(0xffffffffu, hit ? 1u << f : 0u);
-                n_frag += (uint32_t)hit;
                 if (hit) atomicAdd(&S.cnt[lp], 1u);
                 continue;
             }
@@ -351,11 +351,8 @@ __global__ void __launch_bounds__(kSplatWarps * 32, 14) splat_raster_kernel(cons
             if (c)
                 icnt[i] = atomicAdd(a.counts + vw.pix_base + (size_t)(ty0 + i / TILE) * cam.width + (size_t)(tx0 + i % TILE), c);
         }
-        const unsigned r0 = __reduce_add_sync(0xffffffffu, n_test), r1 = __reduce_add_sync(0xffffffffu, n_frag);
-        if (lane == 0) {
-            atomicAdd(&a.st->rect_tests, (unsigned long long)r0);
-            atomicAdd(&a.st->fragments, (unsigned long long)r1);
-        }
+        const unsigned r0 = __reduce_add_sync(0xffffffffu, n_test);
+        if (lane == 0) atomicAdd(a.tests + item % kMaskRegions, r0);
     }
 }
 
@@ -386,6 +383,7 @@ cudaError_t launch(const RenderArgs &ra, cudaStream_t st) {
     a.st = reinterpret_cast<Status *>(ra.ws + L.off_status);
     a.dec = reinterpret_cast<const float4 *>(ra.ws + L.off_dec);
     a.V = L.V;
+    a.tests = reinterpret_cast<uint32_t *>(ra.ws + L.off_mask_cursor);
     a.pinfo = reinterpret_cast<uint2 *>(ra.ws + L.off_maskoff);
     a.coef = ra.splat_coef;
     a.r2 = (float)(ra.spl.trunc * ra.spl.trunc);
