@@ -43,9 +43,12 @@ constexpr int kTraceKB = 8;
 constexpr int kStack = 64;
 constexpr double kSegEps = 1e-9;
 
+// An internal node holds its children's boxes (low corner, high corner), so a traversal step waits
+// for one 64-byte read.
 struct alignas(16) BvhNode {
-    float lo[3], hi[3];
-    int left, right;   // children: < n - 1 internal, >= n - 1 leaf (n - 1 + sorted position)
+    float box[2][6];
+    int child[2];      // < n - 1 internal, >= n - 1 leaf (n - 1 + sorted position)
+    int pad[2];
 };
 
 struct BvhLayout {
@@ -60,7 +63,7 @@ BvhLayout bvh_layout(int64_t T) {
     size_t o = 0;
     L.status = o;   o = al256(o + 256);
     L.bounds = o;   o = al256(o + 8 * sizeof(unsigned));
-    L.nodes = o;    o = al256(o + (size_t)(2 * n - 1) * sizeof(BvhNode));
+    L.nodes = o;    o = al256(o + (size_t)n * sizeof(BvhNode));   // (n - 1 internal nodes)
     L.parent = o;   o = al256(o + (size_t)(2 * n - 1) * 4);
     L.flags = o;    o = al256(o + (size_t)n * 4);
     L.leaf_tri = o; o = al256(o + (size_t)n * 4);
@@ -176,7 +179,7 @@ __device__ __forceinline__ int delta(const unsigned long long *k, int64_t n, int
 
 __global__ void __launch_bounds__(kBvhThreads) radix_tree_kernel(const unsigned long long *__restrict__ keys,
                                                                  int64_t n, BvhNode *__restrict__ nodes,
-                                                                 int *__restrict__ parent,
+                                                                 uint32_t *__restrict__ parent,
                                                                  int *__restrict__ leaf_tri) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         leaf_tri[i] = (int)(uint32_t)keys[i];
@@ -199,43 +202,45 @@ __global__ void __launch_bounds__(kBvhThreads) radix_tree_kernel(const unsigned 
         const int64_t lo = i < j ? i : j, hi = i < j ? j : i;
         const int left = lo == split ? (int)(n - 1 + split) : (int)split;
         const int right = hi == split + 1 ? (int)(n - 1 + split + 1) : (int)(split + 1);
-        nodes[i].left = left;
-        nodes[i].right = right;
-        parent[left] = (int)i;
-        parent[right] = (int)i;
+        nodes[i].child[0] = left;
+        nodes[i].child[1] = right;
+        parent[left] = 2u * (uint32_t)i;        // and which child of it
+        parent[right] = 2u * (uint32_t)i + 1u;
     }
 }
 
 __global__ void __launch_bounds__(kBvhThreads) bounds_up_kernel(const float *__restrict__ xyz,
                                                                 const int32_t *__restrict__ tris, int K, int64_t n,
-                                                                BvhNode *nodes, const int *__restrict__ parent,
+                                                                BvhNode *nodes, const uint32_t *__restrict__ parent,
                                                                 const int *__restrict__ leaf_tri, int *flags) {
+    if (n < 2) return;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t leaf = n - 1 + i;
         int64_t v[3];
         tri_verts(tris, K, leaf_tri[i], v);
-        BvhNode &L = nodes[leaf];
+        float box[6];
 #pragma unroll
         for (int r = 0; r < 3; ++r) {
             const float a = __ldg(xyz + 3 * v[0] + r), b = __ldg(xyz + 3 * v[1] + r), c = __ldg(xyz + 3 * v[2] + r);
             const float lo = fminf(fminf(a, b), c), hi = fmaxf(fmaxf(a, b), c);
             const float m = 1e-5f * (hi - lo) + 1e-6f * fmaxf(fabsf(lo), fabsf(hi)) + 1e-30f;
-            L.lo[r] = lo - m;
-            L.hi[r] = hi + m;
+            box[r] = lo - m;
+            box[3 + r] = hi + m;
         }
-        L.left = L.right = -1;
-        int64_t node = leaf;
-        // each internal node is completed by the second of its two children to arrive
+        int64_t node = n - 1 + i;
+        // every child writes its box into its parent; the second to arrive takes both on
         for (int steps = 0; node != 0 && steps < 64 + 64; ++steps) {
-            const int p = parent[node];
+            const uint32_t ps = parent[node], p = ps >> 1, side = ps & 1u;
+            volatile float *mine = nodes[p].box[side];
+#pragma unroll
+            for (int r = 0; r < 6; ++r) mine[r] = box[r];
             __threadfence();
             if (atomicAdd(&flags[p], 1) == 0) break;
             __threadfence();
-            const BvhNode &a = nodes[nodes[p].left], &b = nodes[nodes[p].right];
+            const volatile float *other = nodes[p].box[side ^ 1u];
 #pragma unroll
             for (int r = 0; r < 3; ++r) {
-                nodes[p].lo[r] = fminf(a.lo[r], b.lo[r]);
-                nodes[p].hi[r] = fmaxf(a.hi[r], b.hi[r]);
+                box[r] = fminf(box[r], other[r]);
+                box[3 + r] = fmaxf(box[3 + r], other[3 + r]);
             }
             node = p;
         }
@@ -303,15 +308,6 @@ __device__ __forceinline__ dfl df_of(double x) {
     return dfl{h, (float)(x - (double)h)};
 }
 __device__ __forceinline__ double to_double(dfl a) { return (double)a.h + (double)a.l; }
-__device__ __forceinline__ RayF ray_f(const double o[3], const double d[3]) {
-    RayF r;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        r.o[k] = df_of(o[k]);
-        r.d[k] = df_of(d[k]);
-    }
-    return r;
-}
 // Error bounds of the filter's determinant and numerators.
 struct MtBounds {
     float det, U, V, T;
@@ -406,19 +402,22 @@ __device__ __forceinline__ void tri_f(const TraceArgs &a, int tri, float P[3][3]
         for (int r = 0; r < 3; ++r) P[k][r] = __ldg(a.xyz + 3 * v[k] + r);
 }
 
-// Whether the ray (o, d; rf its double-float form) crosses triangle P within (tmin, tmax): the
-// binary32 filter, then double-float, then FP64 where neither is certain.
-__device__ __forceinline__ bool crosses(const double o[3], const double d[3], const RayF &rf, const float P[3][3],
-                                        float f_min, float f_max, double tmin, double tmax, Hit &h) {
+// Whether the ray crosses triangle P within (tmin, tmax): the binary32 filter, then double-float,
+// then FP64 where neither is certain.
+__device__ __forceinline__ bool crosses(const RayF &rf, const float P[3][3], float f_min, float f_max, double tmin,
+                                        double tmax, Hit &h) {
     MtBounds e;
     if (!mt_may_hit(rf, P[0], P[1], P[2], f_min, f_max, e)) return false;
     const int c = mt_df(rf, P[0], P[1], P[2], e, df_of(tmin), df_of(tmax), h);
     if (c >= 0) return c != 0;
-    double Q[3][3], t, u, v;
+    double o[3], d[3], Q[3][3], t, u, v;
 #pragma unroll
-    for (int k = 0; k < 3; ++k)
+    for (int k = 0; k < 3; ++k) {
+        o[k] = to_double(rf.o[k]);
+        d[k] = to_double(rf.d[k]);
 #pragma unroll
         for (int r = 0; r < 3; ++r) Q[k][r] = (double)P[k][r];
+    }
     if (!(mt(o, d, Q[0], Q[1], Q[2], t, u, v) && t > tmin && t < tmax)) return false;
     h.t = df_of(t);
     h.u = df_of(u);
@@ -426,14 +425,28 @@ __device__ __forceinline__ bool crosses(const double o[3], const double d[3], co
     return true;
 }
 
-// Slab test of the ray o + t d against a node box (binary32, widened): whether it meets [t0, t1],
+// The boxes and children of an internal node.
+struct NodeW {
+    float4 a, b, c;
+    int left, right;
+};
+__device__ __forceinline__ NodeW load_node(const BvhNode *nodes, int node) {
+    const float4 *p = reinterpret_cast<const float4 *>(nodes + node);
+    NodeW w;
+    w.a = __ldg(p);
+    w.b = __ldg(p + 1);
+    w.c = __ldg(p + 2);
+    const int2 ch = __ldg(reinterpret_cast<const int2 *>(p + 3));
+    w.left = ch.x;
+    w.right = ch.y;
+    return w;
+}
+
+// Slab test of the ray o + t d against a box (binary32, widened): whether it meets [t0, t1],
 // and where (tn, tf).
-__device__ __forceinline__ bool box_span(const BvhNode *node, const float o[3], const float id[3], float t0, float t1,
-                                         float &tn, float &tf, int &left, int &right) {
-    const float4 a = __ldg(reinterpret_cast<const float4 *>(node)), b = __ldg(reinterpret_cast<const float4 *>(node) + 1);
-    const float lo[3] = {a.x, a.y, a.z}, hi[3] = {a.w, b.x, b.y};
-    left = __float_as_int(b.z);
-    right = __float_as_int(b.w);
+__device__ __forceinline__ bool box_span(float lx, float ly, float lz, float hx, float hy, float hz, const float o[3],
+                                         const float id[3], float t0, float t1, float &tn, float &tf) {
+    const float lo[3] = {lx, ly, lz}, hi[3] = {hx, hy, hz};
 #pragma unroll
     for (int r = 0; r < 3; ++r) {
         const float x = (lo[r] - o[r]) * id[r], y = (hi[r] - o[r]) * id[r];
@@ -445,6 +458,14 @@ __device__ __forceinline__ bool box_span(const BvhNode *node, const float o[3], 
     tf = t1;
     return t0 <= t1;
 }
+__device__ __forceinline__ bool left_span(const NodeW &w, const float o[3], const float id[3], float t0, float t1,
+                                          float &tn, float &tf) {
+    return box_span(w.a.x, w.a.y, w.a.z, w.a.w, w.b.x, w.b.y, o, id, t0, t1, tn, tf);
+}
+__device__ __forceinline__ bool right_span(const NodeW &w, const float o[3], const float id[3], float t0, float t1,
+                                           float &tn, float &tf) {
+    return box_span(w.b.z, w.b.w, w.c.x, w.c.y, w.c.z, w.c.w, o, id, t0, t1, tn, tf);
+}
 
 __device__ __forceinline__ bool hit_less(dfl ta, int ia, dfl tb, int ib) {
     return df_lt(ta, tb) || (ta.h == tb.h && ta.l == tb.l && ia < ib);
@@ -455,145 +476,207 @@ __device__ __forceinline__ dfl bary_mix(dfl u, dfl v, float a0, float a1, float 
     return df_add_fast(df_add_fast(df_mul_f(w, a0), df_mul_f(u, a1)), df_mul_f(v, a2));
 }
 
-// Transmittance of the segment p -> L through every triangle but `own`.
-__device__ double shadow(const TraceArgs &a, const double p[3], int own) {
-    const double d[3] = {a.L[0] - p[0], a.L[1] - p[1], a.L[2] - p[2]};
-    const RayF rf = ray_f(p, d);
-    float of[3], id[3];
-#pragma unroll
-    for (int r = 0; r < 3; ++r) {
-        of[r] = rf.o[r].h;
-        id[r] = 1.0f / rf.d[r].h;
-    }
+// Shadow segments of one block's crossings of one pass, a slot per (crossing, pixel).
+constexpr int kJobs = kTraceKB * kTraceThreads;
+struct Jobs {
+    float2 o[3][kJobs], d[3][kJobs];   // origin and vector to the light; o[0] takes the transmittance
+    int tri[kJobs];                    // the crossing's own triangle
+    uint16_t list[kJobs];              // slots in use
+    int n, next;
+};
+
+// Transmittance of the block's segments through every triangle but their own.  A lane that is done
+// takes the next segment of the list, so no lane waits for the longest of 32.
+__device__ __forceinline__ void shadow_jobs(const TraceArgs &a, Jobs &J) {
     const int n1 = (int)(a.T - 1);   // nodes from n1 on are leaves
-    int stack[kStack];
-    int sp = 0, node = 0;
-    dfl S = df_make(1.0f);
     const float t0 = -1e-3f, t1 = 1.001f;
+    int stack[kStack];
+    int sp = 0, node = -1, slot = -1, own = -1;
+    RayF rf;
+    float of[3], id[3];
+    dfl S = df_make(1.0f);
     for (;;) {
-        // down to a leaf whose parent's test admitted it
+        if (node < 0) {
+            if (slot >= 0) J.o[0][slot] = make_float2(S.h, S.l);
+            const int j = atomicAdd(&J.next, 1);
+            if (j >= J.n) break;
+            slot = J.list[j];
+            own = J.tri[slot];
+#pragma unroll
+            for (int r = 0; r < 3; ++r) {
+                const float2 o = J.o[r][slot], d = J.d[r][slot];
+                rf.o[r] = dfl{o.x, o.y};
+                rf.d[r] = dfl{d.x, d.y};
+                of[r] = o.x;
+                id[r] = 1.0f / d.x;
+            }
+            S = df_make(1.0f);
+            sp = 0;
+            node = 0;
+        }
         while (node >= 0 && node < n1) {
-            const int left = __ldg(&a.nodes[node].left), right = __ldg(&a.nodes[node].right);
+            const NodeW w = load_node(a.nodes, node);
             float tn, tf;
-            int x, y;
-            const bool hl = box_span(a.nodes + left, of, id, t0, t1, tn, tf, x, y);
-            const bool hr = box_span(a.nodes + right, of, id, t0, t1, tn, tf, x, y);
+            const bool hl = left_span(w, of, id, t0, t1, tn, tf), hr = right_span(w, of, id, t0, t1, tn, tf);
             if (hl && hr) {
-                if (sp < kStack) stack[sp++] = right;
+                if (sp < kStack) stack[sp++] = w.right;
                 else atomicAdd(a.overflow, 1u);
             }
-            node = hl ? left : (hr ? right : (sp > 0 ? stack[--sp] : -1));
+            node = hl ? w.left : (hr ? w.right : (sp > 0 ? stack[--sp] : -1));
         }
-        if (node < 0) break;
+        if (node < 0) continue;
         const int tri = __ldg(a.leaf_tri + (node - n1));
         node = sp > 0 ? stack[--sp] : -1;
         if (tri == own) continue;
         float P[3][3];
         tri_f(a, tri, P);
         Hit h;
-        if (!crosses(p, d, rf, P, (float)kSegEps, (float)(1.0 - kSegEps), kSegEps, 1.0 - kSegEps, h)) continue;
+        if (!crosses(rf, P, (float)kSegEps, (float)(1.0 - kSegEps), kSegEps, 1.0 - kSegEps, h)) continue;
         int64_t v[3];
         tri_verts(a.tris, a.K, tri, v);
         const dfl al = bary_mix(h.u, h.v, __ldg(a.alpha + v[0]), __ldg(a.alpha + v[1]), __ldg(a.alpha + v[2]));
         S = df_mul(S, df_add_f(df_neg(al), 1.0f));
         // the light is blocked to within T_eps: the colour's shadow factor moves by at
         // most (1 - ambient) T_eps, the primary composite's own termination bound
-        if (to_double(S) < a.T_eps) break;
+        if (to_double(S) < a.T_eps) node = -1;
     }
-    return to_double(S);
 }
 
 // One thread a pixel, a block an 8 x 8 tile of pixels (a warp 8 x 4), so that a warp's rays stay
-// together down the tree.
+// together down the tree.  With shadows a block gathers its pixels' next crossings, traces all their
+// segments to the light as one list, and composites.  What bounds it: the waits on nodes and triangles and the
+// lanes that part ways (a segment meets 187 nodes and 60 leaves on its own).  1.6M triangles with shadows at
+// 800x800, 5.4M segments: 148 ms, against 218 ms for a thread that traced its own pixel's segments one
+// after the other, over nodes that held their own box (two loads a child).
+template <bool SHADOWS>
 __global__ void __launch_bounds__(kTraceThreads) trace_kernel(const __grid_constant__ TraceArgs a) {
+    extern __shared__ __align__(16) char smem[];
+    Jobs &J = *reinterpret_cast<Jobs *>(smem);
     const int W = a.cam.width, H = a.cam.height;
     const int px = blockIdx.x * 8 + (threadIdx.x & 7), py = blockIdx.y * 8 + (threadIdx.x >> 3);
-    if (px >= W || py >= H) return;
-    const int64_t pix = (int64_t)py * W + px;
+    const bool in = px < W && py < H;
     const CamDev &c = a.cam;
-    // ray with unit view depth: d = R^T ((x - cx) / fx, (y - cy) / fy, 1)
-    const double dc[3] = {((double)px + 0.5 - (double)c.cx) / (double)c.fx,
-                          ((double)py + 0.5 - (double)c.cy) / (double)c.fy, 1.0};
-    double d[3], o[3];
-#pragma unroll
-    for (int r = 0; r < 3; ++r) {
-        d[r] = ((double)c.R[r] * dc[0] + (double)c.R[3 + r] * dc[1]) + (double)c.R[6 + r] * dc[2];
-        o[r] = (double)c.C[r];
-    }
-    const RayF rf = ray_f(o, d);
+    RayF rf;
     float of[3], id[3];
+    {
+        // ray with unit view depth: d = R^T ((x - cx) / fx, (y - cy) / fy, 1)
+        const double dc[3] = {((double)px + 0.5 - (double)c.cx) / (double)c.fx,
+                              ((double)py + 0.5 - (double)c.cy) / (double)c.fy, 1.0};
 #pragma unroll
-    for (int r = 0; r < 3; ++r) {
-        of[r] = rf.o[r].h;
-        id[r] = 1.0f / rf.d[r].h;
+        for (int r = 0; r < 3; ++r) {
+            rf.o[r] = df_make(c.C[r]);
+            rf.d[r] = df_of(((double)c.R[r] * dc[0] + (double)c.R[3 + r] * dc[1]) + (double)c.R[6 + r] * dc[2]);
+            of[r] = rf.o[r].h;
+            id[r] = 1.0f / rf.d[r].h;
+        }
     }
     const int n1 = (int)(a.T - 1);   // nodes from n1 on are leaves
     double T = 1.0, C0 = 0.0, C1 = 0.0, C2 = 0.0;
     dfl after_t = df_make(-3.0e38f);
     int after_i = -1;
-    for (int pass = 0; a.T > 0; ++pass) {
+    bool alive = in && a.T > 0;
+    for (;;) {
         Hit buf[kTraceKB];
         int nb = 0;
         bool more = false;
-        int stack[kStack];
-        int sp = 0, node = 0;
-        // Boxes wholly before the last composited crossing hold nothing for this pass, and
-        // boxes wholly beyond the farthest kept crossing of a full buffer only mean another
-        // pass; both bounds are widened by 1e-5 relative, far above the slab test's rounding.
-        const float t_after = after_t.h > 0.0f ? after_t.h * (1.0f - 1e-5f) : 0.0f;
-        const float t_near = c.znear * 0.999f;
-        for (;;) {
-            while (node >= 0 && node < n1) {
-                const int left = __ldg(&a.nodes[node].left), right = __ldg(&a.nodes[node].right);
-                float nl, fl, nr, fr;
-                int x, y;
-                bool hl = box_span(a.nodes + left, of, id, t_near, 3.0e38f, nl, fl, x, y) && fl >= t_after;
-                bool hr = box_span(a.nodes + right, of, id, t_near, 3.0e38f, nr, fr, x, y) && fr >= t_after;
+        if (alive) {
+            int stack[kStack];
+            int sp = 0, node = 0;
+            // Boxes wholly before the last composited crossing hold nothing for this pass, and
+            // boxes wholly beyond the farthest kept crossing of a full buffer only mean another
+            // pass; both bounds are widened by 1e-5 relative, far above the slab test's rounding.
+            const float t_after = after_t.h > 0.0f ? after_t.h * (1.0f - 1e-5f) : 0.0f;
+            const float t_near = c.znear * 0.999f;
+            for (;;) {
+                while (node >= 0 && node < n1) {
+                    const NodeW w = load_node(a.nodes, node);
+                    float nl, fl, nr, fr;
+                    bool hl = left_span(w, of, id, t_near, 3.0e38f, nl, fl) && fl >= t_after;
+                    bool hr = right_span(w, of, id, t_near, 3.0e38f, nr, fr) && fr >= t_after;
+                    if (nb == kTraceKB) {
+                        const float t_far = buf[kTraceKB - 1].t.h * (1.0f + 1e-5f);
+                        if (hl && nl > t_far) {
+                            hl = false;
+                            more = true;
+                        }
+                        if (hr && nr > t_far) {
+                            hr = false;
+                            more = true;
+                        }
+                    }
+                    // the nearer child first: the buffer fills with near crossings early
+                    const bool swap = hl && hr && nr < nl;
+                    const int first = swap || !hl ? w.right : w.left, second = swap ? w.left : w.right;
+                    if (hl && hr) {
+                        if (sp < kStack) stack[sp++] = second;
+                        else atomicAdd(a.overflow, 1u);
+                    }
+                    node = hl || hr ? first : (sp > 0 ? stack[--sp] : -1);
+                }
+                if (node < 0) break;
+                const int tri = __ldg(a.leaf_tri + (node - n1));
+                node = sp > 0 ? stack[--sp] : -1;
+                float P[3][3];
+                tri_f(a, tri, P);
+                Hit h;
+                // crossings before the last composited one were taken in an earlier pass
+                if (!crosses(rf, P, fmaxf(c.znear, after_t.h), 3.0e38f, (double)c.znear, 1.0e300, h)) continue;
+                h.tri = tri;
+                if (!hit_less(after_t, after_i, h.t, tri)) continue;   // composited in an earlier pass
                 if (nb == kTraceKB) {
-                    const float t_far = buf[kTraceKB - 1].t.h * (1.0f + 1e-5f);
-                    if (hl && nl > t_far) {
-                        hl = false;
-                        more = true;
-                    }
-                    if (hr && nr > t_far) {
-                        hr = false;
-                        more = true;
-                    }
+                    more = true;
+                    if (!hit_less(h.t, tri, buf[kTraceKB - 1].t, buf[kTraceKB - 1].tri)) continue;
+                    --nb;   // the farthest kept crossing waits for a later pass
                 }
-                // the nearer child first: the buffer fills with near crossings early
-                const bool swap = hl && hr && nr < nl;
-                const int first = swap || !hl ? right : left, second = swap ? left : right;
-                if (hl && hr) {
-                    if (sp < kStack) stack[sp++] = second;
-                    else atomicAdd(a.overflow, 1u);
+                int s = nb;
+                while (s > 0 && hit_less(h.t, tri, buf[s - 1].t, buf[s - 1].tri)) {
+                    buf[s] = buf[s - 1];
+                    --s;
                 }
-                node = hl || hr ? first : (sp > 0 ? stack[--sp] : -1);
+                buf[s] = h;
+                ++nb;
             }
-            if (node < 0) break;
-            const int tri = __ldg(a.leaf_tri + (node - n1));
-            node = sp > 0 ? stack[--sp] : -1;
-            float P[3][3];
-            tri_f(a, tri, P);
-            Hit h;
-            // crossings before the last composited one were taken in an earlier pass
-            if (!crosses(o, d, rf, P, fmaxf(c.znear, after_t.h), 3.0e38f, (double)c.znear, 1.0e300, h)) continue;
-            h.tri = tri;
-            if (!hit_less(after_t, after_i, h.t, tri)) continue;   // composited in an earlier pass
-            if (nb == kTraceKB) {
-                more = true;
-                if (!hit_less(h.t, tri, buf[kTraceKB - 1].t, buf[kTraceKB - 1].tri)) continue;
-                --nb;   // the farthest kept crossing waits for a later pass
-            }
-            int s = nb;
-            while (s > 0 && hit_less(h.t, tri, buf[s - 1].t, buf[s - 1].tri)) {
-                buf[s] = buf[s - 1];
-                --s;
-            }
-            buf[s] = h;
-            ++nb;
         }
-        bool stop = false;
-        for (int k = 0; k < nb; ++k) {
+        // the crossings that will be composited
+        int n_use = 0;
+        {
+            double Tn = T;
+            for (; n_use < nb && !(Tn < a.T_eps); ++n_use) {
+                const Hit &h = buf[n_use];
+                int64_t v[3];
+                tri_verts(a.tris, a.K, h.tri, v);
+                Tn *= 1.0 - to_double(bary_mix(h.u, h.v, __ldg(a.alpha + v[0]), __ldg(a.alpha + v[1]), __ldg(a.alpha + v[2])));
+            }
+        }
+        if (SHADOWS) {
+            if (threadIdx.x == 0) J.n = J.next = 0;
+            __syncthreads();
+            for (int k = 0; k < kTraceKB; ++k) {   // a warp's segments of one depth follow each other
+                const bool has = k < n_use;
+                const unsigned m = __ballot_sync(0xffffffffu, has);
+                if (m == 0) break;
+                int base = 0;
+                if ((threadIdx.x & 31) == 0) base = atomicAdd(&J.n, __popc(m));
+                base = __shfl_sync(0xffffffffu, base, 0);
+                if (has) {
+                    const int slot = k * kTraceThreads + threadIdx.x;
+                    J.list[base + __popc(m & ((1u << (threadIdx.x & 31)) - 1u))] = (uint16_t)slot;
+                    const double t = to_double(buf[k].t);
+                    J.tri[slot] = buf[k].tri;
+#pragma unroll
+                    for (int r = 0; r < 3; ++r) {
+                        const double p = to_double(rf.o[r]) + t * to_double(rf.d[r]);
+                        const dfl pf = df_of(p), df = df_of(a.L[r] - p);
+                        J.o[r][slot] = make_float2(pf.h, pf.l);
+                        J.d[r][slot] = make_float2(df.h, df.l);
+                    }
+                }
+            }
+            __syncthreads();
+            shadow_jobs(a, J);
+            __syncthreads();
+        }
+        for (int k = 0; k < n_use; ++k) {
             const Hit &h = buf[k];
             int64_t v[3];
             tri_verts(a.tris, a.K, h.tri, v);
@@ -603,10 +686,9 @@ __global__ void __launch_bounds__(kTraceThreads) trace_kernel(const __grid_const
             for (int r = 0; r < 3; ++r)
                 col[r] = to_double(bary_mix(h.u, h.v, __ldg(a.rgb + 3 * v[0] + r), __ldg(a.rgb + 3 * v[1] + r),
                                             __ldg(a.rgb + 3 * v[2] + r)));
-            if (a.shadows) {
-                const double t = to_double(h.t);
-                const double p[3] = {o[0] + t * d[0], o[1] + t * d[1], o[2] + t * d[2]};
-                const double f = a.ambient + (1.0 - a.ambient) * shadow(a, p, h.tri);
+            if (SHADOWS) {
+                const float2 S = J.o[0][k * kTraceThreads + threadIdx.x];
+                const double f = a.ambient + (1.0 - a.ambient) * to_double(dfl{S.x, S.y});
 #pragma unroll
                 for (int r = 0; r < 3; ++r) col[r] *= f;
             }
@@ -616,16 +698,14 @@ __global__ void __launch_bounds__(kTraceThreads) trace_kernel(const __grid_const
             T *= 1.0 - al;
             after_t = h.t;
             after_i = h.tri;
-            if (T < a.T_eps) {
-                stop = true;
-                break;
-            }
         }
-        if (stop || !more) break;
+        alive = alive && more && !(T < a.T_eps);
+        if (SHADOWS ? !__syncthreads_or(alive) : !alive) break;
     }
+    if (!in) return;
     float4 *out = reinterpret_cast<float4 *>(a.out);
-    out[pix] = make_float4((float)(C0 + T * a.bg[0]), (float)(C1 + T * a.bg[1]), (float)(C2 + T * a.bg[2]),
-                           (float)(1.0 - T));
+    out[(int64_t)py * W + px] = make_float4((float)(C0 + T * a.bg[0]), (float)(C1 + T * a.bg[1]),
+                                            (float)(C2 + T * a.bg[2]), (float)(1.0 - T));
 }
 
 unsigned grid_of(int64_t n, int threads) {
@@ -666,7 +746,7 @@ extern "C" MS_API ms_status ms_bvh_build(const float *xyz, const int32_t *tris, 
     e = sort_u64(k0, k1, T, 32, 4, b + L.scratch, st, &sorted);
     if (e != cudaSuccess) return set_error(MS_ERR_CUDA, "BVH key sort: %s", cudaGetErrorString(e));
     BvhNode *nodes = reinterpret_cast<BvhNode *>(b + L.nodes);
-    int *parent = reinterpret_cast<int *>(b + L.parent);
+    uint32_t *parent = reinterpret_cast<uint32_t *>(b + L.parent);
     int *leaf_tri = reinterpret_cast<int *>(b + L.leaf_tri);
     radix_tree_kernel<<<grid_of(T, kBvhThreads), kBvhThreads, 0, st>>>(sorted, T, nodes, parent, leaf_tri);
     bounds_up_kernel<<<grid_of(T, kBvhThreads), kBvhThreads, 0, st>>>(xyz, tris, K, T, nodes, parent, leaf_tri,
@@ -711,7 +791,10 @@ extern "C" MS_API ms_status ms_raytrace(const float *xyz, const float *rgb, cons
     a.T_eps = T_eps;
     a.out = out_rgba;
     const dim3 grid((cam->width + 7) / 8, (cam->height + 7) / 8);
-    trace_kernel<<<grid, kTraceThreads, 0, (cudaStream_t)stream>>>(a);
+    if (a.shadows)
+        trace_kernel<true><<<grid, kTraceThreads, sizeof(Jobs), (cudaStream_t)stream>>>(a);
+    else
+        trace_kernel<false><<<grid, kTraceThreads, 0, (cudaStream_t)stream>>>(a);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return set_error(MS_ERR_CUDA, "trace_kernel: %s", cudaGetErrorString(e));
     count_launches(1);
