@@ -159,12 +159,9 @@ __device__ __noinline__ uint32_t cover_direct(const float4 *__restrict__ dv, int
 }
 
 template <int TILE, int KT>
-__global__ void __launch_bounds__(kFillWarps * 32) fill_kernel(const __grid_constant__ FillArgs a) {
-    extern __shared__ __align__(16) char smem[];
+__device__ __forceinline__ void fill_item(const FillArgs &a, char *smem, uint32_t item) {
     const int K = KT > 0 ? KT : a.K;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t item = blockIdx.x * kFillWarps + warp;
-    if (item >= a.st->n_items) return;   // whole warp; nothing below synchronises the block
     const uint4 it = a.items[item];
     const int view = view_of_tile(a.vt, it.x);
     const ViewDev &vw = a.vt.v[view];
@@ -341,12 +338,29 @@ __global__ void __launch_bounds__(kFillWarps * 32) fill_kernel(const __grid_cons
     }
 }
 
+template <int TILE, int KT, bool STRIDED>
+__global__ void __launch_bounds__(kFillWarps * 32) fill_kernel(const __grid_constant__ FillArgs a) {
+    extern __shared__ __align__(16) char smem[];
+    const uint32_t n_items = a.st->n_items;
+    uint32_t item = blockIdx.x * kFillWarps + threadIdx.x / 32;   // (whole warps: nothing synchronises the block)
+    if (!STRIDED) {
+        if (item < n_items) fill_item<TILE, KT>(a, smem, item);
+    } else {
+        for (; item < n_items; item += gridDim.x * kFillWarps) {
+            fill_item<TILE, KT>(a, smem, item);
+            __syncwarp();   // the stage is free again
+        }
+    }
+}
+
 template <int TILE, int KT>
 cudaError_t launch_t(const FillArgs &fa, int64_t max_items, int K, cudaStream_t st) {
     const size_t smem = kFillWarps * fill_warp_bytes<TILE>(K);
-    auto fn = fill_kernel<TILE, KT>;
+    const int64_t blocks = (max_items + kFillWarps - 1) / kFillWarps;
+    const bool strided = blocks > kItemBlocks;
+    auto fn = strided ? fill_kernel<TILE, KT, true> : fill_kernel<TILE, KT, false>;
     cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    fn<<<(unsigned)((max_items + kFillWarps - 1) / kFillWarps), kFillWarps * 32, smem, st>>>(fa);
+    fn<<<(unsigned)(strided ? kStrideBlocks : blocks), kFillWarps * 32, smem, st>>>(fa);
     return cudaGetLastError();
 }
 

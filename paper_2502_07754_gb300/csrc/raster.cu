@@ -118,12 +118,9 @@ __device__ __forceinline__ uint32_t cover_mask(const CountMem &S, int K, int f, 
 }
 
 template <int TILE, int KT>
-__global__ void __launch_bounds__(kRastWarps * 32) count_kernel(const __grid_constant__ RastArgs a) {
-    extern __shared__ __align__(16) char smem[];
+__device__ __forceinline__ void count_item(const RastArgs &a, char *smem, uint32_t item) {
     const int K = KT > 0 ? KT : a.K;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t item = blockIdx.x * kRastWarps + warp;
-    if (item >= a.st->n_items) return;   // whole warp; nothing below synchronises the block
     const uint4 it = a.items[item];
     const int view = view_of_tile(a.vt, it.x);
     const ViewDev &vw = a.vt.v[view];
@@ -263,12 +260,29 @@ __global__ void __launch_bounds__(kRastWarps * 32) count_kernel(const __grid_con
     }
 }
 
+template <int TILE, int KT, bool STRIDED>
+__global__ void __launch_bounds__(kRastWarps * 32) count_kernel(const __grid_constant__ RastArgs a) {
+    extern __shared__ __align__(16) char smem[];
+    const uint32_t n_items = a.st->n_items;
+    uint32_t item = blockIdx.x * kRastWarps + threadIdx.x / 32;   // (whole warps: nothing synchronises the block)
+    if (!STRIDED) {
+        if (item < n_items) count_item<TILE, KT>(a, smem, item);
+    } else {
+        for (; item < n_items; item += gridDim.x * kRastWarps) {
+            count_item<TILE, KT>(a, smem, item);
+            __syncwarp();   // the stage is free again
+        }
+    }
+}
+
 template <int TILE, int KT>
 cudaError_t launch_t(const RastArgs &ra, int64_t max_items, int K, cudaStream_t st) {
     const size_t smem = kRastWarps * count_warp_bytes<TILE>(K);
-    auto fn = count_kernel<TILE, KT>;
+    const int64_t blocks = (max_items + kRastWarps - 1) / kRastWarps;
+    const bool strided = blocks > kItemBlocks;
+    auto fn = strided ? count_kernel<TILE, KT, true> : count_kernel<TILE, KT, false>;
     cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    fn<<<(unsigned)((max_items + kRastWarps - 1) / kRastWarps), kRastWarps * 32, smem, st>>>(ra);
+    fn<<<(unsigned)(strided ? kStrideBlocks : blocks), kRastWarps * 32, smem, st>>>(ra);
     return cudaGetLastError();
 }
 

@@ -13,6 +13,13 @@ __device__ __forceinline__ int count_bucket(uint32_t n) {
     return n < (uint32_t)kCountBuckets ? (int)n : kCountBuckets - 1;
 }
 
+// The passes over the work items launch a warp an item up to kItemBlocks blocks; beyond, kStrideBlocks
+// blocks stride over the items.  The items are counted on the device, their capacity is many times what a
+// scene needs, and a block without an item still takes a launch slot: the 16 views of 3M fans have 0.9M items
+// and room for 6.3M, and forward and adjoint took 19.7 ms with a warp for each, 17.5 ms with the stride.
+// Below the bound the loop costs more (2% of 8 views of 250k Gaussians) than the empty blocks do.
+constexpr int64_t kItemBlocks = 256 * 1024, kStrideBlocks = 64 * 1024;
+
 // A pair's pixel rectangle clipped to its tile, relative to the tile's corner: x0 | y0 << 6 |
 // (w - 1) << 12 | (h - 1) << 18, bit 31 set; 0 for a pair with no pixel to test.
 __device__ __forceinline__ uint32_t pair_geo(int rx0, int ry0, int w, int h) {

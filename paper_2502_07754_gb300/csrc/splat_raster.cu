@@ -205,12 +205,9 @@ struct SplatMem {
 
 // (14 blocks: the FP64 test's registers spill instead of halving the warps in flight; it is rare)
 template <int TILE, bool FILL>
-__global__ void __launch_bounds__(kSplatWarps * 32, 14) splat_raster_kernel(const __grid_constant__ SplatArgs a) {
-    extern __shared__ __align__(16) char smem[];
+__device__ __forceinline__ void splat_item(const SplatArgs &a, char *smem, uint32_t item) {
     using Mem = SplatMem<TILE, FILL>;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t item = blockIdx.x * kSplatWarps + warp;
-    if (item >= a.st->n_items) return;   // whole warp; nothing below synchronises the block
     Mem &S = reinterpret_cast<Mem *>(smem)[warp];
     const uint4 it = a.items[item];
     const int view = view_of_tile(a.vt, it.x);
@@ -356,12 +353,29 @@ __global__ void __launch_bounds__(kSplatWarps * 32, 14) splat_raster_kernel(cons
     }
 }
 
+template <int TILE, bool FILL, bool STRIDED>
+__global__ void __launch_bounds__(kSplatWarps * 32, 14) splat_raster_kernel(const __grid_constant__ SplatArgs a) {
+    extern __shared__ __align__(16) char smem[];
+    const uint32_t n_items = a.st->n_items;
+    uint32_t item = blockIdx.x * kSplatWarps + threadIdx.x / 32;   // (whole warps: nothing synchronises the block)
+    if (!STRIDED) {
+        if (item < n_items) splat_item<TILE, FILL>(a, smem, item);
+    } else {
+        for (; item < n_items; item += gridDim.x * kSplatWarps) {
+            splat_item<TILE, FILL>(a, smem, item);
+            __syncwarp();   // the stage is free again
+        }
+    }
+}
+
 template <int TILE, bool FILL>
 cudaError_t launch_t(const SplatArgs &sa, int64_t max_items, cudaStream_t st) {
     const size_t smem = kSplatWarps * sizeof(SplatMem<TILE, FILL>);
-    auto fn = splat_raster_kernel<TILE, FILL>;
+    const int64_t blocks = (max_items + kSplatWarps - 1) / kSplatWarps;
+    const bool strided = blocks > kItemBlocks;
+    auto fn = strided ? splat_raster_kernel<TILE, FILL, true> : splat_raster_kernel<TILE, FILL, false>;
     cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    fn<<<(unsigned)((max_items + kSplatWarps - 1) / kSplatWarps), kSplatWarps * 32, smem, st>>>(sa);
+    fn<<<(unsigned)(strided ? kStrideBlocks : blocks), kSplatWarps * 32, smem, st>>>(sa);
     return cudaGetLastError();
 }
 
