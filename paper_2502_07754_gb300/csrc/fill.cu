@@ -3,7 +3,7 @@
 // running index.  It walks the same work items as the count pass (raster.cu), whose coverage
 // masks and rectangles say which centres each pair covers.
 //
-// One warp takes one item (at most kItemFans fans of one tile), 32 pairs at a time:
+// One warp takes one item (at most kItemFans fans of one tile):
 //  1. pairs that cover no centre drop out; the others, kFillFans at a time, are staged with
 //     all lanes: one lane a fan for the centre's double-float projection, then one lane a
 //     (fan, boundary vertex) for the vertices' screen and view offsets, 1 / depth, colour and
@@ -43,7 +43,10 @@ struct FillArgs {
 };
 
 constexpr int kFillWarps = 2;    // warps (work items) per block: items differ widely in cost
-constexpr int kFillFans = 16;    // fans staged together
+// Fans staged together: many where a pair has few centres (8-pixel tiles; 16 views of 3M fans: 18.7 ms with 16,
+// 20.1 with 8), else few, for the shared memory of more warps (200k fans at 800x800: 889 us with 16, 869 with 8).
+template <int TILE>
+constexpr int kFillFans = TILE == 8 ? 16 : 8;
 
 // Words of one warp.  Arrays of one 16-byte word per fan or vertex, so that a job's loads are
 // few and its lanes, on fans in any order, spread over the banks.
@@ -52,22 +55,23 @@ struct FillMem {
     uint32_t *next;      // [TILE^2] next record of each pixel
     uint32_t *fits;      // [TILE^2 / 32] pixels whose records fit the buffer
     uint2 *ring;         // [64] jobs: fan slot | triangle << 4 | x << 8 | y << 13, record
-    uint4 *info;         // [kFillFans] first index in the packed space, first mask, rectangle, fan id
-    float4 *m;           // [kFillFans] centre position, its 1 / depth
-    float4 *P;           // [kFillFans] view position of the centre (high parts), 0
-    float4 *c;           // [kFillFans] double-float screen position of the centre (x, then y)
-    float4 *pc;          // [kFillFans] fx X_c, fy Y_c in double-float
-    float4 *zc;          // [kFillFans] Z_c in double-float, fan id (bits), 0
-    float4 *col;         // [kFillFans] the centre's colour and opacity
-    float4 *va;          // [kFillFans][K] screen offset du, dv, 1 / depth, opacity
-    float4 *vb;          // [kFillFans][K] view offset x, y in double-float
-    float4 *vc;          // [kFillFans][K] view offset z in double-float, red, green
-    float *vd;           // [kFillFans][K] blue
+    uint8_t *live;       // [kItemFans] the item's pairs that cover a centre
+    uint4 *info;         // [kFillFans<TILE>] first index in the packed space, first mask, rectangle, fan id
+    float4 *m;           // [kFillFans<TILE>] centre position, its 1 / depth
+    float4 *P;           // [kFillFans<TILE>] view position of the centre (high parts), 0
+    float4 *c;           // [kFillFans<TILE>] double-float screen position of the centre (x, then y)
+    float4 *pc;          // [kFillFans<TILE>] fx X_c, fy Y_c in double-float
+    float4 *zc;          // [kFillFans<TILE>] Z_c in double-float, fan id (bits), 0
+    float4 *col;         // [kFillFans<TILE>] the centre's colour and opacity
+    float4 *va;          // [kFillFans<TILE>][K] screen offset du, dv, 1 / depth, opacity
+    float4 *vb;          // [kFillFans<TILE>][K] view offset x, y in double-float
+    float4 *vc;          // [kFillFans<TILE>][K] view offset z in double-float, red, green
+    float *vd;           // [kFillFans<TILE>][K] blue
 };
 
 template <int TILE>
 __host__ __device__ constexpr size_t fill_warp_bytes(int K) {
-    return (size_t)TILE * TILE * 4 + 32 * 4 + 64 * 8 + (size_t)kFillFans * (7 * 16 + (size_t)K * 52);
+    return (size_t)TILE * TILE * 4 + 32 * 4 + 64 * 8 + kItemFans + (size_t)kFillFans<TILE> * (7 * 16 + (size_t)K * 52);
 }
 
 template <int TILE>
@@ -76,17 +80,18 @@ __device__ __forceinline__ FillMem<TILE> fill_mem(char *p, int K) {
     s.next = reinterpret_cast<uint32_t *>(p);
     s.fits = s.next + TILE * TILE;
     s.ring = reinterpret_cast<uint2 *>(s.fits + 32);
-    s.info = reinterpret_cast<uint4 *>(s.ring + 64);
-    s.m = reinterpret_cast<float4 *>(s.info + kFillFans);
-    s.P = s.m + kFillFans;
-    s.c = s.P + kFillFans;
-    s.pc = s.c + kFillFans;
-    s.zc = s.pc + kFillFans;
-    s.col = s.zc + kFillFans;
-    s.va = s.col + kFillFans;
-    s.vb = s.va + kFillFans * K;
-    s.vc = s.vb + kFillFans * K;
-    s.vd = reinterpret_cast<float *>(s.vc + kFillFans * K);
+    s.live = reinterpret_cast<uint8_t *>(s.ring + 64);
+    s.info = reinterpret_cast<uint4 *>(s.live + kItemFans);
+    s.m = reinterpret_cast<float4 *>(s.info + kFillFans<TILE>);
+    s.P = s.m + kFillFans<TILE>;
+    s.c = s.P + kFillFans<TILE>;
+    s.pc = s.c + kFillFans<TILE>;
+    s.zc = s.pc + kFillFans<TILE>;
+    s.col = s.zc + kFillFans<TILE>;
+    s.va = s.col + kFillFans<TILE>;
+    s.vb = s.va + kFillFans<TILE> * K;
+    s.vc = s.vb + kFillFans<TILE> * K;
+    s.vd = reinterpret_cast<float *>(s.vc + kFillFans<TILE> * K);
     return s;
 }
 
@@ -192,148 +197,153 @@ __device__ __forceinline__ void fill_item(const FillArgs &a, char *smem, uint32_
     }
     const uint32_t lt = (1u << lane) - 1u, le = 0xffffffffu >> (31 - lane);
     uint32_t head = 0, queued = 0;   // the ring
+    // the pairs that cover a pixel centre, by their place in the item
+    int n_live = 0;
     for (uint32_t cb = it.y; cb < it.z; cb += 32) {
+        const bool covers = cb + lane < it.z && __ldg(&a.pinfo[cb + lane].y) != 0u;
+        const uint32_t live = __ballot_sync(0xffffffffu, covers);
+        if (covers) S.live[n_live + __popc(live & lt)] = (uint8_t)(cb - it.y + lane);
+        n_live += __popc(live);
+    }
+    for (int l0 = 0; l0 < n_live; l0 += kFillFans<TILE>) {
+        const int nl = min(kFillFans<TILE>, n_live - l0), slot = lane;
+        const bool in = lane < nl;
+        __syncwarp();   // the list is written, the previous fans' jobs are done
         uint2 pinf = make_uint2(0u, 0u);
-        uint32_t fan = 0;
-        if (cb + lane < it.z) {
-            pinf = __ldg(a.pinfo + cb + lane);
-            fan = __ldg(a.list + cb + lane);
+        uint32_t fan = 0, excl = 0;
+        if (in) {
+            const uint32_t at = it.y + S.live[l0 + lane];
+            pinf = __ldg(a.pinfo + at);
+            fan = __ldg(a.list + at);
+            excl = (((pinf.y >> 12) & 63u) + 1u) * (((pinf.y >> 18) & 63u) + 1u);
         }
-        const uint32_t n_mine = pinf.y ? (((pinf.y >> 12) & 63u) + 1u) * (((pinf.y >> 18) & 63u) + 1u) : 0u;
-        const uint32_t live = __ballot_sync(0xffffffffu, n_mine != 0u);
-        const int rank = __popc(live & lt), n_live = __popc(live);
-        for (int l0 = 0; l0 < n_live; l0 += kFillFans) {
-            const int nl = min(kFillFans, n_live - l0), slot = rank - l0;
-            const bool in = n_mine != 0u && slot >= 0 && slot < kFillFans;
-            uint32_t excl = in ? n_mine : 0u;
+        const uint32_t n_mine = excl;
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t y = __shfl_up_sync(0xffffffffu, excl, o);
-                if (lane >= o) excl += y;
+        for (int o = 1; o < kFillFans<TILE>; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, excl, o);
+            if (lane >= o) excl += y;
+        }
+        const uint32_t total = __shfl_sync(0xffffffffu, excl, kFillFans<TILE> - 1);
+        excl -= n_mine;
+        if (in) {
+            const float *p = a.xyz + (size_t)fan * (K + 1) * 3;
+            const float m[3] = {__ldg(p), __ldg(p + 1), __ldg(p + 2)};
+            const float *col = a.rgb + (size_t)fan * (K + 1) * 3;
+            S.col[slot] = make_float4(__ldg(col), __ldg(col + 1), __ldg(col + 2),
+                                      __ldg(a.alpha + (size_t)fan * (K + 1)));
+            const CentreProj cp = project_centre(cam, m);
+            const dfl zc = df_fast_two_sum(cp.Zh, cp.Zl);
+            const dfl xf = df_mul_f(df_fast_two_sum(cp.Xh, cp.Xl), cam.fx);
+            const dfl yf = df_mul_f(df_fast_two_sum(cp.Yh, cp.Yl), cam.fy);
+            S.info[slot] = make_uint4(excl, pinf.x, pinf.y, fan);
+            S.m[slot] = make_float4(m[0], m[1], m[2], 1.0f / zc.h);
+            S.P[slot] = make_float4(cp.Xh, cp.Yh, cp.Zh, 0.0f);
+            S.c[slot] = make_float4(cp.xh, cp.xl, cp.yh, cp.yl);
+            S.pc[slot] = make_float4(xf.h, xf.l, yf.h, yf.l);
+            S.zc[slot] = make_float4(zc.h, zc.l, __uint_as_float(fan), 0.0f);
+        }
+        __syncwarp();
+        for (int i = lane; i < nl * K; i += 32) {   // one (fan, boundary vertex) a lane
+            const int f = i / K, k = i - f * K;
+            const float4 mm = S.m[f], PP = S.P[f], zz = S.zc[f];
+            const size_t v = (size_t)__float_as_uint(zz.z) * (K + 1) + 1 + k;
+            const float *pi = a.xyz + 3 * v, *col = a.rgb + 3 * v;
+            const float r = __ldg(col), g = __ldg(col + 1), b = __ldg(col + 2), al = __ldg(a.alpha + v);
+            const float m[3] = {mm.x, mm.y, mm.z};
+            const float d[3] = {__ldg(pi) - m[0], __ldg(pi + 1) - m[1], __ldg(pi + 2) - m[2]};
+            CentreProj cp;
+            cp.Xh = PP.x;
+            cp.Yh = PP.y;
+            cp.Zh = PP.z;
+            float du, dv, X, Y, Z;
+            vertex_offset(cam, cp, d, du, dv, X, Y, Z);
+            // the exact view offset e = R (b_i - c) in double-float, for the fragment depths
+            const DfVec e = df_view_offset(cam, m, pi);
+            S.va[i] = make_float4(du, dv, 1.0f / df_add(dfl{zz.x, zz.y}, e.z).h, al);
+            S.vb[i] = make_float4(e.x.h, e.x.l, e.y.h, e.y.l);
+            S.vc[i] = make_float4(e.z.h, e.z.l, r, g);
+            S.vd[i] = b;
+        }
+        __syncwarp();
+        for (uint32_t base = 0; base < total; base += 32) {
+            // the fan of each index: the fans start one after another, so an index's fan is the
+            // last one that starts at or before it
+            const int before = __popc(__ballot_sync(0xffffffffu, in && excl < base));
+            const uint32_t here = in && excl >= base && excl < base + 32 ? 1u << (excl - base) : 0u;
+            const uint32_t starts = __reduce_or_sync(0xffffffffu, here);
+            const int f = before + __popc(starts & le) - 1;
+            const uint32_t idx = base + lane;
+            uint32_t hits = 0, x = 0, y = 0, rec = 0;
+            if (idx < total) {
+                const uint4 inf = S.info[f];
+                const uint32_t local = idx - inf.x, w = ((inf.z >> 12) & 63u) + 1u;
+                // (local + 0.5) / w is at least 1/(2w) away from an integer: exact row
+                const uint32_t yy = (uint32_t)__fdividef((float)local + 0.5f, (float)w);
+                x = (inf.z & 63u) + (local - yy * w);
+                y = ((inf.z >> 6) & 63u) + yy;
+                if (inf.y != ~0u)
+                    hits = __ldg(a.masks + inf.y + local);
+                else
+                    hits = cover_direct(a.dec + (size_t)view * (size_t)a.V + (size_t)inf.w * (K + 1), K,
+                                        a.face_mask ? __ldg(a.face_mask + inf.w) : ~0u, tx0 + (int)x, ty0 + (int)y);
+                const uint32_t lp = y * TILE + x;
+                if (!all_fit && !((S.fits[lp >> 5] >> (lp & 31u)) & 1u)) hits = 0;
+                if (hits) rec = atomicAdd(&S.next[lp], (uint32_t)__popc(hits));
             }
-            const uint32_t total = __shfl_sync(0xffffffffu, excl, 31);
-            excl -= in ? n_mine : 0u;
-            __syncwarp();   // the previous fans' jobs are done
-            if (in) {
-                const float *p = a.xyz + (size_t)fan * (K + 1) * 3;
-                const float m[3] = {__ldg(p), __ldg(p + 1), __ldg(p + 2)};
-                const float *col = a.rgb + (size_t)fan * (K + 1) * 3;
-                S.col[slot] = make_float4(__ldg(col), __ldg(col + 1), __ldg(col + 2),
-                                          __ldg(a.alpha + (size_t)fan * (K + 1)));
-                const CentreProj cp = project_centre(cam, m);
-                const dfl zc = df_fast_two_sum(cp.Zh, cp.Zl);
-                const dfl xf = df_mul_f(df_fast_two_sum(cp.Xh, cp.Xl), cam.fx);
-                const dfl yf = df_mul_f(df_fast_two_sum(cp.Yh, cp.Yl), cam.fy);
-                S.info[slot] = make_uint4(excl, pinf.x, pinf.y, fan);
-                S.m[slot] = make_float4(m[0], m[1], m[2], 1.0f / zc.h);
-                S.P[slot] = make_float4(cp.Xh, cp.Yh, cp.Zh, 0.0f);
-                S.c[slot] = make_float4(cp.xh, cp.xl, cp.yh, cp.yl);
-                S.pc[slot] = make_float4(xf.h, xf.l, yf.h, yf.l);
-                S.zc[slot] = make_float4(zc.h, zc.l, __uint_as_float(fan), 0.0f);
-            }
-            __syncwarp();
-            for (int i = lane; i < nl * K; i += 32) {   // one (fan, boundary vertex) a lane
-                const int f = i / K, k = i - f * K;
-                const float4 mm = S.m[f], PP = S.P[f], zz = S.zc[f];
-                const size_t v = (size_t)__float_as_uint(zz.z) * (K + 1) + 1 + k;
-                const float *pi = a.xyz + 3 * v, *col = a.rgb + 3 * v;
-                const float r = __ldg(col), g = __ldg(col + 1), b = __ldg(col + 2), al = __ldg(a.alpha + v);
-                const float m[3] = {mm.x, mm.y, mm.z};
-                const float d[3] = {__ldg(pi) - m[0], __ldg(pi + 1) - m[1], __ldg(pi + 2) - m[2]};
-                CentreProj cp;
-                cp.Xh = PP.x;
-                cp.Yh = PP.y;
-                cp.Zh = PP.z;
-                float du, dv, X, Y, Z;
-                vertex_offset(cam, cp, d, du, dv, X, Y, Z);
-                // the exact view offset e = R (b_i - c) in double-float, for the fragment depths
-                const DfVec e = df_view_offset(cam, m, pi);
-                S.va[i] = make_float4(du, dv, 1.0f / df_add(dfl{zz.x, zz.y}, e.z).h, al);
-                S.vb[i] = make_float4(e.x.h, e.x.l, e.y.h, e.y.l);
-                S.vc[i] = make_float4(e.z.h, e.z.l, r, g);
-                S.vd[i] = b;
-            }
-            __syncwarp();
-            for (uint32_t base = 0; base < total; base += 32) {
-                // the fan of each index: the fans start one after another, so an index's fan is the
-                // last one that starts at or before it
-                const int before = __popc(__ballot_sync(0xffffffffu, in && excl < base));
-                const uint32_t here = in && excl >= base && excl < base + 32 ? 1u << (excl - base) : 0u;
-                const uint32_t starts = __reduce_or_sync(0xffffffffu, here);
-                const int f = before + __popc(starts & le) - 1;
-                const uint32_t idx = base + lane;
-                uint32_t hits = 0, x = 0, y = 0, rec = 0;
-                if (idx < total) {
-                    const uint4 inf = S.info[f];
-                    const uint32_t local = idx - inf.x, w = ((inf.z >> 12) & 63u) + 1u;
-                    // (local + 0.5) / w is at least 1/(2w) away from an integer: exact row
-                    const uint32_t yy = (uint32_t)__fdividef((float)local + 0.5f, (float)w);
-                    x = (inf.z & 63u) + (local - yy * w);
-                    y = ((inf.z >> 6) & 63u) + yy;
-                    if (inf.y != ~0u)
-                        hits = __ldg(a.masks + inf.y + local);
-                    else
-                        hits = cover_direct(a.dec + (size_t)view * (size_t)a.V + (size_t)inf.w * (K + 1), K,
-                                            a.face_mask ? __ldg(a.face_mask + inf.w) : ~0u, tx0 + (int)x, ty0 + (int)y);
-                    const uint32_t lp = y * TILE + x;
-                    if (!all_fit && !((S.fits[lp >> 5] >> (lp & 31u)) & 1u)) hits = 0;
-                    if (hits) rec = atomicAdd(&S.next[lp], (uint32_t)__popc(hits));
+            bool more;
+            do {
+                const uint32_t pend = __ballot_sync(0xffffffffu, hits != 0u);
+                if (hits) {
+                    const uint32_t j = (uint32_t)__ffs(hits) - 1u;
+                    S.ring[(head + queued + __popc(pend & lt)) & 63u] =
+                        make_uint2((uint32_t)f | j << 4 | x << 8 | y << 13, rec);
+                    hits &= hits - 1;
+                    ++rec;
                 }
-                bool more;
-                do {
-                    const uint32_t pend = __ballot_sync(0xffffffffu, hits != 0u);
-                    if (hits) {
-                        const uint32_t j = (uint32_t)__ffs(hits) - 1u;
-                        S.ring[(head + queued + __popc(pend & lt)) & 63u] =
-                            make_uint2((uint32_t)f | j << 4 | x << 8 | y << 13, rec);
-                        hits &= hits - 1;
-                        ++rec;
+                queued += __popc(pend);
+                more = __any_sync(0xffffffffu, hits != 0u);
+                __syncwarp();
+                // whole warps of jobs, and what is left once these fans' centres are done
+                while (queued >= 32u || (queued && !more && base + 32 >= total)) {
+                    const uint32_t nj = min(queued, 32u);
+                    if (lane < nj) {
+                        const uint2 job = S.ring[(head + lane) & 63u];
+                        const int jf = (int)(job.x & 15u), j = (int)((job.x >> 4) & 15u);
+                        const float pxc = (float)(tx0 + (int)((job.x >> 8) & 31u)) + 0.5f;
+                        const float pyc = (float)(ty0 + (int)((job.x >> 13) & 31u)) + 0.5f;
+                        const int vj = jf * K + j, vn = j + 1 == K ? jf * K : vj + 1;
+                        const float4 jb = S.vb[vj], jc = S.vc[vj], nb = S.vb[vn], nc = S.vc[vn];
+                        const float4 pc = S.pc[jf], zc = S.zc[jf];
+                        const DfVec e1 = {{jb.x, jb.y}, {jb.z, jb.w}, {jc.x, jc.y}};
+                        const DfVec e2 = {{nb.x, nb.y}, {nb.z, nb.w}, {nc.x, nc.y}};
+                        const dfl zf = frag_depth_df(e1, e2, dfl{pc.x, pc.y}, dfl{pc.z, pc.w}, dfl{zc.x, zc.y}, pxc,
+                                                     pyc, cam);
+                        // perspective-correct barycentrics from the accurate centre offsets
+                        const float4 c = S.c[jf], ja = S.va[vj], na = S.va[vn], cc = S.col[jf];
+                        const float izc = S.m[jf].w, izj = ja.z, izn = na.z;
+                        const float ox = __fsub_rn(c.x, pxc) + c.y;
+                        const float oy = __fsub_rn(c.z, pyc) + c.w;
+                        const float ujx = ox + ja.x, ujy = oy + ja.y;
+                        const float unx = ox + na.x, uny = oy + na.y;
+                        const float w0 = (ujx * uny - ujy * unx) * izc;
+                        const float w1 = (unx * oy - uny * ox) * izj;
+                        const float w2 = (ox * ujy - oy * ujx) * izn;
+                        const float iW = 1.0f / (w0 + w1 + w2);
+                        const float m0 = w0 * iW, m1 = w1 * iW, m2 = w2 * iW;
+                        const float al = m0 * cc.w + m1 * ja.w + m2 * na.w;
+                        const float c0 = m0 * cc.x + m1 * jc.z + m2 * nc.z;
+                        const float c1 = m0 * cc.y + m1 * jc.w + m2 * nc.w;
+                        const float c2 = m0 * cc.z + m1 * S.vd[vj] + m2 * S.vd[vn];
+                        const uint32_t tri = __float_as_uint(zc.z) * (uint32_t)K + (uint32_t)j;
+                        float4 *out = a.frags + (size_t)kRecFwd * (size_t)job.y;
+                        out[0] = make_float4(zf.h, __uint_as_float(tri), 0.0f, zf.l);
+                        out[1] = make_float4(c0, c1, c2, al);
                     }
-                    queued += __popc(pend);
-                    more = __any_sync(0xffffffffu, hits != 0u);
+                    head += nj;
+                    queued -= nj;
                     __syncwarp();
-                    // whole warps of jobs, and what is left once these fans' centres are done
-                    while (queued >= 32u || (queued && !more && base + 32 >= total)) {
-                        const uint32_t nj = min(queued, 32u);
-                        if (lane < nj) {
-                            const uint2 job = S.ring[(head + lane) & 63u];
-                            const int jf = (int)(job.x & 15u), j = (int)((job.x >> 4) & 15u);
-                            const float pxc = (float)(tx0 + (int)((job.x >> 8) & 31u)) + 0.5f;
-                            const float pyc = (float)(ty0 + (int)((job.x >> 13) & 31u)) + 0.5f;
-                            const int vj = jf * K + j, vn = j + 1 == K ? jf * K : vj + 1;
-                            const float4 jb = S.vb[vj], jc = S.vc[vj], nb = S.vb[vn], nc = S.vc[vn];
-                            const float4 pc = S.pc[jf], zc = S.zc[jf];
-                            const DfVec e1 = {{jb.x, jb.y}, {jb.z, jb.w}, {jc.x, jc.y}};
-                            const DfVec e2 = {{nb.x, nb.y}, {nb.z, nb.w}, {nc.x, nc.y}};
-                            const dfl zf = frag_depth_df(e1, e2, dfl{pc.x, pc.y}, dfl{pc.z, pc.w}, dfl{zc.x, zc.y}, pxc,
-                                                         pyc, cam);
-                            // perspective-correct barycentrics from the accurate centre offsets
-                            const float4 c = S.c[jf], ja = S.va[vj], na = S.va[vn], cc = S.col[jf];
-                            const float izc = S.m[jf].w, izj = ja.z, izn = na.z;
-                            const float ox = __fsub_rn(c.x, pxc) + c.y;
-                            const float oy = __fsub_rn(c.z, pyc) + c.w;
-                            const float ujx = ox + ja.x, ujy = oy + ja.y;
-                            const float unx = ox + na.x, uny = oy + na.y;
-                            const float w0 = (ujx * uny - ujy * unx) * izc;
-                            const float w1 = (unx * oy - uny * ox) * izj;
-                            const float w2 = (ox * ujy - oy * ujx) * izn;
-                            const float iW = 1.0f / (w0 + w1 + w2);
-                            const float m0 = w0 * iW, m1 = w1 * iW, m2 = w2 * iW;
-                            const float al = m0 * cc.w + m1 * ja.w + m2 * na.w;
-                            const float c0 = m0 * cc.x + m1 * jc.z + m2 * nc.z;
-                            const float c1 = m0 * cc.y + m1 * jc.w + m2 * nc.w;
-                            const float c2 = m0 * cc.z + m1 * S.vd[vj] + m2 * S.vd[vn];
-                            const uint32_t tri = __float_as_uint(zc.z) * (uint32_t)K + (uint32_t)j;
-                            float4 *out = a.frags + (size_t)kRecFwd * (size_t)job.y;
-                            out[0] = make_float4(zf.h, __uint_as_float(tri), 0.0f, zf.l);
-                            out[1] = make_float4(c0, c1, c2, al);
-                        }
-                        head += nj;
-                        queued -= nj;
-                        __syncwarp();
-                    }
-                } while (more);
-            }
+                }
+            } while (more);
         }
     }
 }
