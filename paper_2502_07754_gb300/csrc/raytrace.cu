@@ -41,6 +41,9 @@ constexpr int kBvhThreads = 256;
 constexpr int kTraceThreads = 64;
 constexpr int kTraceKB = 8;
 constexpr int kStack = 64;
+constexpr int kWalkShare = 1;   // a warp leaves the tree when at most this many of its lanes walk for each that waits
+constexpr int kTraceBlocks = 10;   // blocks an SM with shadows (6, 8, 12: within 5%)
+
 constexpr double kSegEps = 1e-9;
 
 // An internal node holds its children's boxes (low corner, high corner), so a traversal step waits
@@ -257,10 +260,11 @@ struct TraceArgs {
     const BvhNode *nodes;
     const int *leaf_tri;
     CamDev cam;
-    double L[3];
+    float Lf[3];       // the light
     int shadows;
     double ambient;
     double T_eps;
+    float T_epsf;      // the same
     float bg[3];
     float *out;
     unsigned *overflow;   // traversal stack overflows (status)
@@ -442,6 +446,10 @@ __device__ __forceinline__ NodeW load_node(const BvhNode *nodes, int node) {
     return w;
 }
 
+// 1 / d, finite: a side that holds the whole ray (0 / 0 otherwise) is then met at t = 0 only, which may
+// lose the box but no crossing, as the sides lie at least 16 roundings outside the triangles.
+__device__ __forceinline__ float finite_rcp(float d) { return fminf(fmaxf(1.0f / d, -3.0e38f), 3.0e38f); }
+
 // Slab test of the ray o + t d against a box (binary32, widened): whether it meets [t0, t1],
 // and where (tn, tf).
 __device__ __forceinline__ bool box_span(float lx, float ly, float lz, float hx, float hy, float hz, const float o[3],
@@ -450,9 +458,8 @@ __device__ __forceinline__ bool box_span(float lx, float ly, float lz, float hx,
 #pragma unroll
     for (int r = 0; r < 3; ++r) {
         const float x = (lo[r] - o[r]) * id[r], y = (hi[r] - o[r]) * id[r];
-        // (0 * inf, a ray in the plane of a side, does not bound the interval)
-        t0 = fmaxf(t0, x == x && y == y ? fminf(x, y) : -3.0e38f);
-        t1 = fminf(t1, x == x && y == y ? fmaxf(x, y) : 3.0e38f);
+        t0 = fmaxf(t0, fminf(x, y));
+        t1 = fminf(t1, fmaxf(x, y));
     }
     tn = t0;
     tf = t1;
@@ -476,82 +483,160 @@ __device__ __forceinline__ dfl bary_mix(dfl u, dfl v, float a0, float a1, float 
     return df_add_fast(df_add_fast(df_mul_f(w, a0), df_mul_f(u, a1)), df_mul_f(v, a2));
 }
 
+// A warp's ring of triangles that passed the filter, and what the double-float test made of 32.
+struct WarpRing {
+    uint2 job[64];            // (lane or segment slot, triangle)
+    float2 t[32], u[32], v[32];
+    unsigned mine[32];        // per lane of the warp: its crossings among the 32
+};
+struct Block {
+    WarpRing ring[kTraceThreads / 32];
+    float2 d[3][kTraceThreads];      // the pixels' ray directions
+    float after[kTraceThreads];      // the last composited crossing
+};
 // Shadow segments of one block's crossings of one pass, a slot per (crossing, pixel).
 constexpr int kJobs = kTraceKB * kTraceThreads;
 struct Jobs {
-    float2 o[3][kJobs], d[3][kJobs];   // origin and vector to the light; o[0] takes the transmittance
+    float2 o[3][kJobs];                // origin (the segment runs to the light)
+    float2 S[kJobs];                   // transmittance
     int tri[kJobs];                    // the crossing's own triangle
     uint16_t list[kJobs];              // slots in use
     int n, next;
 };
 
+__device__ __forceinline__ void segment(const TraceArgs &a, const Jobs &J, int slot, RayF &rf) {
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+        const float2 o = J.o[r][slot];
+        rf.o[r] = dfl{o.x, o.y};
+        rf.d[r] = df_add_f(df_neg(rf.o[r]), a.Lf[r]);
+    }
+}
+
 // Transmittance of the block's segments through every triangle but their own.  A lane that is done
-// takes the next segment of the list, so no lane waits for the longest of 32.
-__device__ __forceinline__ void shadow_jobs(const TraceArgs &a, Jobs &J) {
+// takes the next segment of the list, so no lane waits for the longest of 32; what passes the filter (one
+// triangle in eight) goes into a ring, and the warp takes 32 of them through the double-float test at
+// once (a lane on its own took it with 3 of 32 lanes: 118 -> 46 ms for the 5.4M segments below).
+__device__ __forceinline__ void shadow_jobs(const TraceArgs &a, Jobs &J, WarpRing &R) {
     const int n1 = (int)(a.T - 1);   // nodes from n1 on are leaves
     const float t0 = -1e-3f, t1 = 1.001f;
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
     int stack[kStack];
-    int sp = 0, node = -1, slot = -1, own = -1;
+    int sp = 0, node = -1, slot = 0, own = -1;
     RayF rf;
     float of[3], id[3];
-    dfl S = df_make(1.0f);
+    bool live = true;                // has a segment, or may find one
+    uint32_t head = 0, queued = 0;   // the ring
     for (;;) {
-        if (node < 0) {
-            if (slot >= 0) J.o[0][slot] = make_float2(S.h, S.l);
+        if (live && node < 0) {
             const int j = atomicAdd(&J.next, 1);
-            if (j >= J.n) break;
-            slot = J.list[j];
-            own = J.tri[slot];
+            live = j < J.n;
+            if (live) {
+                slot = J.list[j];
+                own = J.tri[slot];
+                segment(a, J, slot, rf);
 #pragma unroll
-            for (int r = 0; r < 3; ++r) {
-                const float2 o = J.o[r][slot], d = J.d[r][slot];
-                rf.o[r] = dfl{o.x, o.y};
-                rf.d[r] = dfl{d.x, d.y};
-                of[r] = o.x;
-                id[r] = 1.0f / d.x;
+                for (int r = 0; r < 3; ++r) {
+                    of[r] = rf.o[r].h;
+                    id[r] = finite_rcp(rf.d[r].h);
+                }
+                J.S[slot] = make_float2(1.0f, 0.0f);
+                sp = 0;
+                node = 0;
             }
-            S = df_make(1.0f);
-            sp = 0;
-            node = 0;
         }
-        while (node >= 0 && node < n1) {
-            const NodeW w = load_node(a.nodes, node);
-            float tn, tf;
-            const bool hl = left_span(w, of, id, t0, t1, tn, tf), hr = right_span(w, of, id, t0, t1, tn, tf);
-            if (hl && hr) {
-                if (sp < kStack) stack[sp++] = w.right;
-                else atomicAdd(a.overflow, 1u);
+        // down the tree, until most lanes wait (at a leaf, or for a segment)
+        for (;;) {
+            const bool inner = node >= 0 && node < n1;
+            const unsigned m = __ballot_sync(0xffffffffu, inner), w = __ballot_sync(0xffffffffu, !inner && live);
+            if (m == 0 || __popc(m) <= kWalkShare * __popc(w)) break;
+            if (inner) {
+                const NodeW nd = load_node(a.nodes, node);
+                float tn, tf;
+                const bool hl = left_span(nd, of, id, t0, t1, tn, tf), hr = right_span(nd, of, id, t0, t1, tn, tf);
+                if (hl && hr) {
+                    if (sp < kStack) stack[sp++] = nd.right;
+                    else atomicAdd(a.overflow, 1u);
+                }
+                node = hl ? nd.left : (hr ? nd.right : (sp > 0 ? stack[--sp] : -1));
             }
-            node = hl ? w.left : (hr ? w.right : (sp > 0 ? stack[--sp] : -1));
         }
-        if (node < 0) continue;
-        const int tri = __ldg(a.leaf_tri + (node - n1));
-        node = sp > 0 ? stack[--sp] : -1;
-        if (tri == own) continue;
-        float P[3][3];
-        tri_f(a, tri, P);
-        Hit h;
-        if (!crosses(rf, P, (float)kSegEps, (float)(1.0 - kSegEps), kSegEps, 1.0 - kSegEps, h)) continue;
-        int64_t v[3];
-        tri_verts(a.tris, a.K, tri, v);
-        const dfl al = bary_mix(h.u, h.v, __ldg(a.alpha + v[0]), __ldg(a.alpha + v[1]), __ldg(a.alpha + v[2]));
-        S = df_mul(S, df_add_f(df_neg(al), 1.0f));
-        // the light is blocked to within T_eps: the colour's shadow factor moves by at
-        // most (1 - ambient) T_eps, the primary composite's own termination bound
-        if (to_double(S) < a.T_eps) node = -1;
+        bool pass = false;
+        int tri = -1;
+        if (node >= n1) {
+            tri = __ldg(a.leaf_tri + (node - n1));
+            node = sp > 0 ? stack[--sp] : -1;
+            if (tri != own) {
+                float P[3][3];
+                tri_f(a, tri, P);
+                MtBounds e;
+                pass = mt_may_hit(rf, P[0], P[1], P[2], (float)kSegEps, (float)(1.0 - kSegEps), e);
+            }
+        }
+        const unsigned c = __ballot_sync(0xffffffffu, pass);
+        if (pass) R.job[(head + queued + __popc(c & lt)) & 63u] = make_uint2((uint32_t)slot, (uint32_t)tri);
+        queued += __popc(c);
+        const bool more = __any_sync(0xffffffffu, live);
+        __syncwarp();
+        if (queued >= 32u || !more) {
+            while (queued >= 32u || (!more && queued)) {
+                const uint32_t nj = min(queued, 32u);
+                int at = -1;
+                if (lane < nj) {
+                    const uint2 job = R.job[(head + lane) & 63u];
+                    RayF jr;
+                    segment(a, J, (int)job.x, jr);
+                    float P[3][3];
+                    tri_f(a, (int)job.y, P);
+                    Hit h;
+                    if (crosses(jr, P, (float)kSegEps, (float)(1.0 - kSegEps), kSegEps, 1.0 - kSegEps, h)) {
+                        int64_t v[3];
+                        tri_verts(a.tris, a.K, (int)job.y, v);
+                        const dfl al = bary_mix(h.u, h.v, __ldg(a.alpha + v[0]), __ldg(a.alpha + v[1]), __ldg(a.alpha + v[2]));
+                        const dfl f = df_add_f(df_neg(al), 1.0f);
+                        R.t[lane] = make_float2(f.h, f.l);
+                        at = (int)job.x;
+                    }
+                }
+                head += nj;
+                queued -= nj;
+                // a segment's factors in the order it met them, by the first of their lanes
+                unsigned same = __match_any_sync(0xffffffffu, at);
+                __syncwarp();
+                if (at >= 0 && lane == __ffs(same) - 1) {
+                    dfl S = dfl{J.S[at].x, J.S[at].y};
+                    for (; same; same &= same - 1) {
+                        const float2 f = R.t[__ffs(same) - 1];
+                        S = df_mul(S, dfl{f.x, f.y});
+                    }
+                    J.S[at] = make_float2(S.h, S.l);
+                }
+                __syncwarp();
+            }
+            // the light is blocked to within T_eps: the colour's shadow factor moves by at
+            // most (1 - ambient) T_eps, the primary composite's own termination bound
+            if (node >= 0 && J.S[slot].x < a.T_epsf) node = -1;
+        }
+        if (!more) break;
     }
 }
 
 // One thread a pixel, a block an 8 x 8 tile of pixels (a warp 8 x 4), so that a warp's rays stay
 // together down the tree.  With shadows a block gathers its pixels' next crossings, traces all their
-// segments to the light as one list, and composites.  What bounds it: the waits on nodes and triangles and the
-// lanes that part ways (a segment meets 187 nodes and 60 leaves on its own).  1.6M triangles with shadows at
-// 800x800, 5.4M segments: 148 ms, against 218 ms for a thread that traced its own pixel's segments one
-// after the other, over nodes that held their own box (two loads a child).
+// segments to the light as one list, and composites.  What bounds it: the waits on nodes, at 9 to 16 warps an
+// SM, and lanes at different depths of the tree (18 of 32 active; a segment meets 187 nodes and 60 leaves).
+// 1.6M triangles at 800x800: 8.6 ms without shadows, 62 ms with the 5.4M segments, against 41 and 148 ms
+// for lanes that each took their triangles through the exact tests alone (4.5 of 32 active), and 218 ms
+// for a thread that also traced its own pixel's segments one after the other.
 template <bool SHADOWS>
-__global__ void __launch_bounds__(kTraceThreads) trace_kernel(const __grid_constant__ TraceArgs a) {
+__global__ void __launch_bounds__(kTraceThreads, SHADOWS ? kTraceBlocks : 0) trace_kernel(const __grid_constant__ TraceArgs a) {
     extern __shared__ __align__(16) char smem[];
-    Jobs &J = *reinterpret_cast<Jobs *>(smem);
+    Block &B = *reinterpret_cast<Block *>(smem);
+    Jobs &J = *reinterpret_cast<Jobs *>(smem + sizeof(Block));   // (with SHADOWS)
+    WarpRing &R = B.ring[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31, warp0 = threadIdx.x & ~31;
+    const unsigned lt = (1u << lane) - 1u;
     const int W = a.cam.width, H = a.cam.height;
     const int px = blockIdx.x * 8 + (threadIdx.x & 7), py = blockIdx.y * 8 + (threadIdx.x >> 3);
     const bool in = px < W && py < H;
@@ -567,7 +652,8 @@ __global__ void __launch_bounds__(kTraceThreads) trace_kernel(const __grid_const
             rf.o[r] = df_make(c.C[r]);
             rf.d[r] = df_of(((double)c.R[r] * dc[0] + (double)c.R[3 + r] * dc[1]) + (double)c.R[6 + r] * dc[2]);
             of[r] = rf.o[r].h;
-            id[r] = 1.0f / rf.d[r].h;
+            id[r] = finite_rcp(rf.d[r].h);
+            B.d[r][threadIdx.x] = make_float2(rf.d[r].h, rf.d[r].l);
         }
     }
     const int n1 = (int)(a.T - 1);   // nodes from n1 on are leaves
@@ -579,63 +665,117 @@ __global__ void __launch_bounds__(kTraceThreads) trace_kernel(const __grid_const
         Hit buf[kTraceKB];
         int nb = 0;
         bool more = false;
-        if (alive) {
-            int stack[kStack];
-            int sp = 0, node = 0;
-            // Boxes wholly before the last composited crossing hold nothing for this pass, and
-            // boxes wholly beyond the farthest kept crossing of a full buffer only mean another
-            // pass; both bounds are widened by 1e-5 relative, far above the slab test's rounding.
-            const float t_after = after_t.h > 0.0f ? after_t.h * (1.0f - 1e-5f) : 0.0f;
-            const float t_near = c.znear * 0.999f;
+        // The warp's pixels walk the tree together, as the segments do (shadow_jobs): triangles that
+        // pass the filter wait in the ring for the double-float test of 32, and each lane sorts its
+        // own crossings of these into its buffer.
+        int stack[kStack];
+        int sp = 0, node = alive ? 0 : -1;
+        uint32_t head = 0, queued = 0;
+        B.after[threadIdx.x] = after_t.h;
+        // Boxes wholly before the last composited crossing hold nothing for this pass, and
+        // boxes wholly beyond the farthest kept crossing of a full buffer only mean another
+        // pass; both bounds are widened by 1e-5 relative, far above the slab test's rounding.
+        const float t_after = after_t.h > 0.0f ? after_t.h * (1.0f - 1e-5f) : 0.0f;
+        const float t_near = c.znear * 0.999f;
+        for (;;) {
             for (;;) {
-                while (node >= 0 && node < n1) {
-                    const NodeW w = load_node(a.nodes, node);
-                    float nl, fl, nr, fr;
-                    bool hl = left_span(w, of, id, t_near, 3.0e38f, nl, fl) && fl >= t_after;
-                    bool hr = right_span(w, of, id, t_near, 3.0e38f, nr, fr) && fr >= t_after;
-                    if (nb == kTraceKB) {
-                        const float t_far = buf[kTraceKB - 1].t.h * (1.0f + 1e-5f);
-                        if (hl && nl > t_far) {
-                            hl = false;
-                            more = true;
-                        }
-                        if (hr && nr > t_far) {
-                            hr = false;
-                            more = true;
-                        }
+                const bool inner = node >= 0 && node < n1;
+                const unsigned m = __ballot_sync(0xffffffffu, inner), w = __ballot_sync(0xffffffffu, node >= n1);
+                if (m == 0 || __popc(m) <= kWalkShare * __popc(w)) break;
+                if (!inner) continue;
+                const NodeW nd = load_node(a.nodes, node);
+                float nl, fl, nr, fr;
+                bool hl = left_span(nd, of, id, t_near, 3.0e38f, nl, fl) && fl >= t_after;
+                bool hr = right_span(nd, of, id, t_near, 3.0e38f, nr, fr) && fr >= t_after;
+                if (nb == kTraceKB) {
+                    const float t_far = buf[kTraceKB - 1].t.h * (1.0f + 1e-5f);
+                    if (hl && nl > t_far) {
+                        hl = false;
+                        more = true;
                     }
-                    // the nearer child first: the buffer fills with near crossings early
-                    const bool swap = hl && hr && nr < nl;
-                    const int first = swap || !hl ? w.right : w.left, second = swap ? w.left : w.right;
-                    if (hl && hr) {
-                        if (sp < kStack) stack[sp++] = second;
-                        else atomicAdd(a.overflow, 1u);
+                    if (hr && nr > t_far) {
+                        hr = false;
+                        more = true;
                     }
-                    node = hl || hr ? first : (sp > 0 ? stack[--sp] : -1);
                 }
-                if (node < 0) break;
-                const int tri = __ldg(a.leaf_tri + (node - n1));
+                // the nearer child first: the buffer fills with near crossings early
+                const bool swap = hl && hr && nr < nl;
+                const int first = swap || !hl ? nd.right : nd.left, second = swap ? nd.left : nd.right;
+                if (hl && hr) {
+                    if (sp < kStack) stack[sp++] = second;
+                    else atomicAdd(a.overflow, 1u);
+                }
+                node = hl || hr ? first : (sp > 0 ? stack[--sp] : -1);
+            }
+            bool pass = false;
+            int tri = -1;
+            if (node >= n1) {
+                tri = __ldg(a.leaf_tri + (node - n1));
                 node = sp > 0 ? stack[--sp] : -1;
                 float P[3][3];
                 tri_f(a, tri, P);
-                Hit h;
-                // crossings before the last composited one were taken in an earlier pass
-                if (!crosses(rf, P, fmaxf(c.znear, after_t.h), 3.0e38f, (double)c.znear, 1.0e300, h)) continue;
-                h.tri = tri;
-                if (!hit_less(after_t, after_i, h.t, tri)) continue;   // composited in an earlier pass
-                if (nb == kTraceKB) {
-                    more = true;
-                    if (!hit_less(h.t, tri, buf[kTraceKB - 1].t, buf[kTraceKB - 1].tri)) continue;
-                    --nb;   // the farthest kept crossing waits for a later pass
-                }
-                int s = nb;
-                while (s > 0 && hit_less(h.t, tri, buf[s - 1].t, buf[s - 1].tri)) {
-                    buf[s] = buf[s - 1];
-                    --s;
-                }
-                buf[s] = h;
-                ++nb;
+                MtBounds e;
+                pass = mt_may_hit(rf, P[0], P[1], P[2], fmaxf(c.znear, after_t.h), 3.0e38f, e);
             }
+            const unsigned cand = __ballot_sync(0xffffffffu, pass);
+            if (pass) R.job[(head + queued + __popc(cand & lt)) & 63u] = make_uint2((uint32_t)lane, (uint32_t)tri);
+            queued += __popc(cand);
+            const bool walking = __any_sync(0xffffffffu, node >= 0);
+            __syncwarp();
+            while (queued >= 32u || (!walking && queued)) {
+                const uint32_t nj = min(queued, 32u);
+                int owner = -1;
+                if (lane < nj) {
+                    const uint2 job = R.job[(head + lane) & 63u];
+                    const int at = warp0 + (int)job.x;
+                    RayF jr;
+#pragma unroll
+                    for (int r = 0; r < 3; ++r) {
+                        jr.o[r] = df_make(c.C[r]);
+                        jr.d[r] = dfl{B.d[r][at].x, B.d[r][at].y};
+                    }
+                    float P[3][3];
+                    tri_f(a, (int)job.y, P);
+                    Hit h;
+                    // crossings before the last composited one were taken in an earlier pass
+                    if (crosses(jr, P, fmaxf(c.znear, B.after[at]), 3.0e38f, (double)c.znear, 1.0e300, h)) {
+                        owner = (int)job.x;
+                        R.t[lane] = make_float2(h.t.h, h.t.l);
+                        R.u[lane] = make_float2(h.u.h, h.u.l);
+                        R.v[lane] = make_float2(h.v.h, h.v.l);
+                    }
+                }
+                R.mine[lane] = 0;
+                const unsigned same = __match_any_sync(0xffffffffu, owner);
+                __syncwarp();
+                if (owner >= 0 && lane == __ffs(same) - 1) R.mine[owner] = same;
+                __syncwarp();
+                for (unsigned b = R.mine[lane]; b; b &= b - 1) {
+                    const int i = __ffs(b) - 1;
+                    Hit h;
+                    h.t = dfl{R.t[i].x, R.t[i].y};
+                    h.u = dfl{R.u[i].x, R.u[i].y};
+                    h.v = dfl{R.v[i].x, R.v[i].y};
+                    h.tri = (int)R.job[(head + i) & 63u].y;
+                    if (!hit_less(after_t, after_i, h.t, h.tri)) continue;   // composited in an earlier pass
+                    if (nb == kTraceKB) {
+                        more = true;
+                        if (!hit_less(h.t, h.tri, buf[kTraceKB - 1].t, buf[kTraceKB - 1].tri)) continue;
+                        --nb;   // the farthest kept crossing waits for a later pass
+                    }
+                    int s = nb;
+                    while (s > 0 && hit_less(h.t, h.tri, buf[s - 1].t, buf[s - 1].tri)) {
+                        buf[s] = buf[s - 1];
+                        --s;
+                    }
+                    buf[s] = h;
+                    ++nb;
+                }
+                __syncwarp();
+                head += nj;
+                queued -= nj;
+            }
+            if (!walking) break;
         }
         // the crossings that will be composited
         int n_use = 0;
@@ -665,15 +805,13 @@ __global__ void __launch_bounds__(kTraceThreads) trace_kernel(const __grid_const
                     J.tri[slot] = buf[k].tri;
 #pragma unroll
                     for (int r = 0; r < 3; ++r) {
-                        const double p = to_double(rf.o[r]) + t * to_double(rf.d[r]);
-                        const dfl pf = df_of(p), df = df_of(a.L[r] - p);
+                        const dfl pf = df_of(to_double(rf.o[r]) + t * to_double(rf.d[r]));
                         J.o[r][slot] = make_float2(pf.h, pf.l);
-                        J.d[r][slot] = make_float2(df.h, df.l);
                     }
                 }
             }
             __syncthreads();
-            shadow_jobs(a, J);
+            shadow_jobs(a, J, R);
             __syncthreads();
         }
         for (int k = 0; k < n_use; ++k) {
@@ -687,7 +825,7 @@ __global__ void __launch_bounds__(kTraceThreads) trace_kernel(const __grid_const
                 col[r] = to_double(bary_mix(h.u, h.v, __ldg(a.rgb + 3 * v[0] + r), __ldg(a.rgb + 3 * v[1] + r),
                                             __ldg(a.rgb + 3 * v[2] + r)));
             if (SHADOWS) {
-                const float2 S = J.o[0][k * kTraceThreads + threadIdx.x];
+                const float2 S = J.S[k * kTraceThreads + threadIdx.x];
                 const double f = a.ambient + (1.0 - a.ambient) * to_double(dfl{S.x, S.y});
 #pragma unroll
                 for (int r = 0; r < 3; ++r) col[r] *= f;
@@ -700,7 +838,7 @@ __global__ void __launch_bounds__(kTraceThreads) trace_kernel(const __grid_const
             after_i = h.tri;
         }
         alive = alive && more && !(T < a.T_eps);
-        if (SHADOWS ? !__syncthreads_or(alive) : !alive) break;
+        if (SHADOWS ? !__syncthreads_or(alive) : !__any_sync(0xffffffffu, alive)) break;
     }
     if (!in) return;
     float4 *out = reinterpret_cast<float4 *>(a.out);
@@ -784,17 +922,17 @@ extern "C" MS_API ms_status ms_raytrace(const float *xyz, const float *rgb, cons
     a.cam = make_cam(*cam);
     a.shadows = light != nullptr && ambient < 1.0f;
     for (int r = 0; r < 3; ++r) {
-        a.L[r] = light ? (double)light[r] : 0.0;
+        a.Lf[r] = light ? light[r] : 0.0f;
         a.bg[r] = bg ? bg[r] : 0.0f;
     }
     a.ambient = ambient;
-    a.T_eps = T_eps;
+    a.T_eps = a.T_epsf = T_eps;
     a.out = out_rgba;
     const dim3 grid((cam->width + 7) / 8, (cam->height + 7) / 8);
     if (a.shadows)
-        trace_kernel<true><<<grid, kTraceThreads, sizeof(Jobs), (cudaStream_t)stream>>>(a);
+        trace_kernel<true><<<grid, kTraceThreads, sizeof(Block) + sizeof(Jobs), (cudaStream_t)stream>>>(a);
     else
-        trace_kernel<false><<<grid, kTraceThreads, 0, (cudaStream_t)stream>>>(a);
+        trace_kernel<false><<<grid, kTraceThreads, sizeof(Block), (cudaStream_t)stream>>>(a);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return set_error(MS_ERR_CUDA, "trace_kernel: %s", cudaGetErrorString(e));
     count_launches(1);
