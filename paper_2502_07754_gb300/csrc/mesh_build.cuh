@@ -113,9 +113,8 @@ __device__ __forceinline__ void block_store(float *dst, const float *src, int n)
 struct Frame {
     float m[3], ax[3][3], col[3], sig;
 };
-template <int DEG, bool BF16, bool THREE>
-__device__ __forceinline__ Frame gaussian_frame(const Gaussians &G, const MeshBuildConst &kc, int64_t g) {
-    Frame F;
+template <bool THREE>
+__device__ __forceinline__ void frame_geometry(const Gaussians &G, const MeshBuildConst &kc, int64_t g, Frame &F) {
     F.m[0] = __ldg(G.means + 3 * g);
     F.m[1] = __ldg(G.means + 3 * g + 1);
     F.m[2] = __ldg(G.means + 3 * g + 2);
@@ -150,10 +149,15 @@ __device__ __forceinline__ Frame gaussian_frame(const Gaussians &G, const MeshBu
             F.ax[2][r] = 0.0f;
         }
     }
+}
+// Colour of Gaussian g at m, one for all of its vertices.
+template <int DEG, bool BF16>
+__device__ __forceinline__ void frame_colour(const Gaussians &G, const MeshBuildConst &kc, int64_t g, const float m[3],
+                                             float col[3]) {
     constexpr int NB = (DEG + 1) * (DEG + 1);
     float Y[NB];
     int nuse = 1;
-    float dx = F.m[0] - kc.cc[0], dy = F.m[1] - kc.cc[1], dz = F.m[2] - kc.cc[2];
+    float dx = m[0] - kc.cc[0], dy = m[1] - kc.cc[1], dz = m[2] - kc.cc[2];
     float dn = dx * dx + dy * dy + dz * dz;
     if (DEG > 0 && kc.has_cam && dn > 0.0f) {
         float inv = rsqrtf(dn);
@@ -162,21 +166,23 @@ __device__ __forceinline__ Frame gaussian_frame(const Gaussians &G, const MeshBu
     } else {
         Y[0] = kc.shc[0];
     }
-    sh_colour<DEG, BF16>(G.sh, g, kc.sh_vec_ok, Y, nuse, F.col);   // one per Gaussian, inherited by its vertices
+    sh_colour<DEG, BF16>(G.sh, g, kc.sh_vec_ok, Y, nuse, col);
+}
+template <int DEG, bool BF16, bool THREE>
+__device__ __forceinline__ Frame gaussian_frame(const Gaussians &G, const MeshBuildConst &kc, int64_t g) {
+    Frame F;
+    frame_geometry<THREE>(G, kc, g, F);
+    frame_colour<DEG, BF16>(G, kc, g, F.m, F.col);
     return F;
 }
 
-// Converts Gaussian g into staging vertices lv .. lv + K (s_xyz, s_rgb: 3 floats per
-// vertex; s_a: one) of a flat fan.  cr: the 2(K+1) corrections of g (radial dr_0..dr_K, then
-// log-opacity do_0..do_K): boundary vertex i goes to
-// m + (1 + dr_i)(cos th_i a + sin th_i b) and alpha_i to clamp(alpha_i exp(do_i), 0, 1).
-template <int DEG, bool BF16>
-__device__ __forceinline__ void convert_gaussian(const Gaussians &G, const MeshBuildConst &kc, int64_t g,
-                                                 const float *cr, float *s_xyz, float *s_rgb, float *s_a,
-                                                 int lv) {
+// Places a flat fan's staging vertices lv .. lv + K (s_xyz: 3 floats per vertex; s_a: one).
+// cr: the 2(K+1) corrections (radial dr_0..dr_K, then log-opacity do_0..do_K): boundary vertex i
+// goes to m + (1 + dr_i)(cos th_i a + sin th_i b) and alpha_i to clamp(alpha_i exp(do_i), 0, 1).
+__device__ __forceinline__ void place_corrected(const Frame &F, const MeshBuildConst &kc, const float *cr, float *s_xyz,
+                                                float *s_a, int lv) {
     const int KV = kc.K + 1;
-    const Frame F = gaussian_frame<DEG, BF16, false>(G, kc, g);
-    const float *m = F.m, *a = F.ax[0], *b = F.ax[1], *col = F.col;
+    const float *m = F.m, *a = F.ax[0], *b = F.ax[1];
     const float sig = F.sig;
     for (int k = 0; k < KV; ++k) {
         float p[3];
@@ -191,12 +197,21 @@ __device__ __forceinline__ void convert_gaussian(const Gaussians &G, const MeshB
         float op = k == 0 ? sig : kc.opac_mul * sig;
         op = fminf(fmaxf(op * expf(cr[KV + k]), 0.0f), 1.0f);
 #pragma unroll
-        for (int r = 0; r < 3; ++r) {
-            s_xyz[3 * (lv + k) + r] = p[r];
-            s_rgb[3 * (lv + k) + r] = col[r];
-        }
+        for (int r = 0; r < 3; ++r) s_xyz[3 * (lv + k) + r] = p[r];
         s_a[lv + k] = op;
     }
+}
+
+// Converts Gaussian g into staging vertices lv .. lv + K (s_rgb: 3 floats per vertex).
+template <int DEG, bool BF16>
+__device__ __forceinline__ void convert_gaussian(const Gaussians &G, const MeshBuildConst &kc, int64_t g,
+                                                 const float *cr, float *s_xyz, float *s_rgb, float *s_a,
+                                                 int lv) {
+    const Frame F = gaussian_frame<DEG, BF16, false>(G, kc, g);
+    place_corrected(F, kc, cr, s_xyz, s_a, lv);
+    for (int i = 3 * lv; i < 3 * (lv + kc.K + 1); i += 3)
+#pragma unroll
+        for (int r = 0; r < 3; ++r) s_rgb[i + r] = F.col[r];
 }
 
 }  // namespace mb

@@ -400,6 +400,13 @@ __global__ void __launch_bounds__(kFwdThreads, 1) mlp_fwd_kernel(const MlpSrc s,
         gelu_cols64(tz, H, r, c0);   // the product has read H1: H2 replaces it
         slot_sync_then(slot, issuer);
         if (issuer) issue(tz0, H, W3, kHid, kOutPad, false, mbar);
+        // the colour needs no product: the row's other thread forms it meanwhile (3M Gaussians 680 -> 671 us;
+        // with the fan's axes formed early and the next features moved as well, registers spill: 738 us)
+        float col[3];
+        if (FUSED && !row_owner && g < N) {
+            const float m[3] = {__ldg(out.G.means + 3 * g), __ldg(out.G.means + 3 * g + 1), __ldg(out.G.means + 3 * g + 2)};
+            mb::frame_colour<DEG, BF16>(out.G, out.kc, g, m, col);
+        }
         ok = wait_mma(mbar, phase, timeouts, issuer) && ok;
         float y[32];
         if (row_owner) {
@@ -423,8 +430,18 @@ __global__ void __launch_bounds__(kFwdThreads, 1) mlp_fwd_kernel(const MlpSrc s,
             for (int r0 = 0; r0 < nloc; r0 += per_chunk) {
                 const int nc = min(per_chunk, nloc - r0);
                 float *s_xyz = stg, *s_rgb = stg + 3 * nc * KV, *s_a = stg + 6 * nc * KV;
-                if (row_owner && r >= r0 && r < r0 + nc)
-                    mb::convert_gaussian<DEG, BF16>(out.G, out.kc, g, y, s_xyz, s_rgb, s_a, (r - r0) * KV);
+                if (r >= r0 && r < r0 + nc) {
+                    const int lv = (r - r0) * KV;
+                    if (row_owner) {
+                        mb::Frame F;
+                        mb::frame_geometry<false>(out.G, out.kc, g, F);
+                        mb::place_corrected(F, out.kc, y, s_xyz, s_a, lv);
+                    } else {
+                        for (int i = 3 * lv; i < 3 * (lv + KV); i += 3)
+#pragma unroll
+                            for (int ch = 0; ch < 3; ++ch) s_rgb[i + ch] = col[ch];
+                    }
+                }
                 slot_sync(slot);
                 const int64_t v0 = (g0 + r0) * KV;
                 slot_store(out.xyz + 3 * v0, s_xyz, 3 * nc * KV, st);
