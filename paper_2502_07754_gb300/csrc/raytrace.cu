@@ -38,11 +38,16 @@ namespace ms {
 namespace {
 
 constexpr int kBvhThreads = 256;
-constexpr int kTraceThreads = 64;
-constexpr int kTraceKB = 8;
+constexpr int kTracePix = 32;      // pixels a block (8 x 4, one warp)
+constexpr int kTraceWarps = 4;     // and the warps that trace their segments to the light
+constexpr int kPlainWarps = 2;     // without shadows: warps of 8 x 4 pixels a block
+// Crossings that a pass keeps (1.6M triangles at 800x800: 8, 16, 24, 32 take 45, 39, 42, 43 ms with
+// shadows and 8.7, 6.9, 5.9, 6.1 ms without).
+template <bool SHADOWS>
+constexpr int kTraceKB = SHADOWS ? 16 : 24;
 constexpr int kStack = 64;
 constexpr int kWalkShare = 1;   // a warp leaves the tree when at most this many of its lanes walk for each that waits
-constexpr int kTraceBlocks = 10;   // blocks an SM with shadows (6, 8, 12: within 5%)
+constexpr int kTraceBlocks = 5;    // blocks an SM with shadows
 
 constexpr double kSegEps = 1e-9;
 
@@ -490,12 +495,12 @@ struct WarpRing {
     unsigned mine[32];        // per lane of the warp: its crossings among the 32
 };
 struct Block {
-    WarpRing ring[kTraceThreads / 32];
-    float2 d[3][kTraceThreads];      // the pixels' ray directions
-    float after[kTraceThreads];      // the last composited crossing
+    float2 d[3][kTracePix];      // the pixels' ray directions
+    float after[kTracePix];      // the last composited crossing
 };
+static_assert(sizeof(Block) % 16 == 0 && sizeof(WarpRing) % 16 == 0, "shared memory alignment");
 // Shadow segments of one block's crossings of one pass, a slot per (crossing, pixel).
-constexpr int kJobs = kTraceKB * kTraceThreads;
+constexpr int kJobs = kTraceKB<true> * kTracePix;
 struct Jobs {
     float2 o[3][kJobs];                // origin (the segment runs to the light)
     float2 S[kJobs];                   // transmittance
@@ -622,24 +627,29 @@ __device__ __forceinline__ void shadow_jobs(const TraceArgs &a, Jobs &J, WarpRin
     }
 }
 
-// One thread a pixel, a block an 8 x 8 tile of pixels (a warp 8 x 4), so that a warp's rays stay
-// together down the tree.  With shadows a block gathers its pixels' next crossings, traces all their
-// segments to the light as one list, and composites.  What bounds it: the waits on nodes, at 9 to 16 warps an
-// SM, and lanes at different depths of the tree (18 of 32 active; a segment meets 187 nodes and 60 leaves).
-// 1.6M triangles at 800x800: 8.6 ms without shadows, 62 ms with the 5.4M segments, against 41 and 148 ms
-// for lanes that each took their triangles through the exact tests alone (4.5 of 32 active), and 218 ms
-// for a thread that also traced its own pixel's segments one after the other.
+// One lane a pixel, a warp 8 x 4 pixels, so that its rays stay together down the tree.  With shadows a
+// block is one such warp and three more: it gathers its pixels' next crossings, all four trace
+// their segments to the light as one list, and it composites.  What bounds it: the waits on nodes, lanes at
+// different depths of the tree (18 of 32 active; a segment meets 187 nodes and 60 leaves), and the blocks with
+// the deepest pixels at the end.  1.6M triangles at 800x800: 5.9 ms without shadows, 39 ms with the 5.4M
+// segments; 41 and 148 ms for lanes that each took their triangles through the exact tests alone
+// (4.5 of 32 active); 62 ms with two warps for 8 x 8 pixels and their segments, whose deepest blocks left
+// two thirds of the chip idle; 218 ms for a thread that traced its own pixel's segments one after the other.
 template <bool SHADOWS>
-__global__ void __launch_bounds__(kTraceThreads, SHADOWS ? kTraceBlocks : 0) trace_kernel(const __grid_constant__ TraceArgs a) {
+__global__ void __launch_bounds__(32 * (SHADOWS ? kTraceWarps : kPlainWarps), SHADOWS ? kTraceBlocks : 0)
+trace_kernel(const __grid_constant__ TraceArgs a) {
     extern __shared__ __align__(16) char smem[];
-    Block &B = *reinterpret_cast<Block *>(smem);
-    Jobs &J = *reinterpret_cast<Jobs *>(smem + sizeof(Block));   // (with SHADOWS)
-    WarpRing &R = B.ring[threadIdx.x >> 5];
-    const int lane = threadIdx.x & 31, warp0 = threadIdx.x & ~31;
+    // a ring for each warp, the block's words, and with shadows its segments
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    WarpRing &R = reinterpret_cast<WarpRing *>(smem)[warp];
+    char *rest = smem + (SHADOWS ? kTraceWarps : kPlainWarps) * sizeof(WarpRing);
+    Block &B = reinterpret_cast<Block *>(rest)[SHADOWS ? 0 : warp];
+    Jobs &J = *reinterpret_cast<Jobs *>(rest + sizeof(Block));
+    const bool lead = !SHADOWS || warp == 0;   // a warp of pixels
     const unsigned lt = (1u << lane) - 1u;
     const int W = a.cam.width, H = a.cam.height;
-    const int px = blockIdx.x * 8 + (threadIdx.x & 7), py = blockIdx.y * 8 + (threadIdx.x >> 3);
-    const bool in = px < W && py < H;
+    const int px = blockIdx.x * 8 + (lane & 7), py = blockIdx.y * (SHADOWS ? 4 : 4 * kPlainWarps) + (SHADOWS ? 0 : 4 * warp) + (lane >> 3);
+    const bool in = lead && px < W && py < H;
     const CamDev &c = a.cam;
     RayF rf;
     float of[3], id[3];
@@ -653,7 +663,7 @@ __global__ void __launch_bounds__(kTraceThreads, SHADOWS ? kTraceBlocks : 0) tra
             rf.d[r] = df_of(((double)c.R[r] * dc[0] + (double)c.R[3 + r] * dc[1]) + (double)c.R[6 + r] * dc[2]);
             of[r] = rf.o[r].h;
             id[r] = finite_rcp(rf.d[r].h);
-            B.d[r][threadIdx.x] = make_float2(rf.d[r].h, rf.d[r].l);
+            if (lead) B.d[r][lane] = make_float2(rf.d[r].h, rf.d[r].l);
         }
     }
     const int n1 = (int)(a.T - 1);   // nodes from n1 on are leaves
@@ -662,152 +672,156 @@ __global__ void __launch_bounds__(kTraceThreads, SHADOWS ? kTraceBlocks : 0) tra
     int after_i = -1;
     bool alive = in && a.T > 0;
     for (;;) {
-        Hit buf[kTraceKB];
+        Hit buf[kTraceKB<SHADOWS>];
         int nb = 0;
         bool more = false;
-        // The warp's pixels walk the tree together, as the segments do (shadow_jobs): triangles that
-        // pass the filter wait in the ring for the double-float test of 32, and each lane sorts its
-        // own crossings of these into its buffer.
-        int stack[kStack];
-        int sp = 0, node = alive ? 0 : -1;
-        uint32_t head = 0, queued = 0;
-        B.after[threadIdx.x] = after_t.h;
-        // Boxes wholly before the last composited crossing hold nothing for this pass, and
-        // boxes wholly beyond the farthest kept crossing of a full buffer only mean another
-        // pass; both bounds are widened by 1e-5 relative, far above the slab test's rounding.
-        const float t_after = after_t.h > 0.0f ? after_t.h * (1.0f - 1e-5f) : 0.0f;
-        const float t_near = c.znear * 0.999f;
-        for (;;) {
-            for (;;) {
-                const bool inner = node >= 0 && node < n1;
-                const unsigned m = __ballot_sync(0xffffffffu, inner), w = __ballot_sync(0xffffffffu, node >= n1);
-                if (m == 0 || __popc(m) <= kWalkShare * __popc(w)) break;
-                if (!inner) continue;
-                const NodeW nd = load_node(a.nodes, node);
-                float nl, fl, nr, fr;
-                bool hl = left_span(nd, of, id, t_near, 3.0e38f, nl, fl) && fl >= t_after;
-                bool hr = right_span(nd, of, id, t_near, 3.0e38f, nr, fr) && fr >= t_after;
-                if (nb == kTraceKB) {
-                    const float t_far = buf[kTraceKB - 1].t.h * (1.0f + 1e-5f);
-                    if (hl && nl > t_far) {
-                        hl = false;
-                        more = true;
-                    }
-                    if (hr && nr > t_far) {
-                        hr = false;
-                        more = true;
-                    }
-                }
-                // the nearer child first: the buffer fills with near crossings early
-                const bool swap = hl && hr && nr < nl;
-                const int first = swap || !hl ? nd.right : nd.left, second = swap ? nd.left : nd.right;
-                if (hl && hr) {
-                    if (sp < kStack) stack[sp++] = second;
-                    else atomicAdd(a.overflow, 1u);
-                }
-                node = hl || hr ? first : (sp > 0 ? stack[--sp] : -1);
-            }
-            bool pass = false;
-            int tri = -1;
-            if (node >= n1) {
-                tri = __ldg(a.leaf_tri + (node - n1));
-                node = sp > 0 ? stack[--sp] : -1;
-                float P[3][3];
-                tri_f(a, tri, P);
-                MtBounds e;
-                pass = mt_may_hit(rf, P[0], P[1], P[2], fmaxf(c.znear, after_t.h), 3.0e38f, e);
-            }
-            const unsigned cand = __ballot_sync(0xffffffffu, pass);
-            if (pass) R.job[(head + queued + __popc(cand & lt)) & 63u] = make_uint2((uint32_t)lane, (uint32_t)tri);
-            queued += __popc(cand);
-            const bool walking = __any_sync(0xffffffffu, node >= 0);
-            __syncwarp();
-            while (queued >= 32u || (!walking && queued)) {
-                const uint32_t nj = min(queued, 32u);
-                int owner = -1;
-                if (lane < nj) {
-                    const uint2 job = R.job[(head + lane) & 63u];
-                    const int at = warp0 + (int)job.x;
-                    RayF jr;
-#pragma unroll
-                    for (int r = 0; r < 3; ++r) {
-                        jr.o[r] = df_make(c.C[r]);
-                        jr.d[r] = dfl{B.d[r][at].x, B.d[r][at].y};
-                    }
-                    float P[3][3];
-                    tri_f(a, (int)job.y, P);
-                    Hit h;
-                    // crossings before the last composited one were taken in an earlier pass
-                    if (crosses(jr, P, fmaxf(c.znear, B.after[at]), 3.0e38f, (double)c.znear, 1.0e300, h)) {
-                        owner = (int)job.x;
-                        R.t[lane] = make_float2(h.t.h, h.t.l);
-                        R.u[lane] = make_float2(h.u.h, h.u.l);
-                        R.v[lane] = make_float2(h.v.h, h.v.l);
-                    }
-                }
-                R.mine[lane] = 0;
-                const unsigned same = __match_any_sync(0xffffffffu, owner);
-                __syncwarp();
-                if (owner >= 0 && lane == __ffs(same) - 1) R.mine[owner] = same;
-                __syncwarp();
-                for (unsigned b = R.mine[lane]; b; b &= b - 1) {
-                    const int i = __ffs(b) - 1;
-                    Hit h;
-                    h.t = dfl{R.t[i].x, R.t[i].y};
-                    h.u = dfl{R.u[i].x, R.u[i].y};
-                    h.v = dfl{R.v[i].x, R.v[i].y};
-                    h.tri = (int)R.job[(head + i) & 63u].y;
-                    if (!hit_less(after_t, after_i, h.t, h.tri)) continue;   // composited in an earlier pass
-                    if (nb == kTraceKB) {
-                        more = true;
-                        if (!hit_less(h.t, h.tri, buf[kTraceKB - 1].t, buf[kTraceKB - 1].tri)) continue;
-                        --nb;   // the farthest kept crossing waits for a later pass
-                    }
-                    int s = nb;
-                    while (s > 0 && hit_less(h.t, h.tri, buf[s - 1].t, buf[s - 1].tri)) {
-                        buf[s] = buf[s - 1];
-                        --s;
-                    }
-                    buf[s] = h;
-                    ++nb;
-                }
-                __syncwarp();
-                head += nj;
-                queued -= nj;
-            }
-            if (!walking) break;
-        }
-        // the crossings that will be composited
         int n_use = 0;
-        {
-            double Tn = T;
-            for (; n_use < nb && !(Tn < a.T_eps); ++n_use) {
-                const Hit &h = buf[n_use];
-                int64_t v[3];
-                tri_verts(a.tris, a.K, h.tri, v);
-                Tn *= 1.0 - to_double(bary_mix(h.u, h.v, __ldg(a.alpha + v[0]), __ldg(a.alpha + v[1]), __ldg(a.alpha + v[2])));
+        if (lead) {
+            // The warp's pixels walk the tree together, as the segments do (shadow_jobs): triangles that
+            // pass the filter wait in the ring for the double-float test of 32, and each lane sorts its
+            // own crossings of these into its buffer.
+            int stack[kStack];
+            int sp = 0, node = alive ? 0 : -1;
+            uint32_t head = 0, queued = 0;
+            B.after[lane] = after_t.h;
+            // Boxes wholly before the last composited crossing hold nothing for this pass, and
+            // boxes wholly beyond the farthest kept crossing of a full buffer only mean another
+            // pass; both bounds are widened by 1e-5 relative, far above the slab test's rounding.
+            const float t_after = after_t.h > 0.0f ? after_t.h * (1.0f - 1e-5f) : 0.0f;
+            const float t_near = c.znear * 0.999f;
+            for (;;) {
+                for (;;) {
+                    const bool inner = node >= 0 && node < n1;
+                    const unsigned m = __ballot_sync(0xffffffffu, inner), w = __ballot_sync(0xffffffffu, node >= n1);
+                    if (m == 0 || __popc(m) <= kWalkShare * __popc(w)) break;
+                    if (!inner) continue;
+                    const NodeW nd = load_node(a.nodes, node);
+                    float nl, fl, nr, fr;
+                    bool hl = left_span(nd, of, id, t_near, 3.0e38f, nl, fl) && fl >= t_after;
+                    bool hr = right_span(nd, of, id, t_near, 3.0e38f, nr, fr) && fr >= t_after;
+                    if (nb == kTraceKB<SHADOWS>) {
+                        const float t_far = buf[kTraceKB<SHADOWS> - 1].t.h * (1.0f + 1e-5f);
+                        if (hl && nl > t_far) {
+                            hl = false;
+                            more = true;
+                        }
+                        if (hr && nr > t_far) {
+                            hr = false;
+                            more = true;
+                        }
+                    }
+                    // the nearer child first: the buffer fills with near crossings early
+                    const bool swap = hl && hr && nr < nl;
+                    const int first = swap || !hl ? nd.right : nd.left, second = swap ? nd.left : nd.right;
+                    if (hl && hr) {
+                        if (sp < kStack) stack[sp++] = second;
+                        else atomicAdd(a.overflow, 1u);
+                    }
+                    node = hl || hr ? first : (sp > 0 ? stack[--sp] : -1);
+                }
+                bool pass = false;
+                int tri = -1;
+                if (node >= n1) {
+                    tri = __ldg(a.leaf_tri + (node - n1));
+                    node = sp > 0 ? stack[--sp] : -1;
+                    float P[3][3];
+                    tri_f(a, tri, P);
+                    MtBounds e;
+                    pass = mt_may_hit(rf, P[0], P[1], P[2], fmaxf(c.znear, after_t.h), 3.0e38f, e);
+                }
+                const unsigned cand = __ballot_sync(0xffffffffu, pass);
+                if (pass) R.job[(head + queued + __popc(cand & lt)) & 63u] = make_uint2((uint32_t)lane, (uint32_t)tri);
+                queued += __popc(cand);
+                const bool walking = __any_sync(0xffffffffu, node >= 0);
+                __syncwarp();
+                while (queued >= 32u || (!walking && queued)) {
+                    const uint32_t nj = min(queued, 32u);
+                    int owner = -1;
+                    if (lane < nj) {
+                        const uint2 job = R.job[(head + lane) & 63u];
+                        const int at = (int)job.x;
+                        RayF jr;
+    #pragma unroll
+                        for (int r = 0; r < 3; ++r) {
+                            jr.o[r] = df_make(c.C[r]);
+                            jr.d[r] = dfl{B.d[r][at].x, B.d[r][at].y};
+                        }
+                        float P[3][3];
+                        tri_f(a, (int)job.y, P);
+                        Hit h;
+                        // crossings before the last composited one were taken in an earlier pass
+                        if (crosses(jr, P, fmaxf(c.znear, B.after[at]), 3.0e38f, (double)c.znear, 1.0e300, h)) {
+                            owner = (int)job.x;
+                            R.t[lane] = make_float2(h.t.h, h.t.l);
+                            R.u[lane] = make_float2(h.u.h, h.u.l);
+                            R.v[lane] = make_float2(h.v.h, h.v.l);
+                        }
+                    }
+                    R.mine[lane] = 0;
+                    const unsigned same = __match_any_sync(0xffffffffu, owner);
+                    __syncwarp();
+                    if (owner >= 0 && lane == __ffs(same) - 1) R.mine[owner] = same;
+                    __syncwarp();
+                    for (unsigned b = R.mine[lane]; b; b &= b - 1) {
+                        const int i = __ffs(b) - 1;
+                        Hit h;
+                        h.t = dfl{R.t[i].x, R.t[i].y};
+                        h.u = dfl{R.u[i].x, R.u[i].y};
+                        h.v = dfl{R.v[i].x, R.v[i].y};
+                        h.tri = (int)R.job[(head + i) & 63u].y;
+                        if (!hit_less(after_t, after_i, h.t, h.tri)) continue;   // composited in an earlier pass
+                        if (nb == kTraceKB<SHADOWS>) {
+                            more = true;
+                            if (!hit_less(h.t, h.tri, buf[kTraceKB<SHADOWS> - 1].t, buf[kTraceKB<SHADOWS> - 1].tri)) continue;
+                            --nb;   // the farthest kept crossing waits for a later pass
+                        }
+                        int s = nb;
+                        while (s > 0 && hit_less(h.t, h.tri, buf[s - 1].t, buf[s - 1].tri)) {
+                            buf[s] = buf[s - 1];
+                            --s;
+                        }
+                        buf[s] = h;
+                        ++nb;
+                    }
+                    __syncwarp();
+                    head += nj;
+                    queued -= nj;
+                }
+                if (!walking) break;
+            }
+            // the crossings that will be composited
+            {
+                double Tn = T;
+                for (; n_use < nb && !(Tn < a.T_eps); ++n_use) {
+                    const Hit &h = buf[n_use];
+                    int64_t v[3];
+                    tri_verts(a.tris, a.K, h.tri, v);
+                    Tn *= 1.0 - to_double(bary_mix(h.u, h.v, __ldg(a.alpha + v[0]), __ldg(a.alpha + v[1]), __ldg(a.alpha + v[2])));
+                }
             }
         }
         if (SHADOWS) {
-            if (threadIdx.x == 0) J.n = J.next = 0;
-            __syncthreads();
-            for (int k = 0; k < kTraceKB; ++k) {   // a warp's segments of one depth follow each other
-                const bool has = k < n_use;
-                const unsigned m = __ballot_sync(0xffffffffu, has);
-                if (m == 0) break;
-                int base = 0;
-                if ((threadIdx.x & 31) == 0) base = atomicAdd(&J.n, __popc(m));
-                base = __shfl_sync(0xffffffffu, base, 0);
-                if (has) {
-                    const int slot = k * kTraceThreads + threadIdx.x;
-                    J.list[base + __popc(m & ((1u << (threadIdx.x & 31)) - 1u))] = (uint16_t)slot;
-                    const double t = to_double(buf[k].t);
-                    J.tri[slot] = buf[k].tri;
+            if (lead) {
+                int n = 0;
+                for (int k = 0; k < kTraceKB<SHADOWS>; ++k) {   // the segments of one depth follow each other
+                    const bool has = k < n_use;
+                    const unsigned m = __ballot_sync(0xffffffffu, has);
+                    if (has) {
+                        const int slot = k * kTracePix + lane;
+                        J.list[n + __popc(m & lt)] = (uint16_t)slot;
+                        const double t = to_double(buf[k].t);
+                        J.tri[slot] = buf[k].tri;
 #pragma unroll
-                    for (int r = 0; r < 3; ++r) {
-                        const dfl pf = df_of(to_double(rf.o[r]) + t * to_double(rf.d[r]));
-                        J.o[r][slot] = make_float2(pf.h, pf.l);
+                        for (int r = 0; r < 3; ++r) {
+                            const dfl pf = df_of(to_double(rf.o[r]) + t * to_double(rf.d[r]));
+                            J.o[r][slot] = make_float2(pf.h, pf.l);
+                        }
                     }
+                    n += __popc(m);
+                }
+                if (lane == 0) {
+                    J.n = n;
+                    J.next = 0;
                 }
             }
             __syncthreads();
@@ -825,7 +839,7 @@ __global__ void __launch_bounds__(kTraceThreads, SHADOWS ? kTraceBlocks : 0) tra
                 col[r] = to_double(bary_mix(h.u, h.v, __ldg(a.rgb + 3 * v[0] + r), __ldg(a.rgb + 3 * v[1] + r),
                                             __ldg(a.rgb + 3 * v[2] + r)));
             if (SHADOWS) {
-                const float2 S = J.S[k * kTraceThreads + threadIdx.x];
+                const float2 S = J.S[k * kTracePix + lane];
                 const double f = a.ambient + (1.0 - a.ambient) * to_double(dfl{S.x, S.y});
 #pragma unroll
                 for (int r = 0; r < 3; ++r) col[r] *= f;
@@ -928,11 +942,12 @@ extern "C" MS_API ms_status ms_raytrace(const float *xyz, const float *rgb, cons
     a.ambient = ambient;
     a.T_eps = a.T_epsf = T_eps;
     a.out = out_rgba;
-    const dim3 grid((cam->width + 7) / 8, (cam->height + 7) / 8);
+    const int rows = a.shadows ? 4 : 4 * kPlainWarps;
+    const dim3 grid((cam->width + 7) / 8, (cam->height + rows - 1) / rows);
     if (a.shadows)
-        trace_kernel<true><<<grid, kTraceThreads, sizeof(Block) + sizeof(Jobs), (cudaStream_t)stream>>>(a);
+        trace_kernel<true><<<grid, 32 * kTraceWarps, kTraceWarps * sizeof(WarpRing) + sizeof(Block) + sizeof(Jobs), (cudaStream_t)stream>>>(a);
     else
-        trace_kernel<false><<<grid, kTraceThreads, sizeof(Block), (cudaStream_t)stream>>>(a);
+        trace_kernel<false><<<grid, 32 * kPlainWarps, kPlainWarps * (sizeof(WarpRing) + sizeof(Block)), (cudaStream_t)stream>>>(a);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return set_error(MS_ERR_CUDA, "trace_kernel: %s", cudaGetErrorString(e));
     count_launches(1);

@@ -63,3 +63,23 @@ def test_rays_through_vertices_and_edges(w, h, cell, light):
     assert ref[..., 3].max() > 0.1
     assert np.abs(img - ref).max() <= 1e-4
     assert rt.status()[1] == 0
+
+
+@pytest.mark.parametrize("layers,light", [(24, None), (25, None), (70, None), (16, (0.5, 0.25, 3.0)), (53, (0.5, 0.25, 3.0))])
+def test_many_crossings_per_pixel(layers, light):
+    """As many crossings as a pass keeps, one more, and several passes; a pixel next to one without any."""
+    parts = [_grid(2, 0.125, -0.01 * i, 5 + i) for i in range(layers)]
+    v = np.concatenate([p[0] for p in parts])
+    v[:, :2] += 0.003   # off the rays: no crossing lies on an edge
+    t = np.concatenate([p[1] + i * len(parts[0][0]) for i, p in enumerate(parts)]).astype(np.int32)
+    c = np.concatenate([p[2] for p in parts])
+    a = np.concatenate([p[3] for p in parts]) * np.float32(0.1)
+    cam = _camera(19, 21)
+    rt = ms.RayTracer(len(t))
+    X, T = dev(v), dev(t)
+    rt.build(X, T)
+    img = rt.trace(X, dev(c), dev(a), cam, tris=T, light=light, ambient=0.25 if light else 1.0).cpu().numpy()
+    ref = ort.render(v, c, a, t, cam, light=np.asarray(light, np.float64) if light else None, ambient=0.25 if light else 1.0)
+    assert ref[..., 3].max() > 0.3
+    assert np.abs(img - ref).max() <= 1e-4
+    assert rt.status()[1] == 0
