@@ -8,8 +8,8 @@
 // its kept faces or shared with them through the centre) and compacted in order, with
 // their vertices' Adam moments (layout [xyz 3V | rgb 3V | alpha V]) and their masks.
 //
-// Three launches, no waits between blocks: per-block counts of kept fans; one block
-// scanning the block counts (and writing the kept total); every block ranks its fans
+// Three launches, no waits between blocks: counts of kept fans per group of rows; one block
+// scanning the counts (and writing the kept total); every block ranks its row of fans
 // again and copies the kept ones to their new slots.  The copy is block-cooperative: the
 // block's kept fans of a row are contiguous in the output, so consecutive threads write
 // consecutive output words (each thread finds its source fan from a shared-memory map).
@@ -131,44 +131,47 @@ __device__ __forceinline__ void copy_rows(const float *__restrict__ src, float *
         if (o + u * kPThreads < words) out[o + u * kPThreads] = v[u];
 }
 
+// A block a row of kPThreads fans; the counts are those of kPItems rows, and the rows before are counted
+// again (from L2).  With a block for all four rows, 977 blocks for 1M fans stood 6.4 to an SM and took the
+// rows' barriers one after another: the whole pruning step 417 us, now 394.
 __global__ void __launch_bounds__(kPThreads) prune_scatter_kernel(PruneIO io, int64_t n_fans, int K, float thr,
                                                                   const uint32_t *__restrict__ boff,
                                                                   const int64_t *__restrict__ n_kept) {
     __shared__ uint32_t s_warp[kPThreads / 32];
     __shared__ uint32_t s_src[kPThreads];
-    const int64_t base = (int64_t)blockIdx.x * kPFans;
+    const int64_t base = (int64_t)(blockIdx.x / kPItems) * kPFans;
+    const int row = blockIdx.x % kPItems;
     const int KV = K + 1;
     const int64_t Vo = n_fans * KV, Vn = *n_kept * KV;
-    uint32_t row_base = boff[blockIdx.x];
-    for (int i = 0; i < kPItems; ++i) {   // rows of kPThreads consecutive fans, in order
+    uint32_t row_base = boff[blockIdx.x / kPItems], faces = 0;
+    for (int i = 0; i <= row; ++i) {   // the kept fans of the rows before, then this row's
+        row_base += (uint32_t)__syncthreads_count(faces != 0u);
         const int64_t f = base + i * kPThreads + threadIdx.x;
-        const uint32_t faces = f < n_fans ? fan_faces(io.alpha, io.mask_in, f, K, thr) : 0u;
-        uint32_t tot;
-        const uint32_t rank = block_excl(faces ? 1u : 0u, s_warp, &tot);
-        if (faces) {
-            s_src[rank] = (uint32_t)(f - base);
-            if (io.mask_o) io.mask_o[row_base + rank] = faces;
-        }
-        __syncthreads();
-        // fan-major arrays: xyz and rgb (3 KV words a fan), alpha (KV)
-        const int64_t f0 = base;   // s_src holds offsets from the block's first fan
-        for (int part = 0; part < 3; ++part) {
-            const int per = part == 2 ? KV : 3 * KV;
-            const float *src = (part == 0 ? io.xyz : part == 1 ? io.rgb : io.alpha) + f0 * per;
-            float *dst = part == 0 ? io.xyz_o : part == 1 ? io.rgb_o : io.alpha_o;
-            copy_rows(src, dst, per, s_src, tot, row_base);
-        }
-        // moments: [xyz 3V | rgb 3V | alpha V] segments, each fan-major like the soup
-        for (int mv = 0; mv < 2; ++mv) {
-            const float *ms_ = mv ? io.v : io.m;
-            float *mo = mv ? io.v_o : io.m_o;
-            if (!ms_) continue;
-            copy_rows(ms_ + f0 * 3 * KV, mo, 3 * KV, s_src, tot, row_base);
-            copy_rows(ms_ + 3 * Vo + f0 * 3 * KV, mo + 3 * Vn, 3 * KV, s_src, tot, row_base);
-            copy_rows(ms_ + 6 * Vo + f0 * KV, mo + 6 * Vn, KV, s_src, tot, row_base);
-        }
-        row_base += tot;
-        __syncthreads();   // s_src is rewritten by the next row
+        faces = f < n_fans ? fan_faces(io.alpha, io.mask_in, f, K, thr) : 0u;
+    }
+    uint32_t tot;
+    const uint32_t rank = block_excl(faces ? 1u : 0u, s_warp, &tot);
+    if (faces) {
+        s_src[rank] = (uint32_t)(row * kPThreads + threadIdx.x);
+        if (io.mask_o) io.mask_o[row_base + rank] = faces;
+    }
+    __syncthreads();
+    // fan-major arrays: xyz and rgb (3 KV words a fan), alpha (KV)
+    const int64_t f0 = base;   // s_src holds offsets from the group's first fan
+    for (int part = 0; part < 3; ++part) {
+        const int per = part == 2 ? KV : 3 * KV;
+        const float *src = (part == 0 ? io.xyz : part == 1 ? io.rgb : io.alpha) + f0 * per;
+        float *dst = part == 0 ? io.xyz_o : part == 1 ? io.rgb_o : io.alpha_o;
+        copy_rows(src, dst, per, s_src, tot, row_base);
+    }
+    // moments: [xyz 3V | rgb 3V | alpha V] segments, each fan-major like the soup
+    for (int mv = 0; mv < 2; ++mv) {
+        const float *ms_ = mv ? io.v : io.m;
+        float *mo = mv ? io.v_o : io.m_o;
+        if (!ms_) continue;
+        copy_rows(ms_ + f0 * 3 * KV, mo, 3 * KV, s_src, tot, row_base);
+        copy_rows(ms_ + 3 * Vo + f0 * 3 * KV, mo + 3 * Vn, 3 * KV, s_src, tot, row_base);
+        copy_rows(ms_ + 6 * Vo + f0 * KV, mo + 6 * Vn, KV, s_src, tot, row_base);
     }
 }
 
@@ -190,7 +193,7 @@ cudaError_t launch_prune(const float *xyz, const float *rgb, const float *alpha,
     prune_count_kernel<<<(unsigned)nblk, kPThreads, 0, st>>>(alpha, mask_in, n_fans, K, thr, bsum);
     prune_scan_kernel<<<1, kPThreads, 0, st>>>(bsum, nblk, boff, n_kept);
     PruneIO io{xyz, rgb, alpha, m, v, mask_in, xyz_o, rgb_o, alpha_o, m_o, v_o, mask_o};
-    prune_scatter_kernel<<<(unsigned)nblk, kPThreads, 0, st>>>(io, n_fans, K, thr, boff, n_kept);
+    prune_scatter_kernel<<<(unsigned)nblk * kPItems, kPThreads, 0, st>>>(io, n_fans, K, thr, boff, n_kept);
     return cudaGetLastError();
 }
 
