@@ -181,6 +181,23 @@ __device__ __forceinline__ bool edge_pass(float E, float ex, float ey) {
 }
 
 // ---------------------------------------------------------------------------------
+// 32-byte records: one 256-bit access of sm_100-class GPUs, p 32-byte aligned.  Used where a pass waits
+// on its records (resolve and its adjoint: view of 200k fans 878 -> 862 us; splat fill); the fan fill's and
+// the chain's accesses gain nothing by it.
+// ---------------------------------------------------------------------------------
+
+__device__ __forceinline__ void ld_rec(const float4 *p, float4 &a, float4 &b) {
+    asm volatile("ld.global.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)
+                 : "l"(p));
+}
+__device__ __forceinline__ void st_rec(float4 *p, const float4 a, const float4 b) {
+    asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "f"(a.x), "f"(a.y), "f"(a.z), "f"(a.w),
+                 "f"(b.x), "f"(b.y), "f"(b.z), "f"(b.w)
+                 : "memory");
+}
+
+// ---------------------------------------------------------------------------------
 // Bounded waits
 // ---------------------------------------------------------------------------------
 

@@ -202,11 +202,7 @@ __device__ __forceinline__ uint32_t resolve_group(const ResolveArgs &a, GroupMem
     const int nmax = __reduce_max_sync(0xffffffffu, n);
     const bool has = sub < n;
     float4 r0 = make_float4(0.f, 0.f, 0.f, 0.f), r1 = r0;
-    if (has) {
-        const float4 *rec = a.frags + (size_t)kRecFwd * (size_t)(off + sub);
-        r0 = rec[0];
-        r1 = rec[1];
-    }
+    if (has) ld_rec(a.frags + (size_t)kRecFwd * (size_t)(off + sub), r0, r1);
     const unsigned long long key = has ? sort_key(r0) : ~0ull;
     __syncwarp();   // the words are still read for the previous unit
     m.key[lane] = key;
@@ -287,8 +283,9 @@ __device__ uint32_t resolve_deep(const ResolveArgs &a, GroupMem &m, const Pixel 
     bool ended = false;
     if (n <= 64) {
         const bool ha = lane < n, hb = lane + 32 < n;
-        const float4 a0 = ha ? rec[kRecFwd * lane] : zero, a1 = ha ? rec[kRecFwd * lane + 1] : zero;
-        const float4 b0 = hb ? rec[kRecFwd * (lane + 32)] : zero, b1 = hb ? rec[kRecFwd * (lane + 32) + 1] : zero;
+        float4 a0 = zero, a1 = zero, b0 = zero, b1 = zero;
+        if (ha) ld_rec(rec + kRecFwd * lane, a0, a1);
+        if (hb) ld_rec(rec + kRecFwd * (lane + 32), b0, b1);
         int ra, rb;
         place64(m, ha ? sort_key(a0) : ~0ull, __float_as_uint(a0.y), hb ? sort_key(b0) : ~0ull, __float_as_uint(b0.y),
                 ra, rb);
@@ -418,20 +415,13 @@ __global__ void __launch_bounds__(kBwdThreads) resolve_bwd_kernel(const __grid_c
     float T = 1.0f, C0 = 0.0f, C1 = 0.0f, C2 = 0.0f;
     // (indices past the last composited fragment are not read as records)
     uint32_t i1 = ord[0], i2 = n > 1 ? ord[1] : kEnd;
-    float tri1 = 0.0f;
-    float4 col1 = zero;
-    if (i1 < n) {
-        tri1 = rec[(size_t)kRecFwd * i1].y;
-        col1 = rec[(size_t)kRecFwd * i1 + 1];
-    }
+    float4 id1 = zero, col1 = zero;
+    if (i1 < n) ld_rec(rec + (size_t)kRecFwd * i1, id1, col1);
     uint32_t c = 0;
     for (; c < n && i1 < n; ++c) {
-        const float tri = tri1;
+        const float tri = id1.y;
         const float4 col = col1;
-        if (i2 < n) {
-            tri1 = rec[(size_t)kRecFwd * i2].y;
-            col1 = rec[(size_t)kRecFwd * i2 + 1];
-        }
+        if (i2 < n) ld_rec(rec + (size_t)kRecFwd * i2, id1, col1);
         i1 = i2;
         i2 = c + 2 < n && i2 < n ? ord[c + 2] : kEnd;
         const float al = col.w;
@@ -440,20 +430,20 @@ __global__ void __launch_bounds__(kBwdThreads) resolve_bwd_kernel(const __grid_c
         const float inv = 1.0f / fmaxf(1.0f - al, 1e-6f);
         const float ga = g.x * (T * col.x - (ov.x - nC0) * inv) + g.y * (T * col.y - (ov.y - nC1) * inv) +
                          g.z * (T * col.z - (ov.z - nC2) * inv) + g.w * Tout * inv;
-        adj[2 * c] = make_float4(g.x * w, g.y * w, g.z * w, ga);
-        adj[2 * c + 1] = make_float4(tri, __uint_as_float(e.pix), 0.0f, 0.0f);
+        st_rec(adj + 2 * c, make_float4(g.x * w, g.y * w, g.z * w, ga), make_float4(tri, __uint_as_float(e.pix), 0.0f, 0.0f));
         C0 = nC0; C1 = nC1; C2 = nC2;
         T *= (1.0f - al);
     }
     // slots past the composited fragments carry a zero gradient (the chain pass reads
     // every slot of the pixel's range)
-    for (; c < n; ++c) adj[2 * c] = adj[2 * c + 1] = zero;
+    for (; c < n; ++c) st_rec(adj + 2 * c, zero, zero);
 }
 
 __global__ void grad_scatter_kernel(const float4 *__restrict__ g, int64_t V, float *__restrict__ dx,
                                     float *__restrict__ dc, float *__restrict__ da) {
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < V; v += (int64_t)gridDim.x * blockDim.x) {
-        const float4 a = g[2 * v], b = g[2 * v + 1];
+        float4 a, b;
+        ld_rec(g + 2 * v, a, b);
         dx[3 * v] += a.x;
         dx[3 * v + 1] += a.y;
         dx[3 * v + 2] += a.z;

@@ -330,8 +330,7 @@ __device__ __forceinline__ void splat_item(const SplatArgs &a, char *smem, uint3
                         splat_exact(a.spl, cam, S.gid[jf], px, py, t, al);
                     const float4 col = S.col[jf];
                     float4 *out = a.frags + (size_t)kRecFwd * (size_t)job.y;
-                    out[0] = make_float4(t, __uint_as_float(S.gid[jf]), 0.0f, 0.0f);
-                    out[1] = make_float4(col.x, col.y, col.z, al);
+                    st_rec(out, make_float4(t, __uint_as_float(S.gid[jf]), 0.0f, 0.0f), make_float4(col.x, col.y, col.z, al));
                 }
                 head += nj;
                 queued -= nj;
