@@ -3,7 +3,7 @@
 
 One step = one pass of the hot path over the 1,000,000-Gaussian clustered scene at
 1920x1080 (SH degree 3 in bfloat16, K = 8): fan conversion with SH colour, render
-(projection, tile binning, radix sort, exact-order composite), L1 loss against a
+(projection, tile binning, tile lists, exact-order composite), L1 loss against a
 jittered-scene target, adjoint, and the two-learning-rate Adam update of the fans.
 
 Prints one JSON line (rank 0).  `value` is rendered megapixels per second of the
@@ -41,16 +41,15 @@ NSTAGE = len(STAGES)
 # ncu DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of one launch of a stage's
 # kernels on the 1M-fan 1080p workload stored in spatial order, with the digest of the kernel
 # sources it was taken on; reported only while the digest still matches.  Measured on that
-# workload itself (one pass per launch): work items 0.2 MB, count 193, tile prefix 24, pixel
-# scan 8, pixel order 8, fill 648, resolve 491.
-TRAFFIC = {"raster": {"bytes": 1.37e9, "digest": "94721382e11f362b"}}
+# workload itself (one pass per launch): count 189 MB, record ranges 12, fill 606, resolve 425.
+TRAFFIC = {"raster": {"bytes": 1.23e9, "digest": "8b4854be00fd263f"}}
 
 
 def kernel_digest():
     """Digest of the sources of the rasterisation stage's kernels."""
     import hashlib
     h = hashlib.sha256()
-    for f in ("raster.cu", "resolve.cu", "raster_common.cuh", "fan_geom.cuh"):
+    for f in ("raster.cu", "fill.cu", "tiles.cu", "resolve.cu", "raster_common.cuh", "fan_geom.cuh"):
         h.update(f.encode())
         h.update(open(os.path.join(ROOT, "paper_2502_07754_gb300", "csrc", f), "rb").read())
     return h.hexdigest()[:16]
@@ -316,8 +315,7 @@ def stage_report(stage_ms, stage_n, info, sc, V, K, npx, local):
     nb = (sc.sh_degree + 1) ** 2 * 3 * (2 if sc.sh_bf16 else 4)
     hbm_bytes = {"mesh_build": sc.n * (44 + nb) + V * 28,
                  "bin": V * 12 + info.pairs * 8,
-                 # one histogram read, then per pass each 8-byte element read and written
-                 "sort": info.pairs * (8 + 16 * ((info.sort_bits + 7) // 8)),
+                 "sort": info.pairs * 16,   # tile lists: tile, fan and rank read, fan written
                  "loss": npx * 48,
                  "adam": V * 7 * 28}
     stages = {}

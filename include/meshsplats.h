@@ -6,7 +6,7 @@
  * order-correct alpha compositing.  This library implements, as CUDA kernels:
  *   ms_mesh_build       Gaussian -> fan conversion with SH colour (Sec. 3, Eq. 2 and the
  *                       vertex / colour / opacity rules that follow it)
- *   ms_render           MVP projection, tile binning, radix sort of (tile, depth) keys,
+ *   ms_render           MVP projection, tile binning, tile lists by counting,
  *                       exact per-pixel depth order, perspective-correct barycentric
  *                       interpolation, front-to-back compositing (Sec. 3 "Rendering
  *                       MeshSplats in Nvdiffrast")
@@ -144,9 +144,9 @@ typedef struct {
 typedef enum {
     MS_STAGE_MESH_BUILD = 0,
     MS_STAGE_BIN = 1,
-    MS_STAGE_SORT = 2,
-    MS_STAGE_RASTER = 3,          /* count, pixel scan, fill and resolve of the forward */
-    MS_STAGE_RASTER_BWD = 4,      /* fill, adjoint resolve and gradient scatter */
+    MS_STAGE_SORT = 2,            /* the tile lists */
+    MS_STAGE_RASTER = 3,          /* count, record ranges, fill and resolve of the forward */
+    MS_STAGE_RASTER_BWD = 4,      /* adjoint resolve, record chain and gradient scatter */
     MS_STAGE_LOSS = 5,
     MS_STAGE_ADAM = 6,
     MS_STAGE_MLP = 7,             /* learned initializer inference */
@@ -348,7 +348,7 @@ MS_API size_t ms_render_workspace_size(int64_t n_fans, int32_t K, const ms_camer
  *   xyz, rgb, alpha: device fan soup; n_fans fans of K (3..16) triangles.
  *   out_rgba: device H x W x 4.
  *   workspace: device, >= ms_render_workspace_size bytes, 256-byte aligned; it keeps
- *   the sorted tile lists and per-pixel transmittance that ms_render_backward reuses.
+ *   the tile lists, the records and per-pixel transmittance that ms_render_backward reuses.
  * MS_ERR_INVALID for bad sizes or pointers, including 2^32 or more pixels over all views
  * of a call (pixel indices are 32-bit in the fragment records).
  * Returns once the work is queued; call ms_render_get_info for device-side errors.
@@ -397,7 +397,7 @@ MS_API size_t ms_batch_workspace_size(int64_t n_fans, int32_t K, const ms_camera
 /*
  * Forward render of one fan soup into n_views images of (possibly) different sizes in
  * one pass of the pipeline: the tiles of all views form one index space, so binning,
- * the key sort, rasterisation and the per-pixel resolve each launch once for the whole
+ * the tile lists, rasterisation and the per-pixel resolve each launch once for the whole
  * batch (the multi-view renders of fine-tuning, Sec. 3 "Fine-tuning", and of the
  * evaluation in Sec. 4).  Image v equals ms_render with cams[v] bit for bit.
  *   cams: host array of n_views cameras (read during the call only).

@@ -216,7 +216,7 @@ static ViewTable make_views(const ms_camera *cams, int n_views, const RenderLayo
 
 static bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
-// Forward of any number of views: one binning launch, one sort, one rasterisation
+// Forward of any number of views: one binning launch, the tile lists, one rasterisation
 // and one resolve over the concatenated tile / pixel index space.
 static ms_status render_views(const float *xyz, const float *rgb, const float *alpha, int64_t n_fans, int K,
                               const ms_camera *cams, int n_views, const ms_render_params *params, float *const *out,
@@ -295,7 +295,7 @@ static ms_status render_views_backward(const float *xyz, const float *rgb, const
 }
 
 // Source-Gaussian splat render: the polygons circumscribing the splats go through the
-// same binning, sort and work-item machinery as fans; the splat passes then evaluate
+// same binning, tile-list and work-item machinery as fans; the splat passes then evaluate
 // the Gaussians themselves.  The polygon soup lives after the render layout.
 constexpr double kSplatTrunc = 2.7;           // truncation radius in scales (the fan's scale_mul)
 

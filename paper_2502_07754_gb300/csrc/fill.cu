@@ -14,10 +14,10 @@
 //  3. every covered (fan, triangle, centre) goes into a ring of jobs, and whole warps of jobs
 //     compute their fragment: perspective-correct barycentrics, values, and the exact-order
 //     depth in double-float.
-// What bounds it: issue slots and the waits of a pair's dependent loads.  Staging with every lane
-// and computing fragments 32 at a time, against four lanes a fan and the lanes whose test hit:
-// 1M fans at 1080p (10.4M fragments) 0.62 -> 0.45 ms, 200k fans at 800x800 0.31 -> 0.21 ms, 3M fans
-// in 16 views (42M pairs, 51M fragments) 9.9 -> 5.9 ms.
+// What bounds it: issue slots (64% of cycles) and the waits of a pair's dependent loads.  Staging with
+// every lane and computing fragments 32 at a time, against four lanes a fan and the lanes whose test hit,
+// with full groups of fans: 1M fans at 1080p (10.4M fragments) 0.62 -> 0.43 ms, 200k fans at 800x800 0.31 ->
+// 0.195 ms, 3M fans in 16 views (42M pairs, 51M fragments) 9.9 -> 4.3 ms (with the strided launch).
 #include "raster_common.cuh"
 
 namespace ms {

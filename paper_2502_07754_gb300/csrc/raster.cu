@@ -7,9 +7,9 @@
 // orientations and the fan's pixel rectangle inside the tile.  The rectangles' rows, cut into runs
 // of two pixels, form one index space, a lane a run: it answers the two (fan, pixel) tests with the
 // binary32 decision formulas, sharing the spoke loads and the row's products.  No block barriers
-// are used.  What bounds it: issue slots (70% busy).  Against two lanes
+// are used.  What bounds it: issue slots (56 to 70% busy).  Against two lanes
 // staging a pair's words one triangle after the other and a lane a test: 200k fans at 800x800 (9M tests)
-// 103 -> 80 us, 3M fans in 16 views (42M pairs, 96M tests) 4.3 -> 3.3 ms
+// 103 -> 78 us, 3M fans in 16 views (42M pairs, 96M tests) 4.3 -> 3.3 ms, and 2.1 ms with the strided launch
 //
 // The pass leaves the coverage mask of every test, per pair its first mask index and its pixel
 // rectangle within the tile (zero when the pair covers no pixel centre, so the fill skips it),
