@@ -31,7 +31,7 @@
 // What bounds them: the forward issues on two thirds of its cycles and waits on scattered
 // record reads otherwise (1M fans at 1080p, 10.4M fragments: 0.26 ms; one thread a pixel with a
 // sorted register buffer, 114 registers and 11 of 32 lanes active: 0.54 ms).  The backward
-// waits on its record reads (0.21 ms there, 72 long-scoreboard cycles an instruction).
+// waits on its record reads (0.19 ms there, 72 long-scoreboard cycles an instruction).
 #include "raster_common.cuh"
 
 namespace ms {
