@@ -509,6 +509,9 @@ struct Jobs {
     int n, next;
 };
 
+// Nodes from here on are leaves; a lane that is not in the tree (node -1) is below it, in an empty scene too.
+__device__ __forceinline__ int first_leaf(const TraceArgs &a) { return a.T > 0 ? (int)(a.T - 1) : 0; }
+
 __device__ __forceinline__ void segment(const TraceArgs &a, const Jobs &J, int slot, RayF &rf) {
 #pragma unroll
     for (int r = 0; r < 3; ++r) {
@@ -523,7 +526,7 @@ __device__ __forceinline__ void segment(const TraceArgs &a, const Jobs &J, int s
 // triangle in eight) goes into a ring, and the warp takes 32 of them through the double-float test at
 // once (a lane on its own took it with 3 of 32 lanes: 118 -> 46 ms for the 5.4M segments below).
 __device__ __forceinline__ void shadow_jobs(const TraceArgs &a, Jobs &J, WarpRing &R) {
-    const int n1 = (int)(a.T - 1);   // nodes from n1 on are leaves
+    const int n1 = first_leaf(a);
     const float t0 = -1e-3f, t1 = 1.001f;
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
@@ -666,7 +669,7 @@ trace_kernel(const __grid_constant__ TraceArgs a) {
             if (lead) B.d[r][lane] = make_float2(rf.d[r].h, rf.d[r].l);
         }
     }
-    const int n1 = (int)(a.T - 1);   // nodes from n1 on are leaves
+    const int n1 = first_leaf(a);
     double T = 1.0, C0 = 0.0, C1 = 0.0, C2 = 0.0;
     dfl after_t = df_make(-3.0e38f);
     int after_i = -1;
