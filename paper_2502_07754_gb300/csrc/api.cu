@@ -130,7 +130,7 @@ RenderLayout render_layout(int64_t n_fans, int K, const ms_camera *cams, int n_v
     L.off_status = o;            o = align_up(o + 256, 256);
     L.off_tscan_state = o;       o = align_up(o + 8 * (size_t)L.tscan_blocks, 256);
     L.off_tile_cnt = o;          o = align_up(o + 4 * (size_t)L.n_tiles, 256);
-    L.off_mask_cursor = o;       o = align_up(o + 4 * (size_t)kMaskRegions, 256);
+    L.off_mask_cursor = o;       o = align_up(o + 8 * (size_t)kMaskRegions, 256);
     L.off_counts = o;            o = align_up(o + 4 * (size_t)npx, 256);
     L.off_zero_end = o;          // (the prefix zeroed per render)
     L.off_pairs = o;             o = align_up(o + 8 * (size_t)cap, 256);

@@ -40,8 +40,10 @@ struct Status {
     unsigned int n_items;            // raster work items (<= 64 fans of one tile each)
     unsigned long long items_total;  // work items the tile scan counted
 };
-// The count pass's coverage masks live in at most this many equal regions, each with its own cursor.
-constexpr int kMaskRegions = 256;
+// The count pass's coverage masks live in at most this many equal regions, each with its own cursor. A
+// cursor counts every test of its region, stored or not: 64 bits, as a small image has one region only and
+// wrapped words would hand out stored masks again.
+constexpr int kMaskRegions = 128;
 static_assert(sizeof(Status) <= 256, "status block");
 
 struct CamDev {

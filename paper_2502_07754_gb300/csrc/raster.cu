@@ -42,7 +42,7 @@ struct RastArgs {
     uint16_t *masks;           // coverage masks (bit j: triangle j) of the tests
     int64_t mask_cap;
     uint32_t mask_regions;
-    uint32_t *mask_cursor;     // [mask_regions] fill levels of the mask regions (zeroed per render)
+    unsigned long long *mask_cursor;   // [mask_regions] tests of the mask regions (zeroed per render)
 };
 
 constexpr int kRastWarps = 2;   // warps (work items) per block: items differ widely in cost
@@ -191,8 +191,8 @@ __device__ __forceinline__ void count_item(const RastArgs &a, char *smem, uint32
         if (lane == 0 && total > 0) {
             const uint32_t reg = item % a.mask_regions;
             const uint32_t rsz = (uint32_t)(a.mask_cap / a.mask_regions);
-            const uint32_t b = atomicAdd(a.mask_cursor + reg, all >> 16);
-            if ((uint64_t)b + (uint64_t)(all >> 16) <= (uint64_t)rsz) mbase = reg * rsz + b;
+            const unsigned long long b = atomicAdd(a.mask_cursor + reg, (unsigned long long)(all >> 16));
+            if (b + (all >> 16) <= rsz) mbase = reg * rsz + (uint32_t)b;
         }
         mbase = __shfl_sync(0xffffffffu, mbase, 0);
         const uint32_t live = __ballot_sync(0xffffffffu, in);   // pairs with tests, in order
@@ -311,7 +311,7 @@ RastArgs make_args(const RenderArgs &ra) {
     a.mask_cap = L.mask_cap;
     // regions of at least 2^19 masks: 32 pairs of a whole tile take 2^15, and few regions fill evenly
     a.mask_regions = (uint32_t)std::min<int64_t>(kMaskRegions, std::max<int64_t>(1, L.mask_cap >> 19));
-    a.mask_cursor = reinterpret_cast<uint32_t *>(ra.ws + L.off_mask_cursor);
+    a.mask_cursor = reinterpret_cast<unsigned long long *>(ra.ws + L.off_mask_cursor);
     return a;
 }
 

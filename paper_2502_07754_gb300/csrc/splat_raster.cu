@@ -44,7 +44,7 @@ struct SplatArgs {
     Status *st;
     const float4 *dec;      // [view][vertex] decided polygon vertices
     int64_t V;
-    uint32_t *tests;        // [kMaskRegions] tests, in parts
+    unsigned long long *tests;   // [kMaskRegions] tests, in parts
     uint2 *pinfo;           // per pair: (0, rectangle within the tile; 0 if no centre is hit)
     const float4 *coef;     // [view][Gaussian][5]
     float r2;               // squared truncation radius in scales
@@ -348,7 +348,7 @@ __device__ __forceinline__ void splat_item(const SplatArgs &a, char *smem, uint3
                 icnt[i] = atomicAdd(a.counts + vw.pix_base + (size_t)(ty0 + i / TILE) * cam.width + (size_t)(tx0 + i % TILE), c);
         }
         const unsigned r0 = __reduce_add_sync(0xffffffffu, n_test);
-        if (lane == 0) atomicAdd(a.tests + item % kMaskRegions, r0);
+        if (lane == 0) atomicAdd(a.tests + item % kMaskRegions, (unsigned long long)r0);
     }
 }
 
@@ -396,7 +396,7 @@ cudaError_t launch(const RenderArgs &ra, cudaStream_t st) {
     a.st = reinterpret_cast<Status *>(ra.ws + L.off_status);
     a.dec = reinterpret_cast<const float4 *>(ra.ws + L.off_dec);
     a.V = L.V;
-    a.tests = reinterpret_cast<uint32_t *>(ra.ws + L.off_mask_cursor);
+    a.tests = reinterpret_cast<unsigned long long *>(ra.ws + L.off_mask_cursor);
     a.pinfo = reinterpret_cast<uint2 *>(ra.ws + L.off_maskoff);
     a.coef = ra.splat_coef;
     a.r2 = (float)(ra.spl.trunc * ra.spl.trunc);

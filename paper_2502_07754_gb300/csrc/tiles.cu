@@ -153,7 +153,7 @@ struct AllocArgs {
     uint32_t *list_b;
     float *tfinal;
     Status *st;
-    const uint32_t *tests;      // [kMaskRegions] tests of the count pass, in parts
+    const unsigned long long *tests;   // [kMaskRegions] tests of the count pass, in parts
     float bg0, bg1, bg2;
     ViewTable vt;
 };
@@ -166,10 +166,11 @@ __global__ void __launch_bounds__(kAllocThreads) pixel_alloc_kernel(const __grid
     s_cnt[tid] = 0;
     if (tid < 4) s_class[tid] = 0;
     if (blockIdx.x == 0) {
-        static_assert(kMaskRegions == kAllocThreads, "one thread per part");
-        const uint32_t lo = __reduce_add_sync(0xffffffffu, a.tests[tid] & 0xffffu);
-        const uint32_t hi = __reduce_add_sync(0xffffffffu, a.tests[tid] >> 16);
-        if (lane == 0) atomicAdd(&a.st->rect_tests, (unsigned long long)lo + ((unsigned long long)hi << 16));
+        static_assert(kMaskRegions <= kAllocThreads, "one thread per part");
+        unsigned long long t = tid < kMaskRegions ? a.tests[tid] : 0ull;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (lane == 0 && t) atomicAdd(&a.st->rect_tests, t);
     }
     // this thread's four slots: neighbours in a row of one tile
     const int64_t s0 = (int64_t)blockIdx.x * kAllocSpan + tid * kAllocSlots;
@@ -293,7 +294,7 @@ cudaError_t launch_pixel_alloc(const RenderArgs &ra, cudaStream_t st) {
     a.list_b = reinterpret_cast<uint32_t *>(ws + L.off_order_b);
     a.tfinal = reinterpret_cast<float *>(ws + L.off_tfinal);
     a.st = reinterpret_cast<Status *>(ws + L.off_status);
-    a.tests = reinterpret_cast<const uint32_t *>(ws + L.off_mask_cursor);
+    a.tests = reinterpret_cast<const unsigned long long *>(ws + L.off_mask_cursor);
     a.bg0 = ra.prm.bg[0];
     a.bg1 = ra.prm.bg[1];
     a.bg2 = ra.prm.bg[2];
