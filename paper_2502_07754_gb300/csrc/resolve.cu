@@ -43,7 +43,6 @@ constexpr uint32_t kEnd = 0xffffffffu;
 struct ResolveArgs {
     int64_t npx;
     const float4 *frags;
-    int64_t frag_cap;
     float T_eps, bg0, bg1, bg2;
     Status *st;
     float *tfinal;
@@ -52,7 +51,7 @@ struct ResolveArgs {
                                // (32 bytes, whole sectors: 16 + 8 bytes in two arrays took twice as long)
     uint32_t *corder;          // per pixel: record indices in commit order (same offsets as records), then
                                // kEnd if fewer were composited than there are records
-    // pixels with fragments: list_b holds those of more than 16 fragments (more than 32 from its
+    // pixels whose fragments have records: list_b holds those of more than 16 (more than 32 from its
     // end, the others from its start), list_a the others with their record offsets (9 to 16 from
     // its end, 1 to 8 from its start); st->classes counts the four
     const uint2 *list_a;
@@ -69,12 +68,11 @@ struct Units {
     uint32_t c16, c8;             // pixels of 9 to 16 and of 1 to 8 records
     uint32_t deep, n32, n16, n8;  // unit bounds of the classes
     __device__ __forceinline__ Units(const ResolveArgs &a) {
-        // (a count past a list's end exists only for a buffer that overflowed its capacity)
         const uint4 c = *reinterpret_cast<const uint4 *>(a.st->classes);
-        deep = (uint32_t)min64(c.x, a.order_b);
-        n32 = deep + (uint32_t)min64(c.y, a.order_b);
-        c16 = (uint32_t)min64(c.z, a.npx);
-        c8 = (uint32_t)min64(c.w, a.npx);
+        deep = c.x;
+        n32 = deep + c.y;
+        c16 = c.z;
+        c8 = c.w;
         n16 = n32 + (c16 + 1) / 2;
         n8 = n16 + (c8 + 3) / 4;
     }
@@ -96,8 +94,7 @@ struct Units {
     }
 };
 
-// A pixel with its records: count 0 where there is none, or where they did not fit the buffer
-// (reported through the status block).
+// A pixel with its records (all of which the buffer holds); count 0 where there is none.
 struct Pixel {
     uint32_t pix, off, n;
 };
@@ -110,9 +107,6 @@ __device__ __forceinline__ Pixel pixel_of(const ResolveArgs &a, const uint2 e, b
     return p;
 }
 __device__ __forceinline__ bool is_pixel(const ResolveArgs &a, const Pixel &p) { return p.pix < (uint64_t)a.npx; }
-__device__ __forceinline__ bool fits(const ResolveArgs &a, const Pixel &p) {
-    return (int64_t)p.off + p.n <= a.frag_cap;
-}
 
 // Shared words of one warp: sort keys and ids by record, then the values in sorted places.
 struct GroupMem {
@@ -189,7 +183,7 @@ __device__ __forceinline__ void write_pixel(const ResolveArgs &a, const Pixel &e
     reinterpret_cast<float4 *>(vw.out)[(int64_t)e.pix - (int64_t)vw.pix_base] =
         make_float4(C0 + T * a.bg0, C1 + T * a.bg1, C2 + T * a.bg2, 1.0f - T);
     a.tfinal[e.pix] = T;
-    if (ncom < e.n && fits(a, e)) a.corder[(size_t)e.off + ncom] = kEnd;
+    if (ncom < e.n) a.corder[(size_t)e.off + ncom] = kEnd;
 }
 
 // One warp's 32 / G pixels (e per group); returns the fragments composited (first lanes).
@@ -198,7 +192,7 @@ __device__ __forceinline__ uint32_t resolve_group(const ResolveArgs &a, GroupMem
     const int lane = threadIdx.x & 31, sub = lane & (G - 1), g0 = lane & ~(G - 1);
     const bool valid = is_pixel(a, e);
     const int64_t off = e.off;
-    const int n = fits(a, e) && e.n <= (uint32_t)G ? (int)e.n : 0;
+    const int n = (int)e.n;   // (at most G)
     const int nmax = __reduce_max_sync(0xffffffffu, n);
     const bool has = sub < n;
     float4 r0 = make_float4(0.f, 0.f, 0.f, 0.f), r1 = r0;
@@ -275,7 +269,7 @@ __device__ uint32_t resolve_deep(const ResolveArgs &a, GroupMem &m, const Pixel 
     const int lane = threadIdx.x & 31;
     if (!is_pixel(a, e)) return 0;
     const int64_t off = e.off;
-    const int n = fits(a, e) ? (int)e.n : 0;
+    const int n = (int)e.n;
     const float4 *rec = a.frags + (size_t)kRecFwd * (size_t)off;
     const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
     float T = 1.0f, C = 0.0f;
@@ -390,8 +384,8 @@ constexpr int kBwdThreads = 64;
 __global__ void __launch_bounds__(kBwdThreads) resolve_bwd_kernel(const __grid_constant__ ResolveArgs a) {
     const int64_t q = (int64_t)blockIdx.x * kBwdThreads + threadIdx.x;
     const uint4 cl = *reinterpret_cast<const uint4 *>(a.st->classes);
-    const int64_t n0 = min64(cl.x, a.order_b), n1 = n0 + min64(cl.y, a.order_b), n2 = n1 + min64(cl.z, a.npx);
-    if (q >= n2 + min64(cl.w, a.npx)) return;
+    const int64_t n0 = cl.x, n1 = n0 + cl.y, n2 = n1 + cl.z;
+    if (q >= n2 + cl.w) return;
     uint2 entry = make_uint2(0u, 0u);
     if (q < n0)
         entry.x = __ldg(a.list_b + (a.order_b - 1 - q));
@@ -400,7 +394,7 @@ __global__ void __launch_bounds__(kBwdThreads) resolve_bwd_kernel(const __grid_c
     else
         entry = __ldg(q < n2 ? a.list_a + (a.npx - 1 - (q - n1)) : a.list_a + (q - n2));
     const Pixel e = pixel_of(a, entry, q < n1);
-    if (!is_pixel(a, e) || !fits(a, e)) return;
+    if (!is_pixel(a, e)) return;
     const int64_t off = e.off;
     const uint32_t n = e.n;
     const float4 zero = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
@@ -463,7 +457,6 @@ ResolveArgs make_args(const RenderArgs &ra) {
     ResolveArgs a;
     a.npx = L.npx;
     a.frags = reinterpret_cast<const float4 *>(ra.ws + L.off_frags);
-    a.frag_cap = L.frag_cap;
     a.T_eps = ra.prm.T_eps;
     a.bg0 = ra.prm.bg[0];
     a.bg1 = ra.prm.bg[1];

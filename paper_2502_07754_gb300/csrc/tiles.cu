@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(256) tile_scatter_kernel(const uint2 *__restri
 constexpr int kAllocThreads = 256, kAllocSlots = 4, kAllocSpan = kAllocThreads * kAllocSlots;
 
 struct AllocArgs {
-    int64_t npx, n_slots, order_b;
+    int64_t npx, n_slots, order_b, frag_cap;
     int tile_shift;
     const uint32_t *counts;
     uint32_t *offsets;
@@ -205,13 +205,20 @@ __global__ void __launch_bounds__(kAllocThreads) pixel_alloc_kernel(const __grid
         total += s_warp[w];
     }
     if (tid == 0) s_first = total ? atomicAdd(&a.st->frags, (unsigned long long)total) : 0ull;
-    // rank of each pixel among the span's pixels of its count
+    __syncthreads();
+    unsigned long long run = s_first + before + x - sum;
+    // rank of each pixel among the span's pixels of its count; a pixel whose records do not fit the buffer
+    // (reported through the status block) is none of them, so the lists cannot overflow
     int bk[kAllocSlots];
     uint32_t rk[kAllocSlots];
+    {
+        unsigned long long end = run;
 #pragma unroll
-    for (int i = 0; i < kAllocSlots; ++i) {
-        bk[i] = count_bucket(n[i]);
-        rk[i] = bk[i] ? atomicAdd(&s_cnt[bk[i]], 1u) : 0u;
+        for (int i = 0; i < kAllocSlots; ++i) {
+            end += n[i];
+            bk[i] = end <= (unsigned long long)a.frag_cap ? count_bucket(n[i]) : 0;
+            rk[i] = bk[i] ? atomicAdd(&s_cnt[bk[i]], 1u) : 0u;
+        }
     }
     __syncthreads();
     // descending prefix over the counts: thread t holds count 255 - t
@@ -234,7 +241,6 @@ __global__ void __launch_bounds__(kAllocThreads) pixel_alloc_kernel(const __grid
     for (int c = 0; c < cls; ++c) skip += s_class[c];
     s_at[mb] = px - h - skip;
     __syncthreads();
-    unsigned long long run = s_first + before + x - sum;
     const ViewDev &vw = a.vt.v[view];
     for (int i = 0; i < in; ++i) {
         // offsets beyond 2^32 are clamped; such a buffer overflows its capacity anyway
@@ -244,13 +250,12 @@ __global__ void __launch_bounds__(kAllocThreads) pixel_alloc_kernel(const __grid
         if (bk[i]) {
             const int c = bk[i] > 32 ? 0 : (bk[i] > 16 ? 1 : (bk[i] > 8 ? 2 : 3));
             const int64_t at = (int64_t)s_base[c] + s_at[bk[i]] + rk[i];
-            // (places past a list's end exist only for a buffer that overflowed its capacity)
             const uint2 e = make_uint2((uint32_t)(pix + i), off);
-            if (c == 0 && at < a.order_b) a.list_b[a.order_b - 1 - at] = e.x;
-            if (c == 1 && at < a.order_b) a.list_b[at] = e.x;
-            if (c == 2 && at < a.npx) a.list_a[a.npx - 1 - at] = e;
-            if (c == 3 && at < a.npx) a.list_a[at] = e;
-        } else {   // no fragments: the background
+            if (c == 0) a.list_b[a.order_b - 1 - at] = e.x;
+            if (c == 1) a.list_b[at] = e.x;
+            if (c == 2) a.list_a[a.npx - 1 - at] = e;
+            if (c == 3) a.list_a[at] = e;
+        } else {   // no fragments, or no room for them: the background
             reinterpret_cast<float4 *>(vw.out)[lpix + i] = make_float4(a.bg0, a.bg1, a.bg2, 0.0f);
             a.tfinal[pix + i] = 1.0f;
         }
@@ -288,6 +293,7 @@ cudaError_t launch_pixel_alloc(const RenderArgs &ra, cudaStream_t st) {
     while ((1 << a.tile_shift) < L.tile) ++a.tile_shift;
     a.n_slots = (int64_t)L.n_tiles << (2 * a.tile_shift);
     a.order_b = L.order_b;
+    a.frag_cap = L.frag_cap;
     a.counts = reinterpret_cast<const uint32_t *>(ws + L.off_counts);
     a.offsets = reinterpret_cast<uint32_t *>(ws + L.off_offsets);
     a.list_a = reinterpret_cast<uint2 *>(ws + L.off_order_a);
