@@ -160,7 +160,7 @@ struct AllocArgs {
 
 __global__ void __launch_bounds__(kAllocThreads) pixel_alloc_kernel(const __grid_constant__ AllocArgs a) {
     __shared__ uint32_t s_cnt[kCountBuckets], s_at[kCountBuckets], s_warp[kAllocThreads / 32], s_class[4], s_base[4];
-    __shared__ unsigned long long s_first;
+    __shared__ unsigned long long s_sum[kAllocThreads / 32], s_first;
     static_assert(kAllocThreads == kCountBuckets, "one thread per bucket");
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     s_cnt[tid] = 0;
@@ -190,21 +190,22 @@ __global__ void __launch_bounds__(kAllocThreads) pixel_alloc_kernel(const __grid
         pix = (int64_t)vw.pix_base + lpix;
         for (int i = 0; i < in; ++i) n[i] = a.counts[pix + i];
     }
-    const uint32_t sum = n[0] + n[1] + n[2] + n[3];
-    uint32_t x = sum;
+    // (64 bits: millions of fans over one span, counted without room for their records, pass 2^32 fragments)
+    const unsigned long long sum = (unsigned long long)n[0] + n[1] + n[2] + n[3];
+    unsigned long long x = sum;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
         if (lane >= o) x += y;
     }
-    if (lane == 31) s_warp[warp] = x;
+    if (lane == 31) s_sum[warp] = x;
     __syncthreads();
-    uint32_t before = 0, total = 0;
+    unsigned long long before = 0, total = 0;
     for (int w = 0; w < kAllocThreads / 32; ++w) {
-        if (w < warp) before += s_warp[w];
-        total += s_warp[w];
+        if (w < warp) before += s_sum[w];
+        total += s_sum[w];
     }
-    if (tid == 0) s_first = total ? atomicAdd(&a.st->frags, (unsigned long long)total) : 0ull;
+    if (tid == 0) s_first = total ? atomicAdd(&a.st->frags, total) : 0ull;
     __syncthreads();
     unsigned long long run = s_first + before + x - sum;
     // rank of each pixel among the span's pixels of its count; a pixel whose records do not fit the buffer

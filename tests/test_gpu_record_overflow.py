@@ -1,5 +1,6 @@
 """A fragment buffer that is too small: the overflow is reported, and every pixel of the image is written --
-with what it holds in full where its records fit, with the background where they do not."""
+with what it holds in full where its records fit, with the background where they do not.  Fragments are
+counted in 64 bits however many there are."""
 import ctypes as C
 
 import numpy as np
@@ -56,3 +57,21 @@ def test_every_pixel_is_written(tile, room):
     assert bool((is_bg | is_full).all())
     held = int((is_full & ~is_bg).sum())
     assert held > 100 if room == 0.5 else held <= room
+
+
+def test_more_than_2_to_32_fragments_of_one_span():
+    """4.3M fans over an image of one 32 x 32 tile: every centre lies in one triangle of each."""
+    n, K = 4_300_000, 3
+    cam = synthetic.make_camera((0.0, 0.0, 3.0), 32, 32)
+    half = 3.0 * 16 / cam.fx
+    fan = half * np.array([[0.01, 0.013, 0], [8.0, 0.3, 0], [-5.0, 7.0, 0], [-4.5, -6.5, 0]])
+    xyz = torch.tensor(fan.astype(np.float32), device="cuda").repeat(n, 1)
+    rgb = torch.full_like(xyz, 0.5)
+    a = torch.full((len(xyz),), 0.25, device="cuda")
+    p = ms.render_params(tile=32, bg=(0.125, 0.25, 0.5), pair_capacity=n)
+    r = ms.BatchRenderer(n, K, [cam], p)
+    flat = r.forward(xyz, rgb, a, flat=r.new_flat(-7.0), check_status=False)
+    st, info = r.info()
+    assert st == _lib.MS_ERR_CAPACITY and info.pairs == n
+    assert info.frags == n * 1024 > info.frag_capacity
+    assert bool((flat == torch.tensor([0.125, 0.25, 0.5, 0.0], device="cuda")).all())
