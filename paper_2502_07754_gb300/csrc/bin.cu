@@ -30,7 +30,19 @@ struct BinArgs {
     float4 *dec;               // [view][vertex] decided (xr, yr, Z or -1, origin), read by the raster passes
     int64_t V;
     const uint32_t *face_mask; // per fan, bit j = face j drawn; NULL = all
+    bool splat;                // the soup holds polygons of splats (polygon_pad)
 };
+
+// How far, in pixels, the rounding of its binary32 vertices p (centre first) can draw the bounds of a splat's
+// polygon inside the splat: a vertex moves by at most 2^-22 of the centre's coordinates (the additions) and
+// 2^-20 of its offset from the centre (the rotated axes), which f + reach pixels at depth zmin magnify.
+// 1e-3 px in a scene of a few units; 0.25 px at coordinates of 1000 seen from a unit away at f = 1000.
+__device__ __forceinline__ float polygon_pad(const float *p, int K, float f_reach, float zmin) {
+    float off = 0.0f;
+    for (int i = 3; i < 3 * (K + 1); ++i) off = fmaxf(off, fabsf(p[i] - p[i % 3]));
+    const float m = fmaxf(fmaxf(fabsf(p[0]), fabsf(p[1])), fabsf(p[2]));
+    return fminf((0x1p-22f * m + 0x1p-20f * off) * f_reach / zmin, 2.0f * kGuardPx);
+}
 
 // What bounds it: arithmetic (the double-float projection, two boundary vertices at a time: 83% of issue
 // slots busy).  16 views of 3M fans, K = 6, forward and adjoint: 16.93 -> 16.62 ms against one vertex at a time in
@@ -117,6 +129,15 @@ __global__ void __launch_bounds__(kBinThreads, 4) bin_kernel(const __grid_consta
                 }
         }
         if (ntri_bad) atomicAdd(&s_culled, ntri_bad);
+        if (a.splat && tmask) {   // (kept for the count pass in the third vertex)
+            float zmin = 3.0e38f;
+            for (int k = 0; k < KV; ++k)
+                if ((vmask >> k) & 1u) zmin = fminf(zmin, dec[k].z);
+            const float reach = fmaxf(fmaxf(cam.cx - mnx, mxx - cam.cx), fmaxf(cam.cy - mny, mxy - cam.cy));
+            const float e = polygon_pad(p, K, fmaxf(fabsf(cam.fx), fabsf(cam.fy)) + fmaxf(reach, 0.0f), zmin);
+            dec[2].w = e;
+            mnx -= e; mxx += e; mny -= e; mxy += e;
+        }
         if (tmask) {
             const FanRect r = rect_from_bounds(mnx, mxx, mny, mxy, cam.width, cam.height);
             if (!r.empty) {
@@ -222,6 +243,7 @@ cudaError_t launch_bin(const RenderArgs &ra, cudaStream_t st) {
     a.dec = reinterpret_cast<float4 *>(ra.ws + L.off_dec);
     a.V = L.V;
     a.face_mask = ra.splat ? nullptr : ra.prm.face_mask;
+    a.splat = ra.splat;
     bin_kernel<<<(unsigned)L.bin_blocks, kBinThreads, smem, st>>>(a);
     return cudaGetLastError();
 }

@@ -1,8 +1,8 @@
 // Polygons that circumscribe the source Gaussians' truncation ellipses, for binning the
 // splat passes (ms_splat_render).  The regular 8-gon whose inscribed circle is the unit
-// circle, mapped by the Gaussian's scaled kept axes, contains the ellipse; the extra
-// 1e-4 relative margin keeps it containing the ellipse after binary32 rounding, so the
-// polygon's pixel rectangle and minimum depth bound every hit of the splat.
+// circle, mapped by the Gaussian's scaled kept axes and widened by 1e-4, contains the ellipse; binning
+// widens its bounds on the screen by what the rounding of the vertices can move them (polygon_pad in
+// bin.cu), so that the pixel rectangle bounds every hit of the splat.
 #include "ms_common.cuh"
 #include "ms_internal.h"
 

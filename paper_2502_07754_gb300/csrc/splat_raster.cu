@@ -153,13 +153,14 @@ __device__ __forceinline__ bool splat_values(const float4 &c, const float4 &A, c
            fabsf(tt.l) < half - tt.h * 0x1p-40f && q.h < 8.0f && q.h >= 0.0f;
 }
 
-// Pixel rectangle of a polygon (decided vertices dv) clipped to the tile, as pair_geo; 0 if empty.
+// Pixel rectangle of a polygon (decided vertices dv) clipped to the tile, as pair_geo; 0 if empty. (Far from
+// the origin the vertices of a small splat may round to one point: its centres are found within the pad.)
 __device__ __forceinline__ uint32_t polygon_geo(const float4 *__restrict__ dv, int W, int H, int tx0, int ty0, int tx1,
                                                 int ty1) {
     constexpr int K = kSplatK;
     float x[K + 1], y[K + 1];
     uint32_t vmask = 0;
-    float ox = 0.0f, oy = 0.0f;
+    float ox = 0.0f, oy = 0.0f, pad = 0.0f;
 #pragma unroll
     for (int k = 0; k <= K; ++k) {
         const float4 d = __ldg(dv + k);
@@ -168,25 +169,19 @@ __device__ __forceinline__ uint32_t polygon_geo(const float4 *__restrict__ dv, i
         if (d.z > 0.0f) vmask |= 1u << k;   // binning marks invalid vertices with Z = -1
         if (k == 0) ox = d.w;
         if (k == 1) oy = d.w;
+        if (k == 2) pad = d.w;
     }
     const uint32_t tmask = tri_valid_mask(vmask, K);
     if (tmask == 0) return 0;
     float mnx = 3.0e38f, mxx = -3.0e38f, mny = 3.0e38f, mxy = -3.0e38f;
-    bool area = false;
 #pragma unroll
     for (int k = 0; k <= K; ++k) {
         if (!vertex_used(tmask, k, K)) continue;
         mnx = fminf(mnx, x[k]); mxx = fmaxf(mxx, x[k]);
         mny = fminf(mny, y[k]); mxy = fmaxf(mxy, y[k]);
     }
-#pragma unroll
-    for (int j = 0; j < K; ++j) {
-        const int b = 1 + j, n = j + 1 == K ? 1 : 2 + j;
-        const float ar = dec_area2(x[0], y[0], x[b], y[b], x[n], y[n]);
-        area |= ar < 0.0f || (((tmask >> j) & 1u) && ar != 0.0f);
-    }
-    const FanRect r = rect_from_bounds_rel(mnx, mxx, mny, mxy, (int)ox, (int)oy, W, H);
-    if (r.empty || !area) return 0;
+    const FanRect r = rect_from_bounds_rel(mnx - pad, mxx + pad, mny - pad, mxy + pad, (int)ox, (int)oy, W, H);
+    if (r.empty) return 0;
     const int x0 = max(r.i0, tx0), x1 = min(r.i1, tx1), y0 = max(r.j0, ty0), y1 = min(r.j1, ty1);
     if (x0 > x1 || y0 > y1) return 0;
     return pair_geo(x0 - tx0, y0 - ty0, x1 - x0 + 1, y1 - y0 + 1);
