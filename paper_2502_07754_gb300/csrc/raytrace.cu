@@ -504,7 +504,7 @@ constexpr int kJobs = kTraceKB<true> * kTracePix;
 struct Jobs {
     float2 o[3][kJobs];                // origin (the segment runs to the light)
     float2 S[kJobs];                   // transmittance
-    int tri[kJobs];                    // the crossing's own triangle
+    int tri[kJobs];                    // the crossing's own triangle; -1 once the light is blocked to within T_eps
     uint16_t list[kJobs];              // slots in use
     int n, next;
 };
@@ -609,22 +609,28 @@ __device__ __forceinline__ void shadow_jobs(const TraceArgs &a, Jobs &J, WarpRin
                 }
                 head += nj;
                 queued -= nj;
-                // a segment's factors in the order it met them, by the first of their lanes
+                // a segment's factors in the order it met them, by the first of their lanes, up to the one
+                // that blocks the light to within T_eps: the colour's shadow factor moves by at most
+                // (1 - ambient) T_eps, the primary composite's own termination bound (what comes after
+                // is left out whenever it is tested, so the product does not depend on the warp's other
+                // segments)
                 unsigned same = __match_any_sync(0xffffffffu, at);
                 __syncwarp();
-                if (at >= 0 && lane == __ffs(same) - 1) {
+                if (at >= 0 && lane == __ffs(same) - 1 && J.tri[at] >= 0) {
                     dfl S = dfl{J.S[at].x, J.S[at].y};
                     for (; same; same &= same - 1) {
                         const float2 f = R.t[__ffs(same) - 1];
                         S = df_mul(S, dfl{f.x, f.y});
+                        if (df_lt(S, df_make(a.T_epsf))) {
+                            J.tri[at] = -1;
+                            break;
+                        }
                     }
                     J.S[at] = make_float2(S.h, S.l);
                 }
                 __syncwarp();
             }
-            // the light is blocked to within T_eps: the colour's shadow factor moves by at
-            // most (1 - ambient) T_eps, the primary composite's own termination bound
-            if (node >= 0 && J.S[slot].x < a.T_epsf) node = -1;
+            if (node >= 0 && J.tri[slot] < 0) node = -1;   // (the lane's own segment: it takes the next)
         }
         if (!more) break;
     }
