@@ -798,10 +798,10 @@ trace_kernel(const __grid_constant__ TraceArgs a) {
                 }
                 if (!walking) break;
             }
-            // the crossings that will be composited
+            // the crossings that will be composited: up to the one that takes T below T_eps
             {
                 double Tn = T;
-                for (; n_use < nb && !(Tn < a.T_eps); ++n_use) {
+                for (bool on = true; on && n_use < nb; ++n_use, on = !(Tn < a.T_eps)) {
                     const Hit &h = buf[n_use];
                     int64_t v[3];
                     tri_verts(a.tris, a.K, h.tri, v);

@@ -1,5 +1,6 @@
 """Where a shadow segment stops: its transmittance is the product of the factors up to the first that takes it
-below T_eps, in the order of the walk -- not of however many the warp had tested by then."""
+below T_eps, in the order of the walk -- not of however many the warp had tested by then; and the first crossing
+of a ray counts whatever the bound."""
 import numpy as np
 import pytest
 
@@ -56,3 +57,10 @@ def test_transmittance_stops_at_the_factor_that_blocks(layer_alpha, T_eps, facto
     got = (img[seen, 0] / (0.75 * 0.5) - 0.25) / 0.75      # transmittance of every segment
     want = (1.0 - layer_alpha) ** factors
     assert np.abs(got - want).max() <= 1e-6
+
+
+def test_first_factor_and_first_crossing_count_whatever_the_bound():
+    """A bound above 1 ends a composite after its first crossing and a segment after its first factor."""
+    img = _trace(0.5, 2.0)
+    assert np.abs(img[..., 3] - 0.75).max() <= 1e-6
+    assert np.abs((img[..., 0] / (0.75 * 0.5) - 0.25) / 0.75 - 0.5).max() <= 1e-6
