@@ -428,8 +428,10 @@ __device__ __forceinline__ bool crosses_exactly(const double o[3], const double 
     return mt(o, d, Q[0], Q[1], Q[2], t, u, v);
 }
 // Whether the segment crosses triangle P inside its ends: the binary32 filter, then double-float, then
-// FP64 where neither is certain.
-__device__ __forceinline__ bool segment_crosses(const RayF &rf, const float P[3][3], SegHit &h) {
+// FP64 where neither is certain, from the segment's own FP64 ends (rest: what its double-float origin
+// leaves of the FP64 one).
+__device__ __forceinline__ bool segment_crosses(const RayF &rf, const float rest[3], const float light[3],
+                                                const float P[3][3], SegHit &h) {
     MtBounds e;
     if (!mt_may_hit(rf, P[0], P[1], P[2], (float)kSegEps, (float)(1.0 - kSegEps), e)) return false;
     const int c = mt_df(rf, P[0], P[1], P[2], e, df_of(kSegEps), df_of(1.0 - kSegEps), h);
@@ -437,8 +439,8 @@ __device__ __forceinline__ bool segment_crosses(const RayF &rf, const float P[3]
     double o[3], d[3], t, u, v;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        o[k] = to_double(rf.o[k]);
-        d[k] = to_double(rf.d[k]);
+        o[k] = to_double(rf.o[k]) + (double)rest[k];
+        d[k] = (double)light[k] - o[k];
     }
     if (!(crosses_exactly(o, d, P, t, u, v) && t > kSegEps && t < 1.0 - kSegEps)) return false;
     h.u = df_of(u);
@@ -509,18 +511,23 @@ __device__ __forceinline__ dfl bary_mix(dfl u, dfl v, float a0, float a1, float 
 // A warp's ring of triangles that passed the filter, and what the exact tests made of 32.
 struct WarpRing {
     uint2 job[64];            // (lane or segment slot, triangle)
-    double t[32], u[32], v[32];   // rays: crossings
+    union {
+        double t[32];         // rays: crossings,
+        float2 f[32];         // segments: factors of their transmittance
+    };
+    double u[32], v[32];
     unsigned mine[32];        // rays: per lane of the warp, its crossings among the 32
-    float2 f[32];             // segments: factors of their transmittance
 };
 struct Block {
     double d[3][kTracePix];      // the pixels' ray directions
 };
 static_assert(sizeof(Block) % 16 == 0 && sizeof(WarpRing) % 16 == 0, "shared memory alignment");
-// Shadow segments of one block's crossings of one pass, a slot per (crossing, pixel).
+// Shadow segments of one block's crossings of one pass, a slot per (crossing, pixel). (With 31 KB a block the SM's
+// five leave the nodes a 92 KB L1; with 33 KB the next size down, and the segments take 6% longer.)
 constexpr int kJobs = kTraceKB<true> * kTracePix;
 struct Jobs {
-    float2 o[3][kJobs];                // origin (the segment runs to the light)
+    float2 o[3][kJobs];                // origin (the segment runs to the light),
+    float rest[3][kJobs];              // and its bits below double-float
     float2 S[kJobs];                   // transmittance
     int tri[kJobs];                    // the crossing's own triangle; -1 once the light is blocked to within T_eps
     uint16_t list[kJobs];              // slots in use
@@ -616,7 +623,8 @@ __device__ __forceinline__ void shadow_jobs(const TraceArgs &a, Jobs &J, WarpRin
                     float P[3][3];
                     tri_f(a, (int)job.y, P);
                     SegHit h;
-                    if (segment_crosses(jr, P, h)) {
+                    const float rest[3] = {J.rest[0][job.x], J.rest[1][job.x], J.rest[2][job.x]};
+                    if (segment_crosses(jr, rest, a.Lf, P, h)) {
                         int64_t v[3];
                         tri_verts(a.tris, a.K, (int)job.y, v);
                         const dfl al = bary_mix(h.u, h.v, __ldg(a.alpha + v[0]), __ldg(a.alpha + v[1]), __ldg(a.alpha + v[2]));
@@ -837,8 +845,10 @@ trace_kernel(const __grid_constant__ TraceArgs a) {
                         J.tri[slot] = buf[k].tri;
 #pragma unroll
                         for (int r = 0; r < 3; ++r) {
-                            const dfl pf = df_of((double)c.C[r] + buf[k].t * B.d[r][lane]);
+                            const double p = (double)c.C[r] + buf[k].t * B.d[r][lane];
+                            const dfl pf = df_of(p);
                             J.o[r][slot] = make_float2(pf.h, pf.l);
+                            J.rest[r][slot] = (float)(p - to_double(pf));
                         }
                     }
                     n += __popc(m);
