@@ -192,7 +192,7 @@ __device__ __forceinline__ uint32_t resolve_group(const ResolveArgs &a, GroupMem
     const int lane = threadIdx.x & 31, sub = lane & (G - 1), g0 = lane & ~(G - 1);
     const bool valid = is_pixel(a, e);
     const int64_t off = e.off;
-    const int n = (int)e.n;   // (at most G)
+    const int n = e.n <= (uint32_t)G ? (int)e.n : 0;   // (it is: a bound the loops below are unrolled by)
     const int nmax = __reduce_max_sync(0xffffffffu, n);
     const bool has = sub < n;
     float4 r0 = make_float4(0.f, 0.f, 0.f, 0.f), r1 = r0;
