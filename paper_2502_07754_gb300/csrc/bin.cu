@@ -33,15 +33,22 @@ struct BinArgs {
     bool splat;                // the soup holds polygons of splats (polygon_pad)
 };
 
-// How far, in pixels, the rounding of its binary32 vertices p (centre first) can draw the bounds of a splat's
-// polygon inside the splat: a vertex moves by at most 2^-22 of the centre's coordinates (the additions) and
-// 2^-20 of its offset from the centre (the rotated axes), which f + reach pixels at depth zmin magnify.
+// How far, in pixels, the rounding of its binary32 vertices p (centre first, at depth zc) can draw the bounds of a
+// splat's polygon inside the splat: a vertex moves by at most 2^-22 of the centre's coordinates (the
+// additions) and 2^-20 of its offset from the centre (the rotated axes; no component of an offset exceeds the sum of
+// those of the first and third boundary vertices, which lie on the axes), magnified by f + reach pixels at the least depth.
 // 1e-3 px in a scene of a few units; 0.25 px at coordinates of 1000 seen from a unit away at f = 1000.
-__device__ __forceinline__ float polygon_pad(const float *p, int K, float f_reach, float zmin) {
-    float off = 0.0f;
-    for (int i = 3; i < 3 * (K + 1); ++i) off = fmaxf(off, fabsf(p[i] - p[i % 3]));
-    const float m = fmaxf(fmaxf(fabsf(p[0]), fabsf(p[1])), fabsf(p[2]));
-    return fminf((0x1p-22f * m + 0x1p-20f * off) * f_reach / zmin, 2.0f * kGuardPx);
+__device__ __forceinline__ float polygon_pad(const float *p, const CamDev &c, float zc, float reach) {
+    float m = 0.0f, off = 0.0f, dz = 0.0f;
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+        const float o = fabsf(p[3 + r] - p[r]) + fabsf(p[9 + r] - p[r]);
+        m = fmaxf(m, fabsf(p[r]));
+        off = fmaxf(off, o);
+        dz = fmaf(fabsf(c.R[6 + r]), o, dz);
+    }
+    const float f = fmaxf(fabsf(c.fx), fabsf(c.fy)) + reach;
+    return fminf(__fdividef((0x1p-22f * m + 0x1p-20f * off) * f, fmaxf(zc - dz, c.znear)), 2.0f * kGuardPx);
 }
 
 // What bounds it: arithmetic (the double-float projection, two boundary vertices at a time: 83% of issue
@@ -130,11 +137,8 @@ __global__ void __launch_bounds__(kBinThreads, 4) bin_kernel(const __grid_consta
         }
         if (ntri_bad) atomicAdd(&s_culled, ntri_bad);
         if (a.splat && tmask) {   // (kept for the count pass in the third vertex)
-            float zmin = 3.0e38f;
-            for (int k = 0; k < KV; ++k)
-                if ((vmask >> k) & 1u) zmin = fminf(zmin, dec[k].z);
             const float reach = fmaxf(fmaxf(cam.cx - mnx, mxx - cam.cx), fmaxf(cam.cy - mny, mxy - cam.cy));
-            const float e = polygon_pad(p, K, fmaxf(fabsf(cam.fx), fabsf(cam.fy)) + fmaxf(reach, 0.0f), zmin);
+            const float e = polygon_pad(p, cam, c0.Z.h, fmaxf(reach, 0.0f));
             dec[2].w = e;
             mnx -= e; mxx += e; mny -= e; mxy += e;
         }
