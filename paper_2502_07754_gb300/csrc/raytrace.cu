@@ -522,8 +522,8 @@ struct Block {
     double d[3][kTracePix];      // the pixels' ray directions
 };
 static_assert(sizeof(Block) % 16 == 0 && sizeof(WarpRing) % 16 == 0, "shared memory alignment");
-// Shadow segments of one block's crossings of one pass, a slot per (crossing, pixel). (With 31 KB a block the SM's
-// five leave the nodes a 92 KB L1; with 33 KB the next size down, and the segments take 6% longer.)
+// Shadow segments of one block's crossings of one pass, a slot per (crossing, pixel). (31 KB a block: with 33 KB, and
+// the smaller L1 that five such blocks leave an SM, the segments take 6% longer.)
 constexpr int kJobs = kTraceKB<true> * kTracePix;
 struct Jobs {
     float2 o[3][kJobs];                // origin (the segment runs to the light),
