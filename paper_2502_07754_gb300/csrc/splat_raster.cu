@@ -15,10 +15,13 @@
 //  * the decision is taken in binary32 where it is certain by a margin of 32 units of 2^-24 of
 //    the summed magnitudes, and by the FP64 test itself in the few cases left (a few per
 //    100,000, plus every degenerate splat: its coefficients are not finite);
-//  * depth and opacity of a hit are computed in double-float by whole warps of hits; where the
-//    depth lies within 2^-40 of a tie of its rounding to the binary32 order key, the FP64
-//    values are taken.  So decisions and order keys are those of the FP64 test, and opacities
-//    are within a 2^-30 of its values before the last rounding.
+//  * depth and opacity of a hit are computed in double-float by whole warps of hits, with a bound on
+//    their error: that of D's summed magnitudes, of the centre's rounded position times the slopes
+//    (a centre at 30000 px of a plane 5 px from edge-on is off by 2^-35 of D), and of FP64's own
+//    cancellation edge-on. Where it exceeds 2^-40 of D, and where the depth lies that close to a tie of its
+//    rounding to the binary32 order key, the FP64 values are taken.  So decisions and order
+//    keys are those of the FP64 test, and opacities are within 2^-30 of its values before the last
+//    rounding.
 // What bounds it: issue slots.  250k Gaussians into eight 1080p views (120M tests, 68M hits): setup
 // 0.60 ms (FP64), count 0.90 ms, fill 1.75 ms; with every test, setup and value in FP64 the two
 // passes took 20 and 34 ms.
@@ -56,7 +59,8 @@ __device__ __forceinline__ float2 split(double x) {
 }
 
 // Coefficients of every (view, Gaussian), one thread a Gaussian: [0] centre x, y; [1] a1, a2;
-// [2] b1, b2; [3] d1, d2 (double-float pairs); [4] Z_c, sigma, 0.
+// [2] b1, b2; [3] d1, d2 (double-float pairs); [4] Z_c, sigma, error of D (and 2^-8 of that of u and v) that
+// does not depend on the pixel.
 constexpr int kSetupThreads = 128;
 __global__ void __launch_bounds__(kSetupThreads) splat_setup_kernel(const SplatSrc s, int64_t N,
                                                                     const __grid_constant__ ViewTable vt,
@@ -83,9 +87,15 @@ __global__ void __launch_bounds__(kSetupThreads) splat_setup_kernel(const SplatS
         const float2 b2 = split((o.mcn * o.ub[1] - mub * o.n[1]) * (iy * isb));
         w[2] = make_float4(b1.x, b1.y, b2.x, b2.y);
         const float2 d1 = split(o.n[0] * ix), d2 = split(o.n[1] * iy);
-        w[3] = make_float4(d1.x, d1.y, d2.x, d2.y);
         const float2 z = split(o.mc[2]);
-        w[4] = make_float4(z.x, z.y, ax.sigma, 0.0f);
+        // the centre's position is rounded by 2^-48 of it, n . d_centre by a few 2^-53 of its terms
+        const float X = fabsf(xc.x), Y = fabsf(yc.x), G = (1.0f + fabsf((xc.x - c.cx) / c.fx) + fabsf((yc.x - c.cy) / c.fy)) * fabsf((float)iD);
+        const float err = 0x1p-48f * (fabsf(d1.x) * X + fabsf(d2.x) * Y) + 0x1p-50f * G +
+                          0x1p-56f * ((fabsf(a1.x) + fabsf(b1.x)) * X + (fabsf(a2.x) + fabsf(b2.x)) * Y);
+        // (a splat whose binary32 decisions that could reach is left to FP64 altogether, like one whose
+        // coefficients are not finite)
+        w[3] = make_float4(err < 0x1p-34f ? d1.x : __int_as_float(0x7fffffff), d1.y, d2.x, d2.y);
+        w[4] = make_float4(z.x, z.y, ax.sigma, err);
     }
 }
 
@@ -137,8 +147,8 @@ __device__ __forceinline__ dfl df_exp(dfl x) {
 __device__ __forceinline__ bool splat_values(const float4 &c, const float4 &A, const float4 &B, const float4 &Dc,
                                              const float4 &Z, float px, float py, float &t, float &al) {
     const dfl dx = df_add_f(df_two_sum(px, -c.x), -c.y), dy = df_add_f(df_two_sum(py, -c.z), -c.w);
-    const dfl Nu = df_add_fast(df_mul(dfl{A.x, A.y}, dx), df_mul(dfl{A.z, A.w}, dy));
-    const dfl Nv = df_add_fast(df_mul(dfl{B.x, B.y}, dx), df_mul(dfl{B.z, B.w}, dy));
+    const dfl p0 = df_mul(dfl{A.x, A.y}, dx), p1 = df_mul(dfl{A.z, A.w}, dy), Nu = df_add_fast(p0, p1);
+    const dfl q0 = df_mul(dfl{B.x, B.y}, dx), q1 = df_mul(dfl{B.z, B.w}, dy), Nv = df_add_fast(q0, q1);
     const dfl e0 = df_mul(dfl{Dc.x, Dc.y}, dx), e1 = df_mul(dfl{Dc.z, Dc.w}, dy);
     const dfl D = df_add_f(df_add_fast(e0, e1), 1.0f);
     const dfl tt = df_div_rcp(dfl{Z.x, Z.y}, D);
@@ -146,11 +156,14 @@ __device__ __forceinline__ bool splat_values(const float4 &c, const float4 &A, c
     const dfl a = df_mul_f(df_exp(dfl{-0.5f * q.h, -0.5f * q.l}), Z.z);
     t = tt.h;
     al = __fadd_rn(a.h, a.l);
+    // errors: of D at most err; of Nu and Nv together 2^8 err; so of t err / D, of q 1400 err / D (q < 8)
+    const float err = Z.w + 0x1p-44f * (1.0f + fabsf(e0.h) + fabsf(e1.h)) +
+                      0x1p-52f * ((fabsf(p0.h) + fabsf(p1.h)) + (fabsf(q0.h) + fabsf(q1.h)));
     // tt.h is the rounding of the depth unless its low part reaches half a unit of tt.h
     const uint32_t tb = __float_as_uint(tt.h);
     const float half = __uint_as_float(tb & 0x7f800000u) * 0x1p-24f;
-    return D.h > 0.001f * (1.0f + fabsf(e0.h) + fabsf(e1.h)) && (tb & 0x007fffffu) != 0u &&
-           fabsf(tt.l) < half - tt.h * 0x1p-40f && q.h < 8.0f && q.h >= 0.0f;
+    return err < 0x1p-40f * D.h && (tb & 0x007fffffu) != 0u &&
+           fabsf(tt.l) * D.h < half * D.h - tt.h * fmaf(D.h, 0x1p-45f, err) && q.h < 8.0f && q.h >= 0.0f;
 }
 
 // Pixel rectangle of a polygon (decided vertices dv) clipped to the tile, as pair_geo; 0 if empty. (Far from
