@@ -300,9 +300,17 @@ static ms_status render_views_backward(const float *xyz, const float *rgb, const
 constexpr double kSplatTrunc = 2.7;           // truncation radius in scales (the fan's scale_mul)
 
 static size_t splat_poly_bytes(int64_t N) { return align_up((size_t)N * (kSplatK + 1) * 12, 256); }
-// what a splat workspace holds beyond the render layout: polygons, then coefficients
-static size_t splat_extra_bytes(int64_t N, int n_views) {
-    return splat_poly_bytes(N) + align_up(splat_coef_bytes(N, n_views), 256);
+// Where the coefficients lie: in the adjoint records or the gradients, which this forward-only render leaves
+// unused, if either holds them, else behind the polygons.
+static size_t splat_coef_offset(const RenderLayout &L) {
+    const size_t bytes = splat_coef_bytes(L.n_fans, L.n_views);
+    if (bytes <= 32 * (size_t)L.frag_cap) return L.off_adj;
+    if (bytes <= 32 * (size_t)L.V) return L.off_grad;
+    return L.total + splat_poly_bytes(L.n_fans);
+}
+static size_t splat_total_bytes(const RenderLayout &L) {
+    const size_t polys = L.total + splat_poly_bytes(L.n_fans);
+    return splat_coef_offset(L) < polys ? polys : polys + align_up(splat_coef_bytes(L.n_fans, L.n_views), 256);
 }
 
 static ms_status splat_views(const float *means, const float *log_scales, const float *quats, const float *opacity,
@@ -317,10 +325,11 @@ static ms_status splat_views(const float *means, const float *log_scales, const 
     if (N >= (1ll << 31)) return fail(MS_ERR_INVALID, "too many Gaussians");
     RenderLayout L;
     // the layout check sees a placeholder soup pointer: the polygons are made below
-    const size_t extra = N > 0 && n_views > 0 ? splat_extra_bytes(N, n_views) : 0;
     ms_status s = check_render_args(N > 0 ? means : nullptr, means, means, N, kSplatK, cams, n_views, p, workspace,
-                                    ws_bytes > extra ? ws_bytes - extra : 0, L);
+                                    ws_bytes, L);
     if (s != MS_OK) return s;
+    if (ws_bytes < splat_total_bytes(L))
+        return fail(MS_ERR_INVALID, "workspace %zu bytes < %zu needed", ws_bytes, splat_total_bytes(L));
     if (!out) return fail(MS_ERR_INVALID, "output image list is NULL");
     for (int v = 0; v < n_views; ++v)
         if (!out[v] || !aligned16(out[v])) return fail(MS_ERR_INVALID, "view %d: output image NULL or not 16-byte aligned", v);
@@ -332,7 +341,7 @@ static ms_status splat_views(const float *means, const float *log_scales, const 
     memset(&a, 0, sizeof(a));
     a.xyz = poly; a.n_fans = N; a.K = kSplatK; a.prm = p; a.L = L; a.ws = ws;
     a.splat = true;
-    a.splat_coef = reinterpret_cast<float4 *>(ws + L.total + splat_poly_bytes(N));
+    a.splat_coef = reinterpret_cast<float4 *>(ws + splat_coef_offset(L));
     a.spl.means = means; a.spl.log_scales = log_scales; a.spl.quats = quats; a.spl.opacity = opacity;
     a.spl.rgb = rgb; a.spl.axis_rule = axis_rule; a.spl.trunc = kSplatTrunc;
     a.vt = make_views(cams, n_views, L, out, nullptr, nullptr);
@@ -549,8 +558,10 @@ MS_API ms_status ms_batch_render_backward(const float *xyz, const float *rgb, co
 
 MS_API size_t ms_splat_workspace_size(int64_t N, const ms_camera *cams, int32_t n_views,
                                       const ms_render_params *params) {
-    const size_t base = ms_batch_workspace_size(N, kSplatK, cams, n_views, params);
-    return base ? base + splat_extra_bytes(N, n_views) : 0;
+    if (ms_batch_workspace_size(N, kSplatK, cams, n_views, params) == 0) return 0;
+    ms_render_params p;
+    params_or_default(params, p);
+    return splat_total_bytes(render_layout(N, kSplatK, cams, n_views, p));
 }
 
 MS_API ms_status ms_splat_render(const float *means, const float *log_scales, const float *quats,
