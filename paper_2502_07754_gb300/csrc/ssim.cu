@@ -2,13 +2,13 @@
 // per colour channel under an 11 x 11 Gaussian window (sigma 1.5, zero padding outside
 // the image, C1 = 0.01^2, C2 = 0.03^2) averaged over the pixels and the three channels.
 //
-// Two launches over 32 x 32 output tiles, each staging a 42 x 42 window of its inputs in
-// shared memory (the forward stages the three channels of image and target in one pass)
-// and applying the separable window as a row pass then a column pass.  A thread takes eight
+// Two launches, over 32 x 16 (forward) and 32 x 32 output tiles, each staging a window of its inputs five
+// pixels wider on each side in shared memory (the forward stages the three channels of image and
+// target in one pass) and applying the separable window as a row pass then a column pass.  A thread takes eight
 // neighbouring outputs of the row pass and four of the column pass, so a staged value is loaded
 // once for the up to eleven products it enters, and the sums go two at a time through packed f32x2
 // multiply-adds.  At 1080p the two launches take
-// 0.083 + 0.080 ms, against 0.157 + 0.161 ms with one output a thread on 16 x 16 tiles (273 shared loads
+// 0.084 + 0.080 ms, against 0.157 + 0.161 ms with one output a thread on 16 x 16 tiles (273 shared loads
 // a pixel); issue slots bound them, at 26% of the HBM bandwidth.
 //
 // ssim_fwd_kernel: per channel the raw local moments (x, y, x^2, y^2, xy), the SSIM map,
@@ -17,8 +17,9 @@
 //     G2 = dS/ds_xx = -S/D,  G3 = dS/ds_xy = 2A/(CD),
 //     G1 = dS/dmu_x - 2 mu_x G2 - mu_y G3,  dS/dmu_x = 2 mu_y B/(CD) - 2 mu_x S/C,
 //   written as nine planes; the block's share of the loss is added to *loss.  The
-//   moments are taken of x - r_x and y - r_y with one reference value per tile (a pixel
-//   near its centre; outside the image the padded zeros become -r): the local
+//   moments are taken of x - r_x and y - r_y with one reference value per 16 x 16 square (a pixel
+//   near its centre; outside the image the padded zeros become -r; one value for 32 x 32 pixels, as forward tiles of
+//   that size had, nearly doubled the gradient's error on steep smooth images, for the same time): the local
 //   (co)variances do not depend on the shift, and E[x^2] - mu^2 then cancels against the
 //   local contrast instead of against the brightness.
 // ssim_bwd_kernel: dSSIM/dx_p = (1/N) [(w * G1)(p) + 2 x_p (w * G2)(p) + y_p (w * G3)(p)],
@@ -38,6 +39,10 @@ constexpr int kIn = kT + 2 * kR;         // staged tile edge (42)
 constexpr int kThreads = 256;
 constexpr int kRow = 8, kCol = kT * kT / kThreads;   // outputs of a thread in the row and column pass
 constexpr int kRowTasks = kIn * (kT / kRow);
+// The forward takes 32 x 16 outputs, two 16 x 16 squares with a reference value each.
+constexpr int kFH = 16, kFIn = kFH + 2 * kR, kFThreads = 128;
+constexpr int kFRowTasks = kFIn * (kT / kRow);
+static_assert(kT * kFH / kFThreads == kCol && kFRowTasks <= kFThreads, "forward tile");
 constexpr float kC1 = 0.0001f, kC2 = 0.0009f;
 
 struct Window {
@@ -63,6 +68,7 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
     return d;
 }
 
+template <int THREADS>
 __device__ __forceinline__ float block_sum(float v, float *s_red) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -71,7 +77,7 @@ __device__ __forceinline__ float block_sum(float v, float *s_red) {
     __syncthreads();
     float t = 0.0f;
     if (tid < 32) {
-        t = tid < kThreads / 32 ? s_red[tid] : 0.0f;
+        t = tid < THREADS / 32 ? s_red[tid] : 0.0f;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
     }
@@ -81,11 +87,12 @@ __device__ __forceinline__ float block_sum(float v, float *s_red) {
 // (rows are consecutive over the lanes of the row pass, columns over those of the column pass: the
 // odd row lengths keep both free of bank conflicts)
 struct FwdMem {
-    float2 in[3][kIn][kIn + 1];      // (x, y) of a channel, shifted
-    float2 h01[kIn][kT + 1];         // row sums of x and y,
-    float2 h23[kIn][kT + 1];         // of x^2 and y^2,
-    float h4[kIn][kT + 1];           // and of x y
-    float red[kThreads / 32];
+    float2 in[3][kFIn][kIn + 1];     // (x, y) of a channel
+    float2 h01[kFIn][kT + 1];        // row sums of x and y, about the square's reference,
+    float2 h23[kFIn][kT + 1];        // of x^2 and y^2,
+    float h4[kFIn][kT + 1];          // and of x y
+    float2 ref[2][3];                // each square's reference (x, y) of a channel
+    float red[kFThreads / 32];
 };
 
 // The loss over the blocks, summed in FP64: thousands of binary32 additions to one word would
@@ -95,38 +102,42 @@ struct LossSum {
     unsigned done, pad;
 };
 
-__global__ void __launch_bounds__(kThreads, 3) ssim_fwd_kernel(const float4 *__restrict__ img, const float4 *__restrict__ tgt,
+__global__ void __launch_bounds__(kFThreads, 5) ssim_fwd_kernel(const float4 *__restrict__ img, const float4 *__restrict__ tgt,
                                                             int H, int W, float lam, float inv_n, Window win,
                                                             float *__restrict__ G, LossSum *total,
                                                             float *__restrict__ loss) {
-    extern __shared__ __align__(16) char smem[];
-    FwdMem &S = *reinterpret_cast<FwdMem *>(smem);
+    __shared__ FwdMem S;
     const int tid = threadIdx.x;
-    const int x0 = blockIdx.x * kT, y0 = blockIdx.y * kT;
+    const int x0 = blockIdx.x * kT, y0 = blockIdx.y * kFH;
     const size_t plane = (size_t)H * W;
     float acc = 0.0f;
-    const size_t ref = (size_t)min(y0 + kT / 2, H - 1) * W + min(x0 + kT / 2, W - 1);
-    const float4 rxv = img[ref], ryv = tgt[ref];
+    if (tid < 2) {
+        const size_t ref = (size_t)min(y0 + kFH / 2, H - 1) * W + min(x0 + kFH / 2 + kFH * tid, W - 1);
+        const float4 rx = img[ref], ry = tgt[ref];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) S.ref[tid][c] = make_float2(chan(rx, c), chan(ry, c));
+    }
     // one pass over the window stages all three channels (each RGBA pixel loaded once)
-    for (int i = tid; i < kIn * kIn; i += kThreads) {
+    for (int i = tid; i < kFIn * kIn; i += kFThreads) {
         const int ly = i / kIn, lx = i - ly * kIn;
         const int gx = x0 - kR + lx, gy = y0 - kR + ly;
         float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
         if (gx >= 0 && gx < W && gy >= 0 && gy < H) {
             a = img[(size_t)gy * W + gx];
             b = tgt[(size_t)gy * W + gx];
-            if (lx >= kR && lx < kR + kT && ly >= kR && ly < kR + kT)
+            if (lx >= kR && lx < kR + kT && ly >= kR && ly < kR + kFH)
                 acc += lam * (fabsf(a.x - b.x) + fabsf(a.y - b.y) + fabsf(a.z - b.z));
         }
 #pragma unroll
-        for (int c = 0; c < 3; ++c) S.in[c][ly][lx] = make_float2(chan(a, c) - chan(rxv, c), chan(b, c) - chan(ryv, c));
+        for (int c = 0; c < 3; ++c) S.in[c][ly][lx] = make_float2(chan(a, c), chan(b, c));
     }
     __syncthreads();
     const int tx = tid & 31, ty = (tid >> 5) * kCol;
     const int px = x0 + tx;
     for (int c = 0; c < 3; ++c) {
-        if (tid < kRowTasks) {
-            const int seg = tid / kIn, r = tid - seg * kIn;
+        if (tid < kFRowTasks) {
+            const int seg = tid / kFIn, r = tid - seg * kFIn;
+            const float2 ref = S.ref[seg * kRow / kFH][c];
             float2 s01[kRow], s23[kRow];
             float s4[kRow];
 #pragma unroll
@@ -136,7 +147,8 @@ __global__ void __launch_bounds__(kThreads, 3) ssim_fwd_kernel(const float4 *__r
             }
 #pragma unroll
             for (int t = 0; t < kRow + 2 * kR; ++t) {
-                const float2 v = S.in[c][r][seg * kRow + t];
+                const float2 in = S.in[c][r][seg * kRow + t];
+                const float2 v = make_float2(in.x - ref.x, in.y - ref.y);
                 const float2 vv = mul2(v, v);
                 const float xy = v.x * v.y;
 #pragma unroll
@@ -176,7 +188,7 @@ __global__ void __launch_bounds__(kThreads, 3) ssim_fwd_kernel(const float4 *__r
                     m4[j] = fmaf(w, d, m4[j]);
                 }
         }
-        const float rx = chan(rxv, c), ry = chan(ryv, c);
+        const float rx = S.ref[tx / kFH][c].x, ry = S.ref[tx / kFH][c].y;
 #pragma unroll
         for (int j = 0; j < kCol; ++j) {
             const int py = y0 + ty + j;
@@ -199,7 +211,7 @@ __global__ void __launch_bounds__(kThreads, 3) ssim_fwd_kernel(const float4 *__r
         }
         __syncthreads();   // the next channel's row pass overwrites the row sums
     }
-    const float t = block_sum(acc, S.red);
+    const float t = block_sum<kFThreads>(acc, S.red);
     if (tid == 0) {
         atomicAdd(&total->sum, (double)t * (double)inv_n);
         __threadfence();
@@ -329,14 +341,12 @@ cudaError_t launch_ssim_loss(const float *img, const float *tgt, int H, int W, f
     float *G = reinterpret_cast<float *>(total + 1);
     cudaError_t e = cudaMemsetAsync(total, 0, sizeof(LossSum), st);
     if (e != cudaSuccess) return e;
-    const dim3 grid((W + kT - 1) / kT, (H + kT - 1) / kT), block(kThreads);
+    const dim3 grid((W + kT - 1) / kT, (H + kT - 1) / kT), fwd_grid(grid.x, (H + kFH - 1) / kFH);
     const float inv_n = (float)(1.0 / (3.0 * (double)H * (double)W));
     const Window win = make_window();
-    e = cudaFuncSetAttribute(ssim_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(FwdMem));
-    if (e != cudaSuccess) return e;
-    ssim_fwd_kernel<<<grid, block, sizeof(FwdMem), st>>>(reinterpret_cast<const float4 *>(img), reinterpret_cast<const float4 *>(tgt),
+    ssim_fwd_kernel<<<fwd_grid, kFThreads, 0, st>>>(reinterpret_cast<const float4 *>(img), reinterpret_cast<const float4 *>(tgt),
                                             H, W, lam, inv_n, win, G, total, loss);
-    ssim_bwd_kernel<<<grid, block, 0, st>>>(reinterpret_cast<const float4 *>(img), reinterpret_cast<const float4 *>(tgt),
+    ssim_bwd_kernel<<<grid, kThreads, 0, st>>>(reinterpret_cast<const float4 *>(img), reinterpret_cast<const float4 *>(tgt),
                                             H, W, lam, inv_n, win, G, reinterpret_cast<float4 *>(dL));
     return cudaGetLastError();
 }
