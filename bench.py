@@ -73,7 +73,7 @@ def parse():
     p.add_argument("--no-other-workloads", action="store_true",
                    help="skip the compact measurements of the other configurations")
     p.add_argument("--tile", type=int, default=16, help="screen tile edge (single-view workloads; batch workloads with --no-autotune)")
-    p.add_argument("--kbuf", type=int, default=8, help="per-pixel pending buffer (single-view workloads; batch workloads with --no-autotune)")
+    p.add_argument("--kbuf", type=int, default=8, help="8 or 16; has no effect on the render (kept with the interface)")
     p.add_argument("--pairs-per-scene", type=int, default=125_000, help="training pairs kept per pair scene")
     p.add_argument("--finetune-steps", type=int, default=150)
     p.add_argument("--mlp-steps", type=int, default=400)
@@ -1133,8 +1133,8 @@ def initializer_experiment(args, w, K, cams, centre, G):
 def run_batch(args, ws, rank, local):
     """The batched multi-view step: 16 cameras of mixed resolution over one fan soup.
     One step = fan conversion, batch render of all views, L1 over all views, batch
-    adjoint and Adam, captured once in a CUDA graph and replayed; tile size, pending
-    buffer and list capacities come from the autotuner.  `value` = pixels of all views
+    adjoint and Adam, captured once in a CUDA graph and replayed; tile size and
+    list capacities come from the autotuner.  `value` = pixels of all views
     per second of the forward+backward step."""
     import torch
 
@@ -1153,7 +1153,7 @@ def run_batch(args, ws, rank, local):
     dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
     sh_host = sc.sh.view(np.int16) if sc.sh_bf16 else sc.sh
     G = [dev(sc.means), dev(sc.log_scales), dev(sc.quats), dev(sc.opacity), dev(sh_host)]
-    # without the autotuner the tile and pending buffer come from the command line
+    # without the autotuner the tile comes from the command line
     br = ms.BatchRenderer(sc.n, K, cams, ms.render_params(tile=args.tile, kbuf=args.kbuf)
                           if args.no_autotune else None)
     npx = br.n_pixels

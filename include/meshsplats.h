@@ -500,7 +500,8 @@ MS_API ms_status ms_mse(const float *img_rgba, const float *target_rgba, int64_t
 MS_API ms_status ms_fan_corrections(const float *xyz0, const float *alpha0, const float *xyz1, const float *alpha1,
                                     int64_t N, int32_t K, float *corr, void *stream);
 
-/* Candidates the autotuner times: tile in {8, 16, 32} x kbuf in {8, 16}. */
+/* Candidates of the autotuner: tile in {8, 16, 32} x kbuf in {8, 16}.  A tile's two candidates render the
+ * same way: the tile is timed once, and the second reports the first's figures. */
 #define MS_TUNE_CANDIDATES 6
 
 typedef struct {
@@ -516,7 +517,7 @@ typedef struct {
 
 /*
  * Autotuner of the batch render (no counterpart in the paper, whose renderer has fixed
- * settings).  For every candidate (tile edge, per-pixel buffer) it renders once to
+ * settings).  For every tile edge it renders once to
  * measure the (tile, fan) pair list and the fragment-record list, sets both capacities
  * to the measured length times (1 + headroom) (headroom >= 0; the "list capacity" of the
  * batch), then times `reps` (>= 1) forward+backward batch steps with CUDA events and

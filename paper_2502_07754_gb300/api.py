@@ -458,7 +458,7 @@ class BatchRenderer:
         raise _lib.MSError(_lib.MS_ERR_CAPACITY, "capacity did not converge")
 
     def autotune(self, xyz, rgb, alpha, reps=3, headroom=0.05, stream=None):
-        """Runs ms_batch_autotune (tile, pending buffer, list capacities) on this scene
+        """Runs ms_batch_autotune (tile, list capacities) on this scene
         and adopts the fastest candidate; returns the ms_tune_result."""
         flat = self.new_flat()
         dL = torch.full_like(flat, 1.0 / flat.numel())

@@ -1,5 +1,6 @@
-// ms_batch_autotune: picks the tile edge, the per-pixel pending buffer and the two list
-// capacities (tile-pair list, fragment-record list) of the batch render by measurement.
+// ms_batch_autotune: picks the tile edge and the two list capacities (tile-pair list,
+// fragment-record list) of the batch render by measurement.  The kbuf values of a tile render the same
+// way, so a tile is timed once and stands for both.
 //
 // Host code only.  Every candidate goes through the public batch entry points, so what
 // is timed is exactly what a caller runs.
@@ -57,6 +58,11 @@ extern "C" MS_API ms_status ms_batch_autotune(const float *xyz, const float *rgb
         ms_render_params p = b0;
         p.tile = 8 << (c / 2);
         p.kbuf = 8 << (c % 2);
+        if (c % 2) {
+            res->cand_ms[c] = res->cand_ms[c - 1];
+            res->cand_ws_bytes[c] = res->cand_ws_bytes[c - 1];
+            continue;
+        }
         res->cand_ms[c] = -1.0f;
         // measure the two list lengths; grow the capacities until a render fits
         bool settled = false;
