@@ -87,7 +87,6 @@ RenderLayout render_layout(int64_t n_fans, int K, const ms_camera *cams, int n_v
     RenderLayout L;
     memset(&L, 0, sizeof(L));
     L.tile = p.tile;
-    L.kbuf = p.kbuf;
     L.n_views = n_views;
     int64_t tiles = 0, npx = 0;
     for (int v = 0; v < n_views; ++v) {

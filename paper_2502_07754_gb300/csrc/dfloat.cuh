@@ -55,8 +55,6 @@ __device__ __forceinline__ dfl df_add(dfl a, dfl b) {
     return df_fast_two_sum(s.h, s.l);
 }
 
-__device__ __forceinline__ dfl df_sub(dfl a, dfl b) { return df_add(a, df_neg(b)); }
-
 // a + b with one two-sum of the high parts and the low parts added in binary32: error
 // O(u^2 (|a| + |b|)), enough wherever the result is not a near-total cancellation that
 // must keep its own full relative precision.
@@ -86,15 +84,6 @@ __device__ __forceinline__ dfl df_mul_f(dfl a, float b) {
     return df_fast_two_sum(p.h, p.l);
 }
 
-// a / b: a first quotient from the high parts, the residual a - q1 b in double-float,
-// and a correction quotient of the residual.
-__device__ __forceinline__ dfl df_div(dfl a, dfl b) {
-    const float q1 = __fdiv_rn(a.h, b.h);
-    const dfl r = df_sub(a, df_mul_f(b, q1));
-    const float q2 = __fdiv_rn(r.h, b.h);
-    return df_fast_two_sum(q1, q2);
-}
-
 // a / b from one reciprocal of b.h: q1 = a.h / b.h to a few units, the residual a - q1 b
 // from two FMAs (the high one exact or nearly so), and a correction quotient.
 __device__ __forceinline__ dfl df_div_rcp(dfl a, dfl b) {
@@ -114,11 +103,6 @@ __device__ __forceinline__ float df_round(dfl a) { return __fadd_rn(a.h, a.l); }
 __device__ __forceinline__ float df_floor(dfl a) {
     const float f = floorf(a.h);
     return (f == a.h && a.l < 0.0f) ? f - 1.0f : f;
-}
-
-// Dot product of a binary32 row r with a double-float vector (dx, dy, dz).
-__device__ __forceinline__ dfl df_dot3(const float *r, dfl dx, dfl dy, dfl dz) {
-    return df_add(df_add(df_mul_f(dx, r[0]), df_mul_f(dy, r[1])), df_mul_f(dz, r[2]));
 }
 
 }  // namespace ms

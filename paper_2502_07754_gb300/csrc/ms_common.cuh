@@ -177,11 +177,6 @@ __device__ __forceinline__ float dec_edge(float ex, float ey, float lx, float ly
     return __fsub_rn(__fmul_rn(ex, __fsub_rn(py, ly)), __fmul_rn(ey, __fsub_rn(px, lx)));
 }
 
-// Top-left acceptance of an oriented edge value E with direction (ex, ey).
-__device__ __forceinline__ bool edge_pass(float E, float ex, float ey) {
-    return E > 0.0f || (E == 0.0f && (ey < 0.0f || (ey == 0.0f && ex > 0.0f)));
-}
-
 // ---------------------------------------------------------------------------------
 // 32-byte records: one 256-bit access of sm_100-class GPUs, p 32-byte aligned.  Used where a pass waits
 // on its records (resolve and its adjoint: view of 200k fans 878 -> 862 us; splat fill); the fan fill's and

@@ -29,7 +29,7 @@ cudaError_t launch_mesh_build(const float *means, const float *log_scales, const
 // Render workspace layout (byte offsets from the workspace base, 256-byte aligned).
 // Tiles and pixels of all views form one index space (see ViewTable).
 struct RenderLayout {
-    int tile, n_views, n_tiles, tile_bits, depth_bits, key_bits, kbuf;
+    int tile, n_views, n_tiles, tile_bits, depth_bits, key_bits;
     int fan_bits;
     int tiles_x[kMaxViews], tile_base[kMaxViews];
     int64_t pix_base[kMaxViews];

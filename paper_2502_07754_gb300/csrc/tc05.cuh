@@ -142,17 +142,6 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *mbar, uint32_t parity, uint3
         if (mbar_try_wait(mbar, parity)) return true;
     return false;
 }
-// Expect `bytes` of bulk-copy data on the mbarrier (one arrival).
-__device__ __forceinline__ void mbar_expect_tx(uint64_t *mbar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(mbar)), "r"(bytes)
-                 : "memory");
-}
-// Bulk copy global -> shared through the TMA engine (16-byte aligned, size % 16 == 0),
-// completing `bytes` of transaction count on the mbarrier.
-__device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t bytes, uint64_t *mbar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(mbar)) : "memory");
-}
 
 }  // namespace tc
 }  // namespace ms
