@@ -54,8 +54,8 @@ __device__ __forceinline__ float polygon_pad(const float *p, const CamDev &c, fl
 // What bounds it: arithmetic (the double-float projection, two boundary vertices at a time: 83% of issue
 // slots busy).  16 views of 3M fans, K = 6, forward and adjoint: 16.93 -> 16.62 ms against one vertex at a time in
 // 48 registers; the pairs want 64 (four blocks an SM; with the 76 they would take, three, they gain nothing).
-// Blocks take virtual ids in start order; id = view * fan_blocks + fan block, so pairs
-// come out view by view and, within a view, in fan order.
+// Block = view * fan_blocks + fan block.  A block's pairs are contiguous and in fan order; the blocks' ranges come
+// in the order in which they reserve them.
 __global__ void __launch_bounds__(kBinThreads, 4) bin_kernel(const __grid_constant__ BinArgs a) {
     const float *__restrict__ xyz = a.xyz;
     const int64_t n_fans = a.n_fans;
@@ -133,7 +133,7 @@ __global__ void __launch_bounds__(kBinThreads, 4) bin_kernel(const __grid_consta
                 const DVert d = decide_vertex(cam, df_project(cam, p[3 * k], p[3 * k + 1], p[3 * k + 2]), ox, oy);
                 mnx = fminf(mnx, d.xs); mxx = fmaxf(mxx, d.xs);
                 mny = fminf(mny, d.ys); mxy = fmaxf(mxy, d.ys);
-                }
+            }
         }
         if (ntri_bad) atomicAdd(&s_culled, ntri_bad);
         if (a.splat && tmask) {   // (kept for the count pass in the third vertex)

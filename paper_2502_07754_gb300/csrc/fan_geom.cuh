@@ -17,9 +17,10 @@ struct FanRect {
 // together below 2^-21 of the bounds' width and height, < 0.07 + 0.03 px for anything in the
 // +-2^17 guard band -- and the absolute positions that binning takes its bounds from are
 // rounded by at most 2^-7 px there.  1/32 px plus 2^-20 of the extent exceeds both; a quarter
-// pixel is the most that any fan needs.  (A constant quarter pixel around fans of about a
-// pixel doubles the centres tested: 3M fans in 16 views, 160M tests and 55.6M pairs with it,
-// 96M and 42.4M with this one; the batch step 32.86 -> 28.81 ms.)
+// pixel is the most that any fan needs.  (The three lines' strips can meet further out only past
+// the tip of a sliver; a centre there is outside the triangle and is left out.  A constant quarter
+// pixel around fans of about a pixel doubles the centres tested: 3M fans in 16 views, 160M tests and
+// 55.6M pairs with it, 96M and 42.4M with this one; the batch step 32.86 -> 28.81 ms.)
 __device__ __forceinline__ float rect_margin(float mnx, float mxx, float mny, float mxy) {
     return fminf(0.25f, 0.03125f + 0x1p-20f * ((mxx - mnx) + (mxy - mny)));
 }

@@ -3,8 +3,8 @@
 // accumulators in tensor memory), standing in for part of the fine-tuning of Sec. 3 by
 // predicting per-vertex radial and log-opacity corrections of each fan.
 //
-//   inference  mlp_fwd_kernel: persistent CTAs of 512 threads (two per SM), one 128-row
-//              tile at a time: features -> X (smem) -> Z1 = X W1 (TMEM) -> H1 = bf16(gelu)
+//   inference  mlp_fwd_kernel: a persistent CTA of 1024 threads per SM with four 128-row
+//              tiles in flight, each: features -> X (smem) -> Z1 = X W1 (TMEM) -> H1 = bf16(gelu)
 //              (smem) -> Z2 -> H2 -> Z3 -> corrections (global FP32), or, fused, the
 //              conversion of each row's Gaussian with its corrections still in registers
 //              (the corrections never reach HBM).

@@ -25,7 +25,7 @@ constexpr uint32_t kSpinLimit = 1u << 20;   // polls before a bounded wait gives
 struct Status {
     unsigned long long pairs;        // pairs produced by binning
     unsigned long long culled;       // culled triangles
-    unsigned long long extra_passes; // pixel passes re-run after buffer overflow
+    unsigned long long extra_passes; // rounds of 32 fragments that pixels took beyond their first
     unsigned long long cap;          // pair capacity of the workspace
     unsigned int timeouts;           // bounded waits that expired
     unsigned int sort_ticket[8];     // virtual block ids of each sort pass (sort_u64)
