@@ -329,7 +329,7 @@ struct MtBounds {
 };
 __device__ __forceinline__ bool mt_may_hit(const RayF &r, const float P0[3], const float P1[3], const float P2[3],
                                            float tmin, float tmax, MtBounds &e) {
-    constexpr float kU = 64.0f * 0x1p-24f;
+    constexpr float kU = 64.0f * 0x1p-24f, kTiny = 0x1p-140f;
     float e1[3], e2[3], tv[3], E1[3], E2[3], TV[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
@@ -345,21 +345,22 @@ __device__ __forceinline__ bool mt_may_hit(const RayF &r, const float P0[3], con
     const float pv[3] = {d1 * e2[2] - d2 * e2[1], d2 * e2[0] - d0 * e2[2], d0 * e2[1] - d1 * e2[0]};
     const float PV[3] = {a1 * E2[2] + a2 * E2[1], a2 * E2[0] + a0 * E2[2], a0 * E2[1] + a1 * E2[0]};
     const float det = e1[0] * pv[0] + e1[1] * pv[1] + e1[2] * pv[2];
-    const float eDet = kU * (E1[0] * PV[0] + E1[1] * PV[1] + E1[2] * PV[2]);
+    // (below 2^-128 the products are rounded in units of 2^-149, above the margins: such triangles go to FP64)
+    const float eDet = fmaf(kU, E1[0] * PV[0] + E1[1] * PV[1] + E1[2] * PV[2], 0x1p-128f);
     e = MtBounds{eDet, 3.0e38f, 3.0e38f, 3.0e38f};   // (undetermined: all of it is left to FP64)
     if (!(fabsf(det) > eDet)) return true;
     const float sg = det > 0.0f ? 1.0f : -1.0f;
     const float U = tv[0] * pv[0] + tv[1] * pv[1] + tv[2] * pv[2];
-    const float eU = kU * (TV[0] * PV[0] + TV[1] * PV[1] + TV[2] * PV[2]);
+    const float eU = fmaf(kU, TV[0] * PV[0] + TV[1] * PV[1] + TV[2] * PV[2], kTiny);
     if (sg * U < -eU) return false;
     const float qv[3] = {tv[1] * e1[2] - tv[2] * e1[1], tv[2] * e1[0] - tv[0] * e1[2], tv[0] * e1[1] - tv[1] * e1[0]};
     const float QV[3] = {TV[1] * E1[2] + TV[2] * E1[1], TV[2] * E1[0] + TV[0] * E1[2], TV[0] * E1[1] + TV[1] * E1[0]};
     const float V = qv[0] * d0 + qv[1] * d1 + qv[2] * d2;
-    const float eV = kU * (QV[0] * a0 + QV[1] * a1 + QV[2] * a2);
+    const float eV = fmaf(kU, QV[0] * a0 + QV[1] * a1 + QV[2] * a2, kTiny);
     if (sg * V < -eV) return false;
     if (sg * (U + V - det) > eU + eV + eDet) return false;
     const float Tn = e2[0] * qv[0] + e2[1] * qv[1] + e2[2] * qv[2];
-    const float eT = kU * (E2[0] * QV[0] + E2[1] * QV[1] + E2[2] * QV[2]);
+    const float eT = fmaf(kU, E2[0] * QV[0] + E2[1] * QV[1] + E2[2] * QV[2], kTiny);
     const float t = Tn / det;
     const float dt = (eT + fabsf(t) * eDet) / (fabsf(det) - eDet) + kU * fabsf(t);
     e = MtBounds{eDet, eU, eV, eT};
