@@ -277,7 +277,7 @@ struct TraceArgs {
 };
 
 // A ray's crossing: `at` is the place of its barycentrics, which stay where they are while a pass sorts the
-// crossings (1.6M triangles at 800x800 without a light: 2.84 ms, 2.97 with all of a crossing moved).
+// crossings (moving all of it took 4% longer without a light).
 struct alignas(16) Hit {
     double t;
     int tri, at;
@@ -667,7 +667,7 @@ __device__ __forceinline__ void shadow_jobs(const TraceArgs &a, Jobs &J, WarpRin
 // block is one such warp and three more: it gathers its pixels' next crossings, all four trace
 // their segments to the light as one list, and it composites.  What bounds it: the waits on nodes, lanes at
 // different depths of the tree (18 of 32 active; a segment meets 187 nodes and 60 leaves), and the blocks with
-// the deepest pixels at the end.  1.6M triangles at 800x800: 5.9 ms without shadows, 39 ms with the 5.4M
+// the deepest pixels at the end.  1.6M triangles at 800x800: 5.1 ms without shadows, 39 ms with the 5.4M
 // segments; 41 and 148 ms for lanes that each took their triangles through the exact tests alone
 // (4.5 of 32 active); 62 ms with two warps for 8 x 8 pixels and their segments, whose deepest blocks left
 // two thirds of the chip idle; 218 ms for a thread that traced its own pixel's segments one after the other.
@@ -823,9 +823,12 @@ trace_kernel(const __grid_constant__ TraceArgs a) {
                 }
                 if (!walking) break;
             }
-            // the crossings that will be composited: up to the one that takes T below T_eps
-            {
+            // the crossings that will be composited: up to the one that takes T below T_eps (known once they are
+            // composited, where there are no segments to trace first)
+            n_use = nb;
+            if (SHADOWS) {
                 double Tn = T;
+                n_use = 0;
                 for (bool on = true; on && n_use < nb; ++n_use, on = !(Tn < a.T_eps)) {
                     const Hit &h = buf[n_use];
                     int64_t v[3];
@@ -885,6 +888,7 @@ trace_kernel(const __grid_constant__ TraceArgs a) {
             T *= 1.0 - al;
             after_t = h.t;
             after_i = h.tri;
+            if (!SHADOWS && T < a.T_eps) break;
         }
         alive = alive && more && !(T < a.T_eps);
         if (SHADOWS ? !__syncthreads_or(alive) : !__any_sync(0xffffffffu, alive)) break;
