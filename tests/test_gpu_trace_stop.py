@@ -64,3 +64,21 @@ def test_first_factor_and_first_crossing_count_whatever_the_bound():
     img = _trace(0.5, 2.0)
     assert np.abs(img[..., 3] - 0.75).max() <= 1e-6
     assert np.abs((img[..., 0] / (0.75 * 0.5) - 0.25) / 0.75 - 0.5).max() <= 1e-6
+
+
+def test_images_repeat_bit_for_bit():
+    """Blocks hand their segments out in any order; a coarse bound must not let that show."""
+    rng = np.random.default_rng(4)
+    n = 3000
+    xyz = (rng.uniform(-1, 1, (n, 1, 3)) + rng.normal(0, 0.15, (n, 3, 3))).astype(np.float32).reshape(-1, 3)
+    tris = np.arange(3 * n, dtype=np.int32).reshape(-1, 3)
+    X, I = dev(xyz), dev(tris)
+    rgb, a = dev(rng.uniform(0, 1, (3 * n, 3)).astype(np.float32)), dev(rng.uniform(0.05, 0.3, 3 * n).astype(np.float32))
+    cam = synthetic.make_camera((0.3, 0.4, 3.0), 200, 160)
+    rt = ms.RayTracer(n)
+    rt.build(X, I)
+    first = None
+    for _ in range(8):
+        img = rt.trace(X, rgb, a, cam, tris=I, light=(2.0, -1.5, 2.5), ambient=0.2, T_eps=0.05)
+        first = img.clone() if first is None else first
+        assert torch.equal(img, first)
