@@ -921,12 +921,12 @@ extern "C" MS_API ms_status ms_bvh_build(const float *xyz, const int32_t *tris, 
     const BvhLayout L = bvh_layout(T);
     if (!bvh || (reinterpret_cast<uintptr_t>(bvh) & 255) || bvh_bytes < L.total)
         return set_error(MS_ERR_INVALID, "BVH workspace NULL, misaligned or < %zu bytes", L.total);
-    if (T == 0) return MS_OK;
     cudaStream_t st = (cudaStream_t)stream;
     char *b = static_cast<char *>(bvh);
     cudaError_t e = cudaMemsetAsync(b, 0, L.nodes, st);   // status and bounds
-    if (e == cudaSuccess) e = cudaMemsetAsync(b + L.flags, 0, (size_t)T * 4, st);
+    if (e == cudaSuccess && T > 0) e = cudaMemsetAsync(b + L.flags, 0, (size_t)T * 4, st);
     if (e != cudaSuccess) return set_error(MS_ERR_CUDA, "memset: %s", cudaGetErrorString(e));
+    if (T == 0) return MS_OK;
     unsigned *bounds = reinterpret_cast<unsigned *>(b + L.bounds);
     bounds_init_kernel<<<1, 32, 0, st>>>(bounds);
     centroid_bounds_kernel<<<grid_of(T, kBvhThreads), kBvhThreads, 0, st>>>(xyz, tris, K, T, bounds);

@@ -42,3 +42,13 @@ def test_scene_of_no_and_of_one_triangle(T, light):
     assert np.abs(img.cpu().numpy() - ref).max() <= 1e-5
     if T:
         assert rt.status()[1] == 0
+
+
+@pytest.mark.parametrize("T", [0, 1])
+def test_status_after_a_build(T):
+    """The build clears the status word, whatever the memory held before, of an empty scene too."""
+    rt = ms.RayTracer(T, K=3)
+    rt.bvh.fill_(255)
+    xyz = dev(np.array([[-0.7, -0.6, 0.0], [0.8, -0.5, 0.1], [0.1, 0.9, -0.1]], np.float32))
+    rt.build(xyz, dev(np.array([[0, 1, 2]], np.int32)[:T]) if T else None)
+    assert rt.status() == (0, 0)
