@@ -129,7 +129,8 @@ typedef struct {
     int64_t pair_capacity;  /* capacity of the workspace */
     int64_t culled_tris;    /* triangles culled at the near plane / guard band */
     int64_t extra_passes;   /* rounds of 32 fragments that pixels took beyond their first */
-    int32_t overflow;       /* 1 if pairs or fragments exceed their capacity (image invalid) */
+    int32_t overflow;       /* 1 if pairs or fragments exceed their capacity (image invalid: pairs left out, and
+                               the background where a pixel's fragments found no room) */
     int32_t timeouts;       /* bounded waits that expired (image invalid) */
     int32_t sort_bits;      /* bits of a tile index (the key the pairs are ordered by) */
     int32_t n_tiles;
@@ -429,8 +430,8 @@ MS_API ms_status ms_batch_render_backward(const float *xyz, const float *rgb, co
  * the two kept unit axes u_a, u_b (axis_rule as in ms_fan_params) at local (u, v):
  * alpha = sigma exp(-(u^2/s_a^2 + v^2/s_b^2)/2), kept where (u/(2.7 s_a))^2 + (v/(2.7 s_b))^2
  * <= 1 (the ellipse the fan is inscribed in) and t > znear; colour rgb[g]; fragments of a
- * pixel ordered by (binary32 t, Gaussian index); compositing as in ms_render.  The hit
- * test runs in FP64.
+ * pixel ordered by (binary32 t, Gaussian index); compositing as in ms_render.  Hits and t
+ * are those of the FP64 test; alpha is within 2^-30 of its value before the last rounding.
  *   means N x 3, log_scales N x 3, quats N x 4 (w, x, y, z; 16-byte aligned), opacity N,
  *   rgb N x 3: device.  cams: host array of n_views cameras.  out_rgba: host array of
  *   n_views device images H_v x W_v x 4.  workspace >= ms_splat_workspace_size bytes.
